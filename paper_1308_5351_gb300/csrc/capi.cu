@@ -101,7 +101,7 @@ int check_prec(int prec) {
 // Frees the handle's device memory once every stream's work on it is done
 // (the device synchronisation that cudaFree would imply), back to the pool.
 void release(Boundary& b) {
-    void* ptrs[] = {b.arena, b.V, b.kry, b.kstate};
+    void* ptrs[] = {b.arena, b.V, b.kry, b.kstate, b.partial_x};
     bool any = b.fmm != nullptr;
     for (void* p : ptrs) any = any || p != nullptr;
     if (!any) return;
@@ -114,6 +114,8 @@ void release(Boundary& b) {
     b.V = nullptr;
     b.kry = nullptr;
     b.kstate = nullptr;
+    b.partial_x = nullptr;
+    b.partial_x_bytes = 0;
 }
 
 // Carves the handle's fixed-size buffers out of one device allocation
@@ -231,6 +233,7 @@ int build(Boundary& b, int m1, int n, const double* et, const double* etp, const
                          kSrcTile32);
     b.plandf = make_plan(b.N, b.sms, pair_blocks_per_sm(GNK_PREC_DF32), kThreadsDF * kTargetsDF,
                          kSrcTile32);
+    b.sym64 = make_sym_plan(b.N, b.sms);
     GNK_TRY(pair_workspace_bytes(b, &b.partial_bytes));
     // every fixed-size buffer of the handle lives in one device allocation
     Arena ar;

@@ -126,6 +126,13 @@ struct PairPlan {
     int tiles_per_chunk = 0;
 };
 
+// Node blocks of the FP64 kernel that takes each pair once (pairsum64_sym_kernel).
+struct SymPlan {
+    int W = 0;   // warps per block (0: the kernel is not used)
+    int G = 1;   // sub-tiles of 32 W nodes per node block
+    int nt = 0;  // node blocks
+};
+
 // Everything a launch of the pair-sum + reduce pipeline needs.
 struct PairJob {
     int R = 1;                    // right-hand sides
@@ -187,7 +194,8 @@ struct Boundary {
     size_t partial_bytes = 0;
     // source-chunk override of the direct pair kernels for the current call
     // (gnk_options.tile_chunks; 0: the plans below) and the larger partial-sum
-    // workspace it may need (from the memory pool, kept until the handle is freed)
+    // workspace that it or the FP64 kernel may need (from the memory pool, kept
+    // until the handle is freed)
     mutable int tile_chunks = 0;
     mutable void* partial_x = nullptr;
     mutable size_t partial_x_bytes = 0;
@@ -211,6 +219,7 @@ struct Boundary {
     double* means = nullptr;    // m1
     double* stage = nullptr;    // host-staging buffers: 4 x 2N doubles
     PairPlan plan64, plan32, plandf;
+    SymPlan sym64;
     int eone_prec = GNK_PREC_FP64;  // arithmetic of the precomputed sums
 
     // Krylov workspace (allocated on first solve, grown as needed)
@@ -223,6 +232,7 @@ struct Boundary {
 
 // ---------------------------------------------------------------- pair sums
 PairPlan make_plan(int N, int sms, int blocks_per_sm, int targets_per_block, int src_tile);
+SymPlan make_sym_plan(int N, int sms);
 int pair_workspace_bytes(const Boundary& b, size_t* bytes);
 int run_pairsum64(const Boundary& b, const PairJob& job, cudaStream_t st);
 int run_pairsum32(const Boundary& b, const PairJob& job, cudaStream_t st);

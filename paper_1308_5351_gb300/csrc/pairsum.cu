@@ -8,9 +8,11 @@
 // [chunk][rhs][N] buffer; a second kernel adds the chunks in a fixed order
 // (deterministic) in FP64 and applies the operator's epilogue.
 //
-// Per pair the FP64 kernel spends 13 FP64-pipe instructions:
+// Per pair the FP64 kernels spend 9 FP64-pipe instructions on 1/d:
 //   2 DADD (d = eta_i - eta_j), DMUL + DFMA (|d|^2), 3 DFMA to refine the
-//   hardware reciprocal seed, 2 DMUL (Re, Im of 1/d), 4 DFMA (w / d);
+//   hardware reciprocal seed, 2 DMUL (Re, Im of 1/d),
+// and 4 DFMA on w / d; the kernels that take each pair once share the 9 between
+// the pair's two directions (below);
 // the FP32 kernel spends 10 FP32-pipe instructions and one MUFU reciprocal;
 // the double-float kernel about 97 FP32-pipe instructions and one MUFU.
 #include <algorithm>
@@ -141,6 +143,285 @@ __global__ void __launch_bounds__(kThreads64) pairsum64_kernel(Pair64Args a) {
             for (int r = 0; r < R; ++r)
                 a.partial[((size_t)blockIdx.y * R + r) * N + idx[t]] = make_double2(ax[t][r], ay[t][r]);
         }
+    }
+}
+
+// ------------------------------------------------------------------ FP64, pairs taken once
+// 1/(eta_j - eta_i) = -1/(eta_i - eta_j): a pair's difference, |d|^2 and
+// reciprocal (9 of the 13 FP64 instructions) serve both directions.  The FP64
+// pipe (2 lanes per SM) bounds the sum, so per unordered pair the kernel spends
+//   9 + 8 R (both parts of z) or 9 + 4 (one part, R = 1)
+// instead of 2 (9 + 4 R).  A block takes one pair (I, J) of node blocks of SB =
+// 32 W G nodes (W >= 2).  A warp holds 32 targets (one per lane) and meets 32 sources in
+// 32 steps: in step k lane l takes source (l + k) mod 32, whose sum travels
+// with it, handed to the next lane by a shuffle (issue slots are free: an
+// FP64 instruction holds the pipe for 16 cycles).  Row sums stay in registers,
+// column sums in shared memory between the warps' turns (warp w takes the
+// 32 sources of slice (w + s) mod W in turn s: no two warps share a slice, and
+// the order is fixed).  Block (I, J) writes I's sums to slot J and J's to slot
+// I, so every node gets nt partial sums, added by the reduction in slot order.
+// Measured: (D - diag(D1) + Lhat) x at N = 16,000, real A, 6.15 -> 3.00 ms
+// (90 % of the pipe's rate for 13 instructions per unordered pair).
+struct Pair64SymArgs {
+    const double2* et;
+    int N;
+    const double2* w0;
+    const double2* w1;
+    const double* x0;
+    const double* x1;
+    const double2* s;
+    double2* partial;  // [slot][rhs][N]
+    int nt;            // node blocks
+    int G;             // sub-tiles of 32 W nodes per node block
+    const int* done;
+};
+
+template <int R, int MODE>
+__device__ __forceinline__ void load_node64(const Pair64SymArgs& a, int j, double2& pos, double2 (&w)[R]) {
+    if (j < a.N) {
+        pos = a.et[j];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            if (MODE == W_COMPLEX) {
+                w[r] = (r == 0) ? a.w0[j] : a.w1[j];
+            } else {
+                const double2 sc = a.s[j];
+                const double x = (r == 0) ? a.x0[j] : a.x1[j];
+                w[r] = make_double2(sc.x * x, sc.y * x);
+            }
+        }
+    } else {
+        pos = make_double2(kFar64, kFar64);
+#pragma unroll
+        for (int r = 0; r < R; ++r) w[r] = make_double2(0.0, 0.0);
+    }
+}
+
+// acc += sign * (the wanted parts of w (ar - i ai)); COMP 0: both, 1: Im, 2: Re
+template <int COMP, bool NEG>
+__device__ __forceinline__ void add_term64(double* acc, double2 w, double ar, double ai) {
+    const double wx = NEG ? -w.x : w.x, wy = NEG ? -w.y : w.y;
+    if (COMP != 1) {
+        acc[0] = fma(wx, ar, acc[0]);
+        acc[0] = fma(wy, ai, acc[0]);
+    }
+    if (COMP != 2) {
+        double& im = acc[COMP == 0 ? 1 : 0];
+        im = fma(wy, ar, im);
+        im = fma(-wx, ai, im);
+    }
+}
+
+// Pair t of node blocks: (I, I + o mod nt) for the full offsets o, the half
+// offset of an even nt, then the diagonal (half the work: last).
+__device__ __forceinline__ void sym_blocks(int nt, int t, int& I, int& J) {
+    const int off = nt * (nt - 1) / 2;
+    if (t < off) {
+        const int o = t / nt + 1;
+        I = t - (o - 1) * nt;
+        J = I + o;
+        if (J >= nt) J -= nt;
+    } else {
+        I = J = t - off;
+    }
+}
+
+template <int R, int MODE, int COMP, int W>
+__global__ void __launch_bounds__(32 * W) pairsum64_sym_kernel(Pair64SymArgs a) {
+    constexpr int NC = COMP == 0 ? 2 : 1;  // parts of z kept
+    constexpr int NT = 32 * W;
+    extern __shared__ __align__(16) double s_dyn64[];
+    double2* s_pos = reinterpret_cast<double2*>(s_dyn64);  // [NT]
+    double2* s_w = s_pos + NT;                             // [R][NT]
+    double* s_col = reinterpret_cast<double*>(s_w + R * NT);  // [R][NC][SB]
+    if (a.done != nullptr && *a.done) return;
+    const int SB = NT * a.G;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int I, J;
+    sym_blocks(a.nt, blockIdx.x, I, J);
+    const bool diag = I == J;
+    for (int e = threadIdx.x; e < R * NC * SB; e += NT) s_col[e] = 0.0;
+    for (int gi = 0; gi < a.G; ++gi) {
+        const int i = I * SB + gi * NT + threadIdx.x;
+        if (I * SB + gi * NT >= a.N) break;
+        double2 p, w[R];
+        load_node64<R, MODE>(a, i, p, w);
+        double acc[R][NC];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) acc[r][c] = 0.0;
+        for (int gj = diag ? gi : 0; gj < a.G; ++gj) {
+            const int j0 = J * SB + gj * NT;
+            if (j0 >= a.N) break;
+            __syncthreads();  // the previous sub-tile is done with s_pos, s_w
+            {
+                double2 pj, wj[R];
+                load_node64<R, MODE>(a, j0 + threadIdx.x, pj, wj);
+                s_pos[threadIdx.x] = pj;
+#pragma unroll
+                for (int r = 0; r < R; ++r) s_w[r * NT + threadIdx.x] = wj[r];
+            }
+            const bool self = diag && gj == gi;
+            const int turns = self ? W / 2 + 1 : W;  // a sub-tile with itself: each slice pair once
+            for (int s = 0; s < turns; ++s) {
+                __syncthreads();
+                const int c = (wid + s) & (W - 1);  // W is a power of two
+                if (self && s == 0) {  // the slice with itself: every ordered pair by its own row
+#pragma unroll 4
+                    for (int k = 0; k < 32; ++k) {
+                        const int q = c * 32 + k;
+                        const double2 sp = s_pos[q];
+                        const double dx = p.x - sp.x, dy = p.y - sp.y;
+                        double inv = recip_f64(fma(dx, dx, dy * dy));
+                        inv = (k == lane) ? 0.0 : inv;  // the i = j term is excluded (Eq. fmm-E)
+                        const double ar = dx * inv, ai = dy * inv;
+#pragma unroll
+                        for (int r = 0; r < R; ++r) add_term64<COMP, false>(acc[r], s_w[r * NT + q], ar, ai);
+                    }
+                    continue;
+                }
+                if (self && s == W / 2 && wid >= W / 2) continue;  // the other warp of the slice pair has it
+                double col[R][NC];
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int q = 0; q < NC; ++q) col[r][q] = s_col[(r * NC + q) * SB + gj * NT + c * 32 + lane];
+#pragma unroll 4
+                for (int k = 0; k < 32; ++k) {
+                    const int q = c * 32 + ((lane + k) & 31);
+                    const double2 sp = s_pos[q];
+                    const double dx = p.x - sp.x, dy = p.y - sp.y;
+                    const double inv = recip_f64(fma(dx, dx, dy * dy));
+                    const double ar = dx * inv, ai = dy * inv;  // 1/d = ar - i ai
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        add_term64<COMP, false>(acc[r], s_w[r * NT + q], ar, ai);
+                        add_term64<COMP, true>(col[r], w[r], ar, ai);  // 1/(eta_j - eta_i) = -1/d
+#pragma unroll
+                        for (int u = 0; u < NC; ++u) col[r][u] = __shfl_sync(0xffffffffu, col[r][u], (lane + 1) & 31);
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int u = 0; u < NC; ++u) s_col[(r * NC + u) * SB + gj * NT + c * 32 + lane] = col[r][u];
+            }
+        }
+        if (diag) {  // with the column sums of the same nodes
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int u = 0; u < NC; ++u) s_col[(r * NC + u) * SB + gi * NT + threadIdx.x] += acc[r][u];
+        } else if (i < a.N) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                a.partial[((size_t)J * R + r) * a.N + i] = make_double2(COMP == 1 ? 0.0 : acc[r][0],
+                                                                        COMP == 2 ? 0.0 : acc[r][NC - 1]);
+        }
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < SB; e += NT) {
+        const int j = J * SB + e;
+        if (j >= a.N) break;
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            a.partial[((size_t)I * R + r) * a.N + j] = make_double2(COMP == 1 ? 0.0 : s_col[(r * NC) * SB + e],
+                                                                    COMP == 2 ? 0.0 : s_col[(r * NC + NC - 1) * SB + e]);
+    }
+}
+
+// The same for blocks of 32 nodes, the 32 steps of a pair of blocks shared by
+// kSymSplit warps (warp v takes the steps from 32 v / kSymSplit on), whose row
+// and column sums are added in warp order.  At N = 768 an SM has two such
+// pairs: with one warp each the FP64 pipe waits for the 64-cycle latency of
+// dependent instructions (a product through the C ABI 30 us), with four it is
+// busy (20 us; the kernel 8.4 us, 0.96 of the pipe's rate; the ordered kernel
+// on 18 SMs took 82 to 125 us).
+constexpr int kSymSplit = 4;
+
+template <int R, int MODE, int COMP>
+__global__ void __launch_bounds__(32 * kSymSplit) pairsum64_sym32_kernel(Pair64SymArgs a) {
+    constexpr int NC = COMP == 0 ? 2 : 1, KS = 32 / kSymSplit;
+    __shared__ double2 s_pos[32], s_w[R][32];
+    __shared__ double s_row[kSymSplit][R * NC][32], s_col[kSymSplit][R * NC][32];
+    if (a.done != nullptr && *a.done) return;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int I, J;
+    sym_blocks(a.nt, blockIdx.x, I, J);
+    const int i = I * 32 + lane, j = J * 32 + lane;
+    double2 p, w[R];
+    load_node64<R, MODE>(a, i, p, w);
+    if (wid == 0) {
+        double2 pj = p, wj[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) wj[r] = w[r];
+        if (I != J) load_node64<R, MODE>(a, j, pj, wj);
+        s_pos[lane] = pj;
+#pragma unroll
+        for (int r = 0; r < R; ++r) s_w[r][lane] = wj[r];
+    }
+    __syncthreads();
+    double acc[R][NC], col[R][NC];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int u = 0; u < NC; ++u) acc[r][u] = col[r][u] = 0.0;
+    const int k0 = wid * KS;
+    if (I == J) {  // every ordered pair by its own row
+#pragma unroll
+        for (int k = k0; k < k0 + KS; ++k) {
+            const double2 sp = s_pos[k];
+            const double dx = p.x - sp.x, dy = p.y - sp.y;
+            double inv = recip_f64(fma(dx, dx, dy * dy));
+            inv = (k == lane) ? 0.0 : inv;  // the i = j term is excluded (Eq. fmm-E)
+            const double ar = dx * inv, ai = dy * inv;
+#pragma unroll
+            for (int r = 0; r < R; ++r) add_term64<COMP, false>(acc[r], s_w[r][k], ar, ai);
+        }
+    } else {
+#pragma unroll
+        for (int k = k0; k < k0 + KS; ++k) {
+            const int q = (lane + k) & 31;
+            const double2 sp = s_pos[q];
+            const double dx = p.x - sp.x, dy = p.y - sp.y;
+            const double inv = recip_f64(fma(dx, dx, dy * dy));
+            const double ar = dx * inv, ai = dy * inv;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                add_term64<COMP, false>(acc[r], s_w[r][q], ar, ai);
+                add_term64<COMP, true>(col[r], w[r], ar, ai);
+#pragma unroll
+                for (int u = 0; u < NC; ++u) col[r][u] = __shfl_sync(0xffffffffu, col[r][u], (lane + 1) & 31);
+            }
+        }
+    }
+    const int held = (lane + k0 + KS) & 31;  // the source whose sum this lane holds now
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int u = 0; u < NC; ++u) {
+            s_row[wid][r * NC + u][lane] = acc[r][u];
+            s_col[wid][r * NC + u][held] = col[r][u];
+        }
+    __syncthreads();
+    // warp 0: row sums to slot J; warp 1: column sums to slot I
+    if (wid > (I != J ? 1 : 0)) return;
+    const int node = wid == 0 ? i : j;
+    if (node >= a.N) return;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        double v[NC];
+#pragma unroll
+        for (int u = 0; u < NC; ++u) {
+            const double(*src)[R * NC][32] = wid == 0 ? s_row : s_col;
+            v[u] = src[0][r * NC + u][lane];
+#pragma unroll
+            for (int q = 1; q < kSymSplit; ++q) v[u] += src[q][r * NC + u][lane];
+        }
+        a.partial[((size_t)(wid == 0 ? J : I) * R + r) * a.N + node] =
+            make_double2(COMP == 1 ? 0.0 : v[0], COMP == 2 ? 0.0 : v[NC - 1]);
     }
 }
 
@@ -672,38 +953,57 @@ __global__ void __launch_bounds__(kThreadsDF) pairsumdf2_kernel(PairDFArgs a) {
 }
 
 // ------------------------------------------------------------------ reduce + epilogue
-__global__ void reduce_epilogue_kernel(ReduceArgs a) {
+// Adds the partial sums of 32 nodes per block and applies the operator's
+// epilogue: warp g takes the chunks g, g + 8, ... (coalesced over the nodes,
+// all loads independent), then the eight sums are added in order by warp 0.
+// Latency bounds it (one thread per node read its chunks one after the other).
+constexpr int kReduceGroups = 8;
+
+__global__ void __launch_bounds__(32 * kReduceGroups) reduce_epilogue_kernel(ReduceArgs a) {
     const PairJob& j = a.job;
+    __shared__ double2 s_sum[kMaxRHS][kReduceGroups][32];
     if (j.done != nullptr && *j.done) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.N) return;
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
     const int N = a.N;
-    double zx[kMaxRHS] = {0.0, 0.0}, zy[kMaxRHS] = {0.0, 0.0};
     for (int r = 0; r < a.R; ++r) {
         double sx = 0.0, sy = 0.0;
-        if (a.ptype == 1) {
-            for (int ch = 0; ch < a.chunks; ++ch) {
-                const float2 p = a.p32[((size_t)ch * a.R + r) * N + i];
-                sx += (double)p.x;
-                sy += (double)p.y;
-            }
-        } else if (a.ptype == 2) {
-            for (int ch = 0; ch < a.chunks; ++ch) {
-                const float4 p = a.pdf[((size_t)ch * a.R + r) * N + i];
-                sx += (double)p.x + (double)p.y;
-                sy += (double)p.z + (double)p.w;
-            }
-        } else {
-            for (int ch = 0; ch < a.chunks; ++ch) {
-                const double2 p = a.p64[((size_t)ch * a.R + r) * N + i];
-                sx += p.x;
-                sy += p.y;
+        if (i < N) {
+            if (a.ptype == 1) {
+#pragma unroll 4
+                for (int ch = g; ch < a.chunks; ch += kReduceGroups) {
+                    const float2 p = a.p32[((size_t)ch * a.R + r) * N + i];
+                    sx += (double)p.x;
+                    sy += (double)p.y;
+                }
+            } else if (a.ptype == 2) {
+#pragma unroll 4
+                for (int ch = g; ch < a.chunks; ch += kReduceGroups) {
+                    const float4 p = a.pdf[((size_t)ch * a.R + r) * N + i];
+                    sx += (double)p.x + (double)p.y;
+                    sy += (double)p.z + (double)p.w;
+                }
+            } else {
+#pragma unroll 8
+                for (int ch = g; ch < a.chunks; ch += kReduceGroups) {
+                    const double2 p = a.p64[((size_t)ch * a.R + r) * N + i];
+                    sx += p.x;
+                    sy += p.y;
+                }
             }
         }
-        zx[r] = sx;
-        zy[r] = sy;
+        s_sum[r][g][lane] = make_double2(sx, sy);
     }
-    epilogue_apply(a, i, make_double2(zx[0], zy[0]), make_double2(zx[1], zy[1]));
+    __syncthreads();
+    if (g != 0 || i >= N) return;
+    double2 z[kMaxRHS] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
+    const int ng = min(kReduceGroups, a.chunks);
+    for (int r = 0; r < a.R; ++r)
+        for (int q = 0; q < ng; ++q) {
+            z[r].x += s_sum[r][q][lane].x;
+            z[r].y += s_sum[r][q][lane].y;
+        }
+    epilogue_apply(a, i, z[0], z[1]);
 }
 
 cudaError_t launch_reduce(const Boundary& b, const PairJob& job, int chunks, int ptype,
@@ -714,9 +1014,8 @@ cudaError_t launch_reduce(const Boundary& b, const PairJob& job, int chunks, int
         ra.p64 = static_cast<const double2*>(partial);
         ra.p32 = static_cast<const float2*>(partial);
     }
-    const int threads = 256;
     const ProfToken tok = prof_begin(st, PK_REDUCE);
-    reduce_epilogue_kernel<<<(b.N + threads - 1) / threads, threads, 0, st>>>(ra);
+    reduce_epilogue_kernel<<<(b.N + 31) / 32, 32 * kReduceGroups, 0, st>>>(ra);
     const cudaError_t e = cudaGetLastError();
     // bytes: the partials read plus about four N-vectors of operands and output
     prof_end(tok, PK_REDUCE,
@@ -753,11 +1052,65 @@ PairPlan make_plan(int N, int sms, int blocks_per_sm, int targets_per_block, int
     return p;
 }
 
+// Node blocks of the FP64 kernel that takes each pair once: SB = 32 W G nodes,
+// the size whose estimated time (FP64 pipe work of the busiest SM, then the
+// partial sums written and read at about 4 TB/s) is least, at most kSymMaxBlocks
+// of them (they give 8,256 pairs of blocks, 54 per SM, and 2 KB of partial
+// sums per node and right-hand side); none (W = 0) beyond 524,288 nodes.  Small
+// domains take 32-node blocks of one warp (N = 768: 300 blocks instead of the
+// 18 of the ordered kernel).
+constexpr int kSymMaxBlocks = 128;
+constexpr size_t kSymArenaBytes = (size_t)64 << 20;
+
+SymPlan make_sym_plan(int N, int sms) {
+    static const int kShape[][2] = {{1, 1}, {2, 1}, {4, 1}, {8, 1}, {8, 2}, {8, 4}, {8, 8}, {8, 16}};
+    SymPlan best;
+    double best_t = 0.0;
+    for (const auto& sh : kShape) {
+        const long long SB = 32LL * sh[0] * sh[1], nt = (N + SB - 1) / SB;
+        if (nt > kSymMaxBlocks) continue;
+        const double blocks = 0.5 * nt * (nt - 1) + 0.5 * nt;  // the diagonal's blocks are half
+        const double rounds = std::ceil(blocks / std::max(1, sms));
+        const double t = rounds * (double)SB * SB * 17.0 / 4.1e9 + (double)nt * N * 32.0 / 4e12;
+        if (best.W == 0 || t < best_t) {
+            best_t = t;
+            best.W = sh[0];
+            best.G = sh[1];
+            best.nt = (int)nt;
+        }
+    }
+    return best;
+}
+
 int pair_workspace_bytes(const Boundary& b, size_t* bytes) {
     const size_t b64 = (size_t)b.plan64.chunks * kMaxRHS * b.N * sizeof(double2);
     const size_t b32 = (size_t)b.plan32.chunks * kMaxRHS * b.N * sizeof(float2);
     const size_t bdf = (size_t)b.plandf.chunks * kMaxRHS * b.N * sizeof(float4);
     *bytes = std::max(std::max(b64, b32), bdf);
+    // the sums of the kernel that takes each pair once, where they are small
+    // (larger ones come from the pool with the first FP64 product)
+    const size_t bs = (size_t)b.sym64.nt * kMaxRHS * b.N * sizeof(double2);
+    if (b.sym64.W > 0 && bs <= kSymArenaBytes) *bytes = std::max(*bytes, bs);
+    return GNK_OK;
+}
+
+// Partial-sum workspace of `need` bytes: the handle's own, or one from the pool
+// that is kept (and grown) with the handle.
+static int partial_workspace(const Boundary& b, size_t need, void** partial, cudaStream_t st) {
+    *partial = b.partial;
+    if (need <= b.partial_bytes) return GNK_OK;
+    if (need > b.partial_x_bytes) {
+        if (b.partial_x) pool_free(b.partial_x, st);
+        b.partial_x = nullptr;
+        b.partial_x_bytes = 0;
+        if (pool_alloc(&b.partial_x, need, st) != cudaSuccess) {
+            cudaGetLastError();
+            set_error("pair-sum workspace of %zu bytes: allocation failed", need);
+            return GNK_ENOMEM;
+        }
+        b.partial_x_bytes = need;
+    }
+    *partial = b.partial_x;
     return GNK_OK;
 }
 
@@ -772,24 +1125,92 @@ static int launch_plan(const Boundary& b, const PairPlan& base, size_t elem_byte
     const int want = std::min(b.tile_chunks, p->tiles_src);
     p->tiles_per_chunk = (p->tiles_src + want - 1) / want;
     p->chunks = (p->tiles_src + p->tiles_per_chunk - 1) / p->tiles_per_chunk;
-    const size_t need = (size_t)p->chunks * kMaxRHS * b.N * elem_bytes;
-    if (need <= b.partial_bytes) return GNK_OK;
-    if (need > b.partial_x_bytes) {
-        if (b.partial_x) pool_free(b.partial_x, st);
-        b.partial_x = nullptr;
-        b.partial_x_bytes = 0;
-        if (pool_alloc(&b.partial_x, need, st) != cudaSuccess) {
-            cudaGetLastError();
-            set_error("pair-sum workspace for %d source chunks: allocation failed", p->chunks);
-            return GNK_ENOMEM;
-        }
-        b.partial_x_bytes = need;
+    return partial_workspace(b, (size_t)p->chunks * kMaxRHS * b.N * elem_bytes, partial, st);
+}
+
+template <int R, int MODE, int COMP, int W>
+static cudaError_t launch_sym64(const Pair64SymArgs& a, cudaStream_t st) {
+    constexpr int NT = 32 * W;
+    const int SB = NT * a.G;
+    const size_t smem = (size_t)NT * (1 + R) * sizeof(double2) + (size_t)R * (COMP == 0 ? 2 : 1) * SB * sizeof(double);
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(pairsum64_sym_kernel<R, MODE, COMP, W>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
     }
-    *partial = b.partial_x;
+    pairsum64_sym_kernel<R, MODE, COMP, W><<<a.nt * (a.nt + 1) / 2, NT, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+template <int R, int MODE, int COMP>
+static cudaError_t launch_sym64_w(int W, const Pair64SymArgs& a, cudaStream_t st) {
+    switch (W) {
+        case 1:
+            pairsum64_sym32_kernel<R, MODE, COMP><<<a.nt * (a.nt + 1) / 2, 32 * kSymSplit, 0, st>>>(a);
+            return cudaGetLastError();
+        case 2: return launch_sym64<R, MODE, COMP, 2>(a, st);
+        case 4: return launch_sym64<R, MODE, COMP, 4>(a, st);
+        default: return launch_sym64<R, MODE, COMP, 8>(a, st);
+    }
+}
+
+// The FP64 sum with each pair taken once.  *ran = false where the ordered kernel
+// serves the call: a source-chunk override, more than 524,288 nodes, or
+// a capturing stream before the handle owns the workspace (an allocation
+// captured into a graph would not outlive it).
+static int run_pairsum64_sym(const Boundary& b, const PairJob& job, cudaStream_t st, bool* ran) {
+    *ran = false;
+    const SymPlan& p = b.sym64;
+    if (p.W == 0 || b.tile_chunks > 0) return GNK_OK;
+    const size_t need = (size_t)p.nt * job.R * b.N * sizeof(double2);
+    if (need > b.partial_bytes && need > b.partial_x_bytes) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        GNK_TRY_CUDA(cudaStreamIsCapturing(st, &cs));
+        if (cs != cudaStreamCaptureStatusNone) return GNK_OK;
+    }
+    void* partial = nullptr;
+    GNK_TRY(partial_workspace(b, need, &partial, st));
+    Pair64SymArgs a;
+    a.et = b.et;
+    a.N = b.N;
+    a.w0 = job.w[0];
+    a.w1 = job.w[1];
+    a.x0 = job.x[0];
+    a.x1 = job.x[1];
+    a.s = job.s;
+    a.partial = static_cast<double2*>(partial);
+    a.nt = p.nt;
+    a.G = p.G;
+    a.done = job.done;
+    const ProfToken tok = prof_begin(st);
+    cudaError_t e;
+    if (job.R == 1 && job.mode == W_SCALED && job.comp == 1)
+        e = launch_sym64_w<1, W_SCALED, 1>(p.W, a, st);
+    else if (job.R == 1 && job.mode == W_SCALED && job.comp == 2)
+        e = launch_sym64_w<1, W_SCALED, 2>(p.W, a, st);
+    else if (job.R == 1 && job.mode == W_SCALED)
+        e = launch_sym64_w<1, W_SCALED, 0>(p.W, a, st);
+    else if (job.R == 1)
+        e = launch_sym64_w<1, W_COMPLEX, 0>(p.W, a, st);
+    else if (job.mode == W_SCALED)
+        e = launch_sym64_w<2, W_SCALED, 0>(p.W, a, st);
+    else
+        e = launch_sym64_w<2, W_COMPLEX, 0>(p.W, a, st);
+    GNK_TRY_CUDA(e);
+    // FP64 pipe per unordered pair: 9 (d, |d|^2, reciprocal, 1/d) and per
+    // right-hand side and direction 4 (one part of z: 2)
+    const double per_pair = 9.0 + ((job.comp && job.R == 1) ? 4.0 : 8.0 * job.R);
+    prof_end(tok, PK_PAIR64, (double)job.R * b.N * (b.N - 1.0), st, 0.5 * per_pair * b.N * (b.N - 1.0));
+    GNK_TRY_CUDA(launch_reduce(b, job, p.nt, 0, st, partial));
+    count_launches(2);
+    *ran = true;
     return GNK_OK;
 }
 
 int run_pairsum64(const Boundary& b, const PairJob& job, cudaStream_t st) {
+    bool ran = false;
+    GNK_TRY(run_pairsum64_sym(b, job, st, &ran));
+    if (ran) return GNK_OK;
     PairPlan p;
     void* partial = nullptr;
     GNK_TRY(launch_plan(b, b.plan64, sizeof(double2), &p, &partial, st));

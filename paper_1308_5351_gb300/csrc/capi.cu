@@ -381,10 +381,11 @@ int gnk_build_boundary_ex(gnk_boundary** out, int m1, int n, const double* et, c
                           int precision, void* stream) {
     const int defer = (precision & GNK_BUILD_DEFER) ? 1 : 0;
     const int plain = (precision & GNK_BUILD_PLAIN) ? 1 : 0;
-    precision &= ~(GNK_BUILD_DEFER | GNK_BUILD_PLAIN);
+    const int diff = (precision & GNK_BUILD_DIFF) ? 1 : 0;
+    precision &= ~(GNK_BUILD_DEFER | GNK_BUILD_PLAIN | GNK_BUILD_DIFF);
     if (precision != GNK_PREC_FP64 && precision != GNK_PREC_DF32 && precision != GNK_PREC_FMM) {
         set_error("gnk_build_boundary_ex: precision must be GNK_PREC_FP64, GNK_PREC_DF32 or "
-                  "GNK_PREC_FMM (optionally | GNK_BUILD_DEFER | GNK_BUILD_PLAIN)");
+                  "GNK_PREC_FMM (optionally | GNK_BUILD_DEFER | GNK_BUILD_PLAIN | GNK_BUILD_DIFF)");
         return GNK_EINVAL;
     }
     if (plain && !etpp) {
@@ -410,6 +411,7 @@ int gnk_build_boundary_ex(gnk_boundary** out, int m1, int n, const double* et, c
         set_error("host allocation failed");
         return GNK_ENOMEM;
     }
+    h->b.diff = diff;
     const int s = build(h->b, m1, n, et, etp, etpp, A, Ap, bounded, precision, defer, plain,
                         (cudaStream_t)stream);
     if (s != GNK_OK) {

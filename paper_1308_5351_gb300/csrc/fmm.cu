@@ -33,6 +33,7 @@
 // nodes on average, interaction and neighbour lists.  Every sum on the device
 // runs in a fixed order, so results are reproducible.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <complex>
 #include <cstdint>
@@ -93,6 +94,7 @@ struct FmmArgs {
     const int* node_box;  // leaf box of each node in sorted order
     int* ucnt;            // per box: children counted in the upward pass
     float2* xs;           // [R][N] x in sorted order as double-float (cached near field), or null
+    int near_scaled;      // zn holds the near field times the operator's factor (cached)
     const float4* tp;     // [N][P] powers t^k of every node about its leaf centre, or null
     int* fault;           // set by a bounded wait that gave up
 };
@@ -476,7 +478,6 @@ __global__ void __launch_bounds__(32) fmm_l2l_kernel(FmmArgs a) {
 }
 
 constexpr int kFmmWarps = kFmmNT / 32;
-constexpr int kFmmMaxNbr = 9;  // a leaf and its eight neighbours
 
 // Near field: one block per chunk of up to 32 targets of a leaf (lane = target).
 // The sources of the (at most nine) neighbour leaves, taken as one list in
@@ -683,49 +684,58 @@ __global__ void fmm_tp_build_kernel(FmmArgs a, float4* __restrict__ tp) {
     }
 }
 
-// ---- Near-field operator cache.  The geometry of a handle is fixed for all
-// its products, so the near-field part of z = E(q x), the matrix
-//   Q_ij = q_j / (eta_i - eta_j)   (i = j: 0)
+// ---- Near-field operator caches.  The geometry of a handle is fixed for all
+// its products, so the near-field part of an operator, the matrix
+//   f_i w_j / (eta_i - eta_j)   (i = j: 0)
 // over each work item's targets i (a chunk of tn <= 32 nodes of a leaf) and
 // sources j (the nodes of its neighbour leaves, in neighbour order), is
 // formed once, in double-float from the exact three-float coordinates like
 // the near-field kernel above, and each product then only reads it:
-//   z_i = sum_j x_j Q_ij.
+//   f_i z_i = sum_j x_j f_i w_j / (eta_i - eta_j).
+// (w, f) = (q, A) for the products z = E(q x), whose operators read A z, and
+// (A, q) for the solves with z = E(A x), whose operators read Im(q z).  With
+// the target's factor inside, an operator that needs one part of f z reads one
+// part of the cache, 8 bytes per pair, whether or not f is real.
 // Layout per item, for source pairs p = (2p, 2p + 1) and targets (lanes):
-//   nq_re[off + p tn + lane] = (Re Q hi of 2p, of 2p+1, Re Q lo of 2p, of 2p+1)
-// and nq_im likewise, so a float4 load gives the packed double-float operand
-// of the two sources.  A product that needs only Im z (f_B with real A)
-// reads nq_im alone: 8 bytes per pair.
+//   re[off + p tn + lane] = (Re hi of 2p, of 2p+1, Re lo of 2p, of 2p+1)
+// and im likewise, so a float4 load gives the packed double-float operand
+// of the two sources.
 
-// S (near sources) and tn (targets) of work item `it`; s_beg/s_cum (when
-// given) receive the first source and the running count of each neighbour leaf.
-__device__ __forceinline__ void nq_item_shape(const FmmArgs& a, int it, int* S, int* tn, int* s_beg, int* s_cum,
-                                              int* nn_out) {
-    const int2 item = a.items[it];
-    const int leaf = item.x;
-    *tn = min(32, a.leaf_start[leaf + 1] - item.y);
-    const int n0 = a.nl_start[leaf], nn = min(a.nl_start[leaf + 1] - n0, kFmmMaxNbr);
-    int c = 0;
-    for (int e = 0; e < nn; ++e) {
-        const int nl = a.nl_leaf[n0 + e];
-        if (s_beg) {
-            s_beg[e] = a.leaf_start[nl];
-            s_cum[e] = c;
-        }
-        c += a.leaf_start[nl + 1] - a.leaf_start[nl];
-    }
-    if (s_cum) s_cum[nn] = c;
-    *S = c;
-    if (nn_out) *nn_out = nn;
-}
-
-__global__ void fmm_nq_count_kernel(FmmArgs a, long long* cnt, long long* scnt) {
+// The shape of every work item: S sources, tn targets, the entries, and the
+// run of sorted nodes that each of its neighbour leaves is.
+__global__ void fmm_nq_shape_kernel(FmmArgs a, long long* cnt, int2* nq_item, int2* nq_run) {
     const int it = blockIdx.x * blockDim.x + threadIdx.x;
     if (it >= a.nitems) return;
-    int S, tn;
-    nq_item_shape(a, it, &S, &tn, nullptr, nullptr, nullptr);
-    cnt[it] = (long long)((S + 1) / 2) * tn;
-    scnt[it] = S + (S & 1);  // lists padded to even length (16-byte aligned chunks of x)
+    const int2 item = a.items[it];
+    const int leaf = item.x;
+    const int tn = min(32, a.leaf_start[leaf + 1] - item.y);
+    const int n0 = a.nl_start[leaf], nn = min(a.nl_start[leaf + 1] - n0, kFmmMaxNbr);
+    int c = 0;
+    for (int e = 0; e < kFmmMaxNbr; ++e) {
+        int2 run = make_int2(0, INT_MAX);
+        if (e < nn) {
+            const int nl = a.nl_leaf[n0 + e];
+            const int j0 = a.leaf_start[nl];
+            run = make_int2(j0, c);
+            c += a.leaf_start[nl + 1] - j0;
+        }
+        nq_run[(size_t)it * kFmmMaxNbr + e] = run;
+    }
+    nq_item[it] = make_int2(c, tn);
+    cnt[it] = (long long)((c + 1) / 2) * tn;
+}
+
+// The sorted node of source q of an item: lane e of the warp holds run e
+// (first source, sources before it).  Every lane of the warp calls it.
+__device__ __forceinline__ int nq_source(int2 run, int q) {
+    const unsigned full = 0xffffffffu;
+    int j = __shfl_sync(full, run.x, 0) + q;
+#pragma unroll
+    for (int e = 1; e < kFmmMaxNbr; ++e) {
+        const int beg = __shfl_sync(full, run.x, e), cum = __shfl_sync(full, run.y, e);
+        if (q >= cum) j = beg + (q - cum);
+    }
+    return j;
 }
 
 // off[i] = cnt[0] + ... + cnt[i - 1] for i <= n (one block of 1024 threads,
@@ -754,42 +764,32 @@ __global__ void __launch_bounds__(1024) fmm_nq_scan_kernel(const long long* __re
     if (t == 1023) off[n] = s[1023];
 }
 
-// One block per work item, warp w taking its share of the source pairs.
-__global__ void __launch_bounds__(kFmmNT) fmm_nq_build_kernel(FmmArgs a, const double2* __restrict__ q,
+// The entries f_i w_j / (eta_i - eta_j): one block per work item, warp w taking
+// its share of the source pairs.  RE: the real parts too; FC: f is complex
+// (else only its real part is used).
+template <bool RE, bool FC>
+__global__ void __launch_bounds__(kFmmNT) fmm_nq_build_kernel(FmmArgs a, const double2* __restrict__ wgt,
+                                                              const double2* __restrict__ fac,
                                                               const long long* __restrict__ off,
-                                                              const long long* __restrict__ soff,
-                                                              float4* __restrict__ nq_re,
-                                                              float4* __restrict__ nq_im,
-                                                              int4* __restrict__ nq_item,
-                                                              int* __restrict__ nq_src) {
+                                                              const int2* __restrict__ nq_item,
+                                                              const int2* __restrict__ nq_run,
+                                                              float4* __restrict__ out_re,
+                                                              float4* __restrict__ out_im) {
     __shared__ float s_c[kFmmWarps][6][32];   // x1, x2, x3, y1, y2, y3 of the tile's sources
-    __shared__ float s_q[kFmmWarps][4][32];   // q: re.h, re.l, im.h, im.l
+    __shared__ float s_q[kFmmWarps][4][32];   // weight: re.h, re.l, im.h, im.l
     __shared__ int s_j[kFmmWarps][32];
-    __shared__ int s_cum[kFmmMaxNbr + 1];
-    __shared__ int s_beg[kFmmMaxNbr];
-    __shared__ int s_S, s_tn, s_nn;
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int it = blockIdx.x;
-    if (threadIdx.x == 0) {
-        int S, tn, nn;
-        nq_item_shape(a, it, &S, &tn, s_beg, s_cum, &nn);
-        s_S = S;
-        s_tn = tn;
-        s_nn = nn;
-    }
-    __syncthreads();
-    const int S = s_S, tn = s_tn, nn = s_nn;
-    const int src0 = (int)soff[it];
-    if (threadIdx.x == 0) nq_item[it] = make_int4(S, tn, src0, 0);
-    for (int qq = threadIdx.x; qq < S; qq += blockDim.x) {  // the item's source list
-        int e = 0;
-        while (e + 1 < nn && s_cum[e + 1] <= qq) ++e;
-        nq_src[src0 + qq] = s_beg[e] + (qq - s_cum[e]);
-    }
+    const int2 shape = nq_item[it];
+    const int S = shape.x, tn = shape.y;
+    const int2 run = (lane < kFmmMaxNbr) ? nq_run[(size_t)it * kFmmMaxNbr + lane] : make_int2(0, INT_MAX);
     const int i = a.items[it].y + min(lane, tn - 1);
     const float4 pa = a.p3[i];
     const float2 pb = a.p3b[i];
     const float2 tx1 = f2(pa.x), tx2 = f2(pa.y), tx3 = f2(pa.z), ty1 = f2(pa.w), ty2 = f2(pb.x), ty3 = f2(pb.y);
+    const double2 fi = fac[a.perm[i]];
+    const df fr = df_split(fi.x), fm = df_split(fi.y);
+    const df2 fre{f2(fr.h), f2(fr.l)}, fim{f2(fm.h), f2(fm.l)};
     const int npair = (S + 1) >> 1;
     const int p0 = (int)((long long)npair * wid / kFmmWarps), p1 = (int)((long long)npair * (wid + 1) / kFmmWarps);
     const long long base = off[it];
@@ -798,10 +798,7 @@ __global__ void __launch_bounds__(kFmmNT) fmm_nq_build_kernel(FmmArgs a, const d
         const int np = min(16, p1 - ps);
         const int cnt = min(2 * np, S - 2 * ps);  // sources of this tile
         {
-            const int qq = 2 * ps + min(lane, cnt - 1);
-            int e = 0;
-            while (e + 1 < nn && s_cum[e + 1] <= qq) ++e;
-            const int j = s_beg[e] + (qq - s_cum[e]);
+            const int j = nq_source(run, 2 * ps + min(lane, cnt - 1));
             const float4 c4 = a.p3[j];
             const float2 c2 = a.p3b[j];
             s_c[wid][0][lane] = c4.x;
@@ -811,7 +808,7 @@ __global__ void __launch_bounds__(kFmmNT) fmm_nq_build_kernel(FmmArgs a, const d
             s_c[wid][4][lane] = c2.x;
             s_c[wid][5][lane] = c2.y;
             s_j[wid][lane] = (lane < cnt) ? j : -1;
-            const double2 qj = q[a.perm[j]];
+            const double2 qj = wgt[a.perm[j]];
             const df qr = df_split(qj.x), qi = df_split(qj.y);
             s_q[wid][0][lane] = qr.h;
             s_q[wid][1][lane] = qr.l;
@@ -847,43 +844,43 @@ __global__ void __launch_bounds__(kFmmNT) fmm_nq_build_kernel(FmmArgs a, const d
             const df2 ar = df2_mul(dx, inv), ai = df2_mul(dy, inv);  // 1/d = ar - i ai
             const df2 qre{reinterpret_cast<const float2*>(s_q[wid][0])[pp], reinterpret_cast<const float2*>(s_q[wid][1])[pp]};
             const df2 qim{reinterpret_cast<const float2*>(s_q[wid][2])[pp], reinterpret_cast<const float2*>(s_q[wid][3])[pp]};
-            // q (ar - i ai) = (qre ar + qim ai) + i (qim ar - qre ai)
+            // w (ar - i ai) = (wre ar + wim ai) + i (wim ar - wre ai)
             df2 Qr = df2_mul(qre, ar), Qi = df2_mul(qim, ar);
             df2_acc(Qr, df2_mul(qim, ai));
             df2_dec(Qi, df2_mul(qre, ai));
+            // times the target's factor
+            df2 Pi = df2_mul(fre, Qi), Pr = df2_mul(fre, Qr);
+            if (FC) {
+                df2_acc(Pi, df2_mul(fim, Qr));
+                df2_dec(Pr, df2_mul(fim, Qi));
+            }
             if (lane < tn) {
                 const size_t o = (size_t)(base + (long long)(ps + pp) * tn + lane);
-                nq_re[o] = make_float4(Qr.h.x, Qr.h.y, Qr.l.x, Qr.l.y);
-                nq_im[o] = make_float4(Qi.h.x, Qi.h.y, Qi.l.x, Qi.l.y);
+                if (RE) out_re[o] = make_float4(Pr.h.x, Pr.h.y, Pr.l.x, Pr.l.y);
+                out_im[o] = make_float4(Pi.h.x, Pi.h.y, Pi.l.x, Pi.l.y);
             }
         }
     }
 }
 
-// x in the items' source-list order for the cached near field:
-// xl[r][q] = xs[r][nq_src[q]] (0 at the lists' padding), so that each chunk of
-// a work item's sources is one contiguous, 16-byte aligned run.
-__global__ void fmm_nq_xlist_kernel(const int* __restrict__ src, long long qb, int R, int N,
-                                    const float2* __restrict__ xs, float2* __restrict__ xl, const int* done) {
-    if (done != nullptr && *done) return;
-    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= qb) return;
-    const int j = src[q];
-    for (int r = 0; r < R; ++r) xl[(size_t)r * qb + q] = (j >= 0) ? xs[(size_t)r * N + j] : make_float2(0.f, 0.f);
-}
-
-// The near field of z = E(q x) from the cache, streamed into shared memory by
-// the Tensor Memory Accelerator: one block per work item; a producer warp
-// issues bulk copies of the item's cache entries (contiguous, pair-major,
-// evict-first in L2: the cache is larger than L2 and read once per product) and
-// of its sources' x (list order) in chunks of kNbPairs source pairs through a
-// ring of kNbStages buffers (full/empty mbarriers); 8 consumer warps, lane =
-// target, warp w taking pairs w, w + 8, ... of each chunk.  Even and odd
-// sources go to the two halves of packed float2 sums, added at the end, then
-// the warps' sums in warp order.  COMP = 1: Im z only (Re z written as 0).
-// Every wait is bounded (kNbSpin polls); one that gives up sets a.fault, and
-// the producer still waits (bounded) for its copies in flight before leaving.
-constexpr int kNbPairs = 32;                 // source pairs per chunk
+// A cached near field, streamed into shared memory by the Tensor Memory
+// Accelerator: one block per work item; a producer warp issues bulk copies of
+// the item's cache entries (contiguous, pair-major) in chunks of kNbPairs
+// source pairs through a ring of kNbStages buffers (full/empty mbarriers) and
+// gathers the x of the chunk's sources itself, one pair per lane, from the
+// sorted x (the sources of an item are at most nine runs of sorted nodes, so the
+// loads are nearly coalesced and come from L2): 8 bytes per source instead of
+// the index read, x written and read back of a gather launch of its own, which
+// took 19 us per product at 65,536 nodes and 350 us at 524,288.  8
+// consumer warps, lane = target, warp w taking pairs w, w + 8, ... of each
+// chunk.  Even and odd sources go to the two halves of packed float2 sums,
+// added at the end, then the warps' sums in warp order.  COMP = 1: the imaginary
+// part only (the real part written as 0).  `stream`: the entries are marked
+// evict-first in L2 (a cache larger than L2 read once per product must not push
+// out what is reused).  Every wait is bounded (kNbSpin polls); one that gives up
+// sets a.fault, and the producer still waits (bounded) for its copies in flight
+// before leaving.
+constexpr int kNbPairs = 32;                 // source pairs per chunk: one per producer lane
 constexpr int kNbStages = 3;
 constexpr int kNbThreads = kFmmNT + 32;      // 8 consumer warps and the producer warp
 constexpr int kNbSpin = 1 << 22;
@@ -899,10 +896,10 @@ struct NbLayout {
 
 template <int R, int COMP>
 __global__ void __launch_bounds__(kNbThreads) fmm_near_bulk_kernel(FmmArgs a, const long long* __restrict__ off,
-                                                                   const int4* __restrict__ nq_item,
+                                                                   const int2* __restrict__ nq_item,
+                                                                   const int2* __restrict__ nq_run,
                                                                    const float4* __restrict__ nq_re,
-                                                                   const float4* __restrict__ nq_im,
-                                                                   const float2* __restrict__ xl, long long qb) {
+                                                                   const float4* __restrict__ nq_im, int stream) {
     using L = NbLayout<R, COMP>;
     extern __shared__ __align__(16) float4 nb_buf[];
     __shared__ __align__(8) unsigned long long full[kNbStages], empty[kNbStages];
@@ -910,39 +907,60 @@ __global__ void __launch_bounds__(kNbThreads) fmm_near_bulk_kernel(FmmArgs a, co
     if (a.done != nullptr && *a.done) return;  // set before this launch: the same in every thread
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int it = blockIdx.x;
-    const int4 d = __ldg(nq_item + it);  // (S, tn, first source)
+    const int2 d = __ldg(nq_item + it);  // (S, tn)
     const long long o0 = __ldg(off + it);
-    const int S = d.x, tn = d.y, src0 = d.z;
+    const int S = d.x, tn = d.y;
     const int npair = (S + 1) >> 1;
     const int nch = (npair + kNbPairs - 1) / kNbPairs;
     if (threadIdx.x == 0) {
         for (int k = 0; k < kNbStages; ++k) {
-            mbar_init(&full[k], 1);
+            mbar_init(&full[k], 2);  // the copies' announcement and the x of the chunk
             mbar_init(&empty[k], kFmmWarps);
         }
     }
     __syncthreads();
     if (wid == kFmmWarps) {  // the producer
-        if (lane == 0) {
-            int c = 0;
-            for (; c < nch; ++c) {
-                const int st = c % kNbStages;
-                if (c >= kNbStages && !mbar_wait(&empty[st], (unsigned)((c / kNbStages - 1) & 1), kNbSpin)) {
-                    atomicExch(a.fault, 1);
-                    break;
-                }
-                const int p0 = c * kNbPairs, np = min(kNbPairs, npair - p0);
-                const unsigned qbytes = (unsigned)(np * tn) * 16u, xbytes = (unsigned)np * 16u;
-                float4* stage = nb_buf + (size_t)st * L::kStage;
-                mbar_expect_tx(&full[st], L::kParts * qbytes + R * xbytes);
-                bulk_load_stream(stage, nq_im + o0 + (long long)p0 * tn, qbytes, &full[st]);
-                if (COMP == 0) bulk_load_stream(stage + L::kQ, nq_re + o0 + (long long)p0 * tn, qbytes, &full[st]);
+        const int2 run = (lane < kFmmMaxNbr) ? __ldg(nq_run + (size_t)it * kFmmMaxNbr + lane) : make_int2(0, INT_MAX);
+        int c = 0;
+        for (; c < nch; ++c) {
+            const int st = c % kNbStages;
+            const int p0 = c * kNbPairs, np = min(kNbPairs, npair - p0);
+            float4* stage = nb_buf + (size_t)st * L::kStage;
+            const int q = 2 * (p0 + lane);
+            const int j0 = nq_source(run, q), j1 = nq_source(run, q + 1);
+            float4 xv[R];
 #pragma unroll
-                for (int r = 0; r < R; ++r)
-                    bulk_load(stage + L::kParts * L::kQ + r * L::kX, xl + (size_t)r * qb + src0 + 2 * p0, xbytes,
-                              &full[st]);
+            for (int r = 0; r < R; ++r) {  // (0, 0) past the item's sources
+                const float2* xr = a.xs + (size_t)r * a.N;
+                const float2 u = (q < S) ? __ldg(xr + j0) : make_float2(0.f, 0.f);
+                const float2 v = (q + 1 < S) ? __ldg(xr + j1) : make_float2(0.f, 0.f);
+                xv[r] = make_float4(u.x, u.y, v.x, v.y);
             }
-            // the copies still in flight land before the warp leaves
+            bool ok = true;
+            if (c >= kNbStages) ok = mbar_wait(&empty[st], (unsigned)((c / kNbStages - 1) & 1), kNbSpin);
+            if (!__all_sync(0xffffffffu, ok)) {
+                if (lane == 0) atomicExch(a.fault, 1);
+                break;
+            }
+            if (lane == 0) {
+                const unsigned qbytes = (unsigned)(np * tn) * 16u;
+                mbar_expect_tx(&full[st], L::kParts * qbytes);
+                const float4* im = nq_im + o0 + (long long)p0 * tn;
+                const float4* re = (COMP == 0) ? nq_re + o0 + (long long)p0 * tn : nullptr;
+                if (stream) {
+                    bulk_load_stream(stage, im, qbytes, &full[st]);
+                    if (COMP == 0) bulk_load_stream(stage + L::kQ, re, qbytes, &full[st]);
+                } else {
+                    bulk_load(stage, im, qbytes, &full[st]);
+                    if (COMP == 0) bulk_load(stage + L::kQ, re, qbytes, &full[st]);
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) stage[L::kParts * L::kQ + r * L::kX + lane] = xv[r];
+            __syncwarp();  // every lane's x before the arrival
+            if (lane == 0) mbar_arrive(&full[st]);
+        }
+        if (lane == 0) {  // the copies still in flight land before the warp leaves
             for (int k = max(0, c - kNbStages); k < c; ++k)
                 mbar_wait(&full[k % kNbStages], (unsigned)((k / kNbStages) & 1), kNbSpin);
         }
@@ -1009,7 +1027,8 @@ __global__ void __launch_bounds__(kNbThreads) fmm_near_bulk_kernel(FmmArgs a, co
 // interleaved Horner chains of 8 coefficients joined by t^8 (a dependent chain
 // of 13 steps instead of 31).  EPI: the operator epilogue of the product is applied at
 // once (epilogue_apply: e.g. f_B(x) = 2x + diag(B1) x + (2/n) Im(A z)), so the
-// sums z never go to memory; otherwise z is written in node order.
+// sums z never go to memory; otherwise z is written in node order.  A cached
+// near field (a.near_scaled) comes already multiplied by the epilogue's factor.
 // EF: also F = -d/dz of the far field (Horner's rule carries the derivative)
 // plus the near-field sums of w/d^2, written to outF.
 template <int R, bool EF, bool EPI, int EK = EPI_Z>
@@ -1024,6 +1043,7 @@ __global__ void __launch_bounds__(256) fmm_l2p_kernel(FmmArgs a, ReduceArgs e) {
     const cdf t = cdf{df_split_fast((p.x - c.x) * ir), df_split_fast((p.y - c.y) * ir)};
     const int node = a.perm[i];
     double zx[kMaxRHS] = {0.0, 0.0}, zy[kMaxRHS] = {0.0, 0.0};
+    double2 near[kMaxRHS] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
     cdf t8{};
     if (!EF) t8 = cdf_sq(cdf_sq(cdf_sq(t)));
 #pragma unroll
@@ -1058,8 +1078,14 @@ __global__ void __launch_bounds__(256) fmm_l2p_kernel(FmmArgs a, ReduceArgs e) {
             }
         }
         const double2 zn = a.zn[(size_t)r * a.N + i];
-        zx[r] = ((double)u.re.h + (double)u.re.l) + zn.x;
-        zy[r] = ((double)u.im.h + (double)u.im.l) + zn.y;
+        zx[r] = (double)u.re.h + (double)u.re.l;
+        zy[r] = (double)u.im.h + (double)u.im.l;
+        if (EPI && a.near_scaled) {
+            near[r] = zn;
+        } else {
+            zx[r] += zn.x;
+            zy[r] += zn.y;
+        }
         if (!EPI) a.out[(size_t)r * a.N + node] = make_double2(zx[r], zy[r]);
         if (EF) {
             const double2 zf = a.zf[(size_t)r * a.N + i];
@@ -1067,7 +1093,8 @@ __global__ void __launch_bounds__(256) fmm_l2p_kernel(FmmArgs a, ReduceArgs e) {
                                                           -ir * ((double)du.im.h + (double)du.im.l) + zf.y);
         }
     }
-    if (EPI) epilogue_apply_as(e, EK, node, make_double2(zx[0], zy[0]), make_double2(zx[1], zy[1]));
+    if (EPI)
+        epilogue_apply_as<true>(e, EK, node, make_double2(zx[0], zy[0]), make_double2(zx[1], zy[1]), near[0], near[1]);
 }
 
 // ---------------------------------------------------------------- host: tables
@@ -1247,20 +1274,19 @@ void release_fmm(Boundary& b) {
         give_stream(false, b.fmm->bst, b.device);
         give_event(b.fmm->ev_nq, b.device);
 
-        if (b.fmm->arena || b.fmm->sync || b.fmm->nq_re || b.fmm->tp || b.fmm->fault) {  // once no stream uses them
+        if (b.fmm->arena || b.fmm->sync || b.fmm->nq_item || b.fmm->tp || b.fmm->fault) {  // once no stream uses them
             cudaDeviceSynchronize();
             cudaGetLastError();
             pool_free(b.fmm->arena, 0);
             pool_free(b.fmm->sync, 0);
             pool_free(b.fmm->nq_cnt, 0);
-            pool_free(b.fmm->nq_soff, 0);
             pool_free(b.fmm->nq_off, 0);
             pool_free(b.fmm->nq_item, 0);
-            pool_free(b.fmm->nq_src, 0);
+            pool_free(b.fmm->nq_run, 0);
             pool_free(b.fmm->nq_re, 0);
             pool_free(b.fmm->nq_im, 0);
+            pool_free(b.fmm->nt_im, 0);
             pool_free(b.fmm->xs, 0);
-            pool_free(b.fmm->xl, 0);
             pool_free(b.fmm->fault, 0);
             pool_free(b.fmm->tp, 0);
         }
@@ -1701,105 +1727,105 @@ double fmm_near_cached_instr(const Boundary& b, int R, int comp) {
 }
 
 double fmm_near_cached_bytes(const Boundary& b, int R, int comp) {
-    // 8 bytes per near pair and part of z read from the cache, x in list order
-    // (8 bytes per list entry, counted at the lists' bound) and z out (16 bytes
-    // per node) per right-hand side
-    return b.fmm ? 8.0 * (double)b.fmm->near_pairs * (comp == 1 ? 1.0 : 2.0) +
-                       8.0 * R * (double)b.fmm->nq_qb + 16.0 * R * b.N
-                 : 0.0;
+    // 8 bytes per near pair and part of z read from the cache, x in (8 bytes per
+    // node) and z out (16 bytes per node) per right-hand side
+    return b.fmm ? 8.0 * (double)b.fmm->near_pairs * (comp == 1 ? 1.0 : 2.0) + 24.0 * R * b.N : 0.0;
 }
 
 const int* fmm_fault_word(const Boundary& b) {
     return b.fmm ? b.fmm->fault : nullptr;
 }
 
-// Forms the near-field operator cache of the products z = E(q x) once per
-// handle (count, scan, allocate, build); state -1 when it would exceed
-// kNqMaxBytes or when its allocation fails (the products then compute the
-// near field directly).
+// The near-field operator caches of a handle, each formed once: allocated here
+// (state 2), formed by near_cache_build on the first product that reads it;
+// state -1 when it would exceed kNqMaxBytes or its allocation fails (the
+// products then compute the near field directly).  `adj`: the cache of the
+// solves with weights A x (imaginary part only), else that of the products with
+// weights q x.
 constexpr double kNqMaxBytes = 16.0 * (1 << 30);
 
-static int ensure_near_cache(const Boundary& b, cudaStream_t st) {
+static int ensure_near_cache(const Boundary& b, bool adj, cudaStream_t st) {
     FmmTree* t = b.fmm;
-    if (t->nq_state != 0) return GNK_OK;
-    t->nq_state = -1;
+    int& state = adj ? t->nt_state : t->nq_state;
+    if (state != 0) return GNK_OK;
+    state = -1;
     if (t->nitems <= 0) return GNK_OK;
     // sizes from bounds the tree already gives, so that nothing waits for the
-    // device: sum_items ceil(S/2) tn <= (near pairs + N)/2 entries, and
-    // sum_items S <= near pairs sources (each source meets at least one target)
+    // device: sum_items ceil(S/2) tn <= (near pairs + N)/2 entries
     const size_t ni = (size_t)t->nitems;
-    // sum_items S = sum_leaves ceil(n_leaf / 32) S_leaf <= near pairs / 32 + sum_leaves S_leaf, and
-    // a leaf is a neighbour of at most kFmmMaxNbr leaves, so sum_leaves S_leaf <= kFmmMaxNbr N;
-    // plus one padding entry per item, rounded up to even
     const long long slots = (t->near_pairs + b.N) / 2 + 1;
-    long long nsrc = t->near_pairs / 32 + (long long)kFmmMaxNbr * b.N + (long long)ni + 2;
-    nsrc += nsrc & 1;
     const size_t bytes = (size_t)slots * sizeof(float4);
-    if (nsrc > INT32_MAX || 2.0 * (double)bytes > kNqMaxBytes) return GNK_OK;
-    long long *cnt = nullptr, *soff = nullptr;
-    if (pool_alloc(reinterpret_cast<void**>(&cnt), 2 * ni * sizeof(long long), st) != cudaSuccess ||
-        pool_alloc(reinterpret_cast<void**>(&soff), (ni + 1) * sizeof(long long), st) != cudaSuccess ||
-        pool_alloc(reinterpret_cast<void**>(&t->nq_off), (ni + 1) * sizeof(long long), st) != cudaSuccess ||
-        pool_alloc(reinterpret_cast<void**>(&t->nq_re), bytes, st) != cudaSuccess ||
-        pool_alloc(reinterpret_cast<void**>(&t->nq_im), bytes, st) != cudaSuccess ||
-        pool_alloc(reinterpret_cast<void**>(&t->nq_item), ni * sizeof(int4), st) != cudaSuccess ||
-        pool_alloc(reinterpret_cast<void**>(&t->nq_src), (size_t)nsrc * sizeof(int), st) != cudaSuccess ||
-        pool_alloc(reinterpret_cast<void**>(&t->xs), (size_t)kMaxRHS * b.N * sizeof(float2), st) != cudaSuccess ||
-        pool_alloc(reinterpret_cast<void**>(&t->xl), (size_t)kMaxRHS * nsrc * sizeof(float2), st) != cudaSuccess) {
-        cudaGetLastError();
-        pool_free(cnt, st);
-        pool_free(soff, st);
-        pool_free(t->nq_off, st);
-        pool_free(t->nq_re, st);
-        pool_free(t->nq_im, st);
-        pool_free(t->nq_item, st);
-        pool_free(t->nq_src, st);
-        pool_free(t->xs, st);
-        pool_free(t->xl, st);
-        t->xl = nullptr;
-        t->nq_off = nullptr;
-        t->nq_re = t->nq_im = nullptr;
-        t->nq_item = nullptr;
-        t->nq_src = nullptr;
-        t->xs = nullptr;
-        return GNK_OK;
+    if (2.0 * (double)bytes > kNqMaxBytes) return GNK_OK;
+    if (t->near_shape == 0) {
+        if (pool_alloc(reinterpret_cast<void**>(&t->nq_cnt), ni * sizeof(long long), st) != cudaSuccess ||
+            pool_alloc(reinterpret_cast<void**>(&t->nq_off), (ni + 1) * sizeof(long long), st) != cudaSuccess ||
+            pool_alloc(reinterpret_cast<void**>(&t->nq_item), ni * sizeof(int2), st) != cudaSuccess ||
+            pool_alloc(reinterpret_cast<void**>(&t->nq_run), ni * kFmmMaxNbr * sizeof(int2), st) != cudaSuccess ||
+            pool_alloc(reinterpret_cast<void**>(&t->xs), (size_t)kMaxRHS * b.N * sizeof(float2), st) != cudaSuccess) {
+            cudaGetLastError();
+            pool_free(t->nq_cnt, st);
+            pool_free(t->nq_off, st);
+            pool_free(t->nq_item, st);
+            pool_free(t->nq_run, st);
+            t->nq_cnt = nullptr;
+            t->nq_off = nullptr;
+            t->nq_item = nullptr;
+            t->nq_run = nullptr;
+            t->xs = nullptr;
+            return GNK_OK;
+        }
+        t->near_shape = 1;
+        t->nq_slots = slots;
     }
-    t->nq_slots = slots;
-    t->nq_qb = nsrc;
-    t->nq_cnt = cnt;
-    t->nq_soff = soff;
-    t->nq_state = 2;  // allocated; formed by near_cache_build before the first cached near field
+    float4** part[2] = {adj ? &t->nt_im : &t->nq_im, adj ? nullptr : &t->nq_re};
+    for (float4** p : part) {
+        if (p && pool_alloc(reinterpret_cast<void**>(p), bytes, st) != cudaSuccess) {
+            cudaGetLastError();
+            *p = nullptr;
+            if (p == part[1]) {
+                pool_free(*part[0], st);
+                *part[0] = nullptr;
+            }
+            return GNK_OK;
+        }
+    }
+    state = 2;
     return GNK_OK;
 }
 
-// The launches that form the cache (count, scans, entries), on `st` after the
-// product has forked its far field, so that they overlap it.
-static int near_cache_build(const Boundary& b, cudaStream_t st) {
+// The launches that form a cache (the items' shapes once, then the entries), on
+// `st` after the product has forked its far field, so that they overlap it.
+static int near_cache_build(const Boundary& b, bool adj, cudaStream_t st) {
     FmmTree* t = b.fmm;
-    if (t->nq_state != 2) return GNK_OK;
+    int& state = adj ? t->nt_state : t->nq_state;
+    if (state != 2) return GNK_OK;
     FmmArgs a;
     fmm_args(b, a);
-    const size_t ni = (size_t)t->nitems;
-    long long* cnt = t->nq_cnt;
-    long long* scnt = cnt + ni;
-    long long* soff = t->nq_soff;
-    GNK_TRY_CUDA(cudaMemsetAsync(t->nq_src, 0xff, (size_t)t->nq_qb * sizeof(int), st));  // -1: padding
-    fmm_nq_count_kernel<<<(t->nitems + 255) / 256, 256, 0, st>>>(a, cnt, scnt);
-    fmm_nq_scan_kernel<<<1, 1024, 0, st>>>(cnt, t->nitems, t->nq_off);
-    fmm_nq_scan_kernel<<<1, 1024, 0, st>>>(scnt, t->nitems, soff);
-    GNK_TRY_CUDA(cudaGetLastError());
-    count_launches(3);
+    if (t->near_shape == 1) {
+        fmm_nq_shape_kernel<<<(t->nitems + 255) / 256, 256, 0, st>>>(a, t->nq_cnt, t->nq_item, t->nq_run);
+        fmm_nq_scan_kernel<<<1, 1024, 0, st>>>(t->nq_cnt, t->nitems, t->nq_off);
+        GNK_TRY_CUDA(cudaGetLastError());
+        count_launches(2);
+        pool_free(t->nq_cnt, st);
+        t->nq_cnt = nullptr;
+        t->near_shape = 2;
+    } else if (t->nq_wait) {  // the shapes are being formed on the stream of the other cache
+        GNK_TRY_CUDA(cudaStreamWaitEvent(st, t->ev_nq, 0));
+    }
     const ProfToken tok = prof_begin(st, PK_OTHER);
-    fmm_nq_build_kernel<<<t->nitems, kFmmNT, 0, st>>>(a, b.q, t->nq_off, soff, t->nq_re, t->nq_im, t->nq_item,
-                                                      t->nq_src);
+    if (adj)
+        fmm_nq_build_kernel<false, true><<<t->nitems, kFmmNT, 0, st>>>(a, b.A, b.q, t->nq_off, t->nq_item,
+                                                                       t->nq_run, nullptr, t->nt_im);
+    else if (b.A_real)
+        fmm_nq_build_kernel<true, false><<<t->nitems, kFmmNT, 0, st>>>(a, b.q, b.A, t->nq_off, t->nq_item,
+                                                                       t->nq_run, t->nq_re, t->nq_im);
+    else
+        fmm_nq_build_kernel<true, true><<<t->nitems, kFmmNT, 0, st>>>(a, b.q, b.A, t->nq_off, t->nq_item,
+                                                                      t->nq_run, t->nq_re, t->nq_im);
     GNK_TRY_CUDA(cudaGetLastError());
     prof_end(tok, PK_OTHER, 0.0, st);
     count_launches(1);
-    pool_free(cnt, st);
-    pool_free(soff, st);
-    t->nq_cnt = nullptr;
-    t->nq_soff = nullptr;
-    t->nq_state = 1;
+    state = 1;
     return GNK_OK;
 }
 
@@ -1834,8 +1860,13 @@ static int l2p_epi(const FmmArgs& a, const ReduceArgs& e, int nb, cudaStream_t s
     return GNK_OK;
 }
 
+// Bytes of cache per product up to which it is left to L2's own policy (a third
+// of the 129 MB, beside the power table and the expansions); a larger one is
+// streamed past it.
+constexpr double kNbKeepBytes = 48e6;
+
 template <int R, int COMP>
-static int launch_near_bulk(const Boundary& b, const FmmArgs& a, cudaStream_t st) {
+static int launch_near_bulk(const Boundary& b, const FmmArgs& a, bool adj, cudaStream_t st) {
     using L = NbLayout<R, COMP>;
     static std::mutex mu;
     static std::vector<char> ready;  // per device: the shared-memory attribute is set
@@ -1851,8 +1882,9 @@ static int launch_near_bulk(const Boundary& b, const FmmArgs& a, cudaStream_t st
         }
     }
     const FmmTree* t = b.fmm;
-    fmm_near_bulk_kernel<R, COMP><<<t->nitems, kNbThreads, L::kBytes, st>>>(a, t->nq_off, t->nq_item, t->nq_re,
-                                                                            t->nq_im, t->xl, t->nq_qb);
+    const int stream = 8.0 * L::kParts * (double)t->near_pairs > kNbKeepBytes;
+    fmm_near_bulk_kernel<R, COMP><<<t->nitems, kNbThreads, L::kBytes, st>>>(
+        a, t->nq_off, t->nq_item, t->nq_run, t->nq_re, adj ? t->nt_im : t->nq_im, stream);
     GNK_TRY_CUDA(cudaGetLastError());
     return GNK_OK;
 }
@@ -1867,7 +1899,7 @@ int fmm_start_near_cache(const Boundary& bc, cudaStream_t st) {
     if (b.plain) return GNK_OK;
     GNK_TRY(ensure_fmm(b, kMaxRHS, st));
     FmmTree* t = b.fmm;
-    GNK_TRY(ensure_near_cache(b, st));
+    GNK_TRY(ensure_near_cache(b, false, st));
     if (t->nq_state != 2) return GNK_OK;
     if (!t->bst) {
         if (take_stream(false, &t->bst) != cudaSuccess || take_event(&t->ev_nq) != cudaSuccess) {
@@ -1878,7 +1910,7 @@ int fmm_start_near_cache(const Boundary& bc, cudaStream_t st) {
     // the cache's buffers were allocated in the order of `st`
     GNK_TRY_CUDA(cudaEventRecord(t->ev_nq, st));
     GNK_TRY_CUDA(cudaStreamWaitEvent(t->bst, t->ev_nq, 0));
-    GNK_TRY(near_cache_build(b, t->bst));
+    GNK_TRY(near_cache_build(b, false, t->bst));
     GNK_TRY_CUDA(cudaEventRecord(t->ev_nq, t->bst));
     t->nq_wait = 1;
     return GNK_OK;
@@ -1888,7 +1920,7 @@ int fmm_start_near_cache(const Boundary& bc, cudaStream_t st) {
 // gather, the far-field chain on the high-priority stream, the near field on
 // `st`, and L2P after they join.  EF: also the sums of w/d^2 (to a.outF).
 static int fmm_product(const Boundary& b, FmmArgs& a, int R, bool EF, const ReduceArgs* epi, cudaStream_t st,
-                       int* nlaunch, int cached = -1) {
+                       int* nlaunch, int cached = -1, bool adj = false) {
     const FmmTree* t = b.fmm;
     fmm_gather_kernel<<<(b.N + 255) / 256, 256, 0, st>>>(a);
     GNK_TRY_CUDA(cudaEventRecord(t->ev_fork, st));
@@ -1929,33 +1961,27 @@ static int fmm_product(const Boundary& b, FmmArgs& a, int R, bool EF, const Redu
         ++launches;
     }
     GNK_TRY_CUDA(cudaEventRecord(t->ev_join, fs));
-    // near field on the caller's stream (from the operator cache when `cached`
-    // is 0 (both parts of z) or 1 (Im z only)); the first cached product forms
-    // the cache here, beside its far field
+    // near field on the caller's stream (from an operator cache when `cached`
+    // is 0 (both parts) or 1 (the imaginary part)); the first product that reads
+    // a cache forms it here, beside its far field
     if (cached >= 0) {
-        if (t->nq_wait) {  // formed on its own stream since the tree was built
+        if (!adj && t->nq_wait) {  // formed on its own stream since the tree was built
             GNK_TRY_CUDA(cudaStreamWaitEvent(st, t->ev_nq, 0));
             b.fmm->nq_wait = 0;
         } else {
-            GNK_TRY(near_cache_build(b, st));
+            GNK_TRY(near_cache_build(b, adj, st));
         }
-    }
-    if (cached >= 0) {  // x in the items' list order
-        fmm_nq_xlist_kernel<<<(unsigned)((t->nq_qb + 255) / 256), 256, 0, st>>>(t->nq_src, t->nq_qb, R, b.N, a.xs,
-                                                                               t->xl, a.done);
-        GNK_TRY_CUDA(cudaGetLastError());
-        ++launches;
     }
     const ProfToken tokn = prof_begin(st, PK_FMMNEAR);
     if (cached >= 0) {
         if (R == 2 && cached == 1)
-            GNK_TRY((launch_near_bulk<2, 1>(b, a, st)));
+            GNK_TRY((launch_near_bulk<2, 1>(b, a, adj, st)));
         else if (R == 2)
-            GNK_TRY((launch_near_bulk<2, 0>(b, a, st)));
+            GNK_TRY((launch_near_bulk<2, 0>(b, a, adj, st)));
         else if (cached == 1)
-            GNK_TRY((launch_near_bulk<1, 1>(b, a, st)));
+            GNK_TRY((launch_near_bulk<1, 1>(b, a, adj, st)));
         else
-            GNK_TRY((launch_near_bulk<1, 0>(b, a, st)));
+            GNK_TRY((launch_near_bulk<1, 0>(b, a, adj, st)));
     } else if (R == 2 && EF)
         fmm_near_kernel<2, true><<<t->nitems, kFmmNT, 0, st>>>(a);
     else if (R == 2)
@@ -2023,6 +2049,7 @@ static void fmm_args(const Boundary& b, FmmArgs& a) {
     a.bUp = t->bUp;
     a.ucnt = t->sync;
     a.xs = nullptr;
+    a.near_scaled = 0;
     a.tp = t->tp;
     a.mult = t->mult;
     a.loc = t->loc;
@@ -2047,18 +2074,26 @@ int run_fmm(const Boundary& b, const PairJob& job, cudaStream_t st) {
     a.out = nullptr;
     a.done = job.done;
     int launches = 0;
-    // products with the handle's own weights q x read the near field from
-    // the operator cache (formed by the first of them)
+    // Products with the handle's own weights q x read the near field from its
+    // operator cache (formed by the first of them), one part of it where the
+    // operator reads Im(A z) alone.  Those with weights A x whose operator reads
+    // Im(q z) do so inside a solve (job.done), which forms the cache: it costs
+    // two or three products and a solve has many.
     int cached = -1;
-    if (job.mode == W_SCALED && job.s == b.q && !b.plain) {
-        GNK_TRY(ensure_near_cache(b, st));
-        if (b.fmm->nq_state >= 1) {
-            cached = pair_component_needed(b, job) == 1 ? 1 : 0;
+    const bool im_only = job.R == 1 && (job.epi == EPI_IMINUSN || job.epi == EPI_RESID);
+    const bool im_adj = job.R == 1 && (job.epi == EPI_ADJ || job.epi == EPI_RESID_ADJ || job.epi == EPI_IMINUSN_T ||
+                                       job.epi == EPI_RESID_T);
+    const bool adj = job.s != b.q && job.s == b.A && im_adj && !b.diff;
+    if (job.mode == W_SCALED && !b.plain && (job.s == b.q || adj)) {
+        if (!adj || job.done != nullptr) GNK_TRY(ensure_near_cache(b, adj, st));
+        if ((adj ? b.fmm->nt_state : b.fmm->nq_state) >= 1) {
+            cached = (adj || im_only) ? 1 : 0;
             a.xs = b.fmm->xs;
+            a.near_scaled = 1;
         }
     }
     const ReduceArgs e = reduce_args(b, job, 1, 0);  // the epilogue runs inside L2P
-    GNK_TRY(fmm_product(b, a, job.R, false, &e, st, &launches, cached));
+    GNK_TRY(fmm_product(b, a, job.R, false, &e, st, &launches, cached, adj));
     count_launches(launches);
     return GNK_OK;
 }

@@ -16,6 +16,7 @@ constexpr int kFmmP = 32;     // expansion order (one warp lane per coefficient)
 #endif
 constexpr int kFmmLeaf = GNK_FMM_LEAF;  // target mean number of nodes per leaf
 constexpr int kFmmNT = 256;   // threads of the near-field kernel: 8 warps
+constexpr int kFmmMaxNbr = 9;  // a leaf and its eight neighbours
 
 struct FmmTree {
     int L = 0, nbox = 0, nleaf = 0, R = 0;
@@ -52,23 +53,24 @@ struct FmmTree {
     double2* zf = nullptr;      // [R][N] near-field sums of w/d^2 (gradient products)
     int* node_box = nullptr;    // leaf box of each node in sorted order
     int* sync = nullptr;        // [nbox]: children counted by the upward pass (zero between products)
-    // near-field operator cache of the products z = E(q x) (fixed geometry):
-    // Q_ij = q_j / (eta_i - eta_j) per work item, double-float, for source
-    // pairs x targets; state 0 not formed, 2 allocated (formed by the first
-    // cached product), 1 formed, -1 not used (too large)
-    int nq_state = 0;
-    long long* nq_cnt = nullptr;   // build temporaries while state is 2
-    long long* nq_soff = nullptr;
-    long long nq_slots = 0;     // float4 entries of each of nq_re, nq_im
+    // near-field operator caches (fixed geometry): per work item the entries of
+    //   A_i q_j / (eta_i - eta_j)  for the products with weights q x (both parts),
+    //   q_i A_j / (eta_i - eta_j)  for the solves with weights A x (imaginary part),
+    // double-float, for source pairs x targets.  The items' shapes are shared.
+    int near_shape = 0;           // 1: nq_off, nq_item, nq_run are allocated; 2: formed
+    long long* nq_cnt = nullptr;  // [nitems] build temporary of the shapes
     long long* nq_off = nullptr;  // per work item: first entry (nitems + 1)
-    int4* nq_item = nullptr;    // per work item: (S sources, tn targets, first source in nq_src, -)
-    int* nq_src = nullptr;      // the items' sources (sorted node indices), item after item, each
-                                // item's list padded to even length with -1 (nq_qb entries)
-    long long nq_qb = 0;        // entries of nq_src (a bound on the lists' total, even)
+    int2* nq_item = nullptr;      // per work item: (S sources, tn targets)
+    int2* nq_run = nullptr;       // [nitems][kFmmMaxNbr]: (first source, sources before) of each
+                                  // neighbour leaf; (0, INT_MAX) past the last
+    float2* xs = nullptr;         // [R][N] x in sorted order, double-float (cached products)
+    long long nq_slots = 0;       // float4 entries of each of the arrays below
+    // state 0 not formed, 2 allocated (formed by the first cached product),
+    // 1 formed, -1 not used (too large)
+    int nq_state = 0, nt_state = 0;
     float4* nq_re = nullptr;
     float4* nq_im = nullptr;
-    float2* xs = nullptr;       // [R][N] x in sorted order, double-float (cached products)
-    float2* xl = nullptr;       // [R][nq_qb] x in the items' source-list order (0 at padding)
+    float4* nt_im = nullptr;
     int* fault = nullptr;       // set by a bounded wait of an FMM kernel that gave up
     float4* tp = nullptr;       // [N][P] powers t^k of each node about its leaf centre (P2M), or null
     cudaStream_t aux = nullptr; // high-priority stream of the far field (the near field runs beside it)

@@ -212,6 +212,7 @@ struct Boundary {
     void* arena = nullptr;      // the one allocation that holds the buffers above
     int eone_pending = 0;       // Eone, diag(B1), diag(D1), e not yet formed
     int plain = 0;              // 1: diagonals of the form without singularity subtraction
+    int diff = 0;               // 1: the FMM keeps one fixed sequence of operations (GNK_BUILD_DIFF)
     int A_real = 0;             // 1: Im A = 0 at every node (then f_B needs only Im E(qx))
     FmmTree* fmm = nullptr;     // quadtree and expansions, built on the first FMM product
     int df_scalar = 0;          // 1: scalar double-float kernel instead of the packed one

@@ -39,6 +39,7 @@ GNK_PREC_FMM = 5
 GNK_PREC_MIXED_FMM = 6
 GNK_BUILD_DEFER = 0x100
 GNK_BUILD_PLAIN = 0x200
+GNK_BUILD_DIFF = 0x400
 
 EXPORTED = (
     "gnk_default_options", "gnk_last_error", "gnk_version", "gnk_build_boundary",

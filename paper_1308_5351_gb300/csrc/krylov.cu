@@ -17,8 +17,11 @@
 // plain FP64, in FP64 (k_arnoldi) for that one.  The norms at the start of a
 // cycle finish in the last block to arrive (atomic ticket + fence, no spinning).
 // Partial sums are added in a fixed order, so results are reproducible.
-// Inside a cycle every kernel first reads the device flag `done`, so the host
-// enqueues a whole cycle without waiting and synchronises once per cycle.
+// Inside a cycle every kernel first reads the device flag `done`, so launches
+// past convergence do nothing, and the host synchronises once per cycle.  It
+// keeps only kAhead steps ahead of the device, whose step count it reads from
+// a pinned word that the Arnoldi step writes: a cycle of 20 steps that needs
+// one or two otherwise cost about 20 us of empty launches for each of the rest.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -48,12 +51,20 @@ struct KState {
     int bar_err;      // a grid barrier wait gave up
     int bar_limit;    // polls before a grid barrier wait gives up
     int bar_skip;     // test hook: this block never arrives at a barrier (-1: none)
+    int* progress;    // pinned host word: steps of this cycle, kProgressDone once it has ended (or null)
     // grid barrier of the Arnoldi step: arrivals and generation on cache lines
     // of their own, away from the fields above and from each other
     alignas(128) unsigned bar_count;
     alignas(128) unsigned bar_gen;
     char pad_[124];
 };
+
+constexpr int kProgressDone = 1 << 30;
+
+// After the step count k and the flag `done` of the cycle are known (one thread).
+__device__ __forceinline__ void report_progress(const KState* s, int k, bool done) {
+    if (s->progress) *(volatile int*)s->progress = k | (done ? kProgressDone : 0);
+}
 
 constexpr int KT = 256;       // threads per block of the vector kernels
 constexpr int KB_MAX = 256;   // maximum blocks of the vector kernels
@@ -145,6 +156,7 @@ __global__ void __launch_bounds__(KT) k_norm(const double* __restrict__ x, int N
             s->k = 0;
             if (!isfinite(nrm)) s->nonfinite = 1;
             s->done = (!(nrm > s->tol * s->bnorm)) ? 1 : 0;  // also stops on NaN
+            if (s->done) report_progress(s, 0, true);
             p.g[0] = nrm;
             for (int k = 1; k <= s->restart; ++k) p.g[k] = 0.0;
         }
@@ -358,7 +370,9 @@ __device__ void givens_step(int j, double hn, double* h1, const double* h2, cons
         s->k = j + 1;
         const bool bad = !isfinite(est) || !isfinite(hn);
         if (bad) s->nonfinite = 1;
-        if (bad || est <= s->tol * s->bnorm || j + 1 == s->restart || hn == 0.0) s->done = 1;
+        const bool end = bad || est <= s->tol * s->bnorm || j + 1 == s->restart || hn == 0.0;
+        if (end) s->done = 1;
+        report_progress(s, j + 1, end);
     }
     __syncthreads();
     double* colg = p.H + (size_t)j * p.ld;
@@ -435,7 +449,9 @@ __device__ void givens_step_warp0(int j, double hn, double* h1, const double* h2
         s->k = j + 1;
         const bool bad = !isfinite(est) || !isfinite(hn);
         if (bad) s->nonfinite = 1;
-        if (bad || est <= s->tol * s->bnorm || j + 1 == s->restart || hn == 0.0) s->done = 1;
+        const bool end = bad || est <= s->tol * s->bnorm || j + 1 == s->restart || hn == 0.0;
+        if (end) s->done = 1;
+        report_progress(s, j + 1, end);
     }
     __syncwarp();
     double* colg = p.H + (size_t)j * p.ld;
@@ -795,7 +811,9 @@ __device__ void givens_df_warp0(int j, df hn, double* hcol, const double* scs, c
         s->k = j + 1;
         const bool bad = !isfinite(est) || !isfinite(hnd) || !isfinite(zj);
         if (bad) s->nonfinite = 1;
-        if (bad || est <= s->tol * s->bnorm || j + 1 == s->restart || hnd == 0.0) s->done = 1;
+        const bool end = bad || est <= s->tol * s->bnorm || j + 1 == s->restart || hnd == 0.0;
+        if (end) s->done = 1;
+        report_progress(s, j + 1, end);
     }
     __syncwarp();
     double* colg = p.H + (size_t)j * p.ld;
@@ -1040,7 +1058,7 @@ __global__ void k_axpy(double* __restrict__ x, const double* __restrict__ d, int
     if (i < N) x[i] += d[i];
 }
 
-__global__ void k_init_state(KState* s, double tol, int restart, int bar_limit, int bar_skip) {
+__global__ void k_init_state(KState* s, double tol, int restart, int bar_limit, int bar_skip, int* progress) {
     s->bnorm = 0.0;
     s->beta = 0.0;
     s->tol = tol;
@@ -1056,7 +1074,85 @@ __global__ void k_init_state(KState* s, double tol, int restart, int bar_limit, 
     s->bar_err = 0;
     s->bar_limit = bar_limit;
     s->bar_skip = bar_skip;
+    s->progress = progress;
 }
+
+// Pinned progress words, one per running solve: one page, allocated with the
+// first solve and kept for the process, handed out and taken back under a lock.
+// With all of them in use (or without pinned memory) a solve gets none and its
+// cycles are enqueued whole.
+constexpr int kProgressSlots = 64, kProgressStride = 64 / sizeof(int);  // a cache line each
+
+struct ProgressPool {
+    std::mutex mu;
+    int* page = nullptr;
+    bool tried = false;
+    unsigned long long used = 0;
+};
+
+ProgressPool& progress_pool() {
+    static ProgressPool* p = new ProgressPool();  // outlives static teardown
+    return *p;
+}
+
+struct Progress {
+    int* word = nullptr;
+    int slot = -1;
+    cudaStream_t st;
+    bool idle = true;  // the stream has been synchronised since the last launch
+    explicit Progress(cudaStream_t stream) : st(stream) {
+        ProgressPool& P = progress_pool();
+        std::lock_guard<std::mutex> lock(P.mu);
+        if (!P.tried) {
+            P.tried = true;
+            void* m = nullptr;
+            if (cudaHostAlloc(&m, kProgressSlots * 64, cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess)
+                P.page = static_cast<int*>(m);
+            else
+                cudaGetLastError();
+        }
+        if (!P.page) return;
+        for (int k = 0; k < kProgressSlots; ++k) {
+            if (P.used >> k & 1) continue;
+            P.used |= 1ULL << k;
+            slot = k;
+            word = P.page + (size_t)k * kProgressStride;
+            break;
+        }
+    }
+    Progress(const Progress&) = delete;
+    // no kernel that could still write the word is in flight when it goes back
+    ~Progress() {
+        if (slot < 0) return;
+        if (!idle && cudaStreamSynchronize(st) != cudaSuccess) cudaGetLastError();
+        ProgressPool& P = progress_pool();
+        std::lock_guard<std::mutex> lock(P.mu);
+        P.used &= ~(1ULL << slot);
+    }
+    // before the launches of a cycle
+    void reset() {
+        if (word) *(volatile int*)word = 0;
+        idle = false;
+    }
+    // Waits until the device has finished `steps` steps of the cycle or ended it;
+    // true when it has ended.  A stream that runs dry (or fails) ends the wait.
+    bool wait(int steps) const {
+        if (!word) return false;
+        for (unsigned spin = 1;; ++spin) {
+            const int v = *(volatile int*)word;
+            if (v & kProgressDone) return true;
+            if (v >= steps) return false;
+            if (spin % 4096 == 0 && cudaStreamQuery(st) != cudaErrorNotReady) {
+                cudaGetLastError();
+                return (*(volatile int*)word & kProgressDone) != 0;
+            }
+        }
+    }
+};
+
+// Steps enqueued ahead of the device: the host needs 10 to 20 us to enqueue one
+// and the device at least 25 us to run it.
+constexpr int kAhead = 2;
 
 // Test hook of gnk_debug_barrier_fault, read by every later solve.
 std::atomic<int> g_bar_limit{kBarSpin};
@@ -1183,7 +1279,9 @@ int gmres(Boundary& b, int adjoint /* OpId */, int prec, const double* rhs, doub
     // Gram-Schmidt in double-float for every operator precision but plain FP64
     const bool dfa = prec != GNK_PREC_FP64;
     KState hs;
-    k_init_state<<<1, 1, 0, st>>>(ks, tol, restart, g_bar_limit.load(), g_bar_skip.load());
+    Progress prog(st);
+    prog.reset();
+    k_init_state<<<1, 1, 0, st>>>(ks, tol, restart, g_bar_limit.load(), g_bar_skip.load(), prog.word);
     KLAUNCH(vb, (k_norm<<<nb, KT, 0, st>>>(rhs, N, p, ks, 0)));
     count_launches(2);
     GNK_TRY_CUDA(cudaMemsetAsync(x, 0, N * sizeof(double), st));
@@ -1215,6 +1313,7 @@ int gmres(Boundary& b, int adjoint /* OpId */, int prec, const double* rhs, doub
             goto steps;
         }
         GNK_TRY(read_state(b, &hs, st));
+        prog.idle = true;
         if (cycle == 1 && hs.last_k == 0 && maxit > 0) res->cycles--;  // the first cycle did no step
         if (hs.bar_err) {
             set_error("GMRES: a grid barrier of the Arnoldi step timed out");
@@ -1245,8 +1344,11 @@ int gmres(Boundary& b, int adjoint /* OpId */, int prec, const double* rhs, doub
             break;
         }
         res->cycles++;
+        prog.reset();
     steps:
+        for (std::vector<long>& ids : step_ids) ids.clear();
         for (int j = 0; j < restart; ++j) {
+            if (j >= kAhead && prog.wait(j - kAhead + 1)) break;  // the cycle has ended: no empty launches
             double* vj = b.V + (size_t)j * N;
             double* w = b.V + (size_t)(j + 1) * N;
             const double nv = j + 1;

@@ -36,6 +36,7 @@
 #include <mutex>
 #include <string>
 #include <thread>
+#include <type_traits>
 #include <vector>
 
 #include "gnk_internal.h"
@@ -46,6 +47,8 @@ namespace {
 
 constexpr int BS = kSrcTile32;  // sources per tile (tile of the reference nodes)
 constexpr int BT = 256;         // threads per block, batched pair kernels
+constexpr int BN = 64;          // of them along the targets; the others split each source tile
+constexpr int BSL = BT / BN;    // source slices
 constexpr int KB = 256;         // threads per block, per-system vector kernels
 constexpr float kFarB = 1e18f;
 
@@ -65,7 +68,7 @@ struct BSys {
     int N, dom;
 };
 
-enum BEpi : int { BE_K = 0, BE_RESID = 1, BE_RESID_FC = 2, BE_RHS_FB = 3, BE_EONE = 4 };
+enum BEpi : int { BE_K = 0, BE_RESID = 1, BE_RESID_FC = 2, BE_RHS_FB = 3, BE_EONE = 4, BE_FC = 5 };
 
 struct BPairArgs {
     const BDom* dom;
@@ -78,12 +81,14 @@ struct BPairArgs {
     const float4* et32;
     const float4* ref32;
     const float2* off32;
-    const double2* q;
+    const float4* qd;    // q as double-float: (re.h, re.l, im.h, im.l)
     const float2* q32;
     const double2* A;
     const double* b1;
     const double* d1;
     const double* x;
+    const float* xf;     // x rounded to FP32 (FP32 kernel)
+    const float2* xd;    // x as double-float (double-float kernel)
     const double* rhs;
     const double* Lx;
     double* out;
@@ -113,6 +118,9 @@ __device__ __forceinline__ void bepilogue(const BPairArgs& a, const BDom& D, lon
             a.out[e] = -(-s2n * (A.x * zx - A.y * zy) - a.d1[node] * x + a.Lx[e]);
             a.out2[e] = fb;
             break;
+        case BE_FC:  // f_C(x), from Re(A z) alone
+            a.out[e] = -s2n * (A.x * zx - A.y * zy) - a.d1[node] * x + a.Lx[e];
+            break;
         case BE_EONE:  // x = 1: z = E q
             a.out[e] = -s2n * (A.x * zy + A.y * zx);
             a.out2[e] = -s2n * (A.x * zx - A.y * zy);
@@ -135,112 +143,167 @@ __device__ __forceinline__ bool group_done(const BPairArgs& a, const BDom& D, in
     return all;
 }
 
-// ---------------------------------------------------------------- FP32 persistent kernel
-template <int T, int RG>
-__global__ void __launch_bounds__(BT) bpair32_kernel(BPairArgs a) {
-    __shared__ float2 s_off[BS];
-    __shared__ float2 s_w[RG][BS];
-    __shared__ int s_it;
-    for (;;) {
-        const int it = next_item(a.counter, &s_it);
-        if (it >= a.nitems) return;
-        const BItem item = a.items[it];
-        const BDom D = a.dom[item.dom];
-        const int r0 = item.g * RG;
-        const int nr = min(RG, D.nrhs - r0);
-        if (group_done(a, D, r0, nr)) continue;
-        const int tgt0 = item.tile * (BT * T);
-        float4 th[T];
-        int idx[T];
-        float ox[T], oy[T], ax[T][RG], ay[T][RG];
-#pragma unroll
-        for (int t = 0; t < T; ++t) {
-            idx[t] = tgt0 + t * BT + threadIdx.x;
-            th[t] = a.et32[D.node_off + min(idx[t], D.N - 1)];
-#pragma unroll
-            for (int r = 0; r < RG; ++r) ax[t][r] = ay[t][r] = 0.f;
-        }
-        for (int tile = 0; tile < D.ntiles; ++tile) {
-            const int j0 = tile * BS;
-            const float4 ref = a.ref32[D.tile_off + tile];
-#pragma unroll
-            for (int t = 0; t < T; ++t) {
-                ox[t] = (th[t].x - ref.x) + (th[t].z - ref.z);
-                oy[t] = (th[t].y - ref.y) + (th[t].w - ref.w);
-            }
-            __syncthreads();
-            {
-                const int k = threadIdx.x, j = j0 + k;
-                if (j < D.N) {
-                    s_off[k] = a.off32[D.node_off + j];
-                    const float2 sc = a.q32[D.node_off + j];
-#pragma unroll
-                    for (int r = 0; r < RG; ++r) {
-                        const float xv = (r < nr) ? (float)a.x[D.vec_off + (long long)(r0 + r) * D.N + j] : 0.f;
-                        s_w[r][k] = make_float2(sc.x * xv, sc.y * xv);
-                    }
-                } else {
-                    s_off[k] = make_float2(kFarB, kFarB);
-#pragma unroll
-                    for (int r = 0; r < RG; ++r) s_w[r][k] = make_float2(0.f, 0.f);
-                }
-            }
-            __syncthreads();
-            const bool diag = (j0 < tgt0 + BT * T) && (tgt0 < j0 + BS);
-            if (!diag) {
-#pragma unroll 4
-                for (int k = 0; k < BS; ++k) {
-                    const float2 so = s_off[k];
-#pragma unroll
-                    for (int t = 0; t < T; ++t) {
-                        const float dx = ox[t] - so.x, dy = oy[t] - so.y;
-                        const float inv = recip_f32(fmaf(dx, dx, dy * dy));
-                        const float ar = dx * inv, ai = dy * inv;
-#pragma unroll
-                        for (int r = 0; r < RG; ++r) {
-                            const float2 w = s_w[r][k];
-                            ax[t][r] = fmaf(w.x, ar, fmaf(w.y, ai, ax[t][r]));
-                            ay[t][r] = fmaf(w.y, ar, fmaf(-w.x, ai, ay[t][r]));
-                        }
-                    }
-                }
-            } else {
-                for (int k = 0; k < BS; ++k) {
-                    const float2 so = s_off[k];
-#pragma unroll
-                    for (int t = 0; t < T; ++t) {
-                        const float dx = ox[t] - so.x, dy = oy[t] - so.y;
-                        float inv = recip_f32(fmaf(dx, dx, dy * dy));
-                        inv = (j0 + k == idx[t]) ? 0.f : inv;
-                        const float ar = dx * inv, ai = dy * inv;
-#pragma unroll
-                        for (int r = 0; r < RG; ++r) {
-                            const float2 w = s_w[r][k];
-                            ax[t][r] = fmaf(w.x, ar, fmaf(w.y, ai, ax[t][r]));
-                            ay[t][r] = fmaf(w.y, ar, fmaf(-w.x, ai, ay[t][r]));
-                        }
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < T; ++t) {
-            if (idx[t] < D.N) {
-#pragma unroll
-                for (int r = 0; r < RG; ++r)
-                    if (r < nr)
-                        bepilogue(a, D, D.vec_off + (long long)(r0 + r) * D.N + idx[t], D.node_off + idx[t],
-                                  (double)ax[t][r], (double)ay[t][r]);
-            }
-        }
+// ---------------------------------------------------------------- pair kernels
+// z_ir = sum_j x_jr Q_ij with Q_ij = q_j / (eta_i - eta_j) and real x: Q_ij is
+// formed once per pair and each right-hand side adds one real multiple of it (a
+// product of complex weights q_j x_jr with 1/d took four multiply-adds per
+// right-hand side, and 48 instructions instead of 12 per part in double-float).
+// With A real an operator K reads Im z alone (MODE 1) and f_C Re z alone (MODE
+// 2; MODE 0: both parts).  Per pair the FP32 kernel spends 6 + 2 shared
+// instructions a part and one per part and right-hand side, the double-float
+// one 49 + 16 a part and 12; two right-hand sides share
+// a packed float2 instruction.  The body is instantiated by the group's size,
+// so that a short last group does not pay for a full one.
+//
+// A block takes BN T targets; its threads split each tile of sources into BSL
+// slices, whose sums are added in slice order at the end.  (With one target per
+// thread and all sources in one thread a batch of 24 domains had 340 items, the
+// longest a serial chain of 8,192 sources: 0.82 ms for a product whose
+// arithmetic takes 0.17 ms; now 0.39 ms, and the double-float one 5.2 ms for both
+// parts and 3.7 ms for one, where it took 6.9 ms.)  x comes converted (bk_convert): conversions run on
+// the FP64 pipe, and every target tile reads every x.
+
+// x of a product in the kernels' own form: FP32, or double-float
+__global__ void bk_convert(long long L, const double* __restrict__ x, float* __restrict__ xf, float2* __restrict__ xd) {
+    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= L) return;
+    const double v = x[e];
+    if (xf) xf[e] = (float)v;
+    if (xd) {
+        const df d = df_split(v);
+        xd[e] = make_float2(d.h, d.l);
     }
 }
 
-// ---------------------------------------------------------------- double-float persistent kernel
-template <int T, int RG>
-__global__ void __launch_bounds__(BT) bpairdf_kernel(BPairArgs a) {
-    __shared__ float4 s_off[BS];
-    __shared__ float4 s_w[RG][BS];
+// FP32: NR right-hand sides (a multiple of 4; nr of them real)
+template <int T, int NR, int MODE>
+__device__ __forceinline__ void b32_item(const BPairArgs& a, const BDom& D, int tile0, int r0, int nr, float4* s_src,
+                                         float4* s_x) {
+    const int tl = threadIdx.x % BN, sl = threadIdx.x / BN;
+    const int tgt0 = tile0 * (BN * T);
+    float4 th[T];
+    int idx[T];
+    constexpr int PARTS = MODE == 0 ? 2 : 1;  // the imaginary part first
+    float2 acc[T][PARTS][NR / 2];
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+        idx[t] = tgt0 + t * BN + tl;
+        th[t] = a.et32[D.node_off + min(idx[t], D.N - 1)];
+#pragma unroll
+        for (int c = 0; c < PARTS; ++c)
+#pragma unroll
+            for (int r = 0; r < NR / 2; ++r) acc[t][c][r] = f2(0.f);
+    }
+    // the next tile's sources are loaded while the current one is summed
+    float4 n_src;
+    float n_x[NR];
+    auto fetch = [&](int tile) {
+        const int j = tile * BS + threadIdx.x;
+        const bool in = j < D.N;
+        float2 off = make_float2(kFarB, kFarB), q = make_float2(0.f, 0.f);
+        if (in) {
+            off = a.off32[D.node_off + j];
+            q = a.q32[D.node_off + j];
+        }
+        n_src = make_float4(off.x, off.y, q.x, q.y);
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+            n_x[r] = (in && r < nr) ? a.xf[D.vec_off + (long long)(r0 + r) * D.N + j] : 0.f;
+    };
+    fetch(0);
+    for (int tile = 0; tile < D.ntiles; ++tile) {
+        const int j0 = tile * BS;
+        const float4 ref = a.ref32[D.tile_off + tile];
+        float ox[T], oy[T];
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            ox[t] = (th[t].x - ref.x) + (th[t].z - ref.z);
+            oy[t] = (th[t].y - ref.y) + (th[t].w - ref.w);
+        }
+        __syncthreads();
+        s_src[threadIdx.x] = n_src;
+#pragma unroll
+        for (int r4 = 0; r4 < NR / 4; ++r4)
+            s_x[threadIdx.x * (NR / 4) + r4] =
+                make_float4(n_x[4 * r4], n_x[4 * r4 + 1], n_x[4 * r4 + 2], n_x[4 * r4 + 3]);
+        __syncthreads();
+        if (tile + 1 < D.ntiles) fetch(tile + 1);
+        const bool diag = (j0 < tgt0 + BN * T) && (tgt0 < j0 + BS);
+        auto pairs = [&](auto on_diag) {
+#pragma unroll 4
+            for (int k = sl * (BS / BSL); k < (sl + 1) * (BS / BSL); ++k) {
+                const float4 so = s_src[k];
+                float2 im[T], re[T];
+#pragma unroll
+                for (int t = 0; t < T; ++t) {
+                    const float dx = ox[t] - so.x, dy = oy[t] - so.y;
+                    float inv = recip_f32(fmaf(dx, dx, dy * dy));
+                    if (decltype(on_diag)::value) inv = (j0 + k == idx[t]) ? 0.f : inv;
+                    const float ar = dx * inv, ai = dy * inv;  // 1/d = ar - i ai
+                    if (MODE != 2) im[t] = f2(fmaf(so.w, ar, -(so.z * ai)));
+                    if (MODE != 1) re[t] = f2(fmaf(so.z, ar, so.w * ai));
+                }
+#pragma unroll
+                for (int r4 = 0; r4 < NR / 4; ++r4) {
+                    const float4 x = s_x[k * (NR / 4) + r4];
+                    const float2 x0 = make_float2(x.x, x.y), x1 = make_float2(x.z, x.w);
+#pragma unroll
+                    for (int t = 0; t < T; ++t) {
+                        if (MODE != 2) {
+                            acc[t][0][2 * r4] = fma2(x0, im[t], acc[t][0][2 * r4]);
+                            acc[t][0][2 * r4 + 1] = fma2(x1, im[t], acc[t][0][2 * r4 + 1]);
+                        }
+                        if (MODE != 1) {
+                            acc[t][PARTS - 1][2 * r4] = fma2(x0, re[t], acc[t][PARTS - 1][2 * r4]);
+                            acc[t][PARTS - 1][2 * r4 + 1] = fma2(x1, re[t], acc[t][PARTS - 1][2 * r4 + 1]);
+                        }
+                    }
+                }
+            }
+        };
+        if (diag)
+            pairs(std::true_type{});
+        else
+            pairs(std::false_type{});
+    }
+    // the slices' sums in slice order; thread (sl, tl) finishes right-hand sides sl, sl + BSL, ...
+    float* red = reinterpret_cast<float*>(s_x);  // [NR][BSL][BN]
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+        double z[PARTS][(NR + BSL - 1) / BSL];
+#pragma unroll
+        for (int c = 0; c < PARTS; ++c) {
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < NR; ++r)
+                red[(r * BSL + sl) * BN + tl] = (r & 1) ? acc[t][c][r / 2].y : acc[t][c][r / 2].x;
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < (NR + BSL - 1) / BSL; ++u) {
+                const int r = u * BSL + sl;
+                float v = red[r * BSL * BN + tl];
+#pragma unroll
+                for (int q = 1; q < BSL; ++q) v += red[(r * BSL + q) * BN + tl];
+                z[c][u] = (double)v;
+            }
+        }
+        if (idx[t] < D.N) {
+#pragma unroll
+            for (int u = 0; u < (NR + BSL - 1) / BSL; ++u) {
+                const int r = u * BSL + sl;
+                if (r < nr)
+                    bepilogue(a, D, D.vec_off + (long long)(r0 + r) * D.N + idx[t], D.node_off + idx[t],
+                              MODE != 1 ? z[PARTS - 1][u] : 0.0, MODE != 2 ? z[0][u] : 0.0);
+            }
+        }
+    }
+    __syncthreads();  // the next item reuses the shared arrays
+}
+
+template <int T, int RG, int MODE>
+__global__ void __launch_bounds__(BT) bpair32_kernel(BPairArgs a) {
+    __shared__ float4 s_src[BS];             // (offset, q)
+    __shared__ float4 s_x[BS * (RG / 4)];    // x of the group, [source][rhs]
     __shared__ int s_it;
     for (;;) {
         const int it = next_item(a.counter, &s_it);
@@ -250,93 +313,178 @@ __global__ void __launch_bounds__(BT) bpairdf_kernel(BPairArgs a) {
         const int r0 = item.g * RG;
         const int nr = min(RG, D.nrhs - r0);
         if (group_done(a, D, r0, nr)) continue;
-        const int tgt0 = item.tile * (BT * T);
-        double2 p[T];
-        int idx[T];
-        df are[T][RG], aim[T][RG];
+        if (RG > 4 && nr > 4)
+            b32_item<T, RG, MODE>(a, D, item.tile, r0, nr, s_src, s_x);
+        else
+            b32_item<T, 4, MODE>(a, D, item.tile, r0, nr, s_src, s_x);
+    }
+}
+
+// Double-float: NR right-hand sides (1 or even), T targets per thread.  At the
+// diagonal Q is multiplied by 0 through the reciprocal.
+template <int T, int NR, int MODE>
+__device__ __forceinline__ void bdf_item(const BPairArgs& a, const BDom& D, int tile0, int r0, int nr, float4* s_off,
+                                         float4* s_q, float4* s_x) {
+    constexpr int NP = (NR + 1) / 2;          // packed pairs of right-hand sides
+    constexpr int PARTS = MODE == 0 ? 2 : 1;  // the imaginary part first
+    const int tl = threadIdx.x % BN, sl = threadIdx.x / BN;
+    const int tgt0 = tile0 * (BN * T);
+    double2 p[T];
+    int idx[T];
+    df2 acc[T][PARTS][NP];
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+        idx[t] = tgt0 + t * BN + tl;
+        p[t] = a.et[D.node_off + min(idx[t], D.N - 1)];
+#pragma unroll
+        for (int c = 0; c < PARTS; ++c)
+#pragma unroll
+            for (int r = 0; r < NP; ++r) acc[t][c][r] = df2{f2(0.f), f2(0.f)};
+    }
+    float4 n_off, n_q, n_x[NP];
+    auto fetch = [&](int tile) {
+        const int j = tile * BS + threadIdx.x;
+        const bool in = j < D.N;
+        n_off = in ? a.offdf[D.node_off + j] : make_float4(kFarB, kFarB, 0.f, 0.f);
+        n_q = in ? a.qd[D.node_off + j] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int r = 0; r < NP; ++r) {
+            float2 v[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int rr = 2 * r + u;
+                v[u] = (in && rr < nr) ? a.xd[D.vec_off + (long long)(r0 + rr) * D.N + j] : make_float2(0.f, 0.f);
+            }
+            n_x[r] = make_float4(v[0].x, v[1].x, v[0].y, v[1].y);
+        }
+    };
+    fetch(0);
+    for (int tile = 0; tile < D.ntiles; ++tile) {
+        const int j0 = tile * BS;
+        const double2 ref = a.ref64[D.tile_off + tile];
+        df ox[T], oy[T];
 #pragma unroll
         for (int t = 0; t < T; ++t) {
-            idx[t] = tgt0 + t * BT + threadIdx.x;
-            p[t] = a.et[D.node_off + min(idx[t], D.N - 1)];
-#pragma unroll
-            for (int r = 0; r < RG; ++r) are[t][r] = aim[t][r] = df{0.f, 0.f};
+            ox[t] = df_split(p[t].x - ref.x);
+            oy[t] = df_split(p[t].y - ref.y);
         }
-        for (int tile = 0; tile < D.ntiles; ++tile) {
-            const int j0 = tile * BS;
-            const double2 ref = a.ref64[D.tile_off + tile];
-            df ox[T], oy[T];
+        __syncthreads();
+        s_off[threadIdx.x] = n_off;
+        s_q[threadIdx.x] = n_q;
+#pragma unroll
+        for (int r = 0; r < NP; ++r) s_x[threadIdx.x * NP + r] = n_x[r];
+        __syncthreads();
+        if (tile + 1 < D.ntiles) fetch(tile + 1);
+        const bool diag = (j0 < tgt0 + BN * T) && (tgt0 < j0 + BS);
+#pragma unroll 2
+        for (int k = sl * (BS / BSL); k < (sl + 1) * (BS / BSL); ++k) {
+            const float4 so = s_off[k], q4 = s_q[k];
+            const df qx{q4.x, q4.y}, qy{q4.z, q4.w};
+            df2 im[T], re[T];
 #pragma unroll
             for (int t = 0; t < T; ++t) {
-                ox[t] = df_split(p[t].x - ref.x);
-                oy[t] = df_split(p[t].y - ref.y);
-            }
-            __syncthreads();
-            {
-                const int k = threadIdx.x, j = j0 + k;
-                if (j < D.N) {
-                    s_off[k] = a.offdf[D.node_off + j];
-                    const double2 sc = a.q[D.node_off + j];
-#pragma unroll
-                    for (int r = 0; r < RG; ++r) {
-                        const double xv = (r < nr) ? a.x[D.vec_off + (long long)(r0 + r) * D.N + j] : 0.0;
-                        const df wx = df_split(sc.x * xv), wy = df_split(sc.y * xv);
-                        s_w[r][k] = make_float4(wx.h, wx.l, wy.h, wy.l);
-                    }
-                } else {
-                    s_off[k] = make_float4(kFarB, kFarB, 0.f, 0.f);
-#pragma unroll
-                    for (int r = 0; r < RG; ++r) s_w[r][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                const df dx = df_sub(ox[t].h, ox[t].l, so.x, so.z);
+                const df dy = df_sub(oy[t].h, oy[t].l, so.y, so.w);
+                const float px = __fmul_rn(dx.h, dx.h);
+                float ex = fmaf(dx.h, dx.h, -px);
+                ex = fmaf(dx.h, dx.l + dx.l, ex);
+                const float py = __fmul_rn(dy.h, dy.h);
+                float ey = fmaf(dy.h, dy.h, -py);
+                ey = fmaf(dy.h, dy.l + dy.l, ey);
+                float rh, rest;
+                two_sum(px, py, rh, rest);
+                const float rl = __fadd_rn(__fadd_rn(ex, ey), rest);
+                float y = recip_f32(rh);
+                if (diag && j0 + k == idx[t]) y = 0.f;
+                float e = fmaf(-rh, y, 1.0f);
+                e = fmaf(-rl, y, e);
+                const df inv = df{y, __fmul_rn(y, e)};
+                const df ar = df_mul(dx, inv);
+                const df ai = df_mul(dy, inv);
+                if (MODE != 2) {
+                    df u = df_mul(qy, ar);
+                    const df v = df_mul(qx, ai);
+                    df_acc(u, df{-v.h, -v.l});
+                    im[t] = df2{f2(u.h), f2(u.l)};
+                }
+                if (MODE != 1) {
+                    df w = df_mul(qx, ar);
+                    df_acc(w, df_mul(qy, ai));
+                    re[t] = df2{f2(w.h), f2(w.l)};
                 }
             }
-            __syncthreads();
-            const bool diag = (j0 < tgt0 + BT * T) && (tgt0 < j0 + BS);
-#pragma unroll 2
-            for (int k = 0; k < BS; ++k) {
-                const float4 so = s_off[k];
+#pragma unroll
+            for (int r = 0; r < NP; ++r) {
+                const float4 xv = s_x[k * NP + r];
+                const df2 x{make_float2(xv.x, xv.y), make_float2(xv.z, xv.w)};
 #pragma unroll
                 for (int t = 0; t < T; ++t) {
-                    const df dx = df_sub(ox[t].h, ox[t].l, so.x, so.z);
-                    const df dy = df_sub(oy[t].h, oy[t].l, so.y, so.w);
-                    const float px = __fmul_rn(dx.h, dx.h);
-                    float ex = fmaf(dx.h, dx.h, -px);
-                    ex = fmaf(dx.h, dx.l + dx.l, ex);
-                    const float py = __fmul_rn(dy.h, dy.h);
-                    float ey = fmaf(dy.h, dy.h, -py);
-                    ey = fmaf(dy.h, dy.l + dy.l, ey);
-                    float rh, re;
-                    two_sum(px, py, rh, re);
-                    const float rl = __fadd_rn(__fadd_rn(ex, ey), re);
-                    float y = recip_f32(rh);
-                    if (diag && j0 + k == idx[t]) y = 0.f;
-                    float e = fmaf(-rh, y, 1.0f);
-                    e = fmaf(-rl, y, e);
-                    const df inv = df{y, __fmul_rn(y, e)};
-                    const df ar = df_mul(dx, inv);
-                    const df ai = df_mul(dy, inv);
-#pragma unroll
-                    for (int r = 0; r < RG; ++r) {
-                        const float4 w = s_w[r][k];
-                        const df wx{w.x, w.y}, wy{w.z, w.w};
-                        df_acc(are[t][r], df_mul(wx, ar));
-                        df_acc(are[t][r], df_mul(wy, ai));
-                        df_acc(aim[t][r], df_mul(wy, ar));
-                        const df qq = df_mul(wx, ai);
-                        df_acc(aim[t][r], df{-qq.h, -qq.l});
-                    }
+                    if (MODE != 2) df2_acc(acc[t][0][r], df2_mul(x, im[t]));
+                    if (MODE != 1) df2_acc(acc[t][PARTS - 1][r], df2_mul(x, re[t]));
                 }
             }
         }
+    }
+    // as in the FP32 kernel; the slices' sums are compensated
+    float2* red = reinterpret_cast<float2*>(s_x);  // [2 NP][BSL][BN]
+    constexpr int NU = (2 * NP + BSL - 1) / BSL;
 #pragma unroll
-        for (int t = 0; t < T; ++t) {
-            if (idx[t] < D.N) {
+    for (int t = 0; t < T; ++t) {
+        double z[PARTS][NU];
 #pragma unroll
-                for (int r = 0; r < RG; ++r)
-                    if (r < nr)
-                        bepilogue(a, D, D.vec_off + (long long)(r0 + r) * D.N + idx[t], D.node_off + idx[t],
-                                  (double)are[t][r].h + (double)are[t][r].l,
-                                  (double)aim[t][r].h + (double)aim[t][r].l);
+        for (int c = 0; c < PARTS; ++c) {
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < NP; ++r) {
+                const df2 v = acc[t][c][r];
+                red[((2 * r) * BSL + sl) * BN + tl] = make_float2(v.h.x, v.l.x);
+                red[((2 * r + 1) * BSL + sl) * BN + tl] = make_float2(v.h.y, v.l.y);
+            }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < NU; ++u) {
+                const int r = min(u * BSL + sl, 2 * NP - 1);
+                const float2 f = red[r * BSL * BN + tl];
+                df v{f.x, f.y};
+#pragma unroll
+                for (int q = 1; q < BSL; ++q) {
+                    const float2 g = red[(r * BSL + q) * BN + tl];
+                    df_acc(v, df{g.x, g.y});
+                }
+                z[c][u] = (double)v.h + (double)v.l;
             }
         }
+        if (idx[t] < D.N) {
+#pragma unroll
+            for (int u = 0; u < NU; ++u) {
+                const int r = u * BSL + sl;
+                if (r < nr)
+                    bepilogue(a, D, D.vec_off + (long long)(r0 + r) * D.N + idx[t], D.node_off + idx[t],
+                              MODE != 1 ? z[PARTS - 1][u] : 0.0, MODE != 2 ? z[0][u] : 0.0);
+            }
+        }
+    }
+    __syncthreads();  // the next item reuses the shared arrays
+}
+
+template <int T, int RG, int MODE>
+__global__ void __launch_bounds__(BT) bpairdf_kernel(BPairArgs a) {
+    __shared__ float4 s_off[BS];
+    __shared__ float4 s_q[BS];
+    __shared__ float4 s_x[BS * ((RG + 1) / 2)];  // x of the group: (h, h, l, l) of two right-hand sides
+    __shared__ int s_it;
+    for (;;) {
+        const int it = next_item(a.counter, &s_it);
+        if (it >= a.nitems) return;
+        const BItem item = a.items[it];
+        const BDom D = a.dom[item.dom];
+        const int r0 = item.g * RG;
+        const int nr = min(RG, D.nrhs - r0);
+        if (group_done(a, D, r0, nr)) continue;
+        if (RG > 2 && nr > 2)
+            bdf_item<T, RG, MODE>(a, D, item.tile, r0, nr, s_off, s_q, s_x);
+        else
+            bdf_item<T, (RG > 2 ? 2 : RG), MODE>(a, D, item.tile, r0, nr, s_off, s_q, s_x);
     }
 }
 
@@ -609,6 +757,7 @@ int dalloc(P** p, size_t count) {
 // ---------------------------------------------------------------- batch handle
 struct BatchImpl {
     int ndom = 0, Ntot = 0, ntiles = 0, nsys = 0, nhk = 0, nmax = 0;
+    int A_real = 0;  // Im A = 0 at every node of the batch
     long long L = 0;
     int sms = 0;
     std::vector<BDom> hdom, hdom1;
@@ -637,6 +786,8 @@ struct BatchImpl {
     BItem* itemsdf1 = nullptr;
     int nitemsdf1 = 0;
     unsigned* counter = nullptr;
+    float4* qd = nullptr;     // q as double-float
+    float2* xconv = nullptr;  // L entries: x of the running product, converted
     float tune_ms[8] = {0};
     // vectors (L doubles each)
     double *rhs = nullptr, *x = nullptr, *r = nullptr, *rr = nullptr, *dd = nullptr, *fb = nullptr,
@@ -665,11 +816,11 @@ namespace {
 std::vector<BItem> make_items(const std::vector<BDom>& D, int T, int RG) {
     std::vector<BItem> v;
     for (int d = 0; d < (int)D.size(); ++d) {
-        const int tiles = (D[d].N + BT * T - 1) / (BT * T);
+        const int tiles = (D[d].N + BN * T - 1) / (BN * T);
         const int groups = (D[d].nrhs + RG - 1) / RG;
         for (int t = 0; t < tiles; ++t)
             for (int g = 0; g < groups; ++g) {
-                const int nt = std::min(BT * T, D[d].N - t * BT * T);
+                const int nt = std::min(BN * T, D[d].N - t * BN * T);
                 const int nr = std::min(RG, D[d].nrhs - g * RG);
                 BItem it{d, t, g, 0};
                 // cost in units of 4096 pair-evaluations (for the longest-first order)
@@ -692,7 +843,7 @@ BPairArgs base_args(const BatchImpl& B, const BDom* dom) {
     a.et32 = B.et32;
     a.ref32 = B.ref32;
     a.off32 = B.off32;
-    a.q = B.q;
+    a.qd = B.qd;
     a.q32 = B.q32;
     a.A = B.A;
     a.b1 = B.b1;
@@ -700,26 +851,50 @@ BPairArgs base_args(const BatchImpl& B, const BDom* dom) {
     return a;
 }
 
+// Parts of z that the epilogue reads with real A: K Im z alone, f_C Re z alone
+// (1, 2); else both (0).
+int mode_needed(const BatchImpl& B, int epi) {
+    if (!B.A_real) return 0;
+    return (epi == BE_K || epi == BE_RESID) ? 1 : (epi == BE_FC ? 2 : 0);
+}
+
+template <int T, int RG, int MODE>
+cudaError_t launch32_shape(const BatchImpl& B, const BPairArgs& a, cudaStream_t st) {
+    int nb = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, bpair32_kernel<T, RG, MODE>, BT, 0);
+    bpair32_kernel<T, RG, MODE><<<std::max(1, nb) * B.sms, BT, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
+template <int T, int RG, int MODE>
+cudaError_t launchdf_shape(const BatchImpl& B, const BPairArgs& a, cudaStream_t st) {
+    int nb = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, bpairdf_kernel<T, RG, MODE>, BT, 0);
+    bpairdf_kernel<T, RG, MODE><<<std::max(1, nb) * B.sms, BT, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
 int launch32(const BatchImpl& B, BPairArgs a, int T, int RG, const BItem* items, int nitems, cudaStream_t st) {
     a.items = items;
     a.nitems = nitems;
     GNK_TRY_CUDA(cudaMemsetAsync(B.counter, 0, sizeof(unsigned), st));
-    int nb = 1;
-    const int slots = B.sms;
+    const int mode = mode_needed(B, a.epi);
+    const long long L = (a.dom == B.dom1) ? B.Ntot : B.L;  // length of x
+    a.xf = reinterpret_cast<float*>(B.xconv);
+    bk_convert<<<(unsigned)((L + 255) / 256), 256, 0, st>>>(L, a.x, reinterpret_cast<float*>(B.xconv), nullptr);
     const ProfToken tok = prof_begin(st);
-#define L32(TT, GG)                                                                                   \
-    if (T == TT && RG == GG) {                                                                        \
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, bpair32_kernel<TT, GG>, BT, 0);           \
-        bpair32_kernel<TT, GG><<<std::max(1, nb) * slots, BT, 0, st>>>(a);                           \
-    }
-    L32(1, 8) else L32(2, 4) else L32(2, 8) else L32(4, 4) else {
-        set_error("batch: no FP32 kernel variant T=%d RG=%d", T, RG);
-        return GNK_EINVAL;
-    }
+    cudaError_t e = cudaErrorInvalidValue;
+#define L32(TT, GG)                                                                                              \
+    if (T == TT && RG == GG)                                                                                     \
+    e = (mode == 1) ? launch32_shape<TT, GG, 1>(B, a, st) : launch32_shape<TT, GG, 0>(B, a, st)
+    L32(1, 8);
+    L32(2, 4);
+    L32(2, 8);
+    L32(4, 4);
 #undef L32
-    GNK_TRY_CUDA(cudaGetLastError());
+    GNK_TRY_CUDA(e);
     prof_end(tok, PK_PAIR32, 0.0, st);
-    count_launches(2);
+    count_launches(3);
     return GNK_OK;
 }
 
@@ -727,22 +902,25 @@ int launchdf(const BatchImpl& B, BPairArgs a, int T, int RG, const BItem* items,
     a.items = items;
     a.nitems = nitems;
     GNK_TRY_CUDA(cudaMemsetAsync(B.counter, 0, sizeof(unsigned), st));
-    int nb = 1;
-    const int slots = B.sms;
+    const int mode = mode_needed(B, a.epi);
+    const long long L = (a.dom == B.dom1) ? B.Ntot : B.L;  // length of x
+    a.xd = B.xconv;
+    bk_convert<<<(unsigned)((L + 255) / 256), 256, 0, st>>>(L, a.x, nullptr, B.xconv);
     const ProfToken tok = prof_begin(st);
-#define LDF(TT, GG)                                                                                   \
-    if (T == TT && RG == GG) {                                                                        \
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, bpairdf_kernel<TT, GG>, BT, 0);           \
-        bpairdf_kernel<TT, GG><<<std::max(1, nb) * slots, BT, 0, st>>>(a);                           \
-    }
-    LDF(1, 1) else LDF(1, 2) else LDF(1, 4) else LDF(2, 2) else {
-        set_error("batch: no double-float kernel variant T=%d RG=%d", T, RG);
-        return GNK_EINVAL;
-    }
+    cudaError_t e = cudaErrorInvalidValue;
+#define LDF(TT, GG)                                                                                              \
+    if (T == TT && RG == GG)                                                                                     \
+    e = (mode == 1)   ? launchdf_shape<TT, GG, 1>(B, a, st)                                                          \
+        : (mode == 2) ? launchdf_shape<TT, GG, 2>(B, a, st)                                                          \
+                      : launchdf_shape<TT, GG, 0>(B, a, st)
+    LDF(1, 1);
+    LDF(1, 2);
+    LDF(1, 4);
+    LDF(2, 2);
 #undef LDF
-    GNK_TRY_CUDA(cudaGetLastError());
+    GNK_TRY_CUDA(e);
     prof_end(tok, PK_PAIRDF, 0.0, st);
-    count_launches(2);
+    count_launches(3);
     return GNK_OK;
 }
 
@@ -805,10 +983,20 @@ float time_variant(F launch, cudaStream_t st) {
 }
 
 int autotune(BatchImpl& B, cudaStream_t st) {
-    // sample: every 8th domain (all of them for small batches)
-    std::vector<BDom> sample;
-    for (int d = 0; d < B.ndom; ++d)
-        if (B.ndom < 16 || d % 8 == 0) sample.push_back(B.hdom[d]);
+    // sample: the domains with the most work, until they hold an eighth of the
+    // batch's; the FP32 shapes, whose products are short, on the whole batch while
+    // that takes a few ms (the balance of its items over the SMs then decides, not
+    // the rate)
+    auto work_of = [](const BDom& D) { return (double)D.N * D.N * D.nrhs; };
+    std::vector<BDom> sampledf = B.hdom;
+    std::stable_sort(sampledf.begin(), sampledf.end(),
+                     [&](const BDom& x, const BDom& y) { return work_of(x) > work_of(y); });
+    double work = 0.0, held = 0.0;
+    for (const BDom& D : B.hdom) work += work_of(D);
+    size_t ns = 0;
+    while (ns < sampledf.size() && held < work / 8.0) held += work_of(sampledf[ns++]);
+    sampledf.resize(ns);
+    const std::vector<BDom>& sample = (work < 1e10) ? B.hdom : sampledf;
     BDom* dsample = nullptr;
     GNK_TRY(dalloc(&dsample, sample.size()));
     GNK_TRY_CUDA(cudaMemcpyAsync(dsample, sample.data(), sample.size() * sizeof(BDom), cudaMemcpyHostToDevice, st));
@@ -835,8 +1023,14 @@ int autotune(BatchImpl& B, cudaStream_t st) {
         }
     }
     best = 1e30f;
+    if (rc == GNK_OK &&
+        cudaMemcpyAsync(dsample, sampledf.data(), sampledf.size() * sizeof(BDom), cudaMemcpyHostToDevice, st) !=
+            cudaSuccess) {
+        set_error("batch: upload of the tuning sample failed");
+        rc = GNK_ECUDA;
+    }
     for (int v = 0; v < 3 && rc == GNK_OK; ++v) {
-        rc = upload_items(make_items(sample, vdf[v][0], vdf[v][1]), &it, &nit, st);
+        rc = upload_items(make_items(sampledf, vdf[v][0], vdf[v][1]), &it, &nit, st);
         if (rc != GNK_OK) break;
         const float ms = time_variant([&] { launchdf(B, a, vdf[v][0], vdf[v][1], it, nit, st); }, st);
         B.tune_ms[4 + v] = ms;
@@ -861,7 +1055,7 @@ void release_batch(BatchImpl& B) {
     B.wstreams.clear();
     void* p[] = {B.dom, B.dom1, B.sys, B.hk_off, B.et, B.etp, B.A, B.q, B.ref64, B.Eone, B.b1, B.d1, B.e, B.ones,
                  B.et32, B.ref32, B.offdf, B.off32, B.q32, B.A32, B.twid, B.lcol, B.cdesc, B.cbase, B.items32,
-                 B.itemsdf, B.itemsdf1, B.counter, B.rhs, B.x, B.r, B.rr, B.dd, B.fb, B.fc, B.Lx, B.k.V, B.k.H,
+                 B.itemsdf, B.itemsdf1, B.counter, B.xconv, B.qd, B.rhs, B.x, B.r, B.rr, B.dd, B.fb, B.fc, B.Lx, B.k.V, B.k.H,
                  B.k.g, B.k.cs, B.k.sn, B.k.y, B.k.h1, B.k.h2, B.k.beta, B.k.done, B.k.kst,
                  B.k.unconv, B.k.nonfinite, B.bnorm_in, B.bnorm_out, B.relres, B.oconv};
     for (void* q : p)
@@ -964,7 +1158,7 @@ int gmres_batch(BatchImpl& B, const double* rhs, double* x, int R, int maxit, do
         GNK_TRY_CUDA(cudaStreamSynchronize(st));
         if (unconv == 0 || cycle == maxit) break;
         GNK_TRY_CUDA(cudaGraphLaunch(B.graph, st));
-        count_launches((unsigned long long)R * 5);
+        count_launches((unsigned long long)R * 6);
         bk_update_x<<<ns, KB, 0, st>>>(B.k, x);
         GNK_TRY_CUDA(cudaGetLastError());
         count_launches(1);
@@ -1232,6 +1426,8 @@ int gnk_build_batch(gnk_batch** out, int ndom, const int* m1, const int* n, cons
     TRYB(dalloc(&B.cbase, base.size()));
     TRYB(dalloc(&B.counter, 1));
     const size_t Lz = (size_t)L;
+    TRYB(dalloc(&B.xconv, std::max(Lz, N)));
+    TRYB(dalloc(&B.qd, N));
     TRYB(dalloc(&B.rhs, Lz));
     TRYB(dalloc(&B.x, Lz));
     TRYB(dalloc(&B.r, Lz));
@@ -1305,6 +1501,10 @@ int gnk_build_batch(gnk_batch** out, int ndom, const int* m1, const int* n, cons
         set_error("gnk_build_batch: non-finite geometry or A = 0 at a node");
         return fail(hflag & 1 ? GNK_ENONFINITE : GNK_EINVAL);
     }
+    B.A_real = (hflag & 4) ? 0 : 1;
+    bk_convert<<<(unsigned)((2 * N + 255) / 256), 256, 0, st>>>(2 * (long long)N, reinterpret_cast<const double*>(B.q),
+                                                                nullptr, reinterpret_cast<float2*>(B.qd));
+    count_launches(1);
     // ones, Eone (double-float), diag(B1), diag(D1)
     {
         std::vector<double> one(N, 1.0);
@@ -1476,7 +1676,6 @@ int gnk_batch_fbie(const gnk_batch* hc, const double* gam, double* mu, double* h
     count_launches(1);
     GNK_TRY_CUDA(cudaMemsetAsync(B.x, 0, Lb, st));
     GNK_TRY_CUDA(cudaMemsetAsync(B.fc, 0, Lb, st));  // f_C(0) = 0 for systems that never move
-    bool fc_valid = false;
     int status = GNK_ENOTCONV;
     for (int it = 0;; ++it) {
         GNK_TRY_CUDA(cudaMemsetAsync(B.k.unconv, 0, sizeof(unsigned), st));
@@ -1502,24 +1701,33 @@ int gnk_batch_fbie(const gnk_batch* hc, const double* gam, double* mu, double* h
         res.matvecs_fp32 += steps;
         bk_axpy<<<(unsigned)((B.L + 255) / 256), 256, 0, st>>>(B.L, B.x, B.dd);
         count_launches(1);
-        // outer residual and f_C(x) in double-float
-        GNK_TRY(run_batch_circulant(B.cdesc, B.cbase, B.ncirc, B.nmax, B.x, B.Lx, B.twid, B.lcol, st));
-        // groups whose systems had all converged are skipped: their x did not
-        // move, their residual stays 0 and their f_C(x) stays valid
+        // outer residual in double-float; with complex A f_C(x) comes from the same
+        // sums, with real A (whose residual reads Im z alone) from one sum of Re z
+        // after the last.  Groups whose systems had all converged are skipped:
+        // their x did not move, their residual stays 0 and their f_C(x) stays valid.
+        if (!B.A_real)
+            GNK_TRY(run_batch_circulant(B.cdesc, B.cbase, B.ncirc, B.nmax, B.x, B.Lx, B.twid, B.lcol, st));
         BPairArgs a = base_args(B, B.dom);
         a.x = B.x;
         a.rhs = B.rhs;
         a.Lx = B.Lx;
         a.out = B.rr;
         a.out2 = B.fc;
-        a.epi = BE_RESID_FC;
+        a.epi = B.A_real ? BE_RESID : BE_RESID_FC;
         a.sys_done = B.oconv;
         GNK_TRY(launchdf(B, a, B.Tdf, B.RGdf, B.itemsdf, B.nitemsdf, st));
         res.matvecs_fp64++;
         res.refinements++;
-        fc_valid = true;
     }
-    (void)fc_valid;
+    if (B.A_real && res.refinements > 0) {
+        GNK_TRY(run_batch_circulant(B.cdesc, B.cbase, B.ncirc, B.nmax, B.x, B.Lx, B.twid, B.lcol, st));
+        BPairArgs a = base_args(B, B.dom);
+        a.x = B.x;
+        a.Lx = B.Lx;
+        a.out = B.fc;
+        a.epi = BE_FC;
+        GNK_TRY(launchdf(B, a, B.Tdf, B.RGdf, B.itemsdf, B.nitemsdf, st));
+    }
     // h = (f_C(mu) - f_B(gamma)) / 2, h_k per system
     bk_half_diff<<<(unsigned)((B.L + 255) / 256), 256, 0, st>>>(B.L, B.fc, B.fb, B.dd);
     count_launches(1);

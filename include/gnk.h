@@ -221,8 +221,9 @@ int gnk_build_boundary(gnk_boundary** out, int m1, int n,
  * will be differentiated keeps to one fixed sequence of operations.  Beside a
  * graded corner the nodes are as close as n^-3 and dL/d eta sums 1/d^2: the last
  * bit of mu or lambda moves it by 1e-7 of its norm at n = 2048.  Other handles
- * take faster sequences of the same accuracy (the solves of the adjoint and the
- * transposed equation read their near field from an operator cache). */
+ * take faster sequences of the same accuracy (multipole-to-local translations on
+ * the tensor cores; the solves of the adjoint and the transposed equation read
+ * their near field from an operator cache). */
 #define GNK_BUILD_DIFF 0x400
 int gnk_build_boundary_ex(gnk_boundary** out, int m1, int n,
                           const double* et, const double* etp, const double* etpp,

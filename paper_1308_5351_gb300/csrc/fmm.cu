@@ -32,6 +32,8 @@
 // level L = the deepest level whose non-empty boxes hold at least kFmmLeaf
 // nodes on average, interaction and neighbour lists.  Every sum on the device
 // runs in a fixed order, so results are reproducible.
+#include <cuda_fp16.h>
+
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -73,6 +75,8 @@ struct FmmArgs {
     const float2* m2lH;   // C(k+l, l), [k][l] double-float
     const float4* m2lS;   // per offset code: (-1)^(k+1) delta^-(k+1), then delta^-l
     const float2* bUp;    // C(l, m) at [l][m] (0 for l < m): the L2L Pascal sums
+    const float4* m2lT;   // per offset code: (-1)^(k+1) (2/delta)^k / delta, then (2/delta)^l
+    const uint4* m2lA;    // digits of C(k+l, l) 2^-(k+l) as mma fragments
     float4* mult;
     float4* loc;
     float4* ws;
@@ -517,6 +521,182 @@ __device__ __forceinline__ df2 df2_add(df2 a, df2 b) {
     r.h = add2(s, e);
     r.l = sub2(e, sub2(r.h, s));
     return r;
+}
+
+// ---- M2L on the tensor cores.  With x_k = (-1)^(k+1) (2/delta)^k / delta a_k
+//   b_l = (1/r) (2/delta)^l sum_k C'(k, l) x_k,   C'(k, l) = C(k+l, l) 2^-(k+l) <= 1:
+// for all pairs of boxes one fixed real 32 x 32 matrix times a real matrix whose
+// columns are the pairs' real and imaginary parts.  Both sides are split into
+// kTcD signed digits of 10 bits (C' once, x per pair below a power of two above
+// its largest entry), exact in FP16; the products of digits i and j with
+// i + j <= kTcD accumulate in FP32 by i + j, and every such sum is an integer
+// below 2^24 (for C' the row sums of its digits bound it), so the tensor cores
+// add them without rounding.  What is dropped is below 2^-49 of the largest
+// entry times the row sum (<= 2); the double-float form rounds at 2^-46 per term.
+// Four pairs make the eight columns of an m16n8k16 tile (lane g = lane / 4 forms
+// the B fragment of column g: pair g / 2, part g mod 2; lane t = lane mod 4
+// receives both parts of pair t), 76 mma per tile of four pairs.  The legacy
+// mma.sync is enough: the tensor work is 2 us of a product, the splits, the
+// scalings and the sums around it bound the kernel, and a tcgen05 tile of 128
+// rows would be three quarters padding.  An M2L pair takes about 150 instructions
+// of a warp; the double-float form 960.  Beside the near field it takes 15.6 us at
+// 65,536 nodes (19,700 pairs) and 78 us at 524,288 (135,500); before 35 and 165 us.
+// A warp takes tiles of four entries of the box's interaction list; the warps'
+// sums are added in warp order.
+constexpr int kTcD = 5;
+constexpr int kTcWarps = 4;
+
+__device__ __forceinline__ void mma_f16(float (&c)[4], const uint4 a, unsigned b0, unsigned b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+
+// round to nearest integer, |v| < 2^22, two lanes
+__device__ __forceinline__ float2 rint2(float2 v) {
+    const float2 M = f2(12582912.f);  // 1.5 2^23
+    return sub2(add2(v, M), M);
+}
+
+__device__ __forceinline__ unsigned half2_bits(float2 v) {
+    const __half2 h = __floats2half2_rn(v.x, v.y);
+    return *reinterpret_cast<const unsigned*>(&h);
+}
+
+template <int R>
+__global__ void __launch_bounds__(32 * kTcWarps) fmm_m2l_tc_kernel(FmmArgs a) {
+    __shared__ float4 s_acc[kTcWarps][32];
+    if (a.done != nullptr && *a.done) return;
+    const int box = blockIdx.x, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g = lane >> 2, t = lane & 3, part = g & 1;
+    const unsigned full = 0xffffffffu;
+    const int e0 = a.il_start[box], e1 = a.il_start[box + 1];
+    const df sc = df_split_fast(recip_f64(a.width[box]));
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        df2 acc[4];  // (re, im) of rows l = g + 8 i
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] = df2{f2(0.f), f2(0.f)};
+        for (int base = e0 + 4 * wid; base < e1; base += 4 * kTcWarps) {
+            // x of pair g / 2, part g mod 2, at k = 2t, 2t + 1 (+ 8, + 16, + 24): two k per float2
+            const int eb = min(base + (g >> 1), e1 - 1);
+            const float4* S = a.m2lT + (size_t)a.il_off[eb] * 2 * kFmmP;
+            const float4* A = a.mult + ((size_t)r * a.nbox + a.il_src[eb]) * kFmmP;
+            const bool live = base + (g >> 1) < e1;
+            df2 x[4];
+            float mx = 0.f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int k = 2 * t + 8 * q;
+                const float4 a0 = __ldcg(A + k), a1 = __ldcg(A + k + 1), s0 = __ldg(S + k), s1 = __ldg(S + k + 1);
+                const df2 ar{make_float2(a0.x, a1.x), make_float2(a0.y, a1.y)};
+                const df2 ai{make_float2(a0.z, a1.z), make_float2(a0.w, a1.w)};
+                const df2 sr{make_float2(s0.x, s1.x), make_float2(s0.y, s1.y)};
+                const df2 si{make_float2(s0.z, s1.z), make_float2(s0.w, s1.w)};
+                // re = sr ar - si ai, im = sr ai + si ar
+                const df2 u = part ? ai : ar, v = part ? ar : df2{neg2(ai.h), neg2(ai.l)};
+                df2 w = df2_mul(sr, u);
+                df2_acc(w, df2_mul(si, v));
+                x[q].h = add2(w.h, w.l);
+                x[q].l = sub2(w.l, sub2(x[q].h, w.h));
+                if (!live) x[q] = df2{f2(0.f), f2(0.f)};
+                mx = fmaxf(mx, fmaxf(fabsf(x[q].h.x), fabsf(x[q].h.y)));
+            }
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(full, mx, o));  // lanes of the pair
+            const int ex = max((int)(__float_as_uint(mx) >> 23), 8);  // mx < 2^(ex - 126)
+            // digits of 2^(135 - ex) x (below 512), as B fragments: k tiles 0 (q = 0, 1) and 1 (q = 2, 3)
+            unsigned B[kTcD][4];
+            {
+                const float2 up = f2(__uint_as_float((unsigned)(262 - ex) << 23)), K = f2(1024.f);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float2 h = mul2(x[q].h, up), l = mul2(mul2(x[q].l, up), f2(1048576.f));
+                    float2 d = rint2(h);
+                    B[0][q] = half2_bits(d);
+                    float2 v = mul2(sub2(h, d), K);
+                    d = rint2(v);
+                    B[1][q] = half2_bits(d);
+                    v = mul2(sub2(v, d), K);
+                    d = rint2(add2(v, l));
+                    B[2][q] = half2_bits(d);
+                    v = mul2(add2(sub2(v, d), l), K);  // exact: d is the nearest integer to v + l
+                    d = rint2(v);
+                    B[3][q] = half2_bits(d);
+                    v = mul2(sub2(v, d), K);
+                    B[4][q] = half2_bits(rint2(v));
+                }
+            }
+            float c[kTcD + 1][2][4];
+#pragma unroll
+            for (int s = 0; s <= kTcD; ++s)
+#pragma unroll
+                for (int m = 0; m < 2; ++m)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) c[s][m][u] = 0.f;
+#pragma unroll
+            for (int i = 0; i < kTcD; ++i) {
+                uint4 H[2][2];
+#pragma unroll
+                for (int m = 0; m < 2; ++m)
+#pragma unroll
+                    for (int kt = 0; kt < 2; ++kt) H[m][kt] = __ldg(a.m2lA + ((i * 2 + m) * 2 + kt) * 32 + lane);
+#pragma unroll
+                for (int j = 0; j < kTcD; ++j) {
+                    if (i + j > kTcD) continue;
+#pragma unroll
+                    for (int m = 0; m < 2; ++m)
+#pragma unroll
+                        for (int kt = 0; kt < 2; ++kt) mma_f16(c[i + j][m], H[m][kt], B[j][2 * kt], B[j][2 * kt + 1]);
+                }
+            }
+            // pair t: y_l = 2^(ex - 126) sum_s c_s 2^(-18 - 10 s), then (2/delta)^l y_l
+            const int ec = base + t < e1 ? base + t : e1 - 1;
+            const float4* Q = a.m2lT + ((size_t)a.il_off[ec] * 2 + 1) * kFmmP;
+            const int ext = __shfl_sync(full, ex, 8 * t);
+            const float2 dn = f2(__uint_as_float((unsigned)(min(ext, 253) + 1) << 23));
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float2 v[kTcD + 1];
+                float w = 1.f / 262144.f;
+#pragma unroll
+                for (int s = 0; s <= kTcD; ++s) {
+                    v[s] = mul2(make_float2(c[s][i >> 1][2 * (i & 1)], c[s][i >> 1][2 * (i & 1) + 1]), f2(w));
+                    w *= 1.f / 1024.f;
+                }
+                float2 h, l0, l1;
+                two_sum2(v[0], v[1], h, l0);
+                two_sum2(h, v[2], h, l1);
+                l0 = add2(add2(l0, l1), add2(v[3], add2(v[4], v[5])));
+                df2 y;
+                y.h = add2(h, l0);
+                y.l = mul2(sub2(l0, sub2(y.h, h)), dn);
+                y.h = mul2(y.h, dn);
+                const float4 q4 = __ldg(Q + g + 8 * i);
+                df2_acc(acc[i], df2_mul(y, df2{f2(q4.x), f2(q4.y)}));
+                const df2 yx{make_float2(y.h.y, y.h.x), make_float2(y.l.y, y.l.x)};
+                df2_acc(acc[i], df2_mul(yx, df2{make_float2(-q4.z, q4.z), make_float2(-q4.w, q4.w)}));
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {  // over the four pairs of the lanes t, in a fixed order
+#pragma unroll
+            for (int o = 1; o < 4; o <<= 1) {
+                df2 v;
+                v.h = make_float2(__shfl_xor_sync(full, acc[i].h.x, o), __shfl_xor_sync(full, acc[i].h.y, o));
+                v.l = make_float2(__shfl_xor_sync(full, acc[i].l.x, o), __shfl_xor_sync(full, acc[i].l.y, o));
+                acc[i] = df2_add(acc[i], v);
+            }
+            if (t == 0) s_acc[wid][g + 8 * i] = make_float4(acc[i].h.x, acc[i].l.x, acc[i].h.y, acc[i].l.y);
+        }
+        __syncthreads();
+        if (wid == 0) {
+            cdf b = cdf_of(s_acc[0][lane]);
+            for (int w = 1; w < kTcWarps; ++w) b = cdf_add(b, cdf_of(s_acc[w][lane]));
+            a.loc[((size_t)r * a.nbox + box) * kFmmP + lane] = cdf_pack(cdf{df_mul(b.re, sc), df_mul(b.im, sc)});
+        }
+        if (R > 1) __syncthreads();
+    }
 }
 
 template <int R, bool EF>
@@ -1109,13 +1289,17 @@ float4 cdf_host(const cld& v) {
 // The M2L tables: the Pascal matrix C(k+l, l) as double-float pairs (P x P
 // float2, in kFmmHSlots float4 slots), then per offset code (dx + 3) 7 + (dy + 3)
 // the scalings (-1)^(k+1) delta^-(k+1) and delta^-l, delta = dx + i dy.
+// After the L2L table: the scalings with their powers of two (m2lT) and the
+// digits of C(k+l, l) 2^-(k+l) as A fragments of m16n8k16 (m2lA).
 // Binomial coefficients by Pascal's triangle and powers by repeated products
 // in long double: no library power functions, whose long double forms are
 // slow where long double is emulated in software.
 constexpr int kFmmHSlots = kFmmP * kFmmP / 2;
 constexpr int kFmmSSlots = 49 * 2 * kFmmP;
 // then the L2L Pascal table C(l,m) at [l][m] (double-float, zero outside the
-// triangle), kFmmHSlots float4 slots
+// triangle), kFmmHSlots float4 slots; kFmmSSlots of m2lT; then m2lA
+constexpr int kFmmASlots = kTcD * 2 * 2 * 32;
+constexpr int kFmmTOff = 2 * kFmmHSlots + kFmmSSlots, kFmmAOff = kFmmTOff + kFmmSSlots;
 
 void translation_tables(std::vector<float4>* tab) {
     const int P = kFmmP, PP = 2 * kFmmP + 1;
@@ -1124,7 +1308,7 @@ void translation_tables(std::vector<float4>* tab) {
         C[(size_t)n * PP] = 1.0L;
         for (int k = 1; k <= n; ++k) C[(size_t)n * PP + k] = C[(size_t)(n - 1) * PP + k - 1] + C[(size_t)(n - 1) * PP + k];
     }
-    tab->assign(2 * kFmmHSlots + kFmmSSlots, make_float4(0.f, 0.f, 0.f, 0.f));
+    tab->assign(kFmmAOff + kFmmASlots, make_float4(0.f, 0.f, 0.f, 0.f));
     float* BU = reinterpret_cast<float*>(tab->data() + kFmmHSlots + kFmmSSlots);  // [l][m] = C(l, m)
     for (int r = 0; r < P; ++r)
         for (int c = 0; c < P; ++c) {
@@ -1146,13 +1330,41 @@ void translation_tables(std::vector<float4>* tab) {
             const int o = (dx + 3) * 7 + (dy + 3);
             const cld iz = 1.0L / cld((long double)dx, (long double)dy);
             float4* S = tab->data() + kFmmHSlots + (size_t)o * 2 * P;
+            float4* T = tab->data() + kFmmTOff + (size_t)o * 2 * P;
+            long double two = 1.0L;  // 2^e
             cld pw(1.0L, 0.0L);  // delta^-e
             for (int e = 0; e <= P; ++e) {
                 if (e < P) S[P + e] = cdf_host(pw);                                       // delta^-l, l = e
                 if (e >= 1) S[e - 1] = cdf_host((e % 2 == 1) ? -pw : pw);                // k = e - 1: (-1)^(k+1) = (-1)^e
+                if (e < P) T[P + e] = cdf_host(pw * two);
+                if (e >= 1) T[e - 1] = cdf_host(((e % 2 == 1) ? -pw : pw) * (0.5L * two));
                 pw *= iz;
+                two *= 2.0L;
             }
         }
+    // digits: round(C(k+l, l) 2^(49 - k - l)) in balanced base 1024, most significant first
+    std::vector<int> dig((size_t)kTcD * P * P);
+    for (int k = 0; k < P; ++k)
+        for (int l = 0; l < P; ++l) {
+            const unsigned __int128 c = (unsigned __int128)(unsigned long long)C[(size_t)(k + l) * PP + l] << 50;
+            long long v = (long long)(((c >> (k + l)) + 1) >> 1);
+            for (int i = kTcD - 1; i >= 0; --i) {
+                const int d = (i > 0) ? (int)((v + 512) & 1023) - 512 : (int)v;
+                dig[((size_t)i * P + l) * P + k] = d;
+                v = (v - d) / 1024;
+            }
+        }
+    __half* F = reinterpret_cast<__half*>(tab->data() + kFmmAOff);
+    for (int i = 0; i < kTcD; ++i)
+        for (int m = 0; m < 2; ++m)
+            for (int kt = 0; kt < 2; ++kt)
+                for (int lane = 0; lane < 32; ++lane)
+                    for (int u = 0; u < 8; ++u) {  // row g (+ 8 for odd registers), column 2t + (u & 1) (+ 8)
+                        const int row = 16 * m + (lane >> 2) + 8 * ((u >> 1) & 1);
+                        const int col = 16 * kt + 2 * (lane & 3) + (u & 1) + 8 * (u >> 2);
+                        F[((((i * 2 + m) * 2 + kt) * 32) + lane) * 8 + u] =
+                            __float2half((float)dig[((size_t)i * P + row) * P + col]);
+                    }
 }
 
 // Pinned host staging for the tree upload (grown on demand, kept for the process).
@@ -1593,7 +1805,7 @@ static int fmm_tree_host(const Boundary& b, FmmTree* t, cudaStream_t st) {
     return GNK_OK;
 }
 
-int fmm_device_tables(const float2** m2lH, const float4** m2lS, const float2** bUp, cudaStream_t st) {
+int fmm_device_tables(FmmTree* t, cudaStream_t st) {
     static std::mutex mu;
     static std::vector<float4*> per_device;  // indexed by device, never freed
     int dev = 0;
@@ -1618,9 +1830,11 @@ int fmm_device_tables(const float2** m2lH, const float4** m2lS, const float2** b
         }
         per_device[dev] = d;
     }
-    *m2lH = reinterpret_cast<const float2*>(per_device[dev]);
-    *m2lS = per_device[dev] + kFmmHSlots;
-    *bUp = reinterpret_cast<const float2*>(per_device[dev] + kFmmHSlots + kFmmSSlots);
+    t->m2lH = reinterpret_cast<const float2*>(per_device[dev]);
+    t->m2lS = per_device[dev] + kFmmHSlots;
+    t->bUp = reinterpret_cast<const float2*>(per_device[dev] + kFmmHSlots + kFmmSSlots);
+    t->m2lT = per_device[dev] + kFmmTOff;
+    t->m2lA = reinterpret_cast<const uint4*>(per_device[dev] + kFmmAOff);
     return GNK_OK;
 }
 
@@ -1652,7 +1866,7 @@ int ensure_fmm(const Boundary& bc, int R, cudaStream_t st) {
     t->R = kMaxRHS;
     int rc = fmm_tree_device(b, t, st);
     if (rc == kFmmUseHost) rc = fmm_tree_host(b, t, st);
-    if (rc == GNK_OK) rc = fmm_device_tables(&t->m2lH, &t->m2lS, &t->bUp, st);
+    if (rc == GNK_OK) rc = fmm_device_tables(t, st);
     if (rc == GNK_OK) {  // the upward pass's child counts, all zero
         const size_t nsync = (size_t)t->nbox;
         if (pool_alloc(reinterpret_cast<void**>(&t->sync), nsync * sizeof(int), st) != cudaSuccess ||
@@ -1943,10 +2157,14 @@ static int fmm_product(const Boundary& b, FmmArgs& a, int R, bool EF, const Redu
     GNK_TRY_CUDA(cudaGetLastError());
     prof_end(toku, PK_FMMUP, 0.0, fs, fmm_instr(b, R, 1));
     const ProfToken tokm = prof_begin(fs, PK_FMM);
-    if (R == 2)
+    if (b.diff && R == 2)
         fmm_m2l_kernel<2><<<t->nbox, kFmmUT, 0, fs>>>(a);
-    else
+    else if (b.diff)
         fmm_m2l_kernel<1><<<t->nbox, kFmmUT, 0, fs>>>(a);
+    else if (R == 2)
+        fmm_m2l_tc_kernel<2><<<t->nbox, 32 * kTcWarps, 0, fs>>>(a);
+    else
+        fmm_m2l_tc_kernel<1><<<t->nbox, 32 * kTcWarps, 0, fs>>>(a);
     GNK_TRY_CUDA(cudaGetLastError());
     prof_end(tokm, PK_FMM, (double)R, fs, fmm_instr(b, R, 0));  // work: Cauchy sums (products)
     launches += 2;
@@ -2047,6 +2265,8 @@ static void fmm_args(const Boundary& b, FmmArgs& a) {
     a.m2lH = t->m2lH;
     a.m2lS = t->m2lS;
     a.bUp = t->bUp;
+    a.m2lT = t->m2lT;
+    a.m2lA = t->m2lA;
     a.ucnt = t->sync;
     a.xs = nullptr;
     a.near_scaled = 0;

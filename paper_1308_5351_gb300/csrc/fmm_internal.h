@@ -46,6 +46,8 @@ struct FmmTree {
     const float2* m2lH = nullptr;  // M2L: the Pascal matrix C(k+l, l) [k][l] as double-float,
     const float4* m2lS = nullptr;  // and per offset code the two complex scalings (per-device cache)
     const float2* bUp = nullptr;   // L2L Pascal table C(l,m) [l][m]
+    const float4* m2lT = nullptr;  // the scalings with their powers of two, and the digits of
+    const uint4* m2lA = nullptr;   // C(k+l, l) 2^-(k+l) as tensor-core fragments
     float4* mult = nullptr;     // [R][nbox][P]
     float4* loc = nullptr;      // [R][nbox][P]
     float4* ws = nullptr;       // [R][N] weights in sorted order, double-float complex
@@ -87,10 +89,10 @@ struct FmmTree {
 constexpr int kFmmUseHost = 1;
 int fmm_tree_device(const Boundary& b, FmmTree* t, cudaStream_t st);
 
-// The double-float translation tables on the current device (formed and
-// uploaded once per device and process): the M2L Pascal matrix C(k+l, l)
+// Points t at the translation tables on the current device (formed and uploaded
+// once per device and process): the M2L Pascal matrix C(k+l, l)
 // [P][P] and, per offset code (dx + 3) 7 + (dy + 3), the scalings
 // (-1)^(k+1) delta^-(k+1) and delta^-l; the L2L Pascal matrix C(l, m).
-int fmm_device_tables(const float2** m2lH, const float4** m2lS, const float2** bUp, cudaStream_t st);
+int fmm_device_tables(FmmTree* t, cudaStream_t st);
 
 }  // namespace gnk

@@ -76,7 +76,12 @@ struct FmmArgs {
     const float4* m2lS;   // per offset code: (-1)^(k+1) delta^-(k+1), then delta^-l
     const float2* bUp;    // C(l, m) at [l][m] (0 for l < m): the L2L Pascal sums
     const float4* m2lT;   // per offset code: (-1)^(k+1) (2/delta)^k / delta, then (2/delta)^l
-    const uint4* m2lA;    // digits of C(k+l, l) 2^-(k+l) as mma fragments
+    const uint4* m2lA;    // digits of C(k+l, l) 2^-(k+l) as mma fragments,
+    const uint4* upA;     // of C(m, k) 2^-m (M2M)
+    const uint4* dnA;     // and of C(l, m) 2^-l (L2L)
+    const unsigned* path; // [nleaf][depth]: box | quadrant << 30 of each leaf and its ancestors
+    int depth;            // levels of the tree: L - l0 + 1
+    int nleaf;
     float4* mult;
     float4* loc;
     float4* ws;
@@ -99,7 +104,8 @@ struct FmmArgs {
     int* ucnt;            // per box: children counted in the upward pass
     float2* xs;           // [R][N] x in sorted order as double-float (cached near field), or null
     int near_scaled;      // zn holds the near field times the operator's factor (cached)
-    const float4* tp;     // [N][P] powers t^k of every node about its leaf centre, or null
+    const float4* tn;     // [N] offset t of every node from its leaf centre in leaf widths (double-float complex)
+    const float4* tp;     // [N][P] powers t^k (handles built for differentiation), or null
     int* fault;           // set by a bounded wait that gave up
 };
 
@@ -164,6 +170,19 @@ __device__ __forceinline__ void cdf_mac(cdf& acc, cdf a, cdf b) {
 }
 
 __device__ __forceinline__ cdf cdf_add(cdf a, cdf b) { return cdf{df_add(a.re, b.re), df_add(a.im, b.im)}; }
+
+__device__ __forceinline__ df2 df2_neg(df2 a) { return df2{neg2(a.h), neg2(a.l)}; }
+
+// a + b (renormalised), two lanes
+__device__ __forceinline__ df2 df2_add(df2 a, df2 b) {
+    float2 s, e;
+    two_sum2(a.h, b.h, s, e);
+    e = add2(e, add2(a.l, b.l));
+    df2 r;
+    r.h = add2(s, e);
+    r.l = sub2(e, sub2(r.h, s));
+    return r;
+}
 
 // Translation kernels use kFmmTW warps per target box.
 constexpr int kFmmTW = 4;
@@ -304,48 +323,91 @@ __device__ __forceinline__ void m2l_box(const FmmArgs& a, int box, int wid, int 
     }
 }
 
-// P2M of one leaf (block of kFmmTW warps): for each chunk of 32 nodes, warp
-// w forms the powers t_j^k of orders 8w .. 8w + 7 (from t^8 by squaring) in
-// shared memory, then sums w_j t_j^k over the chunk's nodes 8w .. 8w + 7 for
-// every k (lane = k); the warps' sums are added in warp order.
+// Packed complex double-float: (re, im) in the lanes of a float2.
+__device__ __forceinline__ df2 pc_of(float4 v) { return df2{make_float2(v.x, v.z), make_float2(v.y, v.w)}; }
+
+__device__ __forceinline__ df2 pc_mul(df2 a, df2 b) {  // a b, renormalised
+    const df2 ax{make_float2(a.h.y, a.h.x), make_float2(a.l.y, a.l.x)};
+    const df2 p = df2_mul(a, df2{f2(b.h.x), f2(b.l.x)});
+    const df2 q = df2_mul(ax, df2{make_float2(-b.h.y, b.h.y), make_float2(-b.l.y, b.l.y)});
+    return df2_add(p, q);
+}
+
+// P2M of one leaf, a_k = sum_j w_j t_j^k: a warp takes chunks of 32 nodes (lane =
+// node) and carries w t^k up four interleaved chains k = 8 c + m (c < 4) of
+// eight products; every two steps the eight values of k in hand go through
+// shared memory, where four lanes per k add eight nodes each.  The powers are
+// formed anew for every product: 19 packed instructions a power, 2 us of the
+// FP32 pipe at 65,536 nodes, where a table of them costs 512 bytes of memory
+// traffic a node beside the near field's stream (the upward pass 41 us with the
+// table at 65,536 nodes, 131 us at 524,288).  The warps' sums are added in warp order.
+constexpr int kP2mStride = 36;  // float4 per row: conflict-free for the column reads below
+
 template <int R>
-__device__ __forceinline__ void p2m_leaf(const FmmArgs& a, int leaf, int box, int wid, int lane,
-                                         float4 (*s_pow)[33], float4 (*s_w)[32], float4 (*s_acc)[32]) {
-    const double2 c = a.center[box];
-    const double ir = 1.0 / a.width[box];
-    cdf acc[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) acc[r] = cdf_zero();
+__device__ __forceinline__ void p2m_leaf(const FmmArgs& a, int leaf, int box, int wid, int lane, float4* s_v,
+                                         float4 (*s_acc)[32]) {
+    const unsigned full = 0xffffffffu;
     const int j0 = a.leaf_start[leaf], j1 = a.leaf_start[leaf + 1];
-    for (int base = j0; base < j1; base += 32) {
-        const int j = base + lane;
-        if (j < j1) {
-            const double2 p = a.ps[j];
-            const cdf t = cdf_split(make_double2((p.x - c.x) * ir, (p.y - c.y) * ir));
-            const cdf t8 = cdf_sq(cdf_sq(cdf_sq(t)));
-            cdf v = cdf{df{1.f, 0.f}, df{0.f, 0.f}};
-            if (wid == 1) v = t8;
-            if (wid >= 2) v = cdf_sq(t8);
-            if (wid == 3) v = cdf_mul(v, t8);
-            for (int k = 8 * wid; k < 8 * wid + 8; ++k) {
-                s_pow[k][lane] = cdf_pack(v);
-                v = cdf_mul(v, t);
-            }
-            if (wid < R) s_w[wid][lane] = a.ws[(size_t)wid * a.N + j];
-        }
-        __syncthreads();
-        const int q1 = min(8 * wid + 8, j1 - base);
-        for (int qn = 8 * wid; qn < q1; ++qn) {
-            const cdf pw = cdf_of(s_pow[lane][qn]);
-#pragma unroll
-            for (int r = 0; r < R; ++r) cdf_mac(acc[r], cdf_of(s_w[r][qn]), pw);
-        }
-        __syncthreads();
-    }
+    const int row = lane >> 2, grp = lane & 3;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const cdf sm = reduce_warps(acc[r], s_acc, wid, lane);
-        if (wid == 0) a.mult[((size_t)r * a.nbox + box) * kFmmP + lane] = cdf_pack(sm);
+        df2 acc[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] = df2{f2(0.f), f2(0.f)};
+        for (int base = j0 + 32 * wid; base < j1; base += 32 * kFmmTW) {
+            const int j = base + lane;
+            df2 t{f2(0.f), f2(0.f)}, v[4];
+            v[0] = t;
+            if (j < j1) {
+                t = pc_of(__ldg(a.tn + j));
+                v[0] = pc_of(__ldcg(a.ws + (size_t)r * a.N + j));
+            }
+            {
+                const df2 t2 = pc_mul(t, t), t4 = pc_mul(t2, t2), t8 = pc_mul(t4, t4), t16 = pc_mul(t8, t8);
+                v[1] = pc_mul(v[0], t8);
+                v[2] = pc_mul(v[0], t16);
+                v[3] = pc_mul(v[1], t16);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {  // m = 2 q, 2 q + 1
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        s_v[(2 * c + u) * kP2mStride + lane] = make_float4(v[c].h.x, v[c].h.y, v[c].l.x, v[c].l.y);
+                        if (q < 3 || u < 1) v[c] = pc_mul(v[c], t);
+                    }
+                __syncwarp();
+                df2 s{f2(0.f), f2(0.f)};
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float4 x = s_v[row * kP2mStride + i * 4 + grp];
+                    df2_acc(s, df2{make_float2(x.x, x.y), make_float2(x.z, x.w)});
+                }
+                acc[q] = df2_add(acc[q], s);
+                __syncwarp();
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {  // the four lanes of a k
+#pragma unroll
+            for (int o = 1; o < 4; o <<= 1) {
+                df2 x;
+                x.h = make_float2(__shfl_xor_sync(full, acc[q].h.x, o), __shfl_xor_sync(full, acc[q].h.y, o));
+                x.l = make_float2(__shfl_xor_sync(full, acc[q].l.x, o), __shfl_xor_sync(full, acc[q].l.y, o));
+                acc[q] = df2_add(acc[q], x);
+            }
+            if (grp == 0)
+                s_acc[wid][8 * (row >> 1) + 2 * q + (row & 1)] =
+                    make_float4(acc[q].h.x, acc[q].l.x, acc[q].h.y, acc[q].l.y);
+        }
+        __syncthreads();
+        if (wid == 0) {
+            cdf m = cdf_of(s_acc[0][lane]);
+            for (int w = 1; w < kFmmTW; ++w) m = cdf_add(m, cdf_of(s_acc[w][lane]));
+            a.mult[((size_t)r * a.nbox + box) * kFmmP + lane] = cdf_pack(m);
+        }
+        __syncthreads();
     }
 }
 
@@ -390,29 +452,24 @@ __device__ __forceinline__ void p2m_leaf_cached(const FmmArgs& a, int leaf, int 
     }
 }
 
-// Upward pass, one block per leaf: P2M (from the cached powers when TP), then
-// the multipoles move up the tree without a launch per level: the block that
+// Upward pass of the handles built for differentiation, one block per leaf: P2M
+// from the cached powers, then the multipoles move up the tree without a launch per level: the block that
 // completes the last child of a box (an atomic count per box; nothing waits)
 // forms that box's M2M from its children (warp w takes child w) and goes on
 // to the parent.
-template <int R, bool TP>
+template <int R>
 __global__ void __launch_bounds__(kFmmUT) fmm_up_kernel(FmmArgs a) {
-    __shared__ float4 s_pow[TP ? 1 : kFmmP][33];
-    __shared__ float4 s_w[R][32];
     __shared__ float4 s_acc[kFmmTW][32];
     __shared__ int s_last;
     if (a.done != nullptr && *a.done) return;
     const int leaf = blockIdx.x, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int box = a.leaf_box[leaf];
-    if (TP)
-        p2m_leaf_cached<R>(a, leaf, box, wid, lane, s_acc);
-    else
-        p2m_leaf<R>(a, leaf, box, wid, lane, s_pow, s_w, s_acc);
+    p2m_leaf_cached<R>(a, leaf, box, wid, lane, s_acc);
     for (;;) {
         if (wid == 0) __threadfence();  // the box's multipole (warp 0's stores) before the count
         __syncthreads();
         const int par = a.parent[box];
-        if (par < 0) break;  // level 2
+        if (par < 0) break;  // the topmost level
         if (threadIdx.x == 0) {
             const int last = atomicAdd(&a.ucnt[par], 1) == a.child_count[par] - 1;
             if (last) {
@@ -510,19 +567,6 @@ __device__ __forceinline__ df2 diff3_2(float2 p1, float2 p2, float2 p3, float2 q
     return r;
 }
 
-__device__ __forceinline__ df2 df2_neg(df2 a) { return df2{neg2(a.h), neg2(a.l)}; }
-
-// a + b (renormalised), two lanes
-__device__ __forceinline__ df2 df2_add(df2 a, df2 b) {
-    float2 s, e;
-    two_sum2(a.h, b.h, s, e);
-    e = add2(e, add2(a.l, b.l));
-    df2 r;
-    r.h = add2(s, e);
-    r.l = sub2(e, sub2(r.h, s));
-    return r;
-}
-
 // ---- M2L on the tensor cores.  With x_k = (-1)^(k+1) (2/delta)^k / delta a_k
 //   b_l = (1/r) (2/delta)^l sum_k C'(k, l) x_k,   C'(k, l) = C(k+l, l) 2^-(k+l) <= 1:
 // for all pairs of boxes one fixed real 32 x 32 matrix times a real matrix whose
@@ -563,13 +607,125 @@ __device__ __forceinline__ unsigned half2_bits(float2 v) {
     return *reinterpret_cast<const unsigned*>(&h);
 }
 
+// y = T x for the eight columns of a tile.  In: x of column g (pair g / 2, part
+// g mod 2) at k = 2t + 8q and the next, two k per float2.  Out: rows l = g + 8 i of
+// pair t, (re, im) per float2.  T: the fixed matrix's digits as A fragments.
+__device__ __forceinline__ void tc_transform(const uint4* __restrict__ T, const df2 (&x)[4], int lane, df2 (&y)[4]) {
+    const unsigned full = 0xffffffffu;
+    const int t = lane & 3;
+    float mx = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) mx = fmaxf(mx, fmaxf(fabsf(x[q].h.x), fabsf(x[q].h.y)));
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(full, mx, o));  // lanes of the pair
+    const int ex = max((int)(__float_as_uint(mx) >> 23), 8);  // mx < 2^(ex - 126)
+    // digits of 2^(135 - ex) x (below 512), as B fragments: k tiles 0 (q = 0, 1) and 1 (q = 2, 3)
+    unsigned B[kTcD][4];
+    const float2 up = f2(__uint_as_float((unsigned)(262 - ex) << 23)), K = f2(1024.f);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float2 h = mul2(x[q].h, up), l = mul2(mul2(x[q].l, up), f2(1048576.f));
+        float2 d = rint2(h);
+        B[0][q] = half2_bits(d);
+        float2 v = mul2(sub2(h, d), K);
+        d = rint2(v);
+        B[1][q] = half2_bits(d);
+        v = mul2(sub2(v, d), K);
+        d = rint2(add2(v, l));
+        B[2][q] = half2_bits(d);
+        v = mul2(add2(sub2(v, d), l), K);  // exact: d is the nearest integer to v + l
+        d = rint2(v);
+        B[3][q] = half2_bits(d);
+        v = mul2(sub2(v, d), K);
+        B[4][q] = half2_bits(rint2(v));
+    }
+    float c[kTcD + 1][2][4];
+#pragma unroll
+    for (int s = 0; s <= kTcD; ++s)
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) c[s][m][u] = 0.f;
+#pragma unroll
+    for (int i = 0; i < kTcD; ++i) {
+        uint4 H[2][2];
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int kt = 0; kt < 2; ++kt) H[m][kt] = __ldg(T + ((i * 2 + m) * 2 + kt) * 32 + lane);
+#pragma unroll
+        for (int j = 0; j < kTcD; ++j) {
+            if (i + j > kTcD) continue;
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int kt = 0; kt < 2; ++kt) mma_f16(c[i + j][m], H[m][kt], B[j][2 * kt], B[j][2 * kt + 1]);
+        }
+    }
+    // pair t: y = 2^(ex - 126) sum_s c_s 2^(-18 - 10 s)
+    const int ext = __shfl_sync(full, ex, 8 * t);
+    const float2 dn = f2(__uint_as_float((unsigned)(min(ext, 253) + 1) << 23));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float2 v[kTcD + 1];
+        float w = 1.f / 262144.f;
+#pragma unroll
+        for (int s = 0; s <= kTcD; ++s) {
+            v[s] = mul2(make_float2(c[s][i >> 1][2 * (i & 1)], c[s][i >> 1][2 * (i & 1) + 1]), f2(w));
+            w *= 1.f / 1024.f;
+        }
+        float2 h, l0, l1;
+        two_sum2(v[0], v[1], h, l0);
+        two_sum2(h, v[2], h, l1);
+        l0 = add2(add2(l0, l1), add2(v[3], add2(v[4], v[5])));
+        y[i].h = add2(h, l0);
+        y[i].l = mul2(sub2(l0, sub2(y[i].h, h)), dn);
+        y[i].h = mul2(y[i].h, dn);
+    }
+}
+
+// acc summed over the lanes t (the pairs of a tile) in a fixed order
+__device__ __forceinline__ df2 tc_sum_pairs(df2 acc) {
+    const unsigned full = 0xffffffffu;
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        df2 v;
+        v.h = make_float2(__shfl_xor_sync(full, acc.h.x, o), __shfl_xor_sync(full, acc.h.y, o));
+        v.l = make_float2(__shfl_xor_sync(full, acc.l.x, o), __shfl_xor_sync(full, acc.l.y, o));
+        acc = df2_add(acc, v);
+    }
+    return acc;
+}
+
+// g^e 2^s for g = sqrt(2) e^{i pi ang / 4} (ang odd): a Gaussian integer times a power of two
+__device__ __forceinline__ float2 gauss_pow(int ang, int e, int s) {
+    const int a8 = (ang * e) & 7;
+    const float m = __uint_as_float((unsigned)(127 + (e >> 1) + s) << 23);
+    return make_float2((a8 == 0 || a8 == 1 || a8 == 7) ? m : ((a8 >= 3 && a8 <= 5) ? -m : 0.f),
+                       (a8 >= 1 && a8 <= 3) ? m : ((a8 >= 5) ? -m : 0.f));
+}
+
+// One part (re, im) of v_k g_k for k and k + 1: v as loaded (re.h, re.l, im.h, im.l), g exact
+__device__ __forceinline__ df2 tc_scale_in(float4 v0, float4 v1, float2 g0, float2 g1, int part) {
+    const float2 gr = make_float2(g0.x, g1.x), gi = make_float2(g0.y, g1.y);
+    const df2 re{make_float2(v0.x, v1.x), make_float2(v0.y, v1.y)}, im{make_float2(v0.z, v1.z), make_float2(v0.w, v1.w)};
+    const df2 u = part ? im : re, w = part ? re : df2{neg2(im.h), neg2(im.l)};
+    return df2_add(df2{mul2(u.h, gr), mul2(u.l, gr)}, df2{mul2(w.h, gi), mul2(w.l, gi)});
+}
+
+// y g for a complex y = (re, im) and an exact factor g
+__device__ __forceinline__ df2 tc_scale_out(df2 y, float2 g) {
+    const float2 gr = f2(g.x), gi = make_float2(-g.y, g.y);
+    const float2 xh = make_float2(y.h.y, y.h.x), xl = make_float2(y.l.y, y.l.x);
+    return df2_add(df2{mul2(y.h, gr), mul2(y.l, gr)}, df2{mul2(xh, gi), mul2(xl, gi)});
+}
+
 template <int R>
 __global__ void __launch_bounds__(32 * kTcWarps) fmm_m2l_tc_kernel(FmmArgs a) {
     __shared__ float4 s_acc[kTcWarps][32];
     if (a.done != nullptr && *a.done) return;
     const int box = blockIdx.x, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3, part = g & 1;
-    const unsigned full = 0xffffffffu;
     const int e0 = a.il_start[box], e1 = a.il_start[box + 1];
     const df sc = df_split_fast(recip_f64(a.width[box]));
 #pragma unroll
@@ -578,13 +734,12 @@ __global__ void __launch_bounds__(32 * kTcWarps) fmm_m2l_tc_kernel(FmmArgs a) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[i] = df2{f2(0.f), f2(0.f)};
         for (int base = e0 + 4 * wid; base < e1; base += 4 * kTcWarps) {
-            // x of pair g / 2, part g mod 2, at k = 2t, 2t + 1 (+ 8, + 16, + 24): two k per float2
-            const int eb = min(base + (g >> 1), e1 - 1);
+            const int eb = min(base + (g >> 1), e1 - 1), ec = min(base + t, e1 - 1);
             const float4* S = a.m2lT + (size_t)a.il_off[eb] * 2 * kFmmP;
             const float4* A = a.mult + ((size_t)r * a.nbox + a.il_src[eb]) * kFmmP;
+            const float4* Q = a.m2lT + ((size_t)a.il_off[ec] * 2 + 1) * kFmmP;
             const bool live = base + (g >> 1) < e1;
-            df2 x[4];
-            float mx = 0.f;
+            df2 x[4], y[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int k = 2 * t + 8 * q;
@@ -600,93 +755,19 @@ __global__ void __launch_bounds__(32 * kTcWarps) fmm_m2l_tc_kernel(FmmArgs a) {
                 x[q].h = add2(w.h, w.l);
                 x[q].l = sub2(w.l, sub2(x[q].h, w.h));
                 if (!live) x[q] = df2{f2(0.f), f2(0.f)};
-                mx = fmaxf(mx, fmaxf(fabsf(x[q].h.x), fabsf(x[q].h.y)));
             }
+            tc_transform(a.m2lA, x, lane, y);
 #pragma unroll
-            for (int o = 1; o < 8; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(full, mx, o));  // lanes of the pair
-            const int ex = max((int)(__float_as_uint(mx) >> 23), 8);  // mx < 2^(ex - 126)
-            // digits of 2^(135 - ex) x (below 512), as B fragments: k tiles 0 (q = 0, 1) and 1 (q = 2, 3)
-            unsigned B[kTcD][4];
-            {
-                const float2 up = f2(__uint_as_float((unsigned)(262 - ex) << 23)), K = f2(1024.f);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float2 h = mul2(x[q].h, up), l = mul2(mul2(x[q].l, up), f2(1048576.f));
-                    float2 d = rint2(h);
-                    B[0][q] = half2_bits(d);
-                    float2 v = mul2(sub2(h, d), K);
-                    d = rint2(v);
-                    B[1][q] = half2_bits(d);
-                    v = mul2(sub2(v, d), K);
-                    d = rint2(add2(v, l));
-                    B[2][q] = half2_bits(d);
-                    v = mul2(add2(sub2(v, d), l), K);  // exact: d is the nearest integer to v + l
-                    d = rint2(v);
-                    B[3][q] = half2_bits(d);
-                    v = mul2(sub2(v, d), K);
-                    B[4][q] = half2_bits(rint2(v));
-                }
-            }
-            float c[kTcD + 1][2][4];
-#pragma unroll
-            for (int s = 0; s <= kTcD; ++s)
-#pragma unroll
-                for (int m = 0; m < 2; ++m)
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) c[s][m][u] = 0.f;
-#pragma unroll
-            for (int i = 0; i < kTcD; ++i) {
-                uint4 H[2][2];
-#pragma unroll
-                for (int m = 0; m < 2; ++m)
-#pragma unroll
-                    for (int kt = 0; kt < 2; ++kt) H[m][kt] = __ldg(a.m2lA + ((i * 2 + m) * 2 + kt) * 32 + lane);
-#pragma unroll
-                for (int j = 0; j < kTcD; ++j) {
-                    if (i + j > kTcD) continue;
-#pragma unroll
-                    for (int m = 0; m < 2; ++m)
-#pragma unroll
-                        for (int kt = 0; kt < 2; ++kt) mma_f16(c[i + j][m], H[m][kt], B[j][2 * kt], B[j][2 * kt + 1]);
-                }
-            }
-            // pair t: y_l = 2^(ex - 126) sum_s c_s 2^(-18 - 10 s), then (2/delta)^l y_l
-            const int ec = base + t < e1 ? base + t : e1 - 1;
-            const float4* Q = a.m2lT + ((size_t)a.il_off[ec] * 2 + 1) * kFmmP;
-            const int ext = __shfl_sync(full, ex, 8 * t);
-            const float2 dn = f2(__uint_as_float((unsigned)(min(ext, 253) + 1) << 23));
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float2 v[kTcD + 1];
-                float w = 1.f / 262144.f;
-#pragma unroll
-                for (int s = 0; s <= kTcD; ++s) {
-                    v[s] = mul2(make_float2(c[s][i >> 1][2 * (i & 1)], c[s][i >> 1][2 * (i & 1) + 1]), f2(w));
-                    w *= 1.f / 1024.f;
-                }
-                float2 h, l0, l1;
-                two_sum2(v[0], v[1], h, l0);
-                two_sum2(h, v[2], h, l1);
-                l0 = add2(add2(l0, l1), add2(v[3], add2(v[4], v[5])));
-                df2 y;
-                y.h = add2(h, l0);
-                y.l = mul2(sub2(l0, sub2(y.h, h)), dn);
-                y.h = mul2(y.h, dn);
+            for (int i = 0; i < 4; ++i) {  // (2/delta)^l y_l
                 const float4 q4 = __ldg(Q + g + 8 * i);
-                df2_acc(acc[i], df2_mul(y, df2{f2(q4.x), f2(q4.y)}));
-                const df2 yx{make_float2(y.h.y, y.h.x), make_float2(y.l.y, y.l.x)};
+                df2_acc(acc[i], df2_mul(y[i], df2{f2(q4.x), f2(q4.y)}));
+                const df2 yx{make_float2(y[i].h.y, y[i].h.x), make_float2(y[i].l.y, y[i].l.x)};
                 df2_acc(acc[i], df2_mul(yx, df2{make_float2(-q4.z, q4.z), make_float2(-q4.w, q4.w)}));
             }
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {  // over the four pairs of the lanes t, in a fixed order
-#pragma unroll
-            for (int o = 1; o < 4; o <<= 1) {
-                df2 v;
-                v.h = make_float2(__shfl_xor_sync(full, acc[i].h.x, o), __shfl_xor_sync(full, acc[i].h.y, o));
-                v.l = make_float2(__shfl_xor_sync(full, acc[i].l.x, o), __shfl_xor_sync(full, acc[i].l.y, o));
-                acc[i] = df2_add(acc[i], v);
-            }
+        for (int i = 0; i < 4; ++i) {
+            acc[i] = tc_sum_pairs(acc[i]);
             if (t == 0) s_acc[wid][g + 8 * i] = make_float4(acc[i].h.x, acc[i].l.x, acc[i].h.y, acc[i].l.y);
         }
         __syncthreads();
@@ -696,6 +777,135 @@ __global__ void __launch_bounds__(32 * kTcWarps) fmm_m2l_tc_kernel(FmmArgs a) {
             a.loc[((size_t)r * a.nbox + box) * kFmmP + lane] = cdf_pack(cdf{df_mul(b.re, sc), df_mul(b.im, sc)});
         }
         if (R > 1) __syncthreads();
+    }
+}
+
+// ---- The upward pass, one block per leaf: P2M, then warp 0 alone carries the
+// multipoles up: the warp that completes the last child of a box (an atomic
+// count per box; nothing waits) forms that box's M2M from its at most four
+// children, one tile of tc_transform, and goes on to the parent.  With g the child's
+// Gaussian integer (above) and C(m,k) 2^-m the fixed matrix,
+//   a0_m = (g/2)^m sum_k C(m,k) 2^-m [conj(g)^k a1_k].
+// Latency bounds it: per level a fence, an atomic, the children's multipoles and
+// one transform.  The leaf's path (boxes, child ranges) is read while the P2M runs.
+template <int R>
+__global__ void __launch_bounds__(kFmmUT) fmm_up_tc_kernel(FmmArgs a) {
+    __shared__ float4 s_v[kFmmTW][8 * kP2mStride];
+    __shared__ float4 s_acc[kFmmTW][32];
+    if (a.done != nullptr && *a.done) return;
+    const unsigned full = 0xffffffffu;
+    const int leaf = blockIdx.x, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // lane d of warp 0: the leaf's ancestor d levels up
+    int pbox = 0, pc0 = 0, pnc = 0;
+    if (wid == 0 && lane < a.depth) {
+        pbox = (int)(a.path[(size_t)leaf * a.depth + lane] & 0x3fffffffu);
+        pc0 = a.child_start[pbox];
+        pnc = a.child_count[pbox];
+    }
+    p2m_leaf<R>(a, leaf, a.leaf_box[leaf], wid, lane, s_v[wid], s_acc);
+    if (wid != 0) return;
+    const int g = lane >> 2, t = lane & 3, part = g & 1;
+    for (int d = 1; d < a.depth; ++d) {
+        const int box = __shfl_sync(full, pbox, d), c0 = __shfl_sync(full, pc0, d), nc = __shfl_sync(full, pnc, d);
+        __threadfence();  // the child's multipole before the count
+        __syncwarp();
+        int last = 0;
+        if (lane == 0) {
+            last = atomicAdd(&a.ucnt[box], 1) == nc - 1;
+            if (last) {
+                a.ucnt[box] = 0;  // every child has counted: ready for the next product
+                __threadfence();
+            }
+        }
+        if (!__shfl_sync(full, last, 0)) return;
+        const int cb = c0 + min(g >> 1, nc - 1);
+        const bool live = (g >> 1) < nc;
+        const int angb = gauss_angle(__ldg(a.quad + cb)), angc = gauss_angle(__ldg(a.quad + c0 + min(t, nc - 1)));
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float4* A = a.mult + ((size_t)r * a.nbox + cb) * kFmmP;
+            df2 x[4], y[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int k = 2 * t + 8 * q;
+                x[q] = tc_scale_in(__ldcg(A + k), __ldcg(A + k + 1), gauss_pow(8 - angb, k, 0),
+                                   gauss_pow(8 - angb, k + 1, 0), part);
+                if (!live) x[q] = df2{f2(0.f), f2(0.f)};
+            }
+            tc_transform(a.upA, x, lane, y);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int m = g + 8 * i;
+                const df2 v = tc_sum_pairs(tc_scale_out(y[i], gauss_pow(angc, m, -m)));
+                if (t == 0)
+                    a.mult[((size_t)r * a.nbox + box) * kFmmP + m] = make_float4(v.h.x, v.l.x, v.h.y, v.l.y);
+            }
+        }
+    }
+}
+
+// ---- L2L, one warp per four leaves (the pairs of a tile): each leaf's local
+// expansion is carried down from its topmost ancestor, one tc_transform per
+// level, the M2L part of the next box added:
+//   b1_m = conj(g)^m sum_l C(l,m) 2^-l [(g/2)^l b0_l].
+// Between levels the result goes from the rows of the accumulators to the
+// columns of the next operand through shared memory.  (One warp per leaf with a
+// 32-term double-float sum per lane and level: 13 us at 65,536 nodes.)
+template <int R>
+__global__ void __launch_bounds__(32) fmm_l2l_tc_kernel(FmmArgs a) {
+    __shared__ float4 s_v[4][33];
+    if (a.done != nullptr && *a.done) return;
+    const int lane = threadIdx.x, g = lane >> 2, t = lane & 3, part = g & 1, pb = g >> 1;
+    const int D = a.depth;
+    const int leafb = min(4 * (int)blockIdx.x + pb, a.nleaf - 1), leafc = min(4 * (int)blockIdx.x + t, a.nleaf - 1);
+    const unsigned *pathb = a.path + (size_t)leafb * D, *pathc = a.path + (size_t)leafc * D;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        float4* loc = a.loc + (size_t)r * a.nbox * kFmmP;
+        df2 v[4];
+        {
+            const float4* b = loc + (size_t)(pathc[D - 1] & 0x3fffffffu) * kFmmP;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = pc_of(b[g + 8 * i]);
+        }
+        for (int d = D - 2; d >= 0; --d) {
+            const unsigned eb = __ldg(pathb + d), ec = __ldg(pathc + d);
+            const int angb = gauss_angle((int)(eb >> 30)), angc = gauss_angle((int)(ec >> 30));
+            const float4* b = loc + (size_t)(ec & 0x3fffffffu) * kFmmP;
+            float4 nxt[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) nxt[i] = b[g + 8 * i];
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) s_v[t][g + 8 * i] = make_float4(v[i].h.x, v[i].l.x, v[i].h.y, v[i].l.y);
+            __syncwarp();
+            df2 x[4], y[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int k = 2 * t + 8 * q;
+                x[q] = tc_scale_in(s_v[pb][k], s_v[pb][k + 1], gauss_pow(angb, k, -k), gauss_pow(angb, k + 1, -k - 1),
+                                   part);
+            }
+            tc_transform(a.dnA, x, lane, y);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = df2_add(pc_of(nxt[i]), tc_scale_out(y[i], gauss_pow(8 - angc, g + 8 * i, 0)));
+        }
+        if (4 * (int)blockIdx.x + t < a.nleaf) {
+            float4* b = loc + (size_t)(pathc[0] & 0x3fffffffu) * kFmmP;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) b[g + 8 * i] = make_float4(v[i].h.x, v[i].l.x, v[i].h.y, v[i].l.y);
+        }
+    }
+}
+
+// The path of every leaf: itself, then its ancestors up to the topmost level.
+__global__ void fmm_path_kernel(FmmArgs a, unsigned* path) {
+    const int leaf = blockIdx.x * blockDim.x + threadIdx.x;
+    if (leaf >= a.nleaf) return;
+    int box = a.leaf_box[leaf];
+    for (int d = 0; d < a.depth; ++d) {
+        path[(size_t)leaf * a.depth + d] = (unsigned)box | ((unsigned)a.quad[box] << 30);
+        box = a.parent[box];
     }
 }
 
@@ -845,10 +1055,11 @@ __global__ void __launch_bounds__(kFmmNT) fmm_near_kernel(FmmArgs a) {
     }
 }
 
-// The powers t^k, k < P, of every node about the centre of its leaf in units
-// of the leaf width (t = (s - c)/r), double-float complex, [node][k] in sorted
-// order: formed once per tree, read by every P2M.
-__global__ void fmm_tp_build_kernel(FmmArgs a, float4* __restrict__ tp) {
+// The offset t = (s - c)/r of every node from the centre of its leaf in leaf
+// widths, double-float complex, in sorted order: formed once per tree, read by
+// P2M and L2P (whose FP64 subtraction and product it replaces).  tp (handles
+// built for differentiation): also the powers t^k, k < P, [node][k].
+__global__ void fmm_tn_build_kernel(FmmArgs a, float4* __restrict__ tn, float4* __restrict__ tp) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.N) return;
     const int box = a.node_box[i];
@@ -856,6 +1067,8 @@ __global__ void fmm_tp_build_kernel(FmmArgs a, float4* __restrict__ tp) {
     const double ir = 1.0 / a.width[box];
     const double2 p = a.ps[i];
     const cdf t = cdf_split(make_double2((p.x - c.x) * ir, (p.y - c.y) * ir));
+    tn[i] = cdf_pack(t);
+    if (!tp) return;
     cdf v = cdf{df{1.f, 0.f}, df{0.f, 0.f}};
     float4* out = tp + (size_t)i * kFmmP;
     for (int k = 0; k < kFmmP; ++k) {
@@ -1217,10 +1430,16 @@ __global__ void __launch_bounds__(256) fmm_l2p_kernel(FmmArgs a, ReduceArgs e) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.N) return;
     const int box = a.node_box[i];
-    const double2 c = a.center[box];
-    const double ir = recip_f64(a.width[box]);  // (GB300's FP64 division is a long dependent chain)
-    const double2 p = a.ps[i];
-    const cdf t = cdf{df_split_fast((p.x - c.x) * ir), df_split_fast((p.y - c.y) * ir)};
+    double ir = 0.0;
+    cdf t;
+    if (EF || a.tp) {  // a handle built for differentiation
+        const double2 c = a.center[box];
+        ir = recip_f64(a.width[box]);  // (GB300's FP64 division is a long dependent chain)
+        const double2 p = a.ps[i];
+        t = cdf{df_split_fast((p.x - c.x) * ir), df_split_fast((p.y - c.y) * ir)};
+    } else {
+        t = cdf_of(__ldg(a.tn + i));
+    }
     const int node = a.perm[i];
     double zx[kMaxRHS] = {0.0, 0.0}, zy[kMaxRHS] = {0.0, 0.0};
     double2 near[kMaxRHS] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
@@ -1287,15 +1506,16 @@ float4 cdf_host(const cld& v) {
 }
 
 // The M2L tables: the Pascal matrix C(k+l, l) as double-float pairs (P x P
-// float2, in kFmmHSlots float4 slots), then per offset code (dx + 3) 7 + (dy + 3)
+// float2, in kFmmHSlots float4 slots), then per offset code (dx + 7) 15 + (dy + 7)
 // the scalings (-1)^(k+1) delta^-(k+1) and delta^-l, delta = dx + i dy.
 // After the L2L table: the scalings with their powers of two (m2lT) and the
-// digits of C(k+l, l) 2^-(k+l) as A fragments of m16n8k16 (m2lA).
+// digits of C(k+l, l) 2^-(k+l), C(m, k) 2^-m and C(l, m) 2^-l as A fragments of
+// m16n8k16 (m2lA).
 // Binomial coefficients by Pascal's triangle and powers by repeated products
 // in long double: no library power functions, whose long double forms are
 // slow where long double is emulated in software.
 constexpr int kFmmHSlots = kFmmP * kFmmP / 2;
-constexpr int kFmmSSlots = 49 * 2 * kFmmP;
+constexpr int kFmmSSlots = kFmmOffs * kFmmOffs * 2 * kFmmP;
 // then the L2L Pascal table C(l,m) at [l][m] (double-float, zero outside the
 // triangle), kFmmHSlots float4 slots; kFmmSSlots of m2lT; then m2lA
 constexpr int kFmmASlots = kTcD * 2 * 2 * 32;
@@ -1308,7 +1528,7 @@ void translation_tables(std::vector<float4>* tab) {
         C[(size_t)n * PP] = 1.0L;
         for (int k = 1; k <= n; ++k) C[(size_t)n * PP + k] = C[(size_t)(n - 1) * PP + k - 1] + C[(size_t)(n - 1) * PP + k];
     }
-    tab->assign(kFmmAOff + kFmmASlots, make_float4(0.f, 0.f, 0.f, 0.f));
+    tab->assign(kFmmAOff + 3 * kFmmASlots, make_float4(0.f, 0.f, 0.f, 0.f));
     float* BU = reinterpret_cast<float*>(tab->data() + kFmmHSlots + kFmmSSlots);  // [l][m] = C(l, m)
     for (int r = 0; r < P; ++r)
         for (int c = 0; c < P; ++c) {
@@ -1324,10 +1544,10 @@ void translation_tables(std::vector<float4>* tab) {
             H[2 * (k * P + l)] = hi;
             H[2 * (k * P + l) + 1] = (float)(v - (long double)hi);
         }
-    for (int dx = -3; dx <= 3; ++dx)
-        for (int dy = -3; dy <= 3; ++dy) {
+    for (int dx = -kFmmOffMax; dx <= kFmmOffMax; ++dx)
+        for (int dy = -kFmmOffMax; dy <= kFmmOffMax; ++dy) {
             if (std::max(std::abs(dx), std::abs(dy)) <= 1) continue;
-            const int o = (dx + 3) * 7 + (dy + 3);
+            const int o = (dx + kFmmOffMax) * kFmmOffs + dy + kFmmOffMax;
             const cld iz = 1.0L / cld((long double)dx, (long double)dy);
             float4* S = tab->data() + kFmmHSlots + (size_t)o * 2 * P;
             float4* T = tab->data() + kFmmTOff + (size_t)o * 2 * P;
@@ -1342,29 +1562,44 @@ void translation_tables(std::vector<float4>* tab) {
                 two *= 2.0L;
             }
         }
-    // digits: round(C(k+l, l) 2^(49 - k - l)) in balanced base 1024, most significant first
-    std::vector<int> dig((size_t)kTcD * P * P);
-    for (int k = 0; k < P; ++k)
-        for (int l = 0; l < P; ++l) {
-            const unsigned __int128 c = (unsigned __int128)(unsigned long long)C[(size_t)(k + l) * PP + l] << 50;
-            long long v = (long long)(((c >> (k + l)) + 1) >> 1);
-            for (int i = kTcD - 1; i >= 0; --i) {
-                const int d = (i > 0) ? (int)((v + 512) & 1023) - 512 : (int)v;
-                dig[((size_t)i * P + l) * P + k] = d;
-                v = (v - d) / 1024;
+    // digits of c 2^-sh (row, column): round(c 2^(49 - sh)) in balanced base 1024,
+    // most significant first
+    for (int w = 0; w < 3; ++w) {
+        std::vector<int> dig((size_t)kTcD * P * P);
+        for (int row = 0; row < P; ++row)
+            for (int col = 0; col < P; ++col) {
+                long double c;
+                int sh;
+                if (w == 0) {  // M2L: row l, column k
+                    c = C[(size_t)(row + col) * PP + row];
+                    sh = row + col;
+                } else if (w == 1) {  // M2M: row m, column k
+                    c = C[(size_t)row * PP + col];
+                    sh = row;
+                } else {  // L2L: row m, column l
+                    c = C[(size_t)col * PP + row];
+                    sh = col;
+                }
+                const unsigned __int128 u = (unsigned __int128)(unsigned long long)c << 50;
+                long long v = (long long)(((u >> sh) + 1) >> 1);
+                for (int i = kTcD - 1; i >= 0; --i) {
+                    const int d = (i > 0) ? (int)((v + 512) & 1023) - 512 : (int)v;
+                    dig[((size_t)i * P + row) * P + col] = d;
+                    v = (v - d) / 1024;
+                }
             }
-        }
-    __half* F = reinterpret_cast<__half*>(tab->data() + kFmmAOff);
-    for (int i = 0; i < kTcD; ++i)
-        for (int m = 0; m < 2; ++m)
-            for (int kt = 0; kt < 2; ++kt)
-                for (int lane = 0; lane < 32; ++lane)
-                    for (int u = 0; u < 8; ++u) {  // row g (+ 8 for odd registers), column 2t + (u & 1) (+ 8)
-                        const int row = 16 * m + (lane >> 2) + 8 * ((u >> 1) & 1);
-                        const int col = 16 * kt + 2 * (lane & 3) + (u & 1) + 8 * (u >> 2);
-                        F[((((i * 2 + m) * 2 + kt) * 32) + lane) * 8 + u] =
-                            __float2half((float)dig[((size_t)i * P + row) * P + col]);
-                    }
+        __half* F = reinterpret_cast<__half*>(tab->data() + kFmmAOff + (size_t)w * kFmmASlots);
+        for (int i = 0; i < kTcD; ++i)
+            for (int m = 0; m < 2; ++m)
+                for (int kt = 0; kt < 2; ++kt)
+                    for (int lane = 0; lane < 32; ++lane)
+                        for (int u = 0; u < 8; ++u) {  // row g (+ 8 for odd registers), column 2t + (u & 1) (+ 8)
+                            const int row = 16 * m + (lane >> 2) + 8 * ((u >> 1) & 1);
+                            const int col = 16 * kt + 2 * (lane & 3) + (u & 1) + 8 * (u >> 2);
+                            F[((((i * 2 + m) * 2 + kt) * 32) + lane) * 8 + u] =
+                                __float2half((float)dig[((size_t)i * P + row) * P + col]);
+                        }
+    }
 }
 
 // Pinned host staging for the tree upload (grown on demand, kept for the process).
@@ -1486,7 +1721,7 @@ void release_fmm(Boundary& b) {
         give_stream(false, b.fmm->bst, b.device);
         give_event(b.fmm->ev_nq, b.device);
 
-        if (b.fmm->arena || b.fmm->sync || b.fmm->nq_item || b.fmm->tp || b.fmm->fault) {  // once no stream uses them
+        if (b.fmm->arena || b.fmm->sync || b.fmm->nq_item || b.fmm->tn || b.fmm->path || b.fmm->tp || b.fmm->fault) {  // once no stream uses them
             cudaDeviceSynchronize();
             cudaGetLastError();
             pool_free(b.fmm->arena, 0);
@@ -1500,6 +1735,8 @@ void release_fmm(Boundary& b) {
             pool_free(b.fmm->nt_im, 0);
             pool_free(b.fmm->xs, 0);
             pool_free(b.fmm->fault, 0);
+            pool_free(b.fmm->tn, 0);
+            pool_free(b.fmm->path, 0);
             pool_free(b.fmm->tp, 0);
         }
         delete b.fmm;
@@ -1566,33 +1803,35 @@ static int fmm_tree_host(const Boundary& b, FmmTree* t, cudaStream_t st) {
         L = l;
     }
     t->L = L;
-    // boxes per level (level index l - 2), sorted by key
-    const int nlev = L - 1;
+    const int l0 = fmm_top_level(b, L);
+    t->l0 = l0;
+    // boxes per level (level index l - l0), sorted by key
+    const int nlev = L - l0 + 1;
     std::vector<std::vector<uint32_t>> keys(nlev);
     std::vector<int> leaf_start;
     for (int i = 0; i < N; ++i) {
         const uint32_t k = key_at(i, L);
-        if (i == 0 || k != keys[L - 2].back()) {
-            keys[L - 2].push_back(k);
+        if (i == 0 || k != keys[L - l0].back()) {
+            keys[L - l0].push_back(k);
             leaf_start.push_back(i);
         }
     }
     leaf_start.push_back(N);
-    for (int l = L - 1; l >= 2; --l)
-        for (uint32_t k : keys[l - 1]) {  // children of level l + 1 are keys[l - 1]
+    for (int l = L - 1; l >= l0; --l)
+        for (uint32_t k : keys[l + 1 - l0]) {  // the boxes of level l + 1
             const uint32_t pk = k >> 2;
-            if (keys[l - 2].empty() || keys[l - 2].back() != pk) keys[l - 2].push_back(pk);
+            if (keys[l - l0].empty() || keys[l - l0].back() != pk) keys[l - l0].push_back(pk);
         }
     t->lvl_off.resize(nlev);
     t->lvl_cnt.resize(nlev);
     int nbox = 0;
-    for (int l = 2; l <= L; ++l) {
-        t->lvl_off[l - 2] = nbox;
-        t->lvl_cnt[l - 2] = (int)keys[l - 2].size();
-        nbox += (int)keys[l - 2].size();
+    for (int l = l0; l <= L; ++l) {
+        t->lvl_off[l - l0] = nbox;
+        t->lvl_cnt[l - l0] = (int)keys[l - l0].size();
+        nbox += (int)keys[l - l0].size();
     }
     t->nbox = nbox;
-    t->nleaf = (int)keys[L - 2].size();
+    t->nleaf = (int)keys[L - l0].size();
     auto compact = [](uint32_t v) {  // inverse of spread16
         v &= 0x55555555u;
         v = (v | (v >> 1)) & 0x33333333u;
@@ -1608,30 +1847,30 @@ static int fmm_tree_host(const Boundary& b, FmmTree* t, cudaStream_t st) {
     // box geometry, parents and children: children of a box are contiguous in
     // key order, so one pass over each level links it to the level above
     std::vector<int> bix(nbox), biy(nbox);
-    for (int l = 2; l <= L; ++l)
-        for (int q = 0; q < t->lvl_cnt[l - 2]; ++q) decode(keys[l - 2][q], &bix[t->lvl_off[l - 2] + q],
-                                                           &biy[t->lvl_off[l - 2] + q]);
+    for (int l = l0; l <= L; ++l)
+        for (int q = 0; q < t->lvl_cnt[l - l0]; ++q) decode(keys[l - l0][q], &bix[t->lvl_off[l - l0] + q],
+                                                           &biy[t->lvl_off[l - l0] + q]);
     std::vector<double2> center(nbox);
     std::vector<double> width(nbox);
     std::vector<int> child_start(nbox, -1), child_count(nbox, 0), parent(nbox, -1), quad(nbox, 0);
-    for (int l = 2; l <= L; ++l) {
+    for (int l = l0; l <= L; ++l) {
         const double r = W / (double)(1 << l);
-        for (int q = 0; q < t->lvl_cnt[l - 2]; ++q) {
-            const int g = t->lvl_off[l - 2] + q;
+        for (int q = 0; q < t->lvl_cnt[l - l0]; ++q) {
+            const int g = t->lvl_off[l - l0] + q;
             center[g] = make_double2(x0 + (bix[g] + 0.5) * r, y0 + (biy[g] + 0.5) * r);
             width[g] = r;
             quad[g] = ((bix[g] & 1) << 1) | (biy[g] & 1);
         }
-        if (l == 2) continue;
+        if (l == l0) continue;
         int pq = -1;
         uint32_t last = 0;
-        for (int q = 0; q < t->lvl_cnt[l - 2]; ++q) {
-            const uint32_t pk = keys[l - 2][q] >> 2;
+        for (int q = 0; q < t->lvl_cnt[l - l0]; ++q) {
+            const uint32_t pk = keys[l - l0][q] >> 2;
             if (pq < 0 || pk != last) {
                 ++pq;
                 last = pk;
             }
-            const int g = t->lvl_off[l - 2] + q, pg = t->lvl_off[l - 3] + pq;
+            const int g = t->lvl_off[l - l0] + q, pg = t->lvl_off[l - 1 - l0] + pq;
             parent[g] = pg;
             if (child_start[pg] < 0) child_start[pg] = g;
             ++child_count[pg];
@@ -1639,7 +1878,7 @@ static int fmm_tree_host(const Boundary& b, FmmTree* t, cudaStream_t st) {
     }
     // neighbour lists (adjacent boxes of the same level, the box itself included)
     // and interaction lists, level by level from the children of the parent's
-    // neighbours; level 2 compares all pairs
+    // neighbours; the topmost level compares all pairs
     std::vector<int> nb_start(nbox + 1, 0), nb;
     std::vector<int> il_start(nbox + 1, 0), il_src, il_off;
     nb.reserve((size_t)nbox * 6);
@@ -1651,13 +1890,13 @@ static int fmm_tree_host(const Boundary& b, FmmTree* t, cudaStream_t st) {
             nb.push_back(c);
         } else {
             il_src.push_back(c);
-            il_off.push_back((dx + 3) * 7 + (dy + 3));
+            il_off.push_back((dx + kFmmOffMax) * kFmmOffs + dy + kFmmOffMax);
         }
     };
-    for (int l = 2; l <= L; ++l)
-        for (int q = 0; q < t->lvl_cnt[l - 2]; ++q) {
-            const int g = t->lvl_off[l - 2] + q;
-            if (l == 2) {
+    for (int l = l0; l <= L; ++l)
+        for (int q = 0; q < t->lvl_cnt[l - l0]; ++q) {
+            const int g = t->lvl_off[l - l0] + q;
+            if (l == l0) {
                 for (int c = t->lvl_off[0]; c < t->lvl_off[0] + t->lvl_cnt[0]; ++c) visit(g, c);
             } else {
                 const int pg = parent[g];
@@ -1672,7 +1911,7 @@ static int fmm_tree_host(const Boundary& b, FmmTree* t, cudaStream_t st) {
     // neighbour leaves of each leaf (the leaf itself included)
     std::vector<int> nl_start(t->nleaf + 1, 0), nl_leaf, leaf_box(t->nleaf);
     long long near_pairs = 0;
-    const int loff = t->lvl_off[L - 2];
+    const int loff = t->lvl_off[L - l0];
     for (int q = 0; q < t->nleaf; ++q) {
         leaf_box[q] = loff + q;
         const long long cnt_t = leaf_start[q + 1] - leaf_start[q];
@@ -1878,17 +2117,32 @@ int ensure_fmm(const Boundary& bc, int R, cudaStream_t st) {
             rc = GNK_ENOMEM;
         }
     }
-    // the powers of the P2M: 512 bytes per node, below kTpMaxBytes (else P2M
-    // forms them itself)
-    if (rc == GNK_OK && (double)b.N * kFmmP * sizeof(float4) <= kTpMaxBytes &&
-        pool_alloc(reinterpret_cast<void**>(&t->tp), (size_t)b.N * kFmmP * sizeof(float4), st) == cudaSuccess) {
+    // the nodes' offsets, and for a handle built for differentiation (whose P2M
+    // reads them) their powers, 512 bytes per node, below kTpMaxBytes
+    if (rc == GNK_OK && pool_alloc(reinterpret_cast<void**>(&t->tn), (size_t)b.N * sizeof(float4), st) != cudaSuccess) {
+        cudaGetLastError();
+        set_error("FMM: allocation of the node offsets failed");
+        rc = GNK_ENOMEM;
+    }
+    if (rc == GNK_OK &&
+        pool_alloc(reinterpret_cast<void**>(&t->path), (size_t)t->nleaf * (t->L - t->l0 + 1) * sizeof(unsigned), st) !=
+            cudaSuccess) {
+        cudaGetLastError();
+        set_error("FMM: allocation of the leaves' paths failed");
+        rc = GNK_ENOMEM;
+    }
+    if (rc == GNK_OK && b.diff && (double)b.N * kFmmP * sizeof(float4) <= kTpMaxBytes &&
+        pool_alloc(reinterpret_cast<void**>(&t->tp), (size_t)b.N * kFmmP * sizeof(float4), st) != cudaSuccess)
+        t->tp = nullptr;
+    if (rc == GNK_OK) {
         FmmArgs a;
         b.fmm = t;
         fmm_args(b, a);
-        fmm_tp_build_kernel<<<(b.N + 255) / 256, 256, 0, st>>>(a, t->tp);
-        count_launches(1);
+        fmm_tn_build_kernel<<<(b.N + 255) / 256, 256, 0, st>>>(a, t->tn, t->tp);
+        fmm_path_kernel<<<(t->nleaf + 127) / 128, 128, 0, st>>>(a, t->path);
+        count_launches(2);
         if (cudaGetLastError() != cudaSuccess) {
-            set_error("FMM: launch of the power table failed");
+            set_error("FMM: launch of the node offsets failed");
             rc = GNK_ECUDA;
         }
     }
@@ -1910,11 +2164,10 @@ int ensure_fmm(const Boundary& bc, int R, cudaStream_t st) {
 // Pascal matrix, the two complex scalings (38 each) and the sum (22); 840 per
 // lane for an L2L transform (32 terms of the Pascal sum at 24 each, two exact
 // scalings at 30 and two double-float additions), 742 for an M2M (31 passes
-// of a double-float complex addition, 22 each, and the two scalings); P2M: 36 per
-// complex double-float power (47 per node: 32 orders, the squarings to t^8 in
-// each warp, t^16 and t^24) and 48 R per node and order for the sums; L2P:
-// 58 R per node and order (a complex product and sum), twice that with the
-// derivative.
+// of a double-float complex addition, 22 each, and the two scalings); P2M: 35
+// complex products a node (38 each) and 16 per order for the sums (from the
+// table of a handle built for differentiation 48 per order); L2P: 58 R per node
+// and order (a complex product and sum), twice that with the derivative.
 // which = 0: M2L; 1: the upward pass (P2M and the M2M climb); 2: L2L; 3: L2P;
 // 4: L2P with the derivative.  (The near field: fmm_near_instr.)
 double fmm_instr(const Boundary& b, int R, int which) {
@@ -1923,8 +2176,8 @@ double fmm_instr(const Boundary& b, int R, int which) {
     const double P = kFmmP, m2m = 742.0 * P, l2l = 840.0 * P, m2l = (24.0 * P + 98.0) * P;
     switch (which) {
         case 0: return R * m2l * (double)t->m2l_pairs;
-        case 1: return R * m2m * (double)t->m2m_pairs + (double)b.N * (t->tp ? 48.0 * R * P : 36.0 * 47.0 + 48.0 * R * P);
-        case 2: return R * l2l * (double)t->nleaf * (t->L - 2);
+        case 1: return R * m2m * (double)t->m2m_pairs + (double)b.N * (t->tp ? 48.0 * R * P : R * (38.0 * 35.0 + 16.0 * P));
+        case 2: return R * l2l * (double)t->nleaf * (t->L - t->l0);
         default: return R * (double)b.N * P * 58.0 * (which == 4 ? 2.0 : 1.0);
     }
 }
@@ -2146,14 +2399,14 @@ static int fmm_product(const Boundary& b, FmmArgs& a, int R, bool EF, const Redu
     // level's M2L on a third stream beside the climb measured slower: the two
     // compete for the same SMs.)
     const ProfToken toku = prof_begin(fs, PK_FMMUP);
-    if (R == 2 && a.tp)
-        fmm_up_kernel<2, true><<<t->nleaf, kFmmUT, 0, fs>>>(a);
-    else if (R == 2)
-        fmm_up_kernel<2, false><<<t->nleaf, kFmmUT, 0, fs>>>(a);
+    if (a.tp && R == 2)  // a handle built for differentiation
+        fmm_up_kernel<2><<<t->nleaf, kFmmUT, 0, fs>>>(a);
     else if (a.tp)
-        fmm_up_kernel<1, true><<<t->nleaf, kFmmUT, 0, fs>>>(a);
+        fmm_up_kernel<1><<<t->nleaf, kFmmUT, 0, fs>>>(a);
+    else if (R == 2)
+        fmm_up_tc_kernel<2><<<t->nleaf, kFmmUT, 0, fs>>>(a);
     else
-        fmm_up_kernel<1, false><<<t->nleaf, kFmmUT, 0, fs>>>(a);
+        fmm_up_tc_kernel<1><<<t->nleaf, kFmmUT, 0, fs>>>(a);
     GNK_TRY_CUDA(cudaGetLastError());
     prof_end(toku, PK_FMMUP, 0.0, fs, fmm_instr(b, R, 1));
     const ProfToken tokm = prof_begin(fs, PK_FMM);
@@ -2168,12 +2421,16 @@ static int fmm_product(const Boundary& b, FmmArgs& a, int R, bool EF, const Redu
     GNK_TRY_CUDA(cudaGetLastError());
     prof_end(tokm, PK_FMM, (double)R, fs, fmm_instr(b, R, 0));  // work: Cauchy sums (products)
     launches += 2;
-    if (t->L > 2) {
+    if (t->L > t->l0) {
         const ProfToken tokd = prof_begin(fs, PK_FMML2L);
-        if (R == 2)
+        if (b.diff && R == 2)
             fmm_l2l_kernel<2><<<t->nleaf, 32, 0, fs>>>(a);
-        else
+        else if (b.diff)
             fmm_l2l_kernel<1><<<t->nleaf, 32, 0, fs>>>(a);
+        else if (R == 2)
+            fmm_l2l_tc_kernel<2><<<(t->nleaf + 3) / 4, 32, 0, fs>>>(a);
+        else
+            fmm_l2l_tc_kernel<1><<<(t->nleaf + 3) / 4, 32, 0, fs>>>(a);
         GNK_TRY_CUDA(cudaGetLastError());
         prof_end(tokd, PK_FMML2L, 0.0, fs, fmm_instr(b, R, 2));
         ++launches;
@@ -2267,9 +2524,15 @@ static void fmm_args(const Boundary& b, FmmArgs& a) {
     a.bUp = t->bUp;
     a.m2lT = t->m2lT;
     a.m2lA = t->m2lA;
+    a.upA = t->m2lA + kFmmASlots;
+    a.dnA = t->m2lA + 2 * kFmmASlots;
+    a.path = t->path;
+    a.depth = t->L - t->l0 + 1;
+    a.nleaf = t->nleaf;
     a.ucnt = t->sync;
     a.xs = nullptr;
     a.near_scaled = 0;
+    a.tn = t->tn;
     a.tp = t->tp;
     a.mult = t->mult;
     a.loc = t->loc;

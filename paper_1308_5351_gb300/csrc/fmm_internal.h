@@ -15,12 +15,16 @@ constexpr int kFmmP = 32;     // expansion order (one warp lane per coefficient)
 #define GNK_FMM_LEAF 64
 #endif
 constexpr int kFmmLeaf = GNK_FMM_LEAF;  // target mean number of nodes per leaf
+// M2L offsets between boxes of the topmost level span the grid of level 3
+constexpr int kFmmOffMax = 7;
+constexpr int kFmmOffs = 2 * kFmmOffMax + 1;  // offset code (dx + 7) 15 + (dy + 7)
 constexpr int kFmmNT = 256;   // threads of the near-field kernel: 8 warps
 constexpr int kFmmMaxNbr = 9;  // a leaf and its eight neighbours
 
 struct FmmTree {
     int L = 0, nbox = 0, nleaf = 0, R = 0;
-    std::vector<int> lvl_off;   // first global box index of level l (index l - 2), size L - 1
+    int l0 = 2;                 // the topmost level with expansions
+    std::vector<int> lvl_off;   // first global box index of level l (index l - l0), size L - l0 + 1
     std::vector<int> lvl_cnt;
     long long near_pairs = 0, m2l_pairs = 0, m2m_pairs = 0;
     void* arena = nullptr;
@@ -34,7 +38,7 @@ struct FmmTree {
     double* width = nullptr;    // per box
     int* child_start = nullptr; // per box: first child (global), level < L
     int* child_count = nullptr;
-    int* parent = nullptr;      // per box, -1 on level 2
+    int* parent = nullptr;      // per box, -1 on level l0
     int* quad = nullptr;        // quadrant of a box in its parent: 2 qa + qb
     int* il_start = nullptr;    // interaction lists (nbox + 1), sources, offset codes
     int* il_src = nullptr;
@@ -74,7 +78,9 @@ struct FmmTree {
     float4* nq_im = nullptr;
     float4* nt_im = nullptr;
     int* fault = nullptr;       // set by a bounded wait of an FMM kernel that gave up
-    float4* tp = nullptr;       // [N][P] powers t^k of each node about its leaf centre (P2M), or null
+    unsigned* path = nullptr;   // [nleaf][L - l0 + 1]: box | quadrant << 30 of each leaf and its ancestors
+    float4* tn = nullptr;       // [N] offset of each node from its leaf centre in leaf widths
+    float4* tp = nullptr;       // [N][P] its powers (handles built for differentiation), or null
     cudaStream_t aux = nullptr; // high-priority stream of the far field (the near field runs beside it)
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaStream_t bst = nullptr; // stream of the near cache's formation when it starts early
@@ -87,11 +93,17 @@ struct FmmTree {
 // GNK_OK, an error code, or kFmmUseHost when the tree is too deep for the
 // device lookup grids (then the host builder runs).
 constexpr int kFmmUseHost = 1;
+
+// The topmost level with expansions.  From level 3 on in trees of level 4 and more (all of whose boxes then
+// interact where they are not adjacent, at most 60 each) the climb and the descent
+// are one level shorter: about 8 us of latency per product against some 2,000
+// more M2L pairs.  Handles built for differentiation keep level 2.
+inline int fmm_top_level(const Boundary& b, int L) { return (b.diff || L < 4) ? 2 : 3; }
 int fmm_tree_device(const Boundary& b, FmmTree* t, cudaStream_t st);
 
 // Points t at the translation tables on the current device (formed and uploaded
 // once per device and process): the M2L Pascal matrix C(k+l, l)
-// [P][P] and, per offset code (dx + 3) 7 + (dy + 3), the scalings
+// [P][P] and, per offset code, the scalings
 // (-1)^(k+1) delta^-(k+1) and delta^-l; the L2L Pascal matrix C(l, m).
 int fmm_device_tables(FmmTree* t, cudaStream_t st);
 

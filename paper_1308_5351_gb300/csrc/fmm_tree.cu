@@ -9,7 +9,8 @@
 //   5. per level, box ids by block counts, a scan over blocks and warp ballots;
 //   6. box centres, widths, parents and child ranges from the first node of each box;
 //   7. dense lookup grids of the boxes of each level, then interaction lists
-//      (children of the parent's neighbours that are not adjacent) and the
+//      (children of the parent's neighbours that are not adjacent; on the topmost
+//      level every box that is not adjacent) and the
 //      neighbour leaves of each leaf, counted, scanned and filled;
 //   8. node order, positions, exact three-float splits and near-field work items.
 // Every step is deterministic (counts and scans in a fixed order), so the tree,
@@ -258,13 +259,13 @@ __global__ void __launch_bounds__(TB) tb_firstdiff(const uint32_t* __restrict__ 
 }
 
 // ---- 5. box ids per level: node i starts a box of level l when fd[i] <= l
-__global__ void __launch_bounds__(LV_BLOCK) tb_lcount(const unsigned char* __restrict__ fd, int N, int L,
+__global__ void __launch_bounds__(LV_BLOCK) tb_lcount(const unsigned char* __restrict__ fd, int N, int l0, int L,
                                                       unsigned* cnt, int nb) {
     const int i = blockIdx.x * LV_BLOCK + threadIdx.x;
     const int f = (i < N) ? fd[i] : 99;
-    for (int l = 2; l <= L; ++l) {
+    for (int l = l0; l <= L; ++l) {
         const int c = __syncthreads_count(f <= l);
-        if (threadIdx.x == 0) cnt[(size_t)(l - 2) * nb + blockIdx.x] = (unsigned)c;
+        if (threadIdx.x == 0) cnt[(size_t)(l - l0) * nb + blockIdx.x] = (unsigned)c;
     }
 }
 
@@ -294,36 +295,36 @@ __global__ void __launch_bounds__(1024) tb_lscan(unsigned* cnt, int nb, unsigned
 }
 
 // box id of every node at every level, and the first node of every box
-__global__ void __launch_bounds__(LV_BLOCK) tb_lids(const unsigned char* __restrict__ fd, int N, int L,
+__global__ void __launch_bounds__(LV_BLOCK) tb_lids(const unsigned char* __restrict__ fd, int N, int l0, int L,
                                                     const unsigned* __restrict__ cnt, int nb, int* boxid,
                                                     int* first) {
     __shared__ unsigned wsum[LV_BLOCK / 32];
     const int i = blockIdx.x * LV_BLOCK + threadIdx.x;
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int f = (i < N) ? fd[i] : 99;
-    for (int l = 2; l <= L; ++l) {
+    for (int l = l0; l <= L; ++l) {
         const bool start = f <= l;
         const unsigned bal = __ballot_sync(0xffffffffu, start);
         if (lane == 0) wsum[wid] = __popc(bal);
         __syncthreads();
-        unsigned before = cnt[(size_t)(l - 2) * nb + blockIdx.x];
+        unsigned before = cnt[(size_t)(l - l0) * nb + blockIdx.x];
         for (int w = 0; w < wid; ++w) before += wsum[w];
         before += __popc(bal & ((1u << lane) - 1u));
         if (i < N) {
             const int id = (int)before + (start ? 1 : 0) - 1;  // node 0 starts every level
-            boxid[(size_t)(l - 2) * N + i] = id;
-            if (start) first[(size_t)(l - 2) * (N + 1) + id] = i;
+            boxid[(size_t)(l - l0) * N + i] = id;
+            if (start) first[(size_t)(l - l0) * (N + 1) + id] = i;
         }
         __syncthreads();
     }
 }
 
 struct TreeDev {
-    int N, L, nbox, nleaf;
+    int N, l0, L, nbox, nleaf;
     const uint32_t* key;     // sorted keys
-    const int* boxid;        // [l - 2][N]
-    const int* first;        // [l - 2][N + 1]
-    const int* lvl_off;      // [L - 1]
+    const int* boxid;        // [l - l0][N]
+    const int* first;        // [l - l0][N + 1]
+    const int* lvl_off;      // [L - l0 + 1]
     const int* lvl_cnt;
     const double* geom;
     double2* center;
@@ -349,8 +350,8 @@ struct TreeDev {
 };
 
 __device__ __forceinline__ int level_of(const TreeDev& t, int g) {
-    int l = 2;
-    while (l < t.L && g >= t.lvl_off[l - 1]) ++l;
+    int l = t.l0;
+    while (l < t.L && g >= t.lvl_off[l + 1 - t.l0]) ++l;
     return l;
 }
 
@@ -359,9 +360,9 @@ __global__ void tb_boxes(TreeDev t) {
     const int g = blockIdx.x * TB + threadIdx.x;
     if (g >= t.nbox) return;
     const int l = level_of(t, g);
-    const int b = g - t.lvl_off[l - 2];
-    const int f = t.first[(size_t)(l - 2) * (t.N + 1) + b];
-    const int fn = (b + 1 < t.lvl_cnt[l - 2]) ? t.first[(size_t)(l - 2) * (t.N + 1) + b + 1] : t.N;
+    const int b = g - t.lvl_off[l - t.l0];
+    const int f = t.first[(size_t)(l - t.l0) * (t.N + 1) + b];
+    const int fn = (b + 1 < t.lvl_cnt[l - t.l0]) ? t.first[(size_t)(l - t.l0) * (t.N + 1) + b + 1] : t.N;
     const uint32_t k = t.key[f] >> (2 * (16 - l));
     const int ix = (int)compact16d(k >> 1), iy = (int)compact16d(k);
     const double W = t.geom[2], r = W / (double)(1 << l);
@@ -370,10 +371,10 @@ __global__ void tb_boxes(TreeDev t) {
     t.quad[g] = ((ix & 1) << 1) | (iy & 1);
     t.bix[g] = ix;
     t.biy[g] = iy;
-    t.parent[g] = (l > 2) ? t.lvl_off[l - 3] + t.boxid[(size_t)(l - 3) * t.N + f] : -1;
+    t.parent[g] = (l > t.l0) ? t.lvl_off[l - 1 - t.l0] + t.boxid[(size_t)(l - 1 - t.l0) * t.N + f] : -1;
     if (l < t.L) {
-        const int c0 = t.boxid[(size_t)(l - 1) * t.N + f], c1 = t.boxid[(size_t)(l - 1) * t.N + fn - 1];
-        t.child_start[g] = t.lvl_off[l - 1] + c0;
+        const int c0 = t.boxid[(size_t)(l + 1 - t.l0) * t.N + f], c1 = t.boxid[(size_t)(l + 1 - t.l0) * t.N + fn - 1];
+        t.child_start[g] = t.lvl_off[l + 1 - t.l0] + c0;
         t.child_count[g] = c1 - c0 + 1;
     } else {
         t.child_start[g] = -1;
@@ -382,13 +383,13 @@ __global__ void tb_boxes(TreeDev t) {
         t.leaf_box[b] = g;
         if (b == t.nleaf - 1) t.leaf_start[t.nleaf] = t.N;
     }
-    t.grid[t.grid_off[l - 2] + (long long)ix * (1 << l) + iy] = g;
+    t.grid[t.grid_off[l - t.l0] + (long long)ix * (1 << l) + iy] = g;
 }
 
 __device__ __forceinline__ int grid_at(const TreeDev& t, int l, int ix, int iy) {
     const int n = 1 << l;
     if (ix < 0 || iy < 0 || ix >= n || iy >= n) return -1;
-    return t.grid[t.grid_off[l - 2] + (long long)ix * n + iy];
+    return t.grid[t.grid_off[l - t.l0] + (long long)ix * n + iy];
 }
 
 // ---- 7. lists: pass 0 counts, pass 1 fills (after the counts are scanned)
@@ -398,22 +399,26 @@ __global__ void tb_lists(TreeDev t, int pass) {
     const int l = level_of(t, g);
     const int ix = t.bix[g], iy = t.biy[g], pa = ix >> 1, pb = iy >> 1;
     unsigned n = 0, pos = pass ? t.il_cnt[g] : 0u;
-    for (int sa = 2 * pa - 2; sa <= 2 * pa + 3; ++sa)
-        for (int sb = 2 * pb - 2; sb <= 2 * pb + 3; ++sb) {
+    // the children of the parent's neighbours; on the topmost level every box
+    const bool top = l == t.l0;
+    const int a0 = top ? 0 : 2 * pa - 2, a1 = top ? (1 << l) - 1 : 2 * pa + 3;
+    const int b0 = top ? 0 : 2 * pb - 2, b1 = top ? (1 << l) - 1 : 2 * pb + 3;
+    for (int sa = a0; sa <= a1; ++sa)
+        for (int sb = b0; sb <= b1; ++sb) {
             const int dx = sa - ix, dy = sb - iy;
             if (dx >= -1 && dx <= 1 && dy >= -1 && dy <= 1) continue;
             const int s = grid_at(t, l, sa, sb);
             if (s < 0) continue;
             if (pass) {
                 t.il_src[pos] = s;
-                t.il_off[pos] = (dx + 3) * 7 + (dy + 3);
+                t.il_off[pos] = (dx + kFmmOffMax) * kFmmOffs + dy + kFmmOffMax;
                 ++pos;
             }
             ++n;
         }
     if (!pass) t.il_cnt[g] = n;
     if (l != t.L) return;
-    const int q = g - t.lvl_off[t.L - 2];
+    const int q = g - t.lvl_off[t.L - t.l0];
     const int cnt_t = t.leaf_start[q + 1] - t.leaf_start[q];
     unsigned m = 0, npos = pass ? t.nl_cnt[q] : 0u;
     unsigned long long pairs = 0;
@@ -421,7 +426,7 @@ __global__ void tb_lists(TreeDev t, int pass) {
         for (int sb = iy - 1; sb <= iy + 1; ++sb) {
             const int s = grid_at(t, l, sa, sb);
             if (s < 0) continue;
-            const int lq = s - t.lvl_off[t.L - 2];
+            const int lq = s - t.lvl_off[t.L - t.l0];
             if (pass) {
                 t.nl_leaf[npos++] = lq;
             } else {
@@ -545,7 +550,9 @@ int fmm_tree_device(const Boundary& b, FmmTree* t, cudaStream_t st) {
     }
     if (L > kMaxGridLevel) return kFmmUseHost;
     t->L = L;
-    const int nlev = L - 1;
+    const int l0 = fmm_top_level(b, L);
+    t->l0 = l0;
+    const int nlev = L - l0 + 1;
     // per-level box ids (second temporary block)
     char* tmp2 = nullptr;
     const size_t o2_boxid = 0;
@@ -559,9 +566,9 @@ int fmm_tree_device(const Boundary& b, FmmTree* t, cudaStream_t st) {
     Free free_tmp2{&tmp2, st};
     int* boxid = (int*)(tmp2 + o2_boxid);
     int* first = (int*)(tmp2 + o2_first);
-    tb_lcount<<<nbl, LV_BLOCK, 0, st>>>(fd, N, L, cnt, nbl);
+    tb_lcount<<<nbl, LV_BLOCK, 0, st>>>(fd, N, l0, L, cnt, nbl);
     tb_lscan<<<nlev, 1024, 0, st>>>(cnt, nbl, tot);
-    tb_lids<<<nbl, LV_BLOCK, 0, st>>>(fd, N, L, cnt, nbl, boxid, first);
+    tb_lids<<<nbl, LV_BLOCK, 0, st>>>(fd, N, l0, L, cnt, nbl, boxid, first);
     GNK_TRY_CUDA(cudaGetLastError());
     std::vector<unsigned> ncnt(nlev);
     GNK_TRY_CUDA(cudaMemcpyAsync(ncnt.data(), tot, nlev * sizeof(unsigned), cudaMemcpyDeviceToHost, st));
@@ -569,23 +576,24 @@ int fmm_tree_device(const Boundary& b, FmmTree* t, cudaStream_t st) {
     t->lvl_off.resize(nlev);
     t->lvl_cnt.resize(nlev);
     int nbox = 0;
-    for (int l = 2; l <= L; ++l) {
-        t->lvl_off[l - 2] = nbox;
-        t->lvl_cnt[l - 2] = (int)ncnt[l - 2];
-        nbox += (int)ncnt[l - 2];
+    for (int l = l0; l <= L; ++l) {
+        t->lvl_off[l - l0] = nbox;
+        t->lvl_cnt[l - l0] = (int)ncnt[l - l0];
+        nbox += (int)ncnt[l - l0];
     }
-    const int nleaf = t->lvl_cnt[L - 2];
+    const int nleaf = t->lvl_cnt[L - l0];
     t->nbox = nbox;
     t->nleaf = nleaf;
     std::vector<long long> goff(nlev);
     long long gcells = 0;
-    for (int l = 2; l <= L; ++l) {
-        goff[l - 2] = gcells;
+    for (int l = l0; l <= L; ++l) {
+        goff[l - l0] = gcells;
         gcells += (1LL << (2 * l));
     }
-    // upper bounds of the list lengths: 27 interactions per box, 9 neighbours per
-    // leaf, one chunk of 32 per leaf plus one per 32 nodes
-    const size_t max_il = (size_t)27 * nbox + 1, max_nl = (size_t)9 * nleaf + 1;
+    // upper bounds of the list lengths: 27 interactions per box (60 on the topmost
+    // level, of at most 64 boxes), 9 neighbours per leaf, one chunk of 32 per leaf
+    // plus one per 32 nodes
+    const size_t max_il = (size_t)27 * nbox + 33 * 64 + 1, max_nl = (size_t)9 * nleaf + 1;
     const size_t max_it = (size_t)nleaf + N / 32 + 1;
     // the handle's tree arena (the same layout as the host builder's)
     const size_t P = kFmmP;
@@ -661,6 +669,7 @@ int fmm_tree_device(const Boundary& b, FmmTree* t, cudaStream_t st) {
     GNK_TRY_CUDA(cudaMemcpyAsync(tmp3 + o3_go, goff.data(), nlev * 8, cudaMemcpyHostToDevice, st));
     TreeDev d;
     d.N = N;
+    d.l0 = l0;
     d.L = L;
     d.nbox = nbox;
     d.nleaf = nleaf;
@@ -708,7 +717,7 @@ int fmm_tree_device(const Boundary& b, FmmTree* t, cudaStream_t st) {
         tb_scan<<<3, 1024, 0, st>>>(sa);
     }
     tb_lists<<<gb, TB, 0, st>>>(d, 1);
-    tb_nodes<<<(N + TB - 1) / TB, TB, 0, st>>>(b.et, N, i0, boxid + (size_t)(L - 2) * N, t->lvl_off[L - 2],
+    tb_nodes<<<(N + TB - 1) / TB, TB, 0, st>>>(b.et, N, i0, boxid + (size_t)(L - l0) * N, t->lvl_off[L - l0],
                                                t->perm, t->ps, t->p3, t->p3b, t->node_box);
     GNK_TRY_CUDA(cudaGetLastError());
     // CSR starts: the scanned counts with their totals appended

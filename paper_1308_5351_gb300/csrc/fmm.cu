@@ -102,34 +102,37 @@ struct FmmArgs {
     double2* outF;      // [R][N] F sums in node order (EF products)
     const int* node_box;  // leaf box of each node in sorted order
     int* ucnt;            // per box: children counted in the upward pass
-    float2* xs;           // [R][N] x in sorted order as double-float (cached near field), or null
+    int nsplit;           // shares of the near field, [share][R][N] in zn
+    int gathered;         // ws holds the weights in sorted order (products with a direct near field)
     int near_scaled;      // zn holds the near field times the operator's factor (cached)
     const float4* tn;     // [N] offset t of every node from its leaf centre in leaf widths (double-float complex)
     const float4* tp;     // [N][P] powers t^k (handles built for differentiation), or null
     int* fault;           // set by a bounded wait that gave up
 };
 
+// The weight of right-hand side r at node j, double-float complex.
+__device__ __forceinline__ float4 fmm_weight(const FmmArgs& a, int r, int j) {
+    double2 w;
+    if (a.mode == W_COMPLEX) {
+        w = (r == 0) ? a.w0[j] : a.w1[j];
+    } else {
+        const double2 sc = a.s[j];
+        const double x = (r == 0) ? a.x0[j] : a.x1[j];
+        w = make_double2(sc.x * x, sc.y * x);
+    }
+    const df wx = df_split_fast(w.x), wy = df_split_fast(w.y);
+    return make_float4(wx.h, wx.l, wy.h, wy.l);
+}
+
+// The weights in sorted order, for the products whose near field is summed
+// directly (every leaf's sources are read by its neighbours); with a cached near
+// field P2M is their only reader and forms them itself.
 __global__ void fmm_gather_kernel(FmmArgs a) {
     if (a.done != nullptr && *a.done) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.N) return;
     const int j = a.perm[i];
-    for (int r = 0; r < a.R; ++r) {
-        double2 w;
-        if (a.mode == W_COMPLEX) {
-            w = (r == 0) ? a.w0[j] : a.w1[j];
-        } else {
-            const double2 sc = a.s[j];
-            const double x = (r == 0) ? a.x0[j] : a.x1[j];
-            w = make_double2(sc.x * x, sc.y * x);
-        }
-        const df wx = df_split_fast(w.x), wy = df_split_fast(w.y);
-        a.ws[(size_t)r * a.N + i] = make_float4(wx.h, wx.l, wy.h, wy.l);
-        if (a.xs != nullptr) {  // x alone for the cached near field (W_SCALED)
-            const df xv = df_split_fast((r == 0) ? a.x0[j] : a.x1[j]);
-            a.xs[(size_t)r * a.N + i] = make_float2(xv.h, xv.l);
-        }
-    }
+    for (int r = 0; r < a.R; ++r) a.ws[(size_t)r * a.N + i] = fmm_weight(a, r, j);
 }
 
 // ---- complex double-float arithmetic for the far field (FP32 pipe).  The
@@ -360,7 +363,7 @@ __device__ __forceinline__ void p2m_leaf(const FmmArgs& a, int leaf, int box, in
             v[0] = t;
             if (j < j1) {
                 t = pc_of(__ldg(a.tn + j));
-                v[0] = pc_of(__ldcg(a.ws + (size_t)r * a.N + j));
+                v[0] = pc_of(a.gathered ? __ldcg(a.ws + (size_t)r * a.N + j) : fmm_weight(a, r, __ldg(a.perm + j)));
             }
             {
                 const df2 t2 = pc_mul(t, t), t4 = pc_mul(t2, t2), t8 = pc_mul(t4, t4), t16 = pc_mul(t8, t8);
@@ -588,7 +591,10 @@ __device__ __forceinline__ df2 diff3_2(float2 p1, float2 p2, float2 p3, float2 q
 // A warp takes tiles of four entries of the box's interaction list; the warps'
 // sums are added in warp order.
 constexpr int kTcD = 5;
-constexpr int kTcWarps = 4;
+// warps per box: two where there are boxes enough to fill the SMs (beside the near
+// field 1, 2 and 4 are within 1.5 % at 1,700 boxes and more), eight in small trees,
+// where the topmost boxes' 60 entries would be a chain of tiles
+constexpr int kTcManyBoxes = 1024;
 
 __device__ __forceinline__ void mma_f16(float (&c)[4], const uint4 a, unsigned b0, unsigned b1) {
     asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -720,9 +726,9 @@ __device__ __forceinline__ df2 tc_scale_out(df2 y, float2 g) {
     return df2_add(df2{mul2(y.h, gr), mul2(y.l, gr)}, df2{mul2(xh, gi), mul2(xl, gi)});
 }
 
-template <int R>
-__global__ void __launch_bounds__(32 * kTcWarps) fmm_m2l_tc_kernel(FmmArgs a) {
-    __shared__ float4 s_acc[kTcWarps][32];
+template <int R, int W>
+__global__ void __launch_bounds__(32 * W) fmm_m2l_tc_kernel(FmmArgs a) {
+    __shared__ float4 s_acc[W][32];
     if (a.done != nullptr && *a.done) return;
     const int box = blockIdx.x, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3, part = g & 1;
@@ -733,11 +739,22 @@ __global__ void __launch_bounds__(32 * kTcWarps) fmm_m2l_tc_kernel(FmmArgs a) {
         df2 acc[4];  // (re, im) of rows l = g + 8 i
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[i] = df2{f2(0.f), f2(0.f)};
-        for (int base = e0 + 4 * wid; base < e1; base += 4 * kTcWarps) {
-            const int eb = min(base + (g >> 1), e1 - 1), ec = min(base + t, e1 - 1);
-            const float4* S = a.m2lT + (size_t)a.il_off[eb] * 2 * kFmmP;
-            const float4* A = a.mult + ((size_t)r * a.nbox + a.il_src[eb]) * kFmmP;
-            const float4* Q = a.m2lT + ((size_t)a.il_off[ec] * 2 + 1) * kFmmP;
+        // the list entries of a tile are loaded during the one before
+        int base = e0 + 4 * wid, ob = 0, sb = 0, oc = 0;
+        if (base < e1) {
+            ob = __ldg(a.il_off + min(base + (g >> 1), e1 - 1));
+            sb = __ldg(a.il_src + min(base + (g >> 1), e1 - 1));
+            oc = __ldg(a.il_off + min(base + t, e1 - 1));
+        }
+        for (; base < e1; base += 4 * W) {
+            const float4* S = a.m2lT + (size_t)ob * 2 * kFmmP;
+            const float4* A = a.mult + ((size_t)r * a.nbox + sb) * kFmmP;
+            const float4* Q = a.m2lT + ((size_t)oc * 2 + 1) * kFmmP;
+            if (base + 4 * W < e1) {
+                ob = __ldg(a.il_off + min(base + 4 * W + (g >> 1), e1 - 1));
+                sb = __ldg(a.il_src + min(base + 4 * W + (g >> 1), e1 - 1));
+                oc = __ldg(a.il_off + min(base + 4 * W + t, e1 - 1));
+            }
             const bool live = base + (g >> 1) < e1;
             df2 x[4], y[4];
 #pragma unroll
@@ -773,7 +790,7 @@ __global__ void __launch_bounds__(32 * kTcWarps) fmm_m2l_tc_kernel(FmmArgs a) {
         __syncthreads();
         if (wid == 0) {
             cdf b = cdf_of(s_acc[0][lane]);
-            for (int w = 1; w < kTcWarps; ++w) b = cdf_add(b, cdf_of(s_acc[w][lane]));
+            for (int w = 1; w < W; ++w) b = cdf_add(b, cdf_of(s_acc[w][lane]));
             a.loc[((size_t)r * a.nbox + box) * kFmmP + lane] = cdf_pack(cdf{df_mul(b.re, sc), df_mul(b.im, sc)});
         }
         if (R > 1) __syncthreads();
@@ -1257,34 +1274,36 @@ __global__ void __launch_bounds__(kFmmNT) fmm_nq_build_kernel(FmmArgs a, const d
 }
 
 // A cached near field, streamed into shared memory by the Tensor Memory
-// Accelerator: one block per work item; a producer warp issues bulk copies of
-// the item's cache entries (contiguous, pair-major) in chunks of kNbPairs
-// source pairs through a ring of kNbStages buffers (full/empty mbarriers) and
-// gathers the x of the chunk's sources itself, one pair per lane, from the
-// sorted x (the sources of an item are at most nine runs of sorted nodes, so the
-// loads are nearly coalesced and come from L2): 8 bytes per source instead of
-// the index read, x written and read back of a gather launch of its own, which
-// took 19 us per product at 65,536 nodes and 350 us at 524,288.  8
-// consumer warps, lane = target, warp w taking pairs w, w + 8, ... of each
-// chunk.  Even and odd sources go to the two halves of packed float2 sums,
+// Accelerator: one block per work item (or, where the items do not fill the
+// SMs, per item and share of its sources); a producer thread issues bulk copies
+// of the item's cache entries (contiguous, pair-major) in chunks of kNbPairs
+// source pairs through a ring of kNbStages buffers (full/empty mbarriers).  The 8
+// consumer warps first gather the x of the item's sources (at most nine runs of
+// sorted nodes) through the node order into shared memory, all loads independent,
+// while the first copies are in flight (lists of x written by a launch of their
+// own took 19 us per product at 65,536 nodes and 350 us at 524,288; a gather by
+// the producer, chunk by chunk, made small items a chain of load latencies, 26 us
+// for 2,560 nodes); then lane = target, warp w taking pairs w, w + 8, ... of
+// each chunk.  Even and odd sources go to the two halves of packed float2 sums,
 // added at the end, then the warps' sums in warp order.  COMP = 1: the imaginary
 // part only (the real part written as 0).  `stream`: the entries are marked
 // evict-first in L2 (a cache larger than L2 read once per product must not push
 // out what is reused).  Every wait is bounded (kNbSpin polls); one that gives up
 // sets a.fault, and the producer still waits (bounded) for its copies in flight
 // before leaving.
-constexpr int kNbPairs = 32;                 // source pairs per chunk: one per producer lane
+constexpr int kNbPairs = 24;                 // source pairs per chunk, three per consumer warp
 constexpr int kNbStages = 3;
 constexpr int kNbThreads = kFmmNT + 32;      // 8 consumer warps and the producer warp
 constexpr int kNbSpin = 1 << 22;
+constexpr int kNbSegChunks = 20;             // chunks whose x is gathered at once
+constexpr int kNbX = 2 * kNbPairs * kNbSegChunks;
 
 template <int R, int COMP>
 struct NbLayout {
     static constexpr int kParts = COMP == 0 ? 2 : 1;
     static constexpr int kQ = kNbPairs * 32;                  // float4 entries of one part (tn <= 32)
-    static constexpr int kX = kNbPairs;                       // float4 of x per right-hand side (a pair each)
-    static constexpr int kStage = kParts * kQ + R * kX;       // float4 per stage
-    static constexpr int kBytes = kNbStages * kStage * 16;    // dynamic shared memory
+    static constexpr int kStage = kParts * kQ;                // float4 per stage
+    static constexpr int kBytes = kNbStages * kStage * 16 + R * kNbX * 8;  // dynamic shared memory
 };
 
 template <int R, int COMP>
@@ -1295,6 +1314,7 @@ __global__ void __launch_bounds__(kNbThreads) fmm_near_bulk_kernel(FmmArgs a, co
                                                                    const float4* __restrict__ nq_im, int stream) {
     using L = NbLayout<R, COMP>;
     extern __shared__ __align__(16) float4 nb_buf[];
+    float2* s_x = reinterpret_cast<float2*>(nb_buf + kNbStages * L::kStage);  // [R][kNbX]
     __shared__ __align__(8) unsigned long long full[kNbStages], empty[kNbStages];
     __shared__ double2 s_z[kFmmWarps][R][32];
     if (a.done != nullptr && *a.done) return;  // set before this launch: the same in every thread
@@ -1305,38 +1325,26 @@ __global__ void __launch_bounds__(kNbThreads) fmm_near_bulk_kernel(FmmArgs a, co
     const int S = d.x, tn = d.y;
     const int npair = (S + 1) >> 1;
     const int nch = (npair + kNbPairs - 1) / kNbPairs;
-    if (threadIdx.x == 0) {
+    const int cb = nch * (int)blockIdx.y / (int)gridDim.y, ce = nch * ((int)blockIdx.y + 1) / (int)gridDim.y;
+    if (threadIdx.x == kFmmNT) {
         for (int k = 0; k < kNbStages; ++k) {
-            mbar_init(&full[k], 2);  // the copies' announcement and the x of the chunk
+            mbar_init(&full[k], 1);
             mbar_init(&empty[k], kFmmWarps);
         }
     }
     __syncthreads();
     if (wid == kFmmWarps) {  // the producer
-        const int2 run = (lane < kFmmMaxNbr) ? __ldg(nq_run + (size_t)it * kFmmMaxNbr + lane) : make_int2(0, INT_MAX);
-        int c = 0;
-        for (; c < nch; ++c) {
-            const int st = c % kNbStages;
-            const int p0 = c * kNbPairs, np = min(kNbPairs, npair - p0);
-            float4* stage = nb_buf + (size_t)st * L::kStage;
-            const int q = 2 * (p0 + lane);
-            const int j0 = nq_source(run, q), j1 = nq_source(run, q + 1);
-            float4 xv[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) {  // (0, 0) past the item's sources
-                const float2* xr = a.xs + (size_t)r * a.N;
-                const float2 u = (q < S) ? __ldg(xr + j0) : make_float2(0.f, 0.f);
-                const float2 v = (q + 1 < S) ? __ldg(xr + j1) : make_float2(0.f, 0.f);
-                xv[r] = make_float4(u.x, u.y, v.x, v.y);
-            }
-            bool ok = true;
-            if (c >= kNbStages) ok = mbar_wait(&empty[st], (unsigned)((c / kNbStages - 1) & 1), kNbSpin);
-            if (!__all_sync(0xffffffffu, ok)) {
-                if (lane == 0) atomicExch(a.fault, 1);
-                break;
-            }
-            if (lane == 0) {
+        if (lane == 0) {
+            int c = cb;
+            for (; c < ce; ++c) {
+                const int u = c - cb, st = u % kNbStages;
+                if (u >= kNbStages && !mbar_wait(&empty[st], (unsigned)((u / kNbStages - 1) & 1), kNbSpin)) {
+                    atomicExch(a.fault, 1);
+                    break;
+                }
+                const int p0 = c * kNbPairs, np = min(kNbPairs, npair - p0);
                 const unsigned qbytes = (unsigned)(np * tn) * 16u;
+                float4* stage = nb_buf + (size_t)st * L::kStage;
                 mbar_expect_tx(&full[st], L::kParts * qbytes);
                 const float4* im = nq_im + o0 + (long long)p0 * tn;
                 const float4* re = (COMP == 0) ? nq_re + o0 + (long long)p0 * tn : nullptr;
@@ -1348,50 +1356,67 @@ __global__ void __launch_bounds__(kNbThreads) fmm_near_bulk_kernel(FmmArgs a, co
                     if (COMP == 0) bulk_load(stage + L::kQ, re, qbytes, &full[st]);
                 }
             }
-#pragma unroll
-            for (int r = 0; r < R; ++r) stage[L::kParts * L::kQ + r * L::kX + lane] = xv[r];
-            __syncwarp();  // every lane's x before the arrival
-            if (lane == 0) mbar_arrive(&full[st]);
-        }
-        if (lane == 0) {  // the copies still in flight land before the warp leaves
-            for (int k = max(0, c - kNbStages); k < c; ++k)
-                mbar_wait(&full[k % kNbStages], (unsigned)((k / kNbStages) & 1), kNbSpin);
+            // the copies still in flight land before the warp leaves
+            for (int k = max(cb, c - kNbStages); k < c; ++k)
+                mbar_wait(&full[(k - cb) % kNbStages], (unsigned)(((k - cb) / kNbStages) & 1), kNbSpin);
         }
         return;
     }
+    const int2 run = (lane < kFmmMaxNbr) ? __ldg(nq_run + (size_t)it * kFmmMaxNbr + lane) : make_int2(0, INT_MAX);
     df2 are[R], aim[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) are[r] = aim[r] = df2{f2(0.f), f2(0.f)};
-    for (int c = 0; c < nch; ++c) {
-        const int st = c % kNbStages;
-        if (!mbar_wait(&full[st], (unsigned)((c / kNbStages) & 1), kNbSpin)) {
-            atomicExch(a.fault, 1);
-            break;
-        }
-        const float4* qi = nb_buf + (size_t)st * L::kStage;
-        const float4* qr = qi + L::kQ;
-        const float4* xv4 = qi + L::kParts * L::kQ;
-        const int np = min(kNbPairs, npair - c * kNbPairs);
-        if (lane < tn) {
-            for (int pp = wid; pp < np; pp += kFmmWarps) {
-                const float4 wi = qi[pp * tn + lane];
-                const df2 Qi{make_float2(wi.x, wi.y), make_float2(wi.z, wi.w)};
-                df2 Qr{f2(0.f), f2(0.f)};
-                if (COMP == 0) {
-                    const float4 wr = qr[pp * tn + lane];
-                    Qr = df2{make_float2(wr.x, wr.y), make_float2(wr.z, wr.w)};
-                }
+    bool ok = true;
+    for (int seg = cb; seg < ce; seg += kNbSegChunks) {
+        const int se = min(ce, seg + kNbSegChunks);
+        if (seg > cb) asm volatile("bar.sync 1, %0;" ::"r"(kFmmNT) : "memory");  // the last segment's x has been read
+        const int q0 = 2 * kNbPairs * seg, q1 = 2 * kNbPairs * se;
+        for (int base = q0 + 32 * wid; base < q1; base += kFmmNT) {
+            const int q = base + lane;
+            const int j = nq_source(run, min(q, S - 1));
+            const int node = __ldg(a.perm + j);
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float4 v = xv4[r * L::kX + pp];  // (hi, lo) of sources 2pp and 2pp + 1
-                    const df2 xv{make_float2(v.x, v.z), make_float2(v.y, v.w)};
-                    if (COMP == 0) df2_acc(are[r], df2_mul(xv, Qr));
-                    df2_acc(aim[r], df2_mul(xv, Qi));
-                }
+            for (int r = 0; r < R; ++r) {  // 0 past the item's sources
+                const df v = df_split_fast((q < S) ? ((r == 0) ? a.x0 : a.x1)[node] : 0.0);
+                if (q < q1) s_x[r * kNbX + q - q0] = make_float2(v.h, v.l);
             }
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[st]);
+        asm volatile("bar.sync 1, %0;" ::"r"(kFmmNT) : "memory");
+        for (int c = seg; ok && c < se; ++c) {
+            const int u = c - cb, st = u % kNbStages;
+            if (!mbar_wait(&full[st], (unsigned)((u / kNbStages) & 1), kNbSpin)) {
+                atomicExch(a.fault, 1);
+                ok = false;
+                break;
+            }
+            const float4* qi = nb_buf + (size_t)st * L::kStage;
+            const float4* qr = qi + L::kQ;
+            const float4* xv4 = reinterpret_cast<const float4*>(s_x) + (c - seg) * kNbPairs;
+            const int np = min(kNbPairs, npair - c * kNbPairs);
+            if (lane < tn) {
+#pragma unroll
+                for (int v = 0; v < kNbPairs / kFmmWarps; ++v) {
+                    const int pp = wid + v * kFmmWarps;
+                    if (pp >= np) break;
+                    const float4 wi = qi[pp * tn + lane];
+                    const df2 Qi{make_float2(wi.x, wi.y), make_float2(wi.z, wi.w)};
+                    df2 Qr{f2(0.f), f2(0.f)};
+                    if (COMP == 0) {
+                        const float4 wr = qr[pp * tn + lane];
+                        Qr = df2{make_float2(wr.x, wr.y), make_float2(wr.z, wr.w)};
+                    }
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const float4 x = xv4[r * (kNbX / 2) + pp];  // (hi, lo) of sources 2pp and 2pp + 1
+                        const df2 xv{make_float2(x.x, x.z), make_float2(x.y, x.w)};
+                        if (COMP == 0) df2_acc(are[r], df2_mul(xv, Qr));
+                        df2_acc(aim[r], df2_mul(xv, Qi));
+                    }
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty[st]);
+        }
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -1409,7 +1434,7 @@ __global__ void __launch_bounds__(kNbThreads) fmm_near_bulk_kernel(FmmArgs a, co
                 v.x += s_z[w][r][lane].x;
                 v.y += s_z[w][r][lane].y;
             }
-            a.zn[(size_t)r * a.N + i] = v;
+            a.zn[((size_t)blockIdx.y * R + r) * a.N + i] = v;
         }
     }
 }
@@ -1476,7 +1501,12 @@ __global__ void __launch_bounds__(256) fmm_l2p_kernel(FmmArgs a, ReduceArgs e) {
                 u = cdf{df_add(mm.re, h[q].re), df_add(mm.im, h[q].im)};
             }
         }
-        const double2 zn = a.zn[(size_t)r * a.N + i];
+        double2 zn = a.zn[(size_t)r * a.N + i];
+        for (int p = 1; p < a.nsplit; ++p) {  // the shares of a split near field
+            const double2 v = a.zn[((size_t)p * R + r) * a.N + i];
+            zn.x += v.x;
+            zn.y += v.y;
+        }
         zx[r] = (double)u.re.h + (double)u.re.l;
         zy[r] = (double)u.im.h + (double)u.im.l;
         if (EPI && a.near_scaled) {
@@ -1718,7 +1748,9 @@ void release_fmm(Boundary& b) {
         give_stream(true, b.fmm->aux, b.device);
         give_event(b.fmm->ev_fork, b.device);
         give_event(b.fmm->ev_join, b.device);
+        give_event(b.fmm->ev_solve, b.device);
         give_stream(false, b.fmm->bst, b.device);
+        give_stream(false, b.fmm->nst, b.device);
         give_event(b.fmm->ev_nq, b.device);
 
         if (b.fmm->arena || b.fmm->sync || b.fmm->nq_item || b.fmm->tn || b.fmm->path || b.fmm->tp || b.fmm->fault) {  // once no stream uses them
@@ -1733,7 +1765,6 @@ void release_fmm(Boundary& b) {
             pool_free(b.fmm->nq_re, 0);
             pool_free(b.fmm->nq_im, 0);
             pool_free(b.fmm->nt_im, 0);
-            pool_free(b.fmm->xs, 0);
             pool_free(b.fmm->fault, 0);
             pool_free(b.fmm->tn, 0);
             pool_free(b.fmm->path, 0);
@@ -1969,7 +2000,7 @@ static int fmm_tree_host(const Boundary& b, FmmTree* t, cudaStream_t st) {
         {(void**)&t->mult, (size_t)t->R * nbox * P * sizeof(float4)},
         {(void**)&t->loc, (size_t)t->R * nbox * P * sizeof(float4)},
         {(void**)&t->ws, (size_t)t->R * N * sizeof(float4)},
-        {(void**)&t->zn, (size_t)t->R * N * sizeof(double2)},
+        {(void**)&t->zn, (size_t)fmm_near_splits(b, t->nitems) * t->R * N * sizeof(double2)},
         {(void**)&t->zf, (size_t)t->R * N * sizeof(double2)},
     };
     size_t total = 0;
@@ -2148,8 +2179,8 @@ int ensure_fmm(const Boundary& bc, int R, cudaStream_t st) {
     }
     cudaGetLastError();
     if (rc == GNK_OK &&
-        (take_stream(true, &t->aux) != cudaSuccess || take_event(&t->ev_fork) != cudaSuccess ||
-         take_event(&t->ev_join) != cudaSuccess)) {
+        (take_stream(true, &t->aux) != cudaSuccess || take_stream(false, &t->nst) != cudaSuccess || take_event(&t->ev_fork) != cudaSuccess ||
+         take_event(&t->ev_join) != cudaSuccess || take_event(&t->ev_solve) != cudaSuccess)) {
         cudaGetLastError();
         set_error("FMM: stream or event creation failed");
         rc = GNK_ECUDA;
@@ -2227,8 +2258,7 @@ static int ensure_near_cache(const Boundary& b, bool adj, cudaStream_t st) {
         if (pool_alloc(reinterpret_cast<void**>(&t->nq_cnt), ni * sizeof(long long), st) != cudaSuccess ||
             pool_alloc(reinterpret_cast<void**>(&t->nq_off), (ni + 1) * sizeof(long long), st) != cudaSuccess ||
             pool_alloc(reinterpret_cast<void**>(&t->nq_item), ni * sizeof(int2), st) != cudaSuccess ||
-            pool_alloc(reinterpret_cast<void**>(&t->nq_run), ni * kFmmMaxNbr * sizeof(int2), st) != cudaSuccess ||
-            pool_alloc(reinterpret_cast<void**>(&t->xs), (size_t)kMaxRHS * b.N * sizeof(float2), st) != cudaSuccess) {
+            pool_alloc(reinterpret_cast<void**>(&t->nq_run), ni * kFmmMaxNbr * sizeof(int2), st) != cudaSuccess) {
             cudaGetLastError();
             pool_free(t->nq_cnt, st);
             pool_free(t->nq_off, st);
@@ -2238,7 +2268,6 @@ static int ensure_near_cache(const Boundary& b, bool adj, cudaStream_t st) {
             t->nq_off = nullptr;
             t->nq_item = nullptr;
             t->nq_run = nullptr;
-            t->xs = nullptr;
             return GNK_OK;
         }
         t->near_shape = 1;
@@ -2350,7 +2379,7 @@ static int launch_near_bulk(const Boundary& b, const FmmArgs& a, bool adj, cudaS
     }
     const FmmTree* t = b.fmm;
     const int stream = 8.0 * L::kParts * (double)t->near_pairs > kNbKeepBytes;
-    fmm_near_bulk_kernel<R, COMP><<<t->nitems, kNbThreads, L::kBytes, st>>>(
+    fmm_near_bulk_kernel<R, COMP><<<dim3(t->nitems, a.nsplit), kNbThreads, L::kBytes, st>>>(
         a, t->nq_off, t->nq_item, t->nq_run, t->nq_re, adj ? t->nt_im : t->nq_im, stream);
     GNK_TRY_CUDA(cudaGetLastError());
     return GNK_OK;
@@ -2389,11 +2418,19 @@ int fmm_start_near_cache(const Boundary& bc, cudaStream_t st) {
 static int fmm_product(const Boundary& b, FmmArgs& a, int R, bool EF, const ReduceArgs* epi, cudaStream_t st,
                        int* nlaunch, int cached = -1, bool adj = false) {
     const FmmTree* t = b.fmm;
-    fmm_gather_kernel<<<(b.N + 255) / 256, 256, 0, st>>>(a);
+    // Inside a solve (st is the handle's own high-priority stream) the far field,
+    // the longer chain, stays on it with the steps around it, and the near field
+    // forks to a stream of its own; a product on a caller's stream forks the far
+    // field instead, whose kernels then have the higher priority as well.
+    const bool inside = st == t->aux;
+    cudaStream_t fs = t->aux, ns = inside ? t->nst : st;
+    int launches = 0;
+    if (a.gathered) {
+        fmm_gather_kernel<<<(b.N + 255) / 256, 256, 0, st>>>(a);
+        launches = 1;
+    }
     GNK_TRY_CUDA(cudaEventRecord(t->ev_fork, st));
-    GNK_TRY_CUDA(cudaStreamWaitEvent(t->aux, t->ev_fork, 0));
-    cudaStream_t fs = t->aux;
-    int launches = 1;
+    GNK_TRY_CUDA(cudaStreamWaitEvent(inside ? ns : fs, t->ev_fork, 0));
     // the far field on its stream: the upward pass (P2M and the M2M climb in
     // one launch), M2L for every box, L2L per leaf.  (Running the finest
     // level's M2L on a third stream beside the climb measured slower: the two
@@ -2414,10 +2451,14 @@ static int fmm_product(const Boundary& b, FmmArgs& a, int R, bool EF, const Redu
         fmm_m2l_kernel<2><<<t->nbox, kFmmUT, 0, fs>>>(a);
     else if (b.diff)
         fmm_m2l_kernel<1><<<t->nbox, kFmmUT, 0, fs>>>(a);
+    else if (t->nbox >= kTcManyBoxes && R == 2)
+        fmm_m2l_tc_kernel<2, 2><<<t->nbox, 64, 0, fs>>>(a);
+    else if (t->nbox >= kTcManyBoxes)
+        fmm_m2l_tc_kernel<1, 2><<<t->nbox, 64, 0, fs>>>(a);
     else if (R == 2)
-        fmm_m2l_tc_kernel<2><<<t->nbox, 32 * kTcWarps, 0, fs>>>(a);
+        fmm_m2l_tc_kernel<2, 8><<<t->nbox, 256, 0, fs>>>(a);
     else
-        fmm_m2l_tc_kernel<1><<<t->nbox, 32 * kTcWarps, 0, fs>>>(a);
+        fmm_m2l_tc_kernel<1, 8><<<t->nbox, 256, 0, fs>>>(a);
     GNK_TRY_CUDA(cudaGetLastError());
     prof_end(tokm, PK_FMM, (double)R, fs, fmm_instr(b, R, 0));  // work: Cauchy sums (products)
     launches += 2;
@@ -2435,41 +2476,42 @@ static int fmm_product(const Boundary& b, FmmArgs& a, int R, bool EF, const Redu
         prof_end(tokd, PK_FMML2L, 0.0, fs, fmm_instr(b, R, 2));
         ++launches;
     }
-    GNK_TRY_CUDA(cudaEventRecord(t->ev_join, fs));
-    // near field on the caller's stream (from an operator cache when `cached`
+    if (!inside) GNK_TRY_CUDA(cudaEventRecord(t->ev_join, fs));
+    // near field on its stream (from an operator cache when `cached`
     // is 0 (both parts) or 1 (the imaginary part)); the first product that reads
     // a cache forms it here, beside its far field
     if (cached >= 0) {
         if (!adj && t->nq_wait) {  // formed on its own stream since the tree was built
-            GNK_TRY_CUDA(cudaStreamWaitEvent(st, t->ev_nq, 0));
+            GNK_TRY_CUDA(cudaStreamWaitEvent(ns, t->ev_nq, 0));
             b.fmm->nq_wait = 0;
         } else {
-            GNK_TRY(near_cache_build(b, adj, st));
+            GNK_TRY(near_cache_build(b, adj, ns));
         }
     }
-    const ProfToken tokn = prof_begin(st, PK_FMMNEAR);
+    const ProfToken tokn = prof_begin(ns, PK_FMMNEAR);
     if (cached >= 0) {
         if (R == 2 && cached == 1)
-            GNK_TRY((launch_near_bulk<2, 1>(b, a, adj, st)));
+            GNK_TRY((launch_near_bulk<2, 1>(b, a, adj, ns)));
         else if (R == 2)
-            GNK_TRY((launch_near_bulk<2, 0>(b, a, adj, st)));
+            GNK_TRY((launch_near_bulk<2, 0>(b, a, adj, ns)));
         else if (cached == 1)
-            GNK_TRY((launch_near_bulk<1, 1>(b, a, adj, st)));
+            GNK_TRY((launch_near_bulk<1, 1>(b, a, adj, ns)));
         else
-            GNK_TRY((launch_near_bulk<1, 0>(b, a, adj, st)));
+            GNK_TRY((launch_near_bulk<1, 0>(b, a, adj, ns)));
     } else if (R == 2 && EF)
-        fmm_near_kernel<2, true><<<t->nitems, kFmmNT, 0, st>>>(a);
+        fmm_near_kernel<2, true><<<t->nitems, kFmmNT, 0, ns>>>(a);
     else if (R == 2)
-        fmm_near_kernel<2, false><<<t->nitems, kFmmNT, 0, st>>>(a);
+        fmm_near_kernel<2, false><<<t->nitems, kFmmNT, 0, ns>>>(a);
     else if (EF)
-        fmm_near_kernel<1, true><<<t->nitems, kFmmNT, 0, st>>>(a);
+        fmm_near_kernel<1, true><<<t->nitems, kFmmNT, 0, ns>>>(a);
     else
-        fmm_near_kernel<1, false><<<t->nitems, kFmmNT, 0, st>>>(a);
+        fmm_near_kernel<1, false><<<t->nitems, kFmmNT, 0, ns>>>(a);
     ++launches;
     GNK_TRY_CUDA(cudaGetLastError());
-    prof_end(tokn, PK_FMMNEAR, (double)R * t->near_pairs, st,
+    prof_end(tokn, PK_FMMNEAR, (double)R * t->near_pairs, ns,
              cached >= 0 ? fmm_near_cached_instr(b, R, cached) : fmm_near_instr(b, R) * (EF ? 2.0 : 1.0),
              cached >= 0 ? fmm_near_cached_bytes(b, R, cached) : 0.0);
+    if (inside) GNK_TRY_CUDA(cudaEventRecord(t->ev_join, ns));
     GNK_TRY_CUDA(cudaStreamWaitEvent(st, t->ev_join, 0));
     const ProfToken tokp = prof_begin(st, PK_FMML2P);
     const int nb = (b.N + 255) / 256;
@@ -2530,7 +2572,8 @@ static void fmm_args(const Boundary& b, FmmArgs& a) {
     a.depth = t->L - t->l0 + 1;
     a.nleaf = t->nleaf;
     a.ucnt = t->sync;
-    a.xs = nullptr;
+    a.gathered = 1;
+    a.nsplit = 1;
     a.near_scaled = 0;
     a.tn = t->tn;
     a.tp = t->tp;
@@ -2541,6 +2584,16 @@ static void fmm_args(const Boundary& b, FmmArgs& a) {
     a.outF = nullptr;
     a.done = nullptr;
     a.fault = t->fault;
+}
+
+// The stream on which a solve with FMM products runs: the far field's, so that
+// the chain product - Arnoldi step - product has no hop between streams (two of
+// about 4 us each per step).  The caller orders it with events (ev_solve).
+int fmm_solve_stream(const Boundary& b, cudaStream_t st, cudaStream_t* own, cudaEvent_t* ev) {
+    GNK_TRY(ensure_fmm(b, kMaxRHS, st));
+    *own = b.fmm->aux;
+    *ev = b.fmm->ev_solve;
+    return GNK_OK;
 }
 
 int run_fmm(const Boundary& b, const PairJob& job, cudaStream_t st) {
@@ -2571,8 +2624,9 @@ int run_fmm(const Boundary& b, const PairJob& job, cudaStream_t st) {
         if (!adj || job.done != nullptr) GNK_TRY(ensure_near_cache(b, adj, st));
         if ((adj ? b.fmm->nt_state : b.fmm->nq_state) >= 1) {
             cached = (adj || im_only) ? 1 : 0;
-            a.xs = b.fmm->xs;
+            a.gathered = (a.tp != nullptr);  // the table form of P2M reads the sorted weights
             a.near_scaled = 1;
+            a.nsplit = fmm_near_splits(b, b.fmm->nitems);
         }
     }
     const ReduceArgs e = reduce_args(b, job, 1, 0);  // the epilogue runs inside L2P

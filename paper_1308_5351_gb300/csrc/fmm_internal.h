@@ -69,7 +69,6 @@ struct FmmTree {
     int2* nq_item = nullptr;      // per work item: (S sources, tn targets)
     int2* nq_run = nullptr;       // [nitems][kFmmMaxNbr]: (first source, sources before) of each
                                   // neighbour leaf; (0, INT_MAX) past the last
-    float2* xs = nullptr;         // [R][N] x in sorted order, double-float (cached products)
     long long nq_slots = 0;       // float4 entries of each of the arrays below
     // state 0 not formed, 2 allocated (formed by the first cached product),
     // 1 formed, -1 not used (too large)
@@ -82,7 +81,8 @@ struct FmmTree {
     float4* tn = nullptr;       // [N] offset of each node from its leaf centre in leaf widths
     float4* tp = nullptr;       // [N][P] its powers (handles built for differentiation), or null
     cudaStream_t aux = nullptr; // high-priority stream of the far field (the near field runs beside it)
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    cudaStream_t nst = nullptr; // the near field's stream inside a solve (which runs on aux)
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_solve = nullptr;
     cudaStream_t bst = nullptr; // stream of the near cache's formation when it starts early
     cudaEvent_t ev_nq = nullptr;
     int nq_wait = 0;            // the next cached product waits for ev_nq
@@ -100,6 +100,15 @@ constexpr int kFmmUseHost = 1;
 // more M2L pairs.  Handles built for differentiation keep level 2.
 inline int fmm_top_level(const Boundary& b, int L) { return (b.diff || L < 4) ? 2 : 3; }
 int fmm_tree_device(const Boundary& b, FmmTree* t, cudaStream_t st);
+
+// Shares that each work item of a cached near field is split into: four blocks run
+// on an SM at once, and fewer items than that leave SMs idle.  Handles built for
+// differentiation keep whole items.  (More items never give more shares, so a
+// lower bound of their number, one per leaf and per 32 nodes, sizes the sums.)
+inline int fmm_near_splits(const Boundary& b, int nitems) {
+    const int want = 4 * b.sms / (nitems > 0 ? nitems : 1);
+    return b.diff ? 1 : (want < 1 ? 1 : (want > 4 ? 4 : want));
+}
 
 // Points t at the translation tables on the current device (formed and uploaded
 // once per device and process): the M2L Pascal matrix C(k+l, l)

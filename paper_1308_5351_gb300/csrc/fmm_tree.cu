@@ -624,7 +624,7 @@ int fmm_tree_device(const Boundary& b, FmmTree* t, cudaStream_t st) {
         {(void**)&t->mult, (size_t)t->R * nbox * P * sizeof(float4)},
         {(void**)&t->loc, (size_t)t->R * nbox * P * sizeof(float4)},
         {(void**)&t->ws, (size_t)t->R * N * sizeof(float4)},
-        {(void**)&t->zn, (size_t)t->R * N * sizeof(double2)},
+        {(void**)&t->zn, (size_t)fmm_near_splits(b, std::max(nleaf, (N + 31) / 32)) * t->R * N * sizeof(double2)},
         {(void**)&t->zf, (size_t)t->R * N * sizeof(double2)},
     };
     size_t total = 0;

@@ -298,6 +298,7 @@ int fbie_backward_nodes(Boundary& b, const double* mu, const double* gam, const 
 
 // ---------------------------------------------------------------- FMM (fmm.cu)
 int run_fmm(const Boundary& b, const PairJob& job, cudaStream_t st);
+int fmm_solve_stream(const Boundary& b, cudaStream_t st, cudaStream_t* own, cudaEvent_t* ev);
 int run_fmm_ef(const Boundary& b, const double2* w0, const double2* w1, double2* E, double2* F, cudaStream_t st);
 int ensure_fmm(const Boundary& b, int R, cudaStream_t st);
 int fmm_start_near_cache(const Boundary& b, cudaStream_t st);

@@ -1265,9 +1265,9 @@ static int arnoldi_blocks(int N) {
 // One restarted GMRES solve of A x = rhs with the operator in precision prec.
 // r is a work vector.  Counters are added to *res; *relres receives the final
 // true relative residual (in prec).
-int gmres(Boundary& b, int adjoint /* OpId */, int prec, const double* rhs, double* x, double* r,
-          int restart, int maxit, double tol, gnk_result* res, double* relres, cudaStream_t st,
-          double* fc_out, int* fc_valid) {
+int gmres_on(Boundary& b, int adjoint /* OpId */, int prec, const double* rhs, double* x, double* r,
+             int restart, int maxit, double tol, gnk_result* res, double* relres, cudaStream_t st,
+             double* fc_out, int* fc_valid) {
     if (fc_valid) *fc_valid = 0;
     GNK_TRY(ensure_krylov(b, restart, st));
     const int N = b.N;
@@ -1383,6 +1383,25 @@ int gmres(Boundary& b, int adjoint /* OpId */, int prec, const double* rhs, doub
         if (fc_valid) *fc_valid = 0;  // x moved
     }
     return status;
+}
+
+// The solve on the caller's stream, or with FMM products on the handle's own,
+// between two events on the caller's.
+int gmres(Boundary& b, int adjoint /* OpId */, int prec, const double* rhs, double* x, double* r,
+          int restart, int maxit, double tol, gnk_result* res, double* relres, cudaStream_t st,
+          double* fc_out, int* fc_valid) {
+    if (prec != GNK_PREC_FMM)
+        return gmres_on(b, adjoint, prec, rhs, x, r, restart, maxit, tol, res, relres, st, fc_out, fc_valid);
+    cudaStream_t own;
+    cudaEvent_t ev;
+    GNK_TRY(fmm_solve_stream(b, st, &own, &ev));
+    GNK_TRY_CUDA(cudaEventRecord(ev, st));
+    GNK_TRY_CUDA(cudaStreamWaitEvent(own, ev, 0));
+    const int s = gmres_on(b, adjoint, prec, rhs, x, r, restart, maxit, tol, res, relres, own, fc_out, fc_valid);
+    // also after a failure: what the caller enqueues next follows the solve's kernels
+    GNK_TRY_CUDA(cudaEventRecord(ev, own));
+    GNK_TRY_CUDA(cudaStreamWaitEvent(st, ev, 0));
+    return s;
 }
 
 int norm_host(Boundary& b, const double* v, double* out, cudaStream_t st) {

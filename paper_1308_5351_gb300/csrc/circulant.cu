@@ -196,6 +196,12 @@ int run_component_means(const Boundary& b, const double* x, double* means, cudaS
     return GNK_OK;
 }
 
+int run_job_sides(const Boundary& b, const PairJob& job, cudaStream_t st) {
+    if (job.Lsrc) GNK_TRY(run_circulant(b, job.Lsrc, b.r3, st));
+    if (job.Msrc) GNK_TRY(run_component_means(b, job.Msrc, b.means, st));
+    return GNK_OK;
+}
+
 int run_prepare_nodes(Boundary& b, const double* etpp, const double* Ap, int* d_flag, cudaStream_t st) {
     PrepArgs a;
     a.N = b.N;

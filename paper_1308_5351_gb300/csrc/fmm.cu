@@ -29,7 +29,7 @@
 // The tree is built once per handle (the geometry is fixed for all products),
 // on the device when its lookup grids fit (fmm_tree.cu), else on the host:
 // Morton keys of 16-bit box coordinates, a sort of (key, node) pairs, leaf
-// level L = the deepest level whose non-empty boxes hold at least kFmmLeaf
+// level L = the deepest level whose non-empty boxes hold enough
 // nodes on average, interaction and neighbour lists.  Every sum on the device
 // runs in a fixed order, so results are reproducible.
 #include <cuda_fp16.h>
@@ -1816,8 +1816,8 @@ static int fmm_tree_host(const Boundary& b, FmmTree* t, cudaStream_t st) {
         ord0.swap(ord1);
     }
     auto key_at = [&](int i, int l) { return key0[i] >> (2 * (16 - l)); };
-    // leaf level: deepest level whose non-empty boxes hold >= kFmmLeaf nodes on
-    // average.  Neighbours in key order first differ at level 16 - msb(x)/2.
+    // leaf level: deepest level whose non-empty boxes hold enough nodes on
+    // average (fmm_level_wanted).  Neighbours in key order first differ at level 16 - msb(x)/2.
     std::vector<long long> first_diff(18, 0);
     for (int i = 1; i < N; ++i) {
         const uint32_t x = key0[i] ^ key0[i - 1];
@@ -1830,7 +1830,7 @@ static int fmm_tree_host(const Boundary& b, FmmTree* t, cudaStream_t st) {
     for (int l = 1; l <= 16; ++l) {
         distinct += first_diff[l];
         if (l < 3) continue;
-        if ((double)N / (double)distinct < kFmmLeaf) break;
+        if (!fmm_level_wanted(b, l, (double)N / (double)distinct)) break;
         L = l;
     }
     t->L = L;
@@ -2476,6 +2476,9 @@ static int fmm_product(const Boundary& b, FmmArgs& a, int R, bool EF, const Redu
         prof_end(tokd, PK_FMML2L, 0.0, fs, fmm_instr(b, R, 2));
         ++launches;
     }
+    // what only the epilogue reads, behind the far field (the circulant product is
+    // 38 us of a few blocks; before the product it held up both fields)
+    if (epi) GNK_TRY(run_job_sides(b, epi->job, fs));
     if (!inside) GNK_TRY_CUDA(cudaEventRecord(t->ev_join, fs));
     // near field on its stream (from an operator cache when `cached`
     // is 0 (both parts) or 1 (the imaginary part)); the first product that reads

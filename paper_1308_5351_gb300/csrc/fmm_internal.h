@@ -11,10 +11,6 @@
 namespace gnk {
 
 constexpr int kFmmP = 32;     // expansion order (one warp lane per coefficient)
-#ifndef GNK_FMM_LEAF
-#define GNK_FMM_LEAF 64
-#endif
-constexpr int kFmmLeaf = GNK_FMM_LEAF;  // target mean number of nodes per leaf
 // M2L offsets between boxes of the topmost level span the grid of level 3
 constexpr int kFmmOffMax = 7;
 constexpr int kFmmOffs = 2 * kFmmOffMax + 1;  // offset code (dx + 7) 15 + (dy + 7)
@@ -100,6 +96,17 @@ constexpr int kFmmUseHost = 1;
 // more M2L pairs.  Handles built for differentiation keep level 2.
 inline int fmm_top_level(const Boundary& b, int L) { return (b.diff || L < 4) ? 2 : 3; }
 int fmm_tree_device(const Boundary& b, FmmTree* t, cudaStream_t st);
+
+// Whether the tree goes down to level l, given the mean number of nodes in its
+// non-empty boxes.  Level 3 (a first M2M and L2L) wants 64 nodes: at N = 2,560 the
+// adjoint slit map takes 8.9 ms with leaves of 160 on level 2, 10.1 with 46 on level
+// 3.  Deeper ones want 44: M2L pairs cost the tensor cores little, near pairs 8
+// bytes each (N = 524,288: 129 nodes per leaf 60.1 ms, 62 nodes 40.9, 30 nodes
+// 45.3; adjoint solve at N = 16,830: 128 nodes 2.20 ms, 55 nodes 2.11; N = 65,536:
+// 68 nodes 3.48 ms, 33 nodes 3.57).  Handles built for differentiation keep 64.
+inline bool fmm_level_wanted(const Boundary& b, int l, double mean_nodes) {
+    return mean_nodes >= ((l >= 4 && !b.diff) ? 44.0 : 64.0);
+}
 
 // Shares that each work item of a cached near field is split into: four blocks run
 // on an SM at once, and fewer items than that leave SMs idle.  Handles built for

@@ -5,7 +5,7 @@
 //   3. stable LSD radix sort of (key, node), three passes of 8 bits (bits 8-31);
 //   4. the level at which each node's key first differs from its predecessor's,
 //      whose histogram fixes the leaf level L (the deepest level whose non-empty
-//      boxes hold >= kFmmLeaf nodes on average);
+//      boxes hold enough nodes on average, fmm_level_wanted);
 //   5. per level, box ids by block counts, a scan over blocks and warp ballots;
 //   6. box centres, widths, parents and child ranges from the first node of each box;
 //   7. dense lookup grids of the boxes of each level, then interaction lists
@@ -545,7 +545,7 @@ int fmm_tree_device(const Boundary& b, FmmTree* t, cudaStream_t st) {
     for (int l = 0; l <= 16; ++l) {
         distinct += h[l];
         if (l < 3) continue;
-        if ((double)N / (double)distinct < kFmmLeaf) break;
+        if (!fmm_level_wanted(b, l, (double)N / (double)distinct)) break;
         L = l;
     }
     if (L > kMaxGridLevel) return kFmmUseHost;

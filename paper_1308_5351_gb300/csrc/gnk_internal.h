@@ -150,6 +150,8 @@ struct PairJob {
     const double* rhs = nullptr;  // EPI_RESID*
     const double* Lx = nullptr;   // EPI_M / EPI_H: Lhat x
     const double* means = nullptr;// EPI_ADJ: per-component means of x
+    const double* Lsrc = nullptr; // when given, Lx = Lhat Lsrc is formed (in r3) with the sum
+    const double* Msrc = nullptr; // when given, the component means of Msrc likewise (in means)
     const int* done = nullptr;    // skip the whole job if *done != 0
     int comp = 0;                 // set by run_pairsum: 0 both parts, 1 only Im z, 2 only Re z
 };
@@ -245,6 +247,8 @@ int pair_blocks_per_sm(int precision);
 
 // ---------------------------------------------------------------- circulant / pointwise
 int run_circulant(const Boundary& b, const double* x, double* y, cudaStream_t st);
+// Lhat Lsrc and the means of Msrc that a job's epilogue reads
+int run_job_sides(const Boundary& b, const PairJob& job, cudaStream_t st);
 int run_component_means(const Boundary& b, const double* x, double* means, cudaStream_t st);
 int run_prepare_geometry(Boundary& b, const double* etpp, const double* Ap, int* d_flag,
                          cudaStream_t st);

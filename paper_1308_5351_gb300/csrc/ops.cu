@@ -1,6 +1,7 @@
 // The discrete operators of Secs. 3 and 4 as sequences of launches on one
-// stream: an optional circulant or mean pass, then one pair-sum job whose
-// epilogue forms the operator's output.
+// stream: one pair-sum job whose epilogue forms the operator's output, with the
+// vector whose circulant product or component means the epilogue reads
+// (job.Lsrc, job.Msrc: formed before a direct sum, beside an FMM product).
 #include "gnk_internal.h"
 
 namespace gnk {
@@ -22,7 +23,6 @@ int op_IminusN(const Boundary& b, const double* x, double* y, int prec, cudaStre
 
 // y = (D - diag(D1) + Lhat) x   (Eqs. y, hD-bt, L-bs)
 int op_M(const Boundary& b, const double* x, double* y, int prec, cudaStream_t st) {
-    GNK_TRY(run_circulant(b, x, b.r3, st));
     PairJob j;
     j.R = 1;
     j.mode = W_SCALED;
@@ -32,13 +32,13 @@ int op_M(const Boundary& b, const double* x, double* y, int prec, cudaStream_t s
     j.out = y;
     j.ex = x;
     j.Lx = b.r3;
+    j.Lsrc = x;
     return run_pairsum(b, j, prec, st);
 }
 
 // y = (diag(e) + B^T + Phat) x   (Eqs. sys*, BTx, g_B)
 int op_adjoint(const Boundary& b, const double* x, double* y, int prec, cudaStream_t st,
                const int* done) {
-    GNK_TRY(run_component_means(b, x, b.means, st));
     PairJob j;
     j.R = 1;
     j.mode = W_SCALED;
@@ -48,6 +48,7 @@ int op_adjoint(const Boundary& b, const double* x, double* y, int prec, cudaStre
     j.out = y;
     j.ex = x;
     j.means = b.means;
+    j.Msrc = x;
     j.done = done;
     return run_pairsum(b, j, prec, st);
 }
@@ -69,7 +70,6 @@ int op_IminusN_T(const Boundary& b, const double* x, double* y, int prec, cudaSt
 
 // y = (D - diag(D1) + Lhat)^T x = (2/n) Re(q E(A x)) - diag(D1) x - Lhat x
 int op_MT(const Boundary& b, const double* x, double* y, int prec, cudaStream_t st) {
-    GNK_TRY(run_circulant(b, x, b.r3, st));
     PairJob j;
     j.R = 1;
     j.mode = W_SCALED;
@@ -79,6 +79,7 @@ int op_MT(const Boundary& b, const double* x, double* y, int prec, cudaStream_t 
     j.out = y;
     j.ex = x;
     j.Lx = b.r3;
+    j.Lsrc = x;
     return run_pairsum(b, j, prec, st);
 }
 
@@ -87,7 +88,6 @@ int op_MT(const Boundary& b, const double* x, double* y, int prec, cudaStream_t 
 int op_resid(const Boundary& b, int op, const double* rhs, const double* x, double* r,
              int prec, cudaStream_t st, double* fc_out) {
     if (op != OP_K) fc_out = nullptr;
-    if (fc_out) GNK_TRY(run_circulant(b, x, b.r3, st));
     PairJob j;
     j.R = 1;
     j.mode = W_SCALED;
@@ -99,15 +99,16 @@ int op_resid(const Boundary& b, int op, const double* rhs, const double* x, doub
         j.s = b.A;
         j.epi = EPI_RESID_T;
     } else if (op == OP_ADJ) {
-        GNK_TRY(run_component_means(b, x, b.means, st));
         j.s = b.A;
         j.epi = EPI_RESID_ADJ;
         j.means = b.means;
+        j.Msrc = x;
     } else {
         j.s = b.q;
         j.epi = fc_out ? EPI_RESID_FC : EPI_RESID;
         j.out2 = fc_out;
         j.Lx = b.r3;
+        j.Lsrc = fc_out ? x : nullptr;
     }
     return run_pairsum(b, j, prec, st);
 }
@@ -116,7 +117,6 @@ int op_resid(const Boundary& b, int op, const double* rhs, const double* x, doub
 // sum E(q gamma) (Eqs. y, sys; f_B(gamma) is the second half of h, Eq. bh).
 int op_rhs_fb(const Boundary& b, const double* gam, double* rhs, double* fb, int prec,
               cudaStream_t st) {
-    GNK_TRY(run_circulant(b, gam, b.r3, st));
     PairJob j;
     j.R = 1;
     j.mode = W_SCALED;
@@ -127,13 +127,13 @@ int op_rhs_fb(const Boundary& b, const double* gam, double* rhs, double* fb, int
     j.out2 = fb;
     j.ex = gam;
     j.Lx = b.r3;
+    j.Lsrc = gam;
     return run_pairsum(b, j, prec, st);
 }
 
 // h = ([D - diag(D1) + Lhat] mu - [2I + diag(B1) - B] gamma) / 2   (Eq. bh);
 // both Cauchy sums E(q mu) and E(q gamma) come from one two-RHS launch.
 int op_h(const Boundary& b, const double* mu, const double* gam, double* h, cudaStream_t st) {
-    GNK_TRY(run_circulant(b, mu, b.r3, st));
     PairJob j;
     j.R = 2;
     j.mode = W_SCALED;
@@ -145,6 +145,7 @@ int op_h(const Boundary& b, const double* mu, const double* gam, double* h, cuda
     j.ex = mu;
     j.ex2 = gam;
     j.Lx = b.r3;
+    j.Lsrc = mu;
     return run_pairsum(b, j, GNK_PREC_FP64, st);
 }
 
@@ -176,7 +177,6 @@ int ensure_eone(const Boundary& bc, cudaStream_t st) {
 int op_eone_rhs_fb(const Boundary& bc, const double* gam, double* rhs, double* fb, int prec,
                    cudaStream_t st) {
     Boundary& b = const_cast<Boundary&>(bc);
-    GNK_TRY(run_circulant(b, gam, b.r3, st));
     PairJob j;
     j.R = 2;
     j.mode = W_SCALED;
@@ -189,6 +189,7 @@ int op_eone_rhs_fb(const Boundary& bc, const double* gam, double* rhs, double* f
     j.out2 = fb;
     j.ex = gam;
     j.Lx = b.r3;
+    j.Lsrc = gam;
     GNK_TRY(run_pairsum(b, j, prec, st));
     b.eone_pending = 0;
     return GNK_OK;

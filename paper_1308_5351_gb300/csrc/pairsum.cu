@@ -1385,6 +1385,7 @@ cudaError_t launch_reduce_public(const Boundary& b, const PairJob& job, int chun
 
 int run_pairsum(const Boundary& b, const PairJob& job, int precision, cudaStream_t st) {
     if (precision == GNK_PREC_FMM) return run_fmm(b, job, st);
+    GNK_TRY(run_job_sides(b, job, st));
     PairJob j = job;
     j.comp = pair_component_needed(b, job);
     if (precision == GNK_PREC_FP32) return run_pairsum32(b, j, st);

@@ -163,8 +163,9 @@ int gnk_profile_mask(unsigned mask);
 int gnk_profile_query(int kind, long long* launches, double* total_ms,
                       double* work);
 /* As gnk_profile_query, plus the launches' algorithmic instruction count on
- * their limiting pipe (pair kernels: per ordered pair, FP64 (9 + 8R)/2 where
- * each pair is taken once (one part of z: 13/2), else 9 + 4R, FP32 6 + 4R,
+ * their limiting pipe (pair kernels: per ordered pair, FP64 (2 + 8R)/2 where
+ * each pair is taken once (one part of z: 6/2; domains of up to about a thousand
+ * nodes: 9 in place of 2), else 9 + 4R, FP32 6 + 4R,
  * double-float 49 + 48R, R the right-hand sides of the launch; the FMM
  * kernels: FP32-pipe instructions of their double-float arithmetic). */
 int gnk_profile_query_ex(int kind, long long* launches, double* total_ms,

@@ -180,4 +180,103 @@ static __device__ __forceinline__ void df2_dec(df2& acc, df2 p) {
     acc.l = sub2(acc.l, sub2(p.l, e));
 }
 
+// ------------------------------------------------------------------ 1/d in FP64, on the FP32 pipe
+// conj(d) / |d|^2 = ar - i ai of an FP64 difference d = dx + i dy, to FP64 accuracy,
+// with no FP64 instruction: GB300's FP64 pipe (2 lanes per SM) bounds the FP64 pair
+// kernels, and |d|^2, its reciprocal and the two products were 7 of the 13 to 17
+// instructions of a pair there; the 220 instructions below take the 128 FP32
+// lanes a third of the time that those 7 took.  dx and dy are split exactly into
+// three floats (24 + 23 + 6 bits), |d|^2, its reciprocal and the products are
+// formed as three-float sums with error-free transformations (relative error
+// below 2^-60), and each result is rounded once to FP64 by integer arithmetic on
+// its bits.  The error is below 1.01 ulp of the larger part, 0.51 away from powers
+// of two (20 million pairs emulated against extended precision; the FP64
+// sequence, with a rounding per step, reaches 2).  For 2^-40 <= max(|dx|, |dy|) < 2^40 with
+// the smaller one zero or at least 2^-70; other pairs (and d = 0) take the FP64
+// sequence, out of line so that the compiler branches to it.
+static __device__ __noinline__ double2 inv_slow_f64(double dx, double dy) {
+    const double inv = recip_f64(fma(dx, dx, dy * dy));
+    return make_double2(dx * inv, dy * inv);
+}
+
+// v = h + m + l exactly (0 where v = 0); e: biased exponent of v, at least 949 or 0
+static __device__ __forceinline__ void split3_bits(double v, float& h, float& m, float& l, unsigned& e) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    e = (hi >> 20) & 0x7ffu;
+    const unsigned sign = hi & 0x80000000u;
+    const bool nz = e != 0u;
+    h = __uint_as_float(nz ? (sign | ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29)) : 0u);
+    const float sc = __uint_as_float(nz ? ((e - 948u) << 23) | sign : 0u);  // 2^(e - 1075)
+    m = __fmul_rn(__fsub_rn(__uint_as_float(0x4b000000u | ((lo & 0x1fffffffu) >> 6)), 8388608.0f), __fmul_rn(sc, 64.0f));
+    l = __fmul_rn(__fsub_rn(__uint_as_float(0x4b000000u | (lo & 63u)), 8388608.0f), sc);
+}
+
+// (h + m + l)(y0 + y1 + y2), rounded to FP64; |h y0| below 2^-75 keeps its leading float
+static __device__ __forceinline__ double mul3_f64(float h, float m, float l, float y0, float y1, float y2) {
+    float p = __fmul_rn(h, y0);
+    const float pe = fmaf(h, y0, -p);
+    const float u = __fmul_rn(h, y1), ue = fmaf(h, y1, -u);
+    const float v = __fmul_rn(m, y0), ve = fmaf(m, y0, -v);
+    float w, we, mid, me;
+    two_sum(u, v, w, we);
+    two_sum(w, pe, mid, me);
+    fast_two_sum(p, mid, p, mid);  // |mid| at most half a unit of p's last place
+    const float low = __fadd_rn(__fadd_rn(__fadd_rn(we, me), __fadd_rn(ue, ve)),
+                                fmaf(h, y2, fmaf(m, y1, __fmul_rn(l, y0))));
+    // p as FP64 bits, plus mid + low in units of its last place
+    const unsigned f = __float_as_uint(p), ef = (f >> 23) & 255u;
+    const float sc = __uint_as_float(ef >= 52u ? (306u - ef) << 23 : 0u);  // 2^(52 - (ef - 127))
+    const float ms = __fmul_rn(mid, sc);                                  // at most 2^29
+    const float tb = __fadd_rn(ms, 1610612736.0f);                        // 1.5 2^30: multiples of 128
+    const float small = __fadd_rn(__fsub_rn(ms, __fsub_rn(tb, 1610612736.0f)), __fmul_rn(low, sc));
+    const float ts = __fadd_rn(small, 12582912.0f);                       // 1.5 2^23: integers
+    int di = ((__float_as_int(tb) - 0x4ec00000) << 7) + (__float_as_int(ts) - 0x4b400000);
+    const int neg = (int)f >> 31;
+    di = (di ^ neg) - neg;
+    if ((f & 0x7fffffu) == 0u && di < 0) di += di;  // below a power of two the units are half
+    const long long bits = (((long long)(f & 0x7fffffffu)) << 29) + (896LL << 52) + (long long)di;
+    return __hiloint2double((int)((unsigned)(bits >> 32) | (f & 0x80000000u)), (int)bits);
+}
+
+static __device__ __forceinline__ void inv_conj_f64(double dx, double dy, double& ar, double& ai) {
+    float hx, mx, lx, hy, my, ly;
+    unsigned ex, ey;
+    split3_bits(dx, hx, mx, lx, ex);
+    split3_bits(dy, hy, my, ly, ey);
+    const unsigned em = max(ex, ey);
+    // (exponents, not comparisons of doubles, which would be FP64 instructions;
+    // a denormal counts as zero)
+    if (em - 983u >= 80u || ex - 1u < 952u || ey - 1u < 952u) {
+        const double2 v = inv_slow_f64(dx, dy);
+        ar = v.x;
+        ai = v.y;
+        return;
+    }
+    // |d|^2 = H + M + L
+    const float ax = __fadd_rn(hx, hx), ay = __fadd_rn(hy, hy);
+    const float p0x = __fmul_rn(hx, hx), e0x = fmaf(hx, hx, -p0x), p0y = __fmul_rn(hy, hy), e0y = fmaf(hy, hy, -p0y);
+    const float p1x = __fmul_rn(ax, mx), e1x = fmaf(ax, mx, -p1x), p1y = __fmul_rn(ay, my), e1y = fmaf(ay, my, -p1y);
+    const float rx = fmaf(ax, lx, __fmul_rn(mx, mx)), ry = fmaf(ay, ly, __fmul_rn(my, my));
+    float H, t, s, u1, v, u2, M, u3, u4;
+    two_sum(p0x, p0y, H, t);
+    two_sum(p1x, p1y, s, u1);
+    two_sum(e0x, e0y, v, u2);
+    two_sum(s, v, M, u3);
+    two_sum(M, t, M, u4);
+    float L = __fadd_rn(__fadd_rn(__fadd_rn(u1, u2), __fadd_rn(u3, u4)), __fadd_rn(__fadd_rn(e1x, e1y), __fadd_rn(rx, ry)));
+    fast_two_sum(H, M, H, M);
+    fast_two_sum(M, L, M, L);
+    // 1/|d|^2 = y0 (1 + e + e^2), e = 1 - (H + M + L) y0 to 2^-70
+    const float y0 = recip_f32(H);
+    const float tp = __fmul_rn(H, y0), te = fmaf(H, y0, -tp);
+    const float mp = __fmul_rn(M, y0), me = fmaf(M, y0, -mp);
+    float a, b, eh, c;
+    two_sum(__fsub_rn(1.0f, tp), -te, a, b);
+    two_sum(a, -mp, eh, c);
+    const float sl = fmaf(eh, eh, __fsub_rn(__fadd_rn(b, c), fmaf(L, y0, me)));
+    const float y1 = __fmul_rn(y0, eh), y2 = fmaf(y0, sl, fmaf(y0, eh, -y1));
+    ar = mul3_f64(hx, mx, lx, y0, y1, y2);
+    ai = mul3_f64(hy, my, ly, y0, y1, y2);
+}
+
 }  // namespace gnk

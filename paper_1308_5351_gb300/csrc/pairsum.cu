@@ -8,11 +8,11 @@
 // [chunk][rhs][N] buffer; a second kernel adds the chunks in a fixed order
 // (deterministic) in FP64 and applies the operator's epilogue.
 //
-// Per pair the FP64 kernels spend 9 FP64-pipe instructions on 1/d:
+// Per pair the ordered FP64 kernel spends 9 FP64-pipe instructions on 1/d:
 //   2 DADD (d = eta_i - eta_j), DMUL + DFMA (|d|^2), 3 DFMA to refine the
 //   hardware reciprocal seed, 2 DMUL (Re, Im of 1/d),
-// and 4 DFMA on w / d; the kernels that take each pair once share the 9 between
-// the pair's two directions (below);
+// and 4 DFMA on w / d; the kernels that take each pair once share 1/d between
+// the pair's two directions and form it on the FP32 pipe (below);
 // the FP32 kernel spends 10 FP32-pipe instructions and one MUFU reciprocal;
 // the double-float kernel about 97 FP32-pipe instructions and one MUFU.
 #include <algorithm>
@@ -147,11 +147,11 @@ __global__ void __launch_bounds__(kThreads64) pairsum64_kernel(Pair64Args a) {
 }
 
 // ------------------------------------------------------------------ FP64, pairs taken once
-// 1/(eta_j - eta_i) = -1/(eta_i - eta_j): a pair's difference, |d|^2 and
-// reciprocal (9 of the 13 FP64 instructions) serve both directions.  The FP64
-// pipe (2 lanes per SM) bounds the sum, so per unordered pair the kernel spends
-//   9 + 8 R (both parts of z) or 9 + 4 (one part, R = 1)
-// instead of 2 (9 + 4 R).  A block takes one pair (I, J) of node blocks of SB =
+// 1/(eta_j - eta_i) = -1/(eta_i - eta_j): a pair's difference and 1/d serve both
+// directions.  The FP64 pipe (2 lanes per SM) bounds the sum; 1/d is formed on the
+// FP32 pipe beside it (inv_conj_f64), so per unordered pair the kernel spends
+//   2 + 8 R (both parts of z) or 2 + 4 (one part, R = 1)
+// FP64 instructions instead of 2 (9 + 4 R).  A block takes one pair (I, J) of node blocks of SB =
 // 32 W G nodes (W >= 2).  A warp holds 32 targets (one per lane) and meets 32 sources in
 // 32 steps: in step k lane l takes source (l + k) mod 32, whose sum travels
 // with it, handed to the next lane by a shuffle (issue slots are free: an
@@ -160,8 +160,8 @@ __global__ void __launch_bounds__(kThreads64) pairsum64_kernel(Pair64Args a) {
 // 32 sources of slice (w + s) mod W in turn s: no two warps share a slice, and
 // the order is fixed).  Block (I, J) writes I's sums to slot J and J's to slot
 // I, so every node gets nt partial sums, added by the reduction in slot order.
-// Measured: (D - diag(D1) + Lhat) x at N = 16,000, real A, 6.15 -> 3.00 ms
-// (90 % of the pipe's rate for 13 instructions per unordered pair).
+// Measured: (D - diag(D1) + Lhat) x at N = 16,000, real A: 6.15 ms by ordered
+// pairs, 3.00 with 9 + 4 FP64 instructions per unordered pair, 1.46 now.
 struct Pair64SymArgs {
     const double2* et;
     int N;
@@ -273,9 +273,9 @@ __global__ void __launch_bounds__(32 * W) pairsum64_sym_kernel(Pair64SymArgs a) 
                         const int q = c * 32 + k;
                         const double2 sp = s_pos[q];
                         const double dx = p.x - sp.x, dy = p.y - sp.y;
-                        double inv = recip_f64(fma(dx, dx, dy * dy));
-                        inv = (k == lane) ? 0.0 : inv;  // the i = j term is excluded (Eq. fmm-E)
-                        const double ar = dx * inv, ai = dy * inv;
+                        double ar, ai;
+                        inv_conj_f64(dx, dy, ar, ai);
+                        if (k == lane) ar = ai = 0.0;  // the i = j term is excluded (Eq. fmm-E)
 #pragma unroll
                         for (int r = 0; r < R; ++r) add_term64<COMP, false>(acc[r], s_w[r * NT + q], ar, ai);
                     }
@@ -292,8 +292,8 @@ __global__ void __launch_bounds__(32 * W) pairsum64_sym_kernel(Pair64SymArgs a) 
                     const int q = c * 32 + ((lane + k) & 31);
                     const double2 sp = s_pos[q];
                     const double dx = p.x - sp.x, dy = p.y - sp.y;
-                    const double inv = recip_f64(fma(dx, dx, dy * dy));
-                    const double ar = dx * inv, ai = dy * inv;  // 1/d = ar - i ai
+                    double ar, ai;  // 1/d = ar - i ai
+                    inv_conj_f64(dx, dy, ar, ai);
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
                         add_term64<COMP, false>(acc[r], s_w[r * NT + q], ar, ai);
@@ -338,10 +338,24 @@ __global__ void __launch_bounds__(32 * W) pairsum64_sym_kernel(Pair64SymArgs a) 
 // pairs: with one warp each the FP64 pipe waits for the 64-cycle latency of
 // dependent instructions (a product through the C ABI 30 us), with four it is
 // busy (20 us; the kernel 8.4 us, 0.96 of the pipe's rate; the ordered kernel
-// on 18 SMs took 82 to 125 us).
+// on 18 SMs took 82 to 125 us).  FAST: 1/d on the FP32 pipe; with few blocks per
+// SM its longer chain is what counts (12.3 us at N = 768), so it is taken from
+// kSymFastBlocks blocks per SM on.
 constexpr int kSymSplit = 4;
+constexpr int kSymFastBlocks = 6;
 
-template <int R, int MODE, int COMP>
+template <bool FAST>
+__device__ __forceinline__ void pair_inv64(double dx, double dy, double& ar, double& ai) {
+    if (FAST) {
+        inv_conj_f64(dx, dy, ar, ai);
+    } else {
+        const double inv = recip_f64(fma(dx, dx, dy * dy));
+        ar = dx * inv;
+        ai = dy * inv;
+    }
+}
+
+template <int R, int MODE, int COMP, bool FAST>
 __global__ void __launch_bounds__(32 * kSymSplit) pairsum64_sym32_kernel(Pair64SymArgs a) {
     constexpr int NC = COMP == 0 ? 2 : 1, KS = 32 / kSymSplit;
     __shared__ double2 s_pos[32], s_w[R][32];
@@ -374,9 +388,9 @@ __global__ void __launch_bounds__(32 * kSymSplit) pairsum64_sym32_kernel(Pair64S
         for (int k = k0; k < k0 + KS; ++k) {
             const double2 sp = s_pos[k];
             const double dx = p.x - sp.x, dy = p.y - sp.y;
-            double inv = recip_f64(fma(dx, dx, dy * dy));
-            inv = (k == lane) ? 0.0 : inv;  // the i = j term is excluded (Eq. fmm-E)
-            const double ar = dx * inv, ai = dy * inv;
+            double ar, ai;
+            pair_inv64<FAST>(dx, dy, ar, ai);
+            if (k == lane) ar = ai = 0.0;  // the i = j term is excluded (Eq. fmm-E)
 #pragma unroll
             for (int r = 0; r < R; ++r) add_term64<COMP, false>(acc[r], s_w[r][k], ar, ai);
         }
@@ -386,8 +400,8 @@ __global__ void __launch_bounds__(32 * kSymSplit) pairsum64_sym32_kernel(Pair64S
             const int q = (lane + k) & 31;
             const double2 sp = s_pos[q];
             const double dx = p.x - sp.x, dy = p.y - sp.y;
-            const double inv = recip_f64(fma(dx, dx, dy * dy));
-            const double ar = dx * inv, ai = dy * inv;
+            double ar, ai;
+            pair_inv64<FAST>(dx, dy, ar, ai);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 add_term64<COMP, false>(acc[r], s_w[r][q], ar, ai);
@@ -1069,9 +1083,10 @@ SymPlan make_sym_plan(int N, int sms) {
     for (const auto& sh : kShape) {
         const long long SB = 32LL * sh[0] * sh[1], nt = (N + SB - 1) / SB;
         if (nt > kSymMaxBlocks) continue;
+        if (best.W == 1) break;  // 32-node blocks wherever they are enough: their kernel splits the steps
         const double blocks = 0.5 * nt * (nt - 1) + 0.5 * nt;  // the diagonal's blocks are half
         const double rounds = std::ceil(blocks / std::max(1, sms));
-        const double t = rounds * (double)SB * SB * 17.0 / 4.1e9 + (double)nt * N * 32.0 / 4e12;
+        const double t = rounds * (double)SB * SB * 10.0 / 4.1e9 + (double)nt * N * 32.0 / 4e12;
         if (best.W == 0 || t < best_t) {
             best_t = t;
             best.W = sh[0];
@@ -1143,10 +1158,13 @@ static cudaError_t launch_sym64(const Pair64SymArgs& a, cudaStream_t st) {
 }
 
 template <int R, int MODE, int COMP>
-static cudaError_t launch_sym64_w(int W, const Pair64SymArgs& a, cudaStream_t st) {
+static cudaError_t launch_sym64_w(int W, int sms, const Pair64SymArgs& a, cudaStream_t st) {
     switch (W) {
         case 1:
-            pairsum64_sym32_kernel<R, MODE, COMP><<<a.nt * (a.nt + 1) / 2, 32 * kSymSplit, 0, st>>>(a);
+            if (a.nt * (a.nt + 1) / 2 >= kSymFastBlocks * sms)
+                pairsum64_sym32_kernel<R, MODE, COMP, true><<<a.nt * (a.nt + 1) / 2, 32 * kSymSplit, 0, st>>>(a);
+            else
+                pairsum64_sym32_kernel<R, MODE, COMP, false><<<a.nt * (a.nt + 1) / 2, 32 * kSymSplit, 0, st>>>(a);
             return cudaGetLastError();
         case 2: return launch_sym64<R, MODE, COMP, 2>(a, st);
         case 4: return launch_sym64<R, MODE, COMP, 4>(a, st);
@@ -1185,21 +1203,22 @@ static int run_pairsum64_sym(const Boundary& b, const PairJob& job, cudaStream_t
     const ProfToken tok = prof_begin(st);
     cudaError_t e;
     if (job.R == 1 && job.mode == W_SCALED && job.comp == 1)
-        e = launch_sym64_w<1, W_SCALED, 1>(p.W, a, st);
+        e = launch_sym64_w<1, W_SCALED, 1>(p.W, b.sms, a, st);
     else if (job.R == 1 && job.mode == W_SCALED && job.comp == 2)
-        e = launch_sym64_w<1, W_SCALED, 2>(p.W, a, st);
+        e = launch_sym64_w<1, W_SCALED, 2>(p.W, b.sms, a, st);
     else if (job.R == 1 && job.mode == W_SCALED)
-        e = launch_sym64_w<1, W_SCALED, 0>(p.W, a, st);
+        e = launch_sym64_w<1, W_SCALED, 0>(p.W, b.sms, a, st);
     else if (job.R == 1)
-        e = launch_sym64_w<1, W_COMPLEX, 0>(p.W, a, st);
+        e = launch_sym64_w<1, W_COMPLEX, 0>(p.W, b.sms, a, st);
     else if (job.mode == W_SCALED)
-        e = launch_sym64_w<2, W_SCALED, 0>(p.W, a, st);
+        e = launch_sym64_w<2, W_SCALED, 0>(p.W, b.sms, a, st);
     else
-        e = launch_sym64_w<2, W_COMPLEX, 0>(p.W, a, st);
+        e = launch_sym64_w<2, W_COMPLEX, 0>(p.W, b.sms, a, st);
     GNK_TRY_CUDA(e);
-    // FP64 pipe per unordered pair: 9 (d, |d|^2, reciprocal, 1/d) and per
-    // right-hand side and direction 4 (one part of z: 2)
-    const double per_pair = 9.0 + ((job.comp && job.R == 1) ? 4.0 : 8.0 * job.R);
+    // FP64 pipe per unordered pair: 2 (d; few blocks: 9) and per right-hand side
+    // and direction 4 (one part of z: 2)
+    const bool fast = p.W > 1 || p.nt * (p.nt + 1) / 2 >= kSymFastBlocks * b.sms;
+    const double per_pair = (fast ? 2.0 : 9.0) + ((job.comp && job.R == 1) ? 4.0 : 8.0 * job.R);
     prof_end(tok, PK_PAIR64, (double)job.R * b.N * (b.N - 1.0), st, 0.5 * per_pair * b.N * (b.N - 1.0));
     GNK_TRY_CUDA(launch_reduce(b, job, p.nt, 0, st, partial));
     count_launches(2);

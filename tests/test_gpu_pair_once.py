@@ -73,3 +73,35 @@ def test_pairs_once(G, m1, n, theta):
     tol = 4 * (64 + d.N) * U64 * (sx + (2 + s1) * np.abs(x[rows]) + lx + np.abs(x).max())
     for y, ref in zip(got, refs):
         assert np.all(np.abs(y[rows] - ref) <= tol)
+
+
+@pytest.mark.parametrize("m1,n", [(1, 768), (1, 4096), (1, 4098)], ids=["fp64_sequence", "split_fast", "blocks_fast"])
+@pytest.mark.parametrize("scale", ["ones", "wide", "huge", "tiny", "axis"])
+def test_one_over_d(G, m1, n, scale):
+    """One unit weight: z_i = 1 / (eta_i - eta_j) within 2^-51 of its modulus (2 ulp
+    of the larger part), for distances over many powers of two, equal
+    coordinates, and ranges that leave the three-float form."""
+    rng = np.random.default_rng([n, len(scale)])
+    e = rng.uniform(-1, 1, n) + 1j * rng.uniform(-1, 1, n)
+    if scale == "wide":
+        e = e * 2.0 ** rng.integers(-60, 60, n)
+    elif scale == "huge":
+        e = e * 2.0 ** 120
+    elif scale == "tiny":
+        e = e * 2.0 ** -120
+    elif scale == "axis":  # a grid: every second difference has an exactly zero part
+        k = np.arange(n)
+        e = (k % 64) * 0.37 + 1j * (k // 64) * 2.0 ** -20
+    one = np.ones(n, dtype=np.complex128)
+    with G.Boundary(m1, n, e, one, one, None, None, False) as b:
+        for j in (0, n // 2 + 1, n - 1):
+            w = torch.zeros(n, dtype=torch.complex128, device="cuda")
+            w[j] = 1.0
+            z = b.cauchy_sum(w).cpu().numpy()
+            d = e - e[j]  # rounded as on the GPU
+            i = np.arange(n) != j
+            x, y = d.real[i].astype(np.longdouble), d.imag[i].astype(np.longdouble)
+            r2 = x * x + y * y
+            err = np.hypot((z.real[i] - x / r2), (z.imag[i] + y / r2))
+            assert np.all(err <= 2.0 ** -51 / np.sqrt(r2)), float((err * np.sqrt(r2)).max())
+            assert z[j] == 0

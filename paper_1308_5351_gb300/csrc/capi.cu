@@ -266,7 +266,7 @@ int build(Boundary& b, int m1, int n, const double* et, const double* etp, const
     ar.add(&b.means, (size_t)m1);
     ar.add(&b.stage, 4 * 2 * N);
     ar.add(reinterpret_cast<char**>(&b.partial), b.partial_bytes);
-    ar.add(&b.flag, 1);
+    ar.add(&b.flag, 1 + kSymCounts);
     GNK_TRY(ar.allocate(&b.arena, st));
 
     // geometry copies (host or device sources; cudaMemcpyDefault infers the direction)
@@ -286,7 +286,8 @@ int build(Boundary& b, int m1, int n, const double* et, const double* etp, const
         }
     }
     int* d_flag = b.flag;
-    GNK_TRY_CUDA(cudaMemsetAsync(d_flag, 0, sizeof(int), st));
+    b.sym_count = b.flag + 1;
+    GNK_TRY_CUDA(cudaMemsetAsync(d_flag, 0, (1 + kSymCounts) * sizeof(int), st));
     GNK_TRY_CUDA(cudaMemsetAsync(b.e, 0, N * sizeof(double), st));
     int s = run_prepare_geometry(b, d_etpp, d_Ap, d_flag, st);
     int flag = 0;

@@ -127,6 +127,7 @@ struct PairPlan {
 };
 
 // Node blocks of the FP64 kernel that takes each pair once (pairsum64_sym_kernel).
+constexpr int kSymCounts = 128;  // node blocks at most
 struct SymPlan {
     int W = 0;   // warps per block (0: the kernel is not used)
     int G = 1;   // sub-tiles of 32 W nodes per node block
@@ -211,6 +212,7 @@ struct Boundary {
     double* r6 = nullptr;
     double* ones = nullptr;     // N ones (weights q = q * 1)
     int* flag = nullptr;        // input checks of the geometry preparation
+    int* sym_count = nullptr;   // [kSymCounts] zero between products (pairsum64_sym32_kernel)
     void* arena = nullptr;      // the one allocation that holds the buffers above
     int eone_pending = 0;       // Eone, diag(B1), diag(D1), e not yet formed
     int plain = 0;              // 1: diagonals of the form without singularity subtraction

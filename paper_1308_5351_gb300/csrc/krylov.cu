@@ -249,16 +249,16 @@ __device__ __forceinline__ void range_dots(const double* __restrict__ V, int N, 
         __syncthreads();
         if (threadIdx.x < kn * 8) {
             const int q = threadIdx.x >> 3, part = threadIdx.x & 7;
-            double t = 0.0;
-#pragma unroll 8
-            for (int e = 0; e < KT / 8; ++e) t += buf[q * KT + e * 8 + part];
-            red[part][q] = t;
+            double t[4] = {0.0, 0.0, 0.0, 0.0};  // four chains: a dependent FP64 addition takes 64 cycles
+#pragma unroll
+            for (int e = 0; e < KT / 8; ++e) t[e & 3] += buf[q * KT + e * 8 + part];
+            red[part][q] = (t[0] + t[1]) + (t[2] + t[3]);
         }
         __syncthreads();
         if (threadIdx.x < kn) {
-            double t = 0.0;
-            for (int part = 0; part < 8; ++part) t += red[part][threadIdx.x];
-            out[k0 + threadIdx.x] = t;
+            const int q = threadIdx.x;
+            out[k0 + q] = ((red[0][q] + red[1][q]) + (red[2][q] + red[3][q])) +
+                          ((red[4][q] + red[5][q]) + (red[6][q] + red[7][q]));
         }
         __syncthreads();
     }
@@ -458,6 +458,20 @@ __device__ void givens_step_warp0(int j, double hn, double* h1, const double* h2
     for (int k = lane; k < j + 2; k += 32) colg[k] = h1[k];
 }
 
+// sum_k V_k[i] h[k] for k < nv in four chains
+__device__ __forceinline__ double column_combo(const double* __restrict__ V, int N, int nv, int i, const double* h) {
+    double t0 = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0;
+    int k = 0;
+    for (; k + 3 < nv; k += 4) {
+        t0 = fma(h[k], V[(size_t)k * N + i], t0);
+        t1 = fma(h[k + 1], V[(size_t)(k + 1) * N + i], t1);
+        t2 = fma(h[k + 2], V[(size_t)(k + 2) * N + i], t2);
+        t3 = fma(h[k + 3], V[(size_t)(k + 3) * N + i], t3);
+    }
+    for (; k < nv; ++k) t0 = fma(h[k], V[(size_t)k * N + i], t0);
+    return (t0 + t1) + (t2 + t3);
+}
+
 __global__ void __launch_bounds__(KT) k_arnoldi(const double* __restrict__ V, int N, int j, double* __restrict__ w,
                                                 KPtrs p, KState* s) {
     if (s->done) return;  // set before this launch: the same in every block
@@ -490,9 +504,7 @@ __global__ void __launch_bounds__(KT) k_arnoldi(const double* __restrict__ V, in
     // (fusing this update with the second pass's dots, the basis entries kept in
     // registers, measured slower: 168 registers per thread)
     for (int i = i0 + threadIdx.x; i < i1; i += KT) {
-        double acc = w[i];
-        for (int k = 0; k < nv; ++k) acc = fma(-h1[k], V[(size_t)k * N + i], acc);
-        w[i] = acc;
+        w[i] -= column_combo(V, N, nv, i, h1);
     }
     __syncthreads();
     range_dots(V, N, nv, w, i0, i1, part2 + (size_t)blockIdx.x * p.ld, red, s_pool, true);
@@ -518,8 +530,7 @@ __global__ void __launch_bounds__(KT) k_arnoldi(const double* __restrict__ V, in
     if (hn < 0.0) {  // the same decision in every block
         double acc = 0.0;
         for (int i = i0 + threadIdx.x; i < i1; i += KT) {
-            double wi = w[i];
-            for (int k = 0; k < nv; ++k) wi = fma(-h2[k], V[(size_t)k * N + i], wi);
+            const double wi = w[i] - column_combo(V, N, nv, i, h2);
             w[i] = wi;
             acc = fma(wi, wi, acc);
         }
@@ -546,9 +557,7 @@ __global__ void __launch_bounds__(KT) k_arnoldi(const double* __restrict__ V, in
         if (blockIdx.x == 0 && threadIdx.x < 32) givens_step_warp0(j, hn, h1, h2, scs, ssn, scs[1023], p, s);
         for (int i = i0 + (int)threadIdx.x - t0; i < i1; i += KT - t0) {
             if ((int)threadIdx.x < t0) break;
-            double wi = w[i];
-            for (int k = 0; k < nv; ++k) wi = fma(-h2[k], V[(size_t)k * N + i], wi);
-            w[i] = wi * inv;
+            w[i] = (w[i] - column_combo(V, N, nv, i, h2)) * inv;
         }
     }
 }

@@ -173,6 +173,7 @@ struct Pair64SymArgs {
     double2* partial;  // [slot][rhs][N]
     int nt;            // node blocks
     int G;             // sub-tiles of 32 W nodes per node block
+    int* count;        // [nt] contributions per node block (32-node blocks; zero between products)
     const int* done;
 };
 
@@ -355,11 +356,16 @@ __device__ __forceinline__ void pair_inv64(double dx, double dy, double& ar, dou
     }
 }
 
+// The block that brings the last partial sums of a node block (an atomic count
+// per node block; nothing waits) adds them in slot order and applies the
+// operator's epilogue: one launch and about 2 us less per product than a
+// reduction of its own, which was half as long as the sums at N = 768.
 template <int R, int MODE, int COMP, bool FAST>
-__global__ void __launch_bounds__(32 * kSymSplit) pairsum64_sym32_kernel(Pair64SymArgs a) {
+__global__ void __launch_bounds__(32 * kSymSplit) pairsum64_sym32_kernel(Pair64SymArgs a, ReduceArgs ra) {
     constexpr int NC = COMP == 0 ? 2 : 1, KS = 32 / kSymSplit;
     __shared__ double2 s_pos[32], s_w[R][32];
     __shared__ double s_row[kSymSplit][R * NC][32], s_col[kSymSplit][R * NC][32];
+    __shared__ double2 s_sums[kSymSplit][R][32];
     if (a.done != nullptr && *a.done) return;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int I, J;
@@ -421,21 +427,65 @@ __global__ void __launch_bounds__(32 * kSymSplit) pairsum64_sym32_kernel(Pair64S
         }
     __syncthreads();
     // warp 0: row sums to slot J; warp 1: column sums to slot I
-    if (wid > (I != J ? 1 : 0)) return;
-    const int node = wid == 0 ? i : j;
-    if (node >= a.N) return;
+    const int mine = wid == 0 ? i : j;
+    if (wid <= (I != J ? 1 : 0) && mine < a.N) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        double v[NC];
+        for (int r = 0; r < R; ++r) {
+            double v[NC];
 #pragma unroll
-        for (int u = 0; u < NC; ++u) {
-            const double(*src)[R * NC][32] = wid == 0 ? s_row : s_col;
-            v[u] = src[0][r * NC + u][lane];
+            for (int u = 0; u < NC; ++u) {
+                const double(*src)[R * NC][32] = wid == 0 ? s_row : s_col;
+                v[u] = src[0][r * NC + u][lane];
 #pragma unroll
-            for (int q = 1; q < kSymSplit; ++q) v[u] += src[q][r * NC + u][lane];
+                for (int q = 1; q < kSymSplit; ++q) v[u] += src[q][r * NC + u][lane];
+            }
+            a.partial[((size_t)(wid == 0 ? J : I) * R + r) * a.N + mine] =
+                make_double2(COMP == 1 ? 0.0 : v[0], COMP == 2 ? 0.0 : v[NC - 1]);
         }
-        a.partial[((size_t)(wid == 0 ? J : I) * R + r) * a.N + node] =
-            make_double2(COMP == 1 ? 0.0 : v[0], COMP == 2 ? 0.0 : v[NC - 1]);
+    }
+    __shared__ int s_last;
+    __threadfence();  // the sums before the counts
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int last = atomicAdd(&a.count[I], 1) == a.nt - 1 ? 1 : 0;
+        if (I != J && atomicAdd(&a.count[J], 1) == a.nt - 1) last |= 2;
+        if (last & 1) a.count[I] = 0;  // every block has counted: ready for the next product
+        if (last & 2) a.count[J] = 0;
+        if (last) __threadfence();
+        s_last = last;
+    }
+    __syncthreads();
+    const int last = s_last;
+    for (int which = 0; which < 2; ++which) {  // the same in every thread
+        if (!(last >> which & 1)) continue;
+        const int node = (which == 0 ? I : J) * 32 + lane;
+        double2(*s_sum)[R][32] = s_sums;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            double sx = 0.0, sy = 0.0;
+            if (node < a.N) {
+#pragma unroll 8
+                for (int q = wid; q < a.nt; q += kSymSplit) {
+                    const double2 v = __ldcg(a.partial + ((size_t)q * R + r) * a.N + node);
+                    sx += v.x;
+                    sy += v.y;
+                }
+            }
+            s_sum[wid][r][lane] = make_double2(sx, sy);
+        }
+        __syncthreads();
+        if (wid == 0 && node < a.N) {
+            double2 z[kMaxRHS] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int q = 0; q < kSymSplit; ++q) {
+                    z[r].x += s_sum[q][r][lane].x;
+                    z[r].y += s_sum[q][r][lane].y;
+                }
+            epilogue_apply(ra, node, z[0], z[1]);
+        }
+        __syncthreads();
     }
 }
 
@@ -1073,7 +1123,7 @@ PairPlan make_plan(int N, int sms, int blocks_per_sm, int targets_per_block, int
 // sums per node and right-hand side); none (W = 0) beyond 524,288 nodes.  Small
 // domains take 32-node blocks of one warp (N = 768: 300 blocks instead of the
 // 18 of the ordered kernel).
-constexpr int kSymMaxBlocks = 128;
+constexpr int kSymMaxBlocks = kSymCounts;
 constexpr size_t kSymArenaBytes = (size_t)64 << 20;
 
 SymPlan make_sym_plan(int N, int sms) {
@@ -1158,13 +1208,13 @@ static cudaError_t launch_sym64(const Pair64SymArgs& a, cudaStream_t st) {
 }
 
 template <int R, int MODE, int COMP>
-static cudaError_t launch_sym64_w(int W, int sms, const Pair64SymArgs& a, cudaStream_t st) {
+static cudaError_t launch_sym64_w(int W, int sms, const Pair64SymArgs& a, const ReduceArgs& ra, cudaStream_t st) {
     switch (W) {
         case 1:
             if (a.nt * (a.nt + 1) / 2 >= kSymFastBlocks * sms)
-                pairsum64_sym32_kernel<R, MODE, COMP, true><<<a.nt * (a.nt + 1) / 2, 32 * kSymSplit, 0, st>>>(a);
+                pairsum64_sym32_kernel<R, MODE, COMP, true><<<a.nt * (a.nt + 1) / 2, 32 * kSymSplit, 0, st>>>(a, ra);
             else
-                pairsum64_sym32_kernel<R, MODE, COMP, false><<<a.nt * (a.nt + 1) / 2, 32 * kSymSplit, 0, st>>>(a);
+                pairsum64_sym32_kernel<R, MODE, COMP, false><<<a.nt * (a.nt + 1) / 2, 32 * kSymSplit, 0, st>>>(a, ra);
             return cudaGetLastError();
         case 2: return launch_sym64<R, MODE, COMP, 2>(a, st);
         case 4: return launch_sym64<R, MODE, COMP, 4>(a, st);
@@ -1199,29 +1249,31 @@ static int run_pairsum64_sym(const Boundary& b, const PairJob& job, cudaStream_t
     a.partial = static_cast<double2*>(partial);
     a.nt = p.nt;
     a.G = p.G;
+    a.count = b.sym_count;
     a.done = job.done;
+    ReduceArgs ra = reduce_args(b, job, p.nt, 0);
     const ProfToken tok = prof_begin(st);
     cudaError_t e;
     if (job.R == 1 && job.mode == W_SCALED && job.comp == 1)
-        e = launch_sym64_w<1, W_SCALED, 1>(p.W, b.sms, a, st);
+        e = launch_sym64_w<1, W_SCALED, 1>(p.W, b.sms, a, ra, st);
     else if (job.R == 1 && job.mode == W_SCALED && job.comp == 2)
-        e = launch_sym64_w<1, W_SCALED, 2>(p.W, b.sms, a, st);
+        e = launch_sym64_w<1, W_SCALED, 2>(p.W, b.sms, a, ra, st);
     else if (job.R == 1 && job.mode == W_SCALED)
-        e = launch_sym64_w<1, W_SCALED, 0>(p.W, b.sms, a, st);
+        e = launch_sym64_w<1, W_SCALED, 0>(p.W, b.sms, a, ra, st);
     else if (job.R == 1)
-        e = launch_sym64_w<1, W_COMPLEX, 0>(p.W, b.sms, a, st);
+        e = launch_sym64_w<1, W_COMPLEX, 0>(p.W, b.sms, a, ra, st);
     else if (job.mode == W_SCALED)
-        e = launch_sym64_w<2, W_SCALED, 0>(p.W, b.sms, a, st);
+        e = launch_sym64_w<2, W_SCALED, 0>(p.W, b.sms, a, ra, st);
     else
-        e = launch_sym64_w<2, W_COMPLEX, 0>(p.W, b.sms, a, st);
+        e = launch_sym64_w<2, W_COMPLEX, 0>(p.W, b.sms, a, ra, st);
     GNK_TRY_CUDA(e);
     // FP64 pipe per unordered pair: 2 (d; few blocks: 9) and per right-hand side
     // and direction 4 (one part of z: 2)
     const bool fast = p.W > 1 || p.nt * (p.nt + 1) / 2 >= kSymFastBlocks * b.sms;
     const double per_pair = (fast ? 2.0 : 9.0) + ((job.comp && job.R == 1) ? 4.0 : 8.0 * job.R);
     prof_end(tok, PK_PAIR64, (double)job.R * b.N * (b.N - 1.0), st, 0.5 * per_pair * b.N * (b.N - 1.0));
-    GNK_TRY_CUDA(launch_reduce(b, job, p.nt, 0, st, partial));
-    count_launches(2);
+    if (p.W > 1) GNK_TRY_CUDA(launch_reduce(b, job, p.nt, 0, st, partial));  // else done by the kernel
+    count_launches(p.W > 1 ? 2 : 1);
     *ran = true;
     return GNK_OK;
 }

@@ -72,6 +72,11 @@ struct FmmTree {
     float4* nq_re = nullptr;
     float4* nq_im = nullptr;
     float4* nt_im = nullptr;
+    // handles built for differentiation: 1/(eta_i - eta_j) of every near pair (state as above)
+    int inv_state = 0;
+    long long* inv_off = nullptr;  // nitems + 1
+    float4* inv_r = nullptr;
+    float4* inv_i = nullptr;
     int* fault = nullptr;       // set by a bounded wait of an FMM kernel that gave up
     unsigned* path = nullptr;   // [nleaf][L - l0 + 1]: box | quadrant << 30 of each leaf and its ancestors
     float4* tn = nullptr;       // [N] offset of each node from its leaf centre in leaf widths

@@ -87,3 +87,19 @@ def test_diff_handle_keeps_its_arithmetic(G):
                                      G.options(precision=G.GNK_PREC_FMM, tol=1e-12))
             out.append(lam.cpu().numpy())
     assert np.abs(out[0] - out[1]).max() <= 1e-10 * np.abs(out[1]).max()
+
+
+@pytest.mark.parametrize("name", list(DOMS))
+def test_inverse_cache_changes_no_bit(G, name):
+    """GNK_BUILD_DIFF: the same product before a solve (1/d formed in the kernel)
+    and after one (1/d read from the cache that the solve formed)."""
+    d = DOMS[name]
+    rng = np.random.default_rng(6)
+    x = torch.as_tensor(rng.normal(size=d.N), device="cuda")
+    gam = torch.as_tensor(Dm.gamma_log(d, d.holes[0]) if d.m1 > 1 else np.cos(Dm.nodes(d.n)), device="cuda")
+    fmm = G.GNK_PREC_FMM
+    with G.Boundary.from_domain(d, adjoint=True, device="cuda", precision=fmm | G.GNK_BUILD_DIFF) as b:
+        before = b.apply_adjoint(x, fmm).cpu().numpy()
+        b.solve_adjoint_ie(gam, precision=fmm, tol=1e-12)
+        after = b.apply_adjoint(x, fmm).cpu().numpy()
+    assert np.array_equal(before, after)

@@ -2393,9 +2393,8 @@ static int near_cache_build(const Boundary& b, bool adj, cudaStream_t st) {
 // every near pair (16 bytes), for the products with weights A x of its solves,
 // whose sums must stay bit for bit those of the direct near field.  Formed by the
 // first of them; a product then reads it instead of spending 49 of 97
-// instructions per pair on 1/d beside the far field on the same pipe: the forward
-and transposed solves of a gradient at N = 40,960 (13.6 million near pairs, 220 MB
-a product) and its three E, F passes 13.3 -> 11.9 ms.
+// instructions per pair on 1/d beside the far field on the same pipe: a forward
+// and a transposed solve at N = 40,960 with the gradient's E, F passes 13.3 -> 11.9 ms.
 static int ensure_inverse_cache(const Boundary& b, cudaStream_t st) {
     FmmTree* t = b.fmm;
     if (t->inv_state != 0) return GNK_OK;

@@ -771,6 +771,173 @@ __global__ void __launch_bounds__(kThreads32) pairsum32x2_kernel(Pair32Args a) {
     }
 }
 
+// Each unordered pair once: one reciprocal (the ordered kernel's bound) serves
+// both directions.  As the double-float kernel below: a block takes a pair (I, J) of
+// blocks of kSrcTile32 nodes; a warp has 128 rows, four per thread in two packs, so
+// that the shared-memory reads and the shuffles of a step serve four pairs.  I - N
+// with real A (a whole product): N = 2,048 23 us against 26 with the ordered kernel,
+// 8,192 29.5 against 42, 16,384 72 against 103, 65,536 915 against 1,079.
+constexpr int kSym32Warps = kSrcTile32 / 128;
+
+template <int R, int MODE, int COMP>
+__global__ void __launch_bounds__(32 * kSym32Warps) pairsum32_sym_kernel(Pair32Args a, int nt) {
+    constexpr int S = kSrcTile32, NT = 32 * kSym32Warps, NS = S / 32, P = 2;
+    constexpr int NC = COMP == 0 ? 2 : 1;  // parts of z kept: both, Im (COMP 1) or Re (COMP 2)
+    static_assert(2 * P * NT == S, "four rows per thread");
+    __shared__ float4 s_src[S];         // (x, y, wx, wy) of the first right-hand side
+    __shared__ float2 s_w1[R > 1 ? S : 1];
+    __shared__ float2 s_col[R][NC][S];  // column sums, one per lane of the packs
+    if (a.done != nullptr && *a.done) return;
+    const int N = a.N, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int I, J;
+    sym_blocks(nt, blockIdx.x, I, J);
+    const float4 ref = a.ref32[J];
+    auto weight = [&](int r, int j) -> float2 {
+        if (MODE == W_COMPLEX) {
+            const double2 wd = (r == 0) ? a.w0[j] : a.w1[j];
+            return make_float2((float)wd.x, (float)wd.y);
+        }
+        const float2 sc = a.s32[j];
+        const float x = (float)((r == 0) ? a.x0[j] : a.x1[j]);
+        return make_float2(sc.x * x, sc.y * x);
+    };
+    // rows; those past the end lie far on the other side than the columns past the
+    // end, with weight 0
+    const int ib = I * S + wid * 128 + lane;
+    float2 ox[P], oy[P], wx[P][R], wy[P][R], acc[P][R][NC];
+#pragma unroll
+    for (int u = 0; u < P; ++u) {
+        float px[2], py[2];
+        float2 w[2][R];
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            const int i = ib + 64 * u + 32 * v;
+            px[v] = py[v] = -kFar32;
+            if (i < N) {
+                const float4 t = a.et32[i];
+                px[v] = (t.x - ref.x) + (t.z - ref.z);
+                py[v] = (t.y - ref.y) + (t.w - ref.w);
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) w[v][r] = i < N ? weight(r, i) : f2(0.f);
+        }
+        ox[u] = make_float2(px[0], px[1]);
+        oy[u] = make_float2(py[0], py[1]);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            wx[u][r] = make_float2(w[0][r].x, w[1][r].x);
+            wy[u][r] = make_float2(w[0][r].y, w[1][r].y);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) acc[u][r][c] = f2(0.f);
+        }
+    }
+    for (int k = threadIdx.x; k < S; k += NT) {
+        const int j = J * S + k;
+        const float2 o = j < N ? a.off32[j] : f2(kFar32);
+        const float2 w = j < N ? weight(0, j) : f2(0.f);
+        s_src[k] = make_float4(o.x, o.y, w.x, w.y);
+        if (R > 1) s_w1[k] = j < N ? weight(R - 1, j) : f2(0.f);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) s_col[r][c][k] = f2(0.f);
+    }
+    // z += w / d = w conj(d) / |d|^2
+    auto add = [&](float2* z, float2 vx, float2 vy, float2 dx, float2 dy, float2 inv) {
+        if (COMP == 0) {
+            const float2 ar = mul2(dx, inv), ai = mul2(dy, inv);
+            z[0] = fma2(vx, ar, fma2(vy, ai, z[0]));
+            z[NC - 1] = fma2(vy, ar, fma2(neg2(vx), ai, z[NC - 1]));
+        } else if (COMP == 1) {
+            z[0] = fma2(fma2(neg2(vx), dy, mul2(vy, dx)), inv, z[0]);
+        } else {
+            z[0] = fma2(fma2(vy, dy, mul2(vx, dx)), inv, z[0]);
+        }
+    };
+    if (I == J) {  // every ordered pair by its own row
+        __syncthreads();
+#pragma unroll 2
+        for (int q = 0; q < S; ++q) {
+            const float4 sv = s_src[q];
+#pragma unroll
+            for (int u = 0; u < P; ++u) {
+                const float2 dx = sub2(ox[u], f2(sv.x)), dy = sub2(oy[u], f2(sv.y));
+                const float2 r2 = fma2(dy, dy, mul2(dx, dx));
+                float2 inv = make_float2(recip_f32(r2.x), recip_f32(r2.y));
+                inv.x = (J * S + q == ib + 64 * u) ? 0.f : inv.x;  // the i = j term is excluded (Eq. fmm-E)
+                inv.y = (J * S + q == ib + 64 * u + 32) ? 0.f : inv.y;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const float2 v = r == 0 ? make_float2(sv.z, sv.w) : s_w1[R > 1 ? q : 0];
+                    add(acc[u][r], f2(v.x), f2(v.y), dx, dy, inv);
+                }
+            }
+        }
+    } else {
+        for (int s = 0; s < NS; ++s) {
+            __syncthreads();  // the slices' sums are back in shared memory
+            const int c0 = ((NS / kSym32Warps * wid + s) & (NS - 1)) * 32;
+            float2 col[R][NC];
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < NC; ++c) col[r][c] = s_col[r][c][c0 + lane];
+#pragma unroll 4
+            for (int k = 0; k < 32; ++k) {
+                const int q = c0 + ((lane + k) & 31);
+                const float4 sv = s_src[q];
+#pragma unroll
+                for (int u = 0; u < P; ++u) {
+                    const float2 dx = sub2(ox[u], f2(sv.x)), dy = sub2(oy[u], f2(sv.y));
+                    const float2 r2 = fma2(dy, dy, mul2(dx, dx));
+                    const float2 inv = make_float2(recip_f32(r2.x), recip_f32(r2.y));
+                    const float2 ninv = neg2(inv);
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const float2 v = r == 0 ? make_float2(sv.z, sv.w) : s_w1[R > 1 ? q : 0];
+                        add(acc[u][r], f2(v.x), f2(v.y), dx, dy, inv);
+                        add(col[r], wx[u][r], wy[u][r], dx, dy, ninv);  // 1/(eta_j - eta_i) = -1/d
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        col[r][c].x = __shfl_sync(0xffffffffu, col[r][c].x, (lane + 1) & 31);
+                        col[r][c].y = __shfl_sync(0xffffffffu, col[r][c].y, (lane + 1) & 31);
+                    }
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < NC; ++c) s_col[r][c][c0 + lane] = col[r][c];
+        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < S; k += NT) {  // column sums to slot I
+            const int j = J * S + k;
+            if (j >= N) break;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const float2 re = s_col[r][0][k], im = s_col[r][NC - 1][k];
+                a.partial[((size_t)I * R + r) * N + j] =
+                    make_float2(COMP == 1 ? 0.f : re.x + re.y, COMP == 2 ? 0.f : im.x + im.y);
+            }
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < P; ++u)  // row sums to slot J
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float2 re = acc[u][r][0], im = acc[u][r][NC - 1];
+            const int i = ib + 64 * u;
+            if (i < N)
+                a.partial[((size_t)J * R + r) * N + i] = make_float2(COMP == 1 ? 0.f : re.x, COMP == 2 ? 0.f : im.x);
+            if (i + 32 < N)
+                a.partial[((size_t)J * R + r) * N + i + 32] =
+                    make_float2(COMP == 1 ? 0.f : re.y, COMP == 2 ? 0.f : im.y);
+        }
+}
+
 // ------------------------------------------------------------------ double-float (df32)
 // (arithmetic helpers in pairmath.cuh)
 struct PairDFArgs {
@@ -1016,6 +1183,218 @@ __global__ void __launch_bounds__(kThreadsDF) pairsumdf2_kernel(PairDFArgs a) {
     }
 }
 
+// Each unordered pair once: 1/d (49 of the FP32 instructions) serves both
+// directions.  A block takes a pair (I, J) of blocks of kSrcTile32 nodes, its four
+// warps 64 rows each (two per thread, one per lane of the packed registers); at turn
+// s warp v has the 32 columns of slice 2 v + s mod 8, whose sums travel round its
+// lanes with the sources and wait in shared memory for the next warp.  At N = 16,384
+// with real A a product takes 447 us (FP32 pipe 323; ordered 694), 644 with complex A
+// (ordered 900); below 4,096 the 256 steps of one block, about 48 us.  The
+// diagonal blocks (1/nt of the pairs) sum every ordered pair by its own row.
+constexpr int kSymDFWarps = kSrcTile32 / 64;
+
+template <int R, int MODE, int COMP>
+__global__ void __launch_bounds__(32 * kSymDFWarps) pairsumdf_sym_kernel(PairDFArgs a, int nt) {
+    constexpr int S = kSrcTile32, NT = 32 * kSymDFWarps, NS = S / 32;
+    constexpr int NC = COMP == 0 ? 2 : 1;  // parts of z kept: both, Im (COMP 1) or Re (COMP 2)
+    static_assert(2 * NT == S, "two rows per thread");
+    __shared__ float4 s_off[2][S];      // (xh, xh, yh, yh), (xl, xl, yl, yl)
+    __shared__ float4 s_w[R][2][S];     // (wxh, wxh, wxl, wxl), (wyh, wyh, wyl, wyl)
+    __shared__ float4 s_col[R][NC][S];  // (h.x, h.y, l.x, l.y): column sums, one per row lane
+    if (a.done != nullptr && *a.done) return;
+    const int N = a.N, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int I, J;
+    sym_blocks(nt, blockIdx.x, I, J);
+    const double2 ref = a.ref64[J];
+    auto weight = [&](int r, int j) -> double2 {
+        if (MODE == W_COMPLEX) return (r == 0) ? a.w0[j] : a.w1[j];
+        const double2 sc = a.s[j];
+        const double x = (r == 0) ? a.x0[j] : a.x1[j];
+        return make_double2(sc.x * x, sc.y * x);
+    };
+    // rows: positions against the column block's reference, in FP64 once; rows past
+    // the end lie far on the other side than the columns past the end, with weight 0
+    const int i0 = I * S + wid * 64 + lane, i1 = i0 + 32;
+    df ox[2], oy[2];
+    df2 wx[R], wy[R];
+    {
+        df px[R][2], py[R][2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int i = u == 0 ? i0 : i1;
+            if (i < N) {
+                const double2 p = a.et[i];
+                ox[u] = df_split(p.x - ref.x);
+                oy[u] = df_split(p.y - ref.y);
+            } else {
+                ox[u] = oy[u] = df{-kFar32, 0.f};
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const double2 w = i < N ? weight(r, i) : make_double2(0.0, 0.0);
+                px[r][u] = df_split(w.x);
+                py[r][u] = df_split(w.y);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            wx[r] = df2{make_float2(px[r][0].h, px[r][1].h), make_float2(px[r][0].l, px[r][1].l)};
+            wy[r] = df2{make_float2(py[r][0].h, py[r][1].h), make_float2(py[r][0].l, py[r][1].l)};
+        }
+    }
+    const float2 oxh = make_float2(ox[0].h, ox[1].h), oxl = make_float2(ox[0].l, ox[1].l);
+    const float2 oyh = make_float2(oy[0].h, oy[1].h), oyl = make_float2(oy[0].l, oy[1].l);
+    for (int k = threadIdx.x; k < S; k += NT) {
+        const int j = J * S + k;
+        const float4 o = j < N ? a.offdf[j] : make_float4(kFar32, kFar32, 0.f, 0.f);
+        s_off[0][k] = make_float4(o.x, o.x, o.y, o.y);
+        s_off[1][k] = make_float4(o.z, o.z, o.w, o.w);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const double2 w = j < N ? weight(r, j) : make_double2(0.0, 0.0);
+            const df vx = df_split(w.x), vy = df_split(w.y);
+            s_w[r][0][k] = make_float4(vx.h, vx.h, vx.l, vx.l);
+            s_w[r][1][k] = make_float4(vy.h, vy.h, vy.l, vy.l);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) s_col[r][c][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
+    df2 acc[R][NC];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) acc[r][c] = df2{f2(0.f), f2(0.f)};
+    // 1/d = ar - i ai of the two rows and column q; `self`: i = j may occur (then 0, Eq. fmm-E)
+    auto inverse = [&](int q, bool self, df2& ar, df2& ai) {
+        const float4 oa = s_off[0][q], ob = s_off[1][q];
+        const df2 dx = df2_sub(oxh, oxl, make_float2(oa.x, oa.y), make_float2(ob.x, ob.y));
+        const df2 dy = df2_sub(oyh, oyl, make_float2(oa.z, oa.w), make_float2(ob.z, ob.w));
+        const float2 px = mul2(dx.h, dx.h);
+        float2 ex = fma2(dx.h, dx.h, neg2(px));
+        ex = fma2(dx.h, add2(dx.l, dx.l), ex);
+        const float2 py = mul2(dy.h, dy.h);
+        float2 ey = fma2(dy.h, dy.h, neg2(py));
+        ey = fma2(dy.h, add2(dy.l, dy.l), ey);
+        float2 rh, re;
+        two_sum2(px, py, rh, re);
+        const float2 rl = add2(add2(ex, ey), re);
+        float y0 = recip_f32(rh.x), y1 = recip_f32(rh.y);
+        if (self) {
+            y0 = (J * S + q == i0) ? 0.f : y0;
+            y1 = (J * S + q == i1) ? 0.f : y1;
+        }
+        const float2 y = make_float2(y0, y1);
+        float2 e = fma2(neg2(rh), y, f2(1.0f));
+        e = fma2(neg2(rl), y, e);
+        const df2 inv{y, mul2(y, e)};
+        ar = df2_mul(dx, inv);
+        ai = df2_mul(dy, inv);
+    };
+    auto row_terms = [&](int q, const df2& ar, const df2& ai) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float4 wa = s_w[r][0][q], wb = s_w[r][1][q];
+            const df2 vx{make_float2(wa.x, wa.y), make_float2(wa.z, wa.w)};
+            const df2 vy{make_float2(wb.x, wb.y), make_float2(wb.z, wb.w)};
+            if (COMP != 1) {
+                df2_acc(acc[r][0], df2_mul(vx, ar));
+                df2_acc(acc[r][0], df2_mul(vy, ai));
+            }
+            if (COMP != 2) {
+                df2_acc(acc[r][NC - 1], df2_mul(vy, ar));
+                df2_dec(acc[r][NC - 1], df2_mul(vx, ai));
+            }
+        }
+    };
+    if (I == J) {
+        __syncthreads();
+#pragma unroll 2
+        for (int q = 0; q < S; ++q) {
+            df2 ar, ai;
+            inverse(q, true, ar, ai);
+            row_terms(q, ar, ai);
+        }
+    } else {
+        for (int s = 0; s < NS; ++s) {
+            __syncthreads();  // the slices' sums are back in shared memory
+            const int c0 = ((2 * wid + s) & (NS - 1)) * 32;
+            df2 col[R][NC];
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    const float4 v = s_col[r][c][c0 + lane];
+                    col[r][c] = df2{make_float2(v.x, v.y), make_float2(v.z, v.w)};
+                }
+#pragma unroll 2
+            for (int k = 0; k < 32; ++k) {
+                const int q = c0 + ((lane + k) & 31);
+                df2 ar, ai;
+                inverse(q, false, ar, ai);
+                row_terms(q, ar, ai);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {  // the other direction: 1/(eta_j - eta_i) = -1/d
+                    if (COMP != 1) {
+                        df2_dec(col[r][0], df2_mul(wx[r], ar));
+                        df2_dec(col[r][0], df2_mul(wy[r], ai));
+                    }
+                    if (COMP != 2) {
+                        df2_dec(col[r][NC - 1], df2_mul(wy[r], ar));
+                        df2_acc(col[r][NC - 1], df2_mul(wx[r], ai));
+                    }
+                    const int next = (lane + 1) & 31;
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        df2& v = col[r][c];
+                        v.h.x = __shfl_sync(0xffffffffu, v.h.x, next);
+                        v.h.y = __shfl_sync(0xffffffffu, v.h.y, next);
+                        v.l.x = __shfl_sync(0xffffffffu, v.l.x, next);
+                        v.l.y = __shfl_sync(0xffffffffu, v.l.y, next);
+                    }
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    const df2 v = col[r][c];
+                    s_col[r][c][c0 + lane] = make_float4(v.h.x, v.h.y, v.l.x, v.l.y);
+                }
+        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < S; k += NT) {  // column sums to slot I
+            const int j = J * S + k;
+            if (j >= N) break;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                df v[NC];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    const float4 t = s_col[r][c][k];
+                    float h, e;
+                    two_sum(t.x, t.y, h, e);
+                    v[c] = df{h, e + (t.z + t.w)};
+                }
+                a.partial[((size_t)I * R + r) * N + j] =
+                    make_float4(COMP == 1 ? 0.f : v[0].h, COMP == 1 ? 0.f : v[0].l, COMP == 2 ? 0.f : v[NC - 1].h,
+                                COMP == 2 ? 0.f : v[NC - 1].l);
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)  // row sums to slot J
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int i = u == 0 ? i0 : i1;
+            if (i >= N) continue;
+            const df2 re = acc[r][0], im = acc[r][NC - 1];
+            const float reh = u ? re.h.y : re.h.x, rel = u ? re.l.y : re.l.x;
+            const float imh = u ? im.h.y : im.h.x, iml = u ? im.l.y : im.l.x;
+            a.partial[((size_t)J * R + r) * N + i] = make_float4(COMP == 1 ? 0.f : reh, COMP == 1 ? 0.f : rel,
+                                                                 COMP == 2 ? 0.f : imh, COMP == 2 ? 0.f : iml);
+        }
+}
+
 // ------------------------------------------------------------------ reduce + epilogue
 // Adds the partial sums of 32 nodes per block and applies the operator's
 // epilogue: warp g takes the chunks g, g + 8, ... (coalesced over the nodes,
@@ -1193,6 +1572,23 @@ static int launch_plan(const Boundary& b, const PairPlan& base, size_t elem_byte
     return partial_workspace(b, (size_t)p->chunks * kMaxRHS * b.N * elem_bytes, partial, st);
 }
 
+// The workspace of the kernels that take each pair once; null where the ordered
+// kernel, which needs far less, is to serve the call: no memory for it, or a
+// capturing stream and more than the handle's own workspace holds (the one from
+// the pool moves when a later product needs more, and a graph keeps its address).
+static int sym_workspace(const Boundary& b, size_t need, void** partial, cudaStream_t st) {
+    *partial = nullptr;
+    if (need > b.partial_bytes) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        GNK_TRY_CUDA(cudaStreamIsCapturing(st, &cs));
+        if (cs != cudaStreamCaptureStatusNone) return GNK_OK;
+    }
+    const int rc = partial_workspace(b, need, partial, st);
+    if (rc == GNK_OK) return GNK_OK;
+    *partial = nullptr;
+    return rc == GNK_ENOMEM ? GNK_OK : rc;
+}
+
 template <int R, int MODE, int COMP, int W>
 static cudaError_t launch_sym64(const Pair64SymArgs& a, cudaStream_t st) {
     constexpr int NT = 32 * W;
@@ -1223,21 +1619,15 @@ static cudaError_t launch_sym64_w(int W, int sms, const Pair64SymArgs& a, const 
 }
 
 // The FP64 sum with each pair taken once.  *ran = false where the ordered kernel
-// serves the call: a source-chunk override, more than 524,288 nodes, or
-// a capturing stream before the handle owns the workspace (an allocation
-// captured into a graph would not outlive it).
+// serves the call: a source-chunk override, more than 524,288 nodes, no memory for
+// the partial sums, or a capturing stream (sym_workspace).
 static int run_pairsum64_sym(const Boundary& b, const PairJob& job, cudaStream_t st, bool* ran) {
     *ran = false;
     const SymPlan& p = b.sym64;
     if (p.W == 0 || b.tile_chunks > 0) return GNK_OK;
-    const size_t need = (size_t)p.nt * job.R * b.N * sizeof(double2);
-    if (need > b.partial_bytes && need > b.partial_x_bytes) {
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        GNK_TRY_CUDA(cudaStreamIsCapturing(st, &cs));
-        if (cs != cudaStreamCaptureStatusNone) return GNK_OK;
-    }
     void* partial = nullptr;
-    GNK_TRY(partial_workspace(b, need, &partial, st));
+    GNK_TRY(sym_workspace(b, (size_t)p.nt * job.R * b.N * sizeof(double2), &partial, st));
+    if (!partial) return GNK_OK;
     Pair64SymArgs a;
     a.et = b.et;
     a.N = b.N;
@@ -1316,7 +1706,60 @@ int run_pairsum64(const Boundary& b, const PairJob& job, cudaStream_t st) {
     return GNK_OK;
 }
 
+constexpr int kSymMaxTiles = 256;  // N <= 65,536: 268 MB of double-float sums
+
+// The FP32 sum with each pair taken once; *ran as for the double-float sum.
+static int run_pairsum32_sym(const Boundary& b, const PairJob& job, cudaStream_t st, bool* ran) {
+    *ran = false;
+    const int nt = (b.N + kSrcTile32 - 1) / kSrcTile32, pairs = nt * (nt + 1) / 2;
+    if (b.tile_chunks > 0 || b.f32_scalar || nt > kSymMaxTiles) return GNK_OK;
+    if (job.mode == W_SCALED && job.s != b.q && job.s != b.A) return GNK_OK;  // refused by the caller
+    void* partial = nullptr;
+    GNK_TRY(sym_workspace(b, (size_t)nt * job.R * b.N * sizeof(float2), &partial, st));
+    if (!partial) return GNK_OK;
+    Pair32Args a;
+    a.et32 = b.et32;
+    a.ref32 = b.ref32;
+    a.off32 = b.off32;
+    a.N = b.N;
+    a.w0 = job.w[0];
+    a.w1 = job.w[1];
+    a.x0 = job.x[0];
+    a.x1 = job.x[1];
+    a.s32 = (job.s == b.q) ? b.q32 : b.A32;
+    a.partial = static_cast<float2*>(partial);
+    a.tiles_src = nt;
+    a.tiles_per_chunk = 1;
+    a.done = job.done;
+    const ProfToken tok = prof_begin(st);
+    constexpr int NT = 32 * kSym32Warps;
+    if (job.R == 1 && job.mode == W_SCALED && job.comp == 1)
+        pairsum32_sym_kernel<1, W_SCALED, 1><<<pairs, NT, 0, st>>>(a, nt);
+    else if (job.R == 1 && job.mode == W_SCALED && job.comp == 2)
+        pairsum32_sym_kernel<1, W_SCALED, 2><<<pairs, NT, 0, st>>>(a, nt);
+    else if (job.R == 1 && job.mode == W_SCALED)
+        pairsum32_sym_kernel<1, W_SCALED, 0><<<pairs, NT, 0, st>>>(a, nt);
+    else if (job.R == 1)
+        pairsum32_sym_kernel<1, W_COMPLEX, 0><<<pairs, NT, 0, st>>>(a, nt);
+    else if (job.mode == W_SCALED)
+        pairsum32_sym_kernel<2, W_SCALED, 0><<<pairs, NT, 0, st>>>(a, nt);
+    else
+        pairsum32_sym_kernel<2, W_COMPLEX, 0><<<pairs, NT, 0, st>>>(a, nt);
+    GNK_TRY_CUDA(cudaGetLastError());
+    // FP32 pipe per unordered pair: 4 (|d|^2), then per direction 2 and 4 per
+    // right-hand side (one part of z: 3)
+    const double per_pair = 4.0 + ((job.comp && job.R == 1) ? 6.0 : 4.0 + 8.0 * job.R);
+    prof_end(tok, PK_PAIR32, (double)job.R * b.N * (b.N - 1.0), st, 0.5 * per_pair * b.N * (b.N - 1.0));
+    GNK_TRY_CUDA(launch_reduce(b, job, nt, 1, st, partial));
+    count_launches(2);
+    *ran = true;
+    return GNK_OK;
+}
+
 int run_pairsum32(const Boundary& b, const PairJob& job, cudaStream_t st) {
+    bool ran = false;
+    GNK_TRY(run_pairsum32_sym(b, job, st, &ran));
+    if (ran) return GNK_OK;
     PairPlan p;
     void* partial = nullptr;
     GNK_TRY(launch_plan(b, b.plan32, sizeof(float2), &p, &partial, st));
@@ -1372,7 +1815,63 @@ int run_pairsum32(const Boundary& b, const PairJob& job, cudaStream_t st) {
     return GNK_OK;
 }
 
+// The double-float sum with each pair taken once; not faster at any size with the
+// ordered kernel (I - N, real A: N = 512 to 4,096 48-50 against 54-56 us, the time of
+// one block's 256 steps; 6,144 78 against 101; 16,384 447 against 694; 32,768 1,671
+// against 2,348).  *ran = false where that one serves the call all the same: a
+// source-chunk override, the scalar variant, partial sums (nt x N) past kSymMaxTiles
+// node blocks, no memory for them, or a capturing stream (sym_workspace).
+
+static int run_pairsumdf_sym(const Boundary& b, const PairJob& job, cudaStream_t st, bool* ran) {
+    *ran = false;
+    const int nt = (b.N + kSrcTile32 - 1) / kSrcTile32, pairs = nt * (nt + 1) / 2;
+    if (b.tile_chunks > 0 || b.df_scalar || nt > kSymMaxTiles) return GNK_OK;
+    void* partial = nullptr;
+    GNK_TRY(sym_workspace(b, (size_t)nt * job.R * b.N * sizeof(float4), &partial, st));
+    if (!partial) return GNK_OK;
+    PairDFArgs a;
+    a.et = b.et;
+    a.ref64 = b.ref64;
+    a.offdf = b.offdf;
+    a.N = b.N;
+    a.w0 = job.w[0];
+    a.w1 = job.w[1];
+    a.x0 = job.x[0];
+    a.x1 = job.x[1];
+    a.s = job.s;
+    a.partial = static_cast<float4*>(partial);
+    a.tiles_src = nt;
+    a.tiles_per_chunk = 1;
+    a.done = job.done;
+    const ProfToken tok = prof_begin(st);
+    constexpr int NT = 32 * kSymDFWarps;
+    if (job.R == 1 && job.mode == W_SCALED && job.comp == 1)
+        pairsumdf_sym_kernel<1, W_SCALED, 1><<<pairs, NT, 0, st>>>(a, nt);
+    else if (job.R == 1 && job.mode == W_SCALED && job.comp == 2)
+        pairsumdf_sym_kernel<1, W_SCALED, 2><<<pairs, NT, 0, st>>>(a, nt);
+    else if (job.R == 1 && job.mode == W_SCALED)
+        pairsumdf_sym_kernel<1, W_SCALED, 0><<<pairs, NT, 0, st>>>(a, nt);
+    else if (job.R == 1)
+        pairsumdf_sym_kernel<1, W_COMPLEX, 0><<<pairs, NT, 0, st>>>(a, nt);
+    else if (job.mode == W_SCALED)
+        pairsumdf_sym_kernel<2, W_SCALED, 0><<<pairs, NT, 0, st>>>(a, nt);
+    else
+        pairsumdf_sym_kernel<2, W_COMPLEX, 0><<<pairs, NT, 0, st>>>(a, nt);
+    GNK_TRY_CUDA(cudaGetLastError());
+    // FP32 pipe per unordered pair: 49 (1/d) and per right-hand side and direction
+    // 48 (one part of z: 24)
+    const double per_pair = 49.0 + ((job.comp && job.R == 1) ? 48.0 : 96.0 * job.R);
+    prof_end(tok, PK_PAIRDF, (double)job.R * b.N * (b.N - 1.0), st, 0.5 * per_pair * b.N * (b.N - 1.0));
+    GNK_TRY_CUDA(launch_reduce(b, job, nt, 2, st, partial));
+    count_launches(2);
+    *ran = true;
+    return GNK_OK;
+}
+
 int run_pairsumdf(const Boundary& b, const PairJob& job, cudaStream_t st) {
+    bool ran = false;
+    GNK_TRY(run_pairsumdf_sym(b, job, st, &ran));
+    if (ran) return GNK_OK;
     PairPlan p;
     void* partial = nullptr;
     GNK_TRY(launch_plan(b, b.plandf, sizeof(float4), &p, &partial, st));

@@ -43,13 +43,11 @@ TOL = 1e-10
 L2_FLUSH_BYTES = 256 << 20
 SMS, SM_MAX_MHZ = 152, 2070.0
 # Pipe peaks derived from unit counts and the maximum SM clock:
-#   FP32: 128 lanes/SM; a pair costs 10 FP32-pipe instructions + 1 MUFU.
-#   FP64: 2 DFMA lanes/SM (1.25 TFLOP/s nominal); a pair costs 13 FP64-pipe
-#   instructions (10 arithmetic + 3 to refine the reciprocal seed).
-#   double-float: ~97 FP32-pipe instructions per pair + 1 MUFU.
+#   FP32 and double-float: 128 lanes/SM; FP64: 2 DFMA lanes/SM (1.25 TFLOP/s nominal).
 # The roofline compares the launches' algorithmic instructions on their limiting
-# pipe (per pair: FP64 9 + 4R, FP32 6 + 4R, double-float 49 + 48R for R
-# right-hand sides) with the pipe's peak instruction rate.
+# pipe with the pipe's peak instruction rate.  Per unordered pair, both directions,
+# for R right-hand sides: FP64 2 + 8R (9 + 8R where few blocks form 1/d on the FP64
+# pipe), FP32 8 + 8R, double-float 49 + 96R.
 PEAK_INSTR = {
     "pair32": SMS * SM_MAX_MHZ * 1e6 * 128,
     "pair64": SMS * SM_MAX_MHZ * 1e6 * 2,
@@ -61,23 +59,25 @@ PEAK_INSTR = {
     "fmm_l2l": SMS * SM_MAX_MHZ * 1e6 * 128,
 }
 PEAK_BASIS = {
-    "pair64": "FP64 pipe: 152 SMs x 2 DFMA lanes x 2070 MHz; 9 + 4R FP64 instr per pair",
-    "pair32": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 6 + 4R FP32 instr per pair (+1 MUFU)",
-    "pairdf": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 49 + 48R FP32 instr per double-float pair",
+    "pair64": "FP64 pipe: 152 SMs x 2 DFMA lanes x 2070 MHz; 2 + 8R FP64 instr per unordered pair (9 + 8R in small domains)",
+    "pair32": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 8 + 8R FP32 instr per unordered pair (+1 MUFU)",
+    "pairdf": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 49 + 96R FP32 instr per unordered double-float pair",
     "fmm": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; per M2L pair and lane 24 FP32 instr for each "
-           "of the 32 double-float products of the real Pascal matrix + 98 for the two complex scalings",
+           "of the 32 double-float products of the real Pascal matrix + 98 for the two complex scalings "
+           "(equivalents: the matrix product itself runs on the tensor cores)",
     "fmm_up": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 742 FP32 instr per lane per binomial M2M "
-              "transform, 36 x 47 per node for the powers and 48R per node and order in P2M",
-    "fmm_l2l": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 840 FP32 instr per lane per Pascal-matrix L2L transform",
+              "transform (equivalents: on the tensor cores), 35 x 38 R + 16R per order and node in P2M",
+    "fmm_l2l": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 840 FP32 instr per lane per Pascal-matrix L2L transform "
+               "(equivalents: on the tensor cores)",
     "fmm_l2p": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 58R FP32 instr per node and order (Horner)",
     "fmm_near": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 49 + 48R FP32 instr per double-float "
                 "near-field pair",
 }
-KERNEL_NAME = {"pair64": "pairsum64_kernel", "pair32": "pairsum32x2_kernel", "pairdf": "pairsumdf2_kernel",
-               "fmm": "fmm_m2l_kernel",
+KERNEL_NAME = {"pair64": "pairsum64_sym_kernel", "pair32": "pairsum32_sym_kernel", "pairdf": "pairsumdf_sym_kernel",
+               "fmm": "fmm_m2l_tc_kernel",
                "fmm_near": "fmm_near_bulk_kernel (near field streamed from the operator cache by bulk copies)",
-               "fmm_l2p": "fmm_l2p_kernel", "fmm_up": "fmm_up_kernel (P2M and the M2M chain)",
-               "fmm_l2l": "fmm_l2l_kernel"}
+               "fmm_l2p": "fmm_l2p_kernel", "fmm_up": "fmm_up_tc_kernel (P2M and the M2M chain)",
+               "fmm_l2l": "fmm_l2l_tc_kernel"}
 # DRAM bytes read + written per launch of the kernel at the headline size
 # (64 ellipses, n = 1024; the R = 1 launches of the solve), from one ncu
 # capture of the same command (ncu's default cache control: caches flushed

@@ -4,9 +4,9 @@
 // * One persistent launch per operator product: a work list of items
 //   (domain, target tile, group of right-hand sides), longest first, that the
 //   resident blocks pull with an atomic ticket.  Each item streams all source
-//   tiles of its domain through shared memory and finishes with the
-//   operator's epilogue (no split-source partials: the list has far more
-//   items than the GPU has block slots).
+//   tiles of its domain through shared memory, slices of a tile's sources going to
+//   different warps, and finishes with the operator's epilogue (no partial sums in
+//   memory: the list has far more items than the GPU has block slots).
 // * The inner products use FP32 pair sums; the refinement residual, the
 //   right-hand side and h use double-float pair sums (FP64-class).
 // * GMRES runs per system (domain, right-hand side), one thread block per

@@ -1,7 +1,7 @@
 // Fast multipole evaluation of the Cauchy sum z_i = sum_{j != i} w_j / (eta_i - eta_j)
 // (Sec. 2.5, Eqs. fmm-1, fmm-E: the paper forms E w with the FMM of zfmm2dpart,
 // O((m+1)n) operations).  Uniform-depth quadtree over the bounding square of the
-// nodes (levels 2..L, empty boxes pruned), expansions of order P scaled by the box
+// nodes (levels 2 or 3..L, empty boxes pruned), expansions of order P scaled by the box
 // width r (Greengard & Rokhlin's complex-analytic 2-D FMM):
 //   multipole  phi(z) = sum_k a_k r^k / (z - c)^(k+1),  a_k = sum_j w_j ((s_j - c)/r)^k
 //   local      phi(z) = sum_l b_l ((z - c)/r)^l
@@ -13,18 +13,20 @@
 // sum_j |w_j / (eta_i - eta_j)| (about 2e-12 at P = 32 including round-off;
 // checked against direct sums in the tests).
 //
-// One product is six or seven launches on two streams.  The weights are
-// gathered into tree order; the far field runs on a high-priority stream: the
-// upward pass (P2M, then the M2M chain carried by the block that completes
-// each box's last child, no launch per level), M2L for every box, L2L per leaf
-// down its ancestor path.  The near field runs beside it on the caller's
-// stream (for the products z = E(q x) streamed from the near-field operator
-// cache by bulk asynchronous copies, after x is gathered in the near lists'
-// order); L2P adds the two after they join.  M2M and L2L are
-// fixed real Pascal matrices between exact Gaussian-integer scalings, M2L a
-// fixed real Pascal matrix between two complex scalings per offset: no P x P
-// table per relative position.  The far field runs in complex double-float on the FP32
-// pipe (GB300's FP64 pipe is 1/64 of it).
+// One product is five to seven launches on two or three streams.  The far field:
+// the upward pass (P2M, then the M2M chain carried by the warp that completes
+// each box's last child, no launch per level), M2L for every box, L2L for four
+// leaves per warp down their ancestor paths.  The near field runs beside it; where
+// its geometry and factors are fixed (weights q x; in a solve also A x) it is
+// streamed from an operator cache by bulk asynchronous copies, else the weights are
+// gathered into tree order first and every pair is formed.  L2P adds the two after
+// they join and applies the operator's epilogue.  M2M and L2L are fixed real Pascal
+// matrices between exact Gaussian-integer scalings, M2L a fixed real Pascal
+// matrix between two complex scalings per offset: no P x P table per relative
+// position.  The fixed matrices multiply on the tensor cores (digits exact in
+// FP16), everything else runs in complex double-float on the FP32 pipe (GB300's
+// FP64 pipe is 1/64 of it).  A handle built for differentiation (GNK_BUILD_DIFF)
+// keeps one fixed sequence of operations, the double-float translations.
 //
 // The tree is built once per handle (the geometry is fixed for all products),
 // on the device when its lookup grids fit (fmm_tree.cu), else on the host:
@@ -2254,7 +2256,8 @@ int ensure_fmm(const Boundary& bc, int R, cudaStream_t st) {
     return rc;
 }
 
-// FP32-pipe instructions of one FMM product, for the roofline.  M2L, per pair
+// FP32-pipe instructions of one FMM product, for the roofline, in the
+// double-float form of the translations whichever form runs.  M2L, per pair
 // and lane: 32 (2 Dekker products and 2 compensated sums, 24) for the real
 // Pascal matrix, the two complex scalings (38 each) and the sum (22); 840 per
 // lane for an L2L transform (32 terms of the Pascal sum at 24 each, two exact

@@ -2,19 +2,23 @@
 // Eqs. fmm-1, fmm-E) and the pointwise operators built on them (Secs. 3.3,
 // 3.4, 4.3, 4.4).
 //
-// Layout of a launch: blocks along x own a tile of targets held in registers
-// (T per thread); blocks along y own a contiguous chunk of source tiles, which
-// they stream through shared memory.  Each block writes its partial sums to a
-// [chunk][rhs][N] buffer; a second kernel adds the chunks in a fixed order
-// (deterministic) in FP64 and applies the operator's epilogue.
+// In every precision one kernel takes each unordered pair once (`_sym`): a block
+// has a pair of node blocks, rows in registers, the columns' sums passed round the
+// lanes, and 1/d serves both directions.  It writes partial sums to a
+// [node block][rhs][N] buffer; a second kernel adds them in a fixed order
+// (deterministic) in FP64 and applies the operator's epilogue (small FP64 sums do
+// this themselves).
 //
-// Per pair the ordered FP64 kernel spends 9 FP64-pipe instructions on 1/d:
+// The ordered kernels serve a source-chunk override and the calls for which the
+// others' partial sums have no room: blocks along x own a tile of targets held in
+// registers (T per thread); blocks along y a contiguous chunk of source tiles, which
+// they stream through shared memory, with a [chunk][rhs][N] buffer.
+//
+// Per ordered pair: FP64 9 FP64-pipe instructions on 1/d
 //   2 DADD (d = eta_i - eta_j), DMUL + DFMA (|d|^2), 3 DFMA to refine the
-//   hardware reciprocal seed, 2 DMUL (Re, Im of 1/d),
-// and 4 DFMA on w / d; the kernels that take each pair once share 1/d between
-// the pair's two directions and form it on the FP32 pipe (below);
-// the FP32 kernel spends 10 FP32-pipe instructions and one MUFU reciprocal;
-// the double-float kernel about 97 FP32-pipe instructions and one MUFU.
+//   hardware reciprocal seed, 2 DMUL (Re, Im of 1/d)
+// (two when it is formed on the FP32 pipe) and 4 DFMA on w / d; FP32 10 FP32-pipe
+// instructions and one MUFU reciprocal; double-float about 97 and one MUFU.
 #include <algorithm>
 #include <cmath>
 

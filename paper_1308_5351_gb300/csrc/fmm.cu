@@ -933,7 +933,11 @@ __global__ void fmm_path_kernel(FmmArgs a, unsigned* path) {
 }
 
 // INV: 0 forms 1/d; 1 forms and stores it (no sums: the build of the inverse
-// cache); 2 reads it (bit for bit the same sums as 0).
+// cache); 2 reads it (bit for bit the same sums as 0); 3 forms it, folded: an item
+// with 16 targets or fewer (the last of a leaf) would leave half its lanes idle, so
+// the lanes form groups of `width`, each with its share of the source pairs (a leaf
+// of 68 nodes takes 2 + 1/8 instead of 3 turns of its sources; one Cauchy sum at
+// N = 65,536 169 -> 164 us).  Handles built for differentiation keep 0.
 template <int R, bool EF, int INV = 0>
 __global__ void __launch_bounds__(kFmmNT) fmm_near_kernel(FmmArgs a) {
     constexpr int RS = EF ? 2 * R : R;
@@ -950,7 +954,13 @@ __global__ void __launch_bounds__(kFmmNT) fmm_near_kernel(FmmArgs a) {
     const int2 it = a.items[blockIdx.x];  // (leaf, first target)
     const int leaf = it.x;
     const int t1 = a.leaf_start[leaf + 1];
-    const int i = it.y + lane;
+    const int tn = min(32, t1 - it.y);
+    int width = 32;  // lanes per group: group lane / width takes the pairs lane / width + (32 / width) u
+    if (INV == 3)
+        while (width > 2 && (width >> 1) >= tn) width >>= 1;
+    const int lt = INV == 3 ? lane & (width - 1) : lane;  // the lane's target
+    const int p0 = INV == 3 ? lane / width : 0, pstep = INV == 3 ? 32 / width : 1;
+    const int i = it.y + lt;
     const bool act = i < t1;
     const float4 pa = (INV != 2) ? a.p3[act ? i : it.y] : make_float4(0.f, 0.f, 0.f, 0.f);
     const float2 pb = (INV != 2) ? a.p3b[act ? i : it.y] : make_float2(0.f, 0.f);
@@ -972,9 +982,8 @@ __global__ void __launch_bounds__(kFmmNT) fmm_near_kernel(FmmArgs a) {
     __syncthreads();
     const int total = s_cum[nn];
     const int q0 = (int)((long long)total * wid / kFmmWarps), q1 = (int)((long long)total * (wid + 1) / kFmmWarps);
-    const int tn = min(32, t1 - it.y);
     long long entry = 0;  // of this warp's pair in hand: the items' entries, warp after warp, pair-major
-    if (INV != 0) {
+    if (INV == 1 || INV == 2) {
         entry = a.inv_off[blockIdx.x];
         for (int w = 0; w < wid; ++w)
             entry += (long long)tn * (((int)((long long)total * (w + 1) / kFmmWarps) -
@@ -1014,7 +1023,7 @@ __global__ void __launch_bounds__(kFmmNT) fmm_near_kernel(FmmArgs a) {
         const int npair = (cnt + 1) >> 1;
         float4 vr[4], vi[4];  // INV == 2: four pairs' entries in flight
 #pragma unroll 4
-        for (int pp = 0; pp < npair; ++pp) {
+        for (int pp = p0; pp < npair; pp += pstep) {
             if (INV == 2 && (pp & 3) == 0) {
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
@@ -1099,10 +1108,16 @@ __global__ void __launch_bounds__(kFmmNT) fmm_near_kernel(FmmArgs a) {
     for (int r = 0; r < RS; ++r) {  // even + odd sums, then to FP64
         const df sr = df_add(df{are[r].h.x, are[r].l.x}, df{are[r].h.y, are[r].l.y});
         const df si = df_add(df{aim[r].h.x, aim[r].l.x}, df{aim[r].h.y, aim[r].l.y});
-        s_z[wid][r][lane] = make_double2((double)sr.h + (double)sr.l, (double)si.h + (double)si.l);
+        double2 v = make_double2((double)sr.h + (double)sr.l, (double)si.h + (double)si.l);
+        if (INV == 3)
+            for (int o = width; o < 32; o <<= 1) {  // the groups' sums
+                v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+                v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+            }
+        s_z[wid][r][lane] = v;
     }
     __syncthreads();
-    if (wid == 0 && act) {
+    if (wid == 0 && act && lane == lt) {
 #pragma unroll
         for (int r = 0; r < RS; ++r) {
             double2 v = s_z[0][r][lane];
@@ -2609,15 +2624,19 @@ static int fmm_product(const Boundary& b, FmmArgs& a, int R, bool EF, const Redu
         else
             GNK_TRY((launch_near_bulk<1, 0>(b, a, adj, ns)));
     } else if (R == 2 && EF)
-        fmm_near_kernel<2, true><<<t->nitems, kFmmNT, 0, ns>>>(a);
+        b.diff ? fmm_near_kernel<2, true><<<t->nitems, kFmmNT, 0, ns>>>(a)
+               : fmm_near_kernel<2, true, 3><<<t->nitems, kFmmNT, 0, ns>>>(a);
     else if (R == 2)
-        fmm_near_kernel<2, false><<<t->nitems, kFmmNT, 0, ns>>>(a);
+        b.diff ? fmm_near_kernel<2, false><<<t->nitems, kFmmNT, 0, ns>>>(a)
+               : fmm_near_kernel<2, false, 3><<<t->nitems, kFmmNT, 0, ns>>>(a);
     else if (a.use_inv)
         fmm_near_kernel<1, false, 2><<<t->nitems, kFmmNT, 0, ns>>>(a);
     else if (EF)
-        fmm_near_kernel<1, true><<<t->nitems, kFmmNT, 0, ns>>>(a);
+        b.diff ? fmm_near_kernel<1, true><<<t->nitems, kFmmNT, 0, ns>>>(a)
+               : fmm_near_kernel<1, true, 3><<<t->nitems, kFmmNT, 0, ns>>>(a);
     else
-        fmm_near_kernel<1, false><<<t->nitems, kFmmNT, 0, ns>>>(a);
+        b.diff ? fmm_near_kernel<1, false><<<t->nitems, kFmmNT, 0, ns>>>(a)
+               : fmm_near_kernel<1, false, 3><<<t->nitems, kFmmNT, 0, ns>>>(a);
     ++launches;
     GNK_TRY_CUDA(cudaGetLastError());
     prof_end(tokn, PK_FMMNEAR, (double)R * t->near_pairs, ns,

@@ -103,3 +103,17 @@ def test_inverse_cache_changes_no_bit(G, name):
         b.solve_adjoint_ie(gam, precision=fmm, tol=1e-12)
         after = b.apply_adjoint(x, fmm).cpu().numpy()
     assert np.array_equal(before, after)
+
+
+@pytest.mark.parametrize("n", [24, 34, 66, 70, 78, 94, 130])
+def test_folded_items(G, n):
+    """The directly summed near field (weights of the caller's) with last items of 1
+    to 32 targets: within the FMM's bound, 1e-11 of sum |w/d|, of the dense sum."""
+    d = Dm.build_domain(Dm.random_ellipses(np.random.default_rng(n), 5, 2.0), n, bounded=False)
+    rng = np.random.default_rng(n)
+    w = rng.normal(size=d.N) + 1j * rng.normal(size=d.N)
+    diff = d.et[:, None] - d.et[None, :]
+    np.fill_diagonal(diff, np.inf)
+    with G.Boundary.from_domain(d, adjoint=False, device="cuda", precision=G.GNK_PREC_FMM) as b:
+        z = b.cauchy_sum(torch.as_tensor(w, device="cuda"), precision=G.GNK_PREC_FMM).cpu().numpy()
+    assert np.abs(z - (w[None, :] / diff).sum(1)).max() <= 1e-11 * (np.abs(w)[None, :] / np.abs(diff)).sum(1).max()

@@ -1908,10 +1908,13 @@ static int fmm_tree_host(const Boundary& b, FmmTree* t, cudaStream_t st) {
     }
     int L = 2;
     long long distinct = 1;
+    double prev = 0.0;  // nodes per box one level up
     for (int l = 1; l <= 16; ++l) {
         distinct += first_diff[l];
+        const double mean = (double)N / (double)distinct, above = prev;
+        prev = mean;
         if (l < 3) continue;
-        if (!fmm_level_wanted(b, l, (double)N / (double)distinct)) break;
+        if (!fmm_level_wanted(b, l, mean, above)) break;
         L = l;
     }
     t->L = L;

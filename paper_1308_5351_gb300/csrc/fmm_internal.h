@@ -109,8 +109,12 @@ int fmm_tree_device(const Boundary& b, FmmTree* t, cudaStream_t st);
 // bytes each (N = 524,288: 129 nodes per leaf 60.1 ms, 62 nodes 40.9, 30 nodes
 // 45.3; adjoint solve at N = 16,830: 128 nodes 2.20 ms, 55 nodes 2.11; N = 65,536:
 // 68 nodes 3.48 ms, 33 nodes 3.57).  Handles built for differentiation keep 64.
-inline bool fmm_level_wanted(const Boundary& b, int l, double mean_nodes) {
-    return mean_nodes >= ((l >= 4 && !b.diff) ? 44.0 : 64.0);
+// Where the boxes fill the plane a level has up to four times the nodes of the next:
+// there the line is the geometric mean of the two (62): 400 close circles at N = 40,000,
+// 156 nodes per leaf 8.58 ms, 39 nodes 5.66; 576 at 36,864, 144 nodes 11.19, 36 nodes 8.14.
+inline bool fmm_level_wanted(const Boundary& b, int l, double mean_nodes, double parent_nodes) {
+    if (l < 4 || b.diff) return mean_nodes >= 64.0;
+    return mean_nodes >= 44.0 || (mean_nodes >= 28.0 && mean_nodes * parent_nodes >= 62.0 * 62.0);
 }
 
 // Shares that each work item of a cached near field is split into: four blocks run

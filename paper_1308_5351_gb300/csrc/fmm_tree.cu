@@ -542,10 +542,13 @@ int fmm_tree_device(const Boundary& b, FmmTree* t, cudaStream_t st) {
     GNK_TRY_CUDA(cudaStreamSynchronize(st));
     int L = 2;
     long long distinct = 0;
+    double prev = 0.0;  // nodes per box one level up
     for (int l = 0; l <= 16; ++l) {
         distinct += h[l];
+        const double mean = distinct > 0 ? (double)N / (double)distinct : 0.0, above = prev;
+        prev = mean;
         if (l < 3) continue;
-        if (!fmm_level_wanted(b, l, (double)N / (double)distinct)) break;
+        if (!fmm_level_wanted(b, l, mean, above)) break;
         L = l;
     }
     if (L > kMaxGridLevel) return kFmmUseHost;

@@ -117,3 +117,15 @@ def test_folded_items(G, n):
     with G.Boundary.from_domain(d, adjoint=False, device="cuda", precision=G.GNK_PREC_FMM) as b:
         z = b.cauchy_sum(torch.as_tensor(w, device="cuda"), precision=G.GNK_PREC_FMM).cpu().numpy()
     assert np.abs(z - (w[None, :] / diff).sum(1)).max() <= 1e-11 * (np.abs(w)[None, :] / np.abs(diff)).sum(1).max()
+
+
+@pytest.mark.parametrize("grid,n", [(20, 80), (20, 100), (22, 64)])
+def test_domains_that_fill_the_plane(G, grid, n):
+    """Trees whose leaf level is chosen against its parent's mean (28 to 44 nodes per
+    leaf, 120 to 160 one level up): the FMM's operator against the double-float direct
+    sums, both within 1e-12 of (2/n) sum |A q x/d| <= 100, so within 1e-10 of |x| <= 1."""
+    d = Dm.close_curves(seed=5, n=n, grid=grid, squares=1)
+    x = torch.as_tensor(np.random.default_rng(n).uniform(-1, 1, d.N), device="cuda")
+    with G.Boundary.from_domain(d, adjoint=False, device="cuda", precision=G.GNK_PREC_FMM) as b:
+        y, z = b.apply_IminusN(x, G.GNK_PREC_FMM), b.apply_IminusN(x, G.GNK_PREC_DF32)
+    assert float((y - z).abs().max()) <= 2e-10

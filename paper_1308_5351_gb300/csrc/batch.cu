@@ -19,7 +19,7 @@
 //   sample of the batch's work list.
 //
 // * With GNK_PREC_FMM the systems are solved by the single-domain FBIE path
-//   with every Cauchy sum by the FMM (one quadtree, power table and near-field
+//   with every Cauchy sum by the FMM (one quadtree and near-field
 //   cache per domain, kept with the batch): worker threads, each with a CUDA
 //   stream of its own, take the domains in turn (largest first) and solve
 //   their right-hand sides one after the other, so that several domains'

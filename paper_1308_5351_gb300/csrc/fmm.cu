@@ -112,7 +112,7 @@ struct FmmArgs {
     int gathered;         // ws holds the weights in sorted order (products with a direct near field)
     int near_scaled;      // zn holds the near field times the operator's factor (cached)
     const float4* tn;     // [N] offset t of every node from its leaf centre in leaf widths (double-float complex)
-    const float4* tp;     // [N][P] powers t^k (handles built for differentiation), or null
+    int diff;             // a handle built for differentiation
     int* fault;           // set by a bounded wait that gave up
 };
 
@@ -420,38 +420,43 @@ __device__ __forceinline__ void p2m_leaf(const FmmArgs& a, int leaf, int box, in
     }
 }
 
-// P2M of one leaf from the cached powers t_j^k (a.tp, [node][k]): warp w
-// sums w_j t_j^k over the leaf's nodes j = j0 + w, j0 + w + kFmmTW, ...
-// (lane = k), with no block barrier until the warps' sums are added in warp
-// order.  The powers (33.5 MB at 65,536 nodes) are read with the default L2
-// policy: with the near-field stream marked evict-first they stay in L2
-// between products.
+// P2M of one leaf for the handles built for differentiation, one fixed sequence of
+// operations: t^k by repeated products, and warp w's sum over the nodes j0 + w,
+// j0 + w + kFmmTW, ... in this order.  Lane u forms the powers of node u of a batch of
+// kPowBatch in shared memory, then lane k sums w_j t_j^k over the batch.  (A table of
+// the powers, 512 bytes a node, gives the same bits and the same time to 0.4 %, 11.92
+// against 11.97 ms for a gradient at N = 40,960; without it no allocation decides which
+// form runs.)
+constexpr int kPowBatch = 16;
+
 template <int R>
-__device__ __forceinline__ void p2m_leaf_cached(const FmmArgs& a, int leaf, int box, int wid, int lane,
-                                                float4 (*s_acc)[32]) {
+__device__ __forceinline__ void p2m_leaf_diff(const FmmArgs& a, int leaf, int box, int wid, int lane,
+                                              float4 (*s_pow)[kPowBatch + 1], float4 (*s_w)[kPowBatch],
+                                              float4 (*s_acc)[32]) {
     cdf acc[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) acc[r] = cdf_zero();
     const int j0 = a.leaf_start[leaf], j1 = a.leaf_start[leaf + 1];
-    constexpr int U = 8;  // rows loaded before they are used: 8 loads in flight per warp
-    for (int j = j0 + wid; j < j1; j += kFmmTW * U) {
-        float4 tv[U], wv[R][U];
+    for (int j = j0 + wid; j < j1; j += kFmmTW * kPowBatch) {
+        const int cnt = min(kPowBatch, (j1 - j + kFmmTW - 1) / kFmmTW);
+        __syncwarp();  // the last batch has been read
+        if (lane < cnt) {
+            const int jj = j + lane * kFmmTW;
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int jj = j + u * kFmmTW;
-            if (jj < j1) {
-                tv[u] = __ldg(a.tp + (size_t)jj * kFmmP + lane);
-#pragma unroll
-                for (int r = 0; r < R; ++r) wv[r][u] = __ldcg(a.ws + (size_t)r * a.N + jj);
+            for (int r = 0; r < R; ++r) s_w[r][lane] = __ldcg(a.ws + (size_t)r * a.N + jj);
+            const cdf t = cdf_of(__ldg(a.tn + jj));
+            cdf v = cdf{df{1.f, 0.f}, df{0.f, 0.f}};
+            for (int k = 0; k < kFmmP; ++k) {
+                s_pow[k][lane] = cdf_pack(v);
+                v = cdf_mul(v, t);
             }
         }
+        __syncwarp();
+#pragma unroll 4
+        for (int u = 0; u < cnt; ++u) {
+            const cdf pw = cdf_of(s_pow[lane][u]);
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (j + u * kFmmTW < j1) {
-                const cdf pw = cdf_of(tv[u]);
-#pragma unroll
-                for (int r = 0; r < R; ++r) cdf_mac(acc[r], cdf_of(wv[r][u]), pw);
-            }
+            for (int r = 0; r < R; ++r) cdf_mac(acc[r], cdf_of(s_w[r][u]), pw);
         }
     }
 #pragma unroll
@@ -461,19 +466,21 @@ __device__ __forceinline__ void p2m_leaf_cached(const FmmArgs& a, int leaf, int 
     }
 }
 
-// Upward pass of the handles built for differentiation, one block per leaf: P2M
-// from the cached powers, then the multipoles move up the tree without a launch per level: the block that
+// Upward pass of the handles built for differentiation, one block per leaf: P2M,
+// then the multipoles move up the tree without a launch per level: the block that
 // completes the last child of a box (an atomic count per box; nothing waits)
 // forms that box's M2M from its children (warp w takes child w) and goes on
 // to the parent.
 template <int R>
 __global__ void __launch_bounds__(kFmmUT) fmm_up_kernel(FmmArgs a) {
+    __shared__ float4 s_pow[kFmmTW][kFmmP][kPowBatch + 1];
+    __shared__ float4 s_w[kFmmTW][R][kPowBatch];
     __shared__ float4 s_acc[kFmmTW][32];
     __shared__ int s_last;
     if (a.done != nullptr && *a.done) return;
     const int leaf = blockIdx.x, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int box = a.leaf_box[leaf];
-    p2m_leaf_cached<R>(a, leaf, box, wid, lane, s_acc);
+    p2m_leaf_diff<R>(a, leaf, box, wid, lane, s_pow[wid], s_w[wid], s_acc);
     for (;;) {
         if (wid == 0) __threadfence();  // the box's multipole (warp 0's stores) before the count
         __syncthreads();
@@ -1135,9 +1142,8 @@ __global__ void __launch_bounds__(kFmmNT) fmm_near_kernel(FmmArgs a) {
 
 // The offset t = (s - c)/r of every node from the centre of its leaf in leaf
 // widths, double-float complex, in sorted order: formed once per tree, read by
-// P2M and L2P (whose FP64 subtraction and product it replaces).  tp (handles
-// built for differentiation): also the powers t^k, k < P, [node][k].
-__global__ void fmm_tn_build_kernel(FmmArgs a, float4* __restrict__ tn, float4* __restrict__ tp) {
+// P2M and L2P (whose FP64 subtraction and product it replaces).
+__global__ void fmm_tn_build_kernel(FmmArgs a, float4* __restrict__ tn) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.N) return;
     const int box = a.node_box[i];
@@ -1146,13 +1152,6 @@ __global__ void fmm_tn_build_kernel(FmmArgs a, float4* __restrict__ tn, float4* 
     const double2 p = a.ps[i];
     const cdf t = cdf_split(make_double2((p.x - c.x) * ir, (p.y - c.y) * ir));
     tn[i] = cdf_pack(t);
-    if (!tp) return;
-    cdf v = cdf{df{1.f, 0.f}, df{0.f, 0.f}};
-    float4* out = tp + (size_t)i * kFmmP;
-    for (int k = 0; k < kFmmP; ++k) {
-        out[k] = cdf_pack(v);
-        v = cdf_mul(v, t);
-    }
 }
 
 // ---- Near-field operator caches.  The geometry of a handle is fixed for all
@@ -1535,7 +1534,7 @@ __global__ void __launch_bounds__(256) fmm_l2p_kernel(FmmArgs a, ReduceArgs e) {
     const int box = a.node_box[i];
     double ir = 0.0;
     cdf t;
-    if (EF || a.tp) {  // a handle built for differentiation
+    if (EF || a.diff) {
         const double2 c = a.center[box];
         ir = recip_f64(a.width[box]);  // (GB300's FP64 division is a long dependent chain)
         const double2 p = a.ps[i];
@@ -1831,7 +1830,7 @@ void release_fmm(Boundary& b) {
         give_stream(false, b.fmm->nst, b.device);
         give_event(b.fmm->ev_nq, b.device);
 
-        if (b.fmm->arena || b.fmm->sync || b.fmm->nq_item || b.fmm->tn || b.fmm->path || b.fmm->tp || b.fmm->fault) {  // once no stream uses them
+        if (b.fmm->arena || b.fmm->sync || b.fmm->nq_item || b.fmm->tn || b.fmm->path || b.fmm->fault) {  // once no stream uses them
             cudaDeviceSynchronize();
             cudaGetLastError();
             pool_free(b.fmm->arena, 0);
@@ -1849,7 +1848,6 @@ void release_fmm(Boundary& b) {
             pool_free(b.fmm->fault, 0);
             pool_free(b.fmm->tn, 0);
             pool_free(b.fmm->path, 0);
-            pool_free(b.fmm->tp, 0);
         }
         delete b.fmm;
         b.fmm = nullptr;
@@ -2204,8 +2202,6 @@ static int fmm_high_priority() {
 
 static void fmm_args(const Boundary& b, FmmArgs& a);
 
-constexpr double kTpMaxBytes = 4.0 * (1 << 30);
-
 // Builds the tree of the handle's nodes (once) with workspace for kMaxRHS
 // right-hand sides: on the device when the lookup grids fit, else on the host.
 int ensure_fmm(const Boundary& bc, int R, cudaStream_t st) {
@@ -2232,8 +2228,6 @@ int ensure_fmm(const Boundary& bc, int R, cudaStream_t st) {
             rc = GNK_ENOMEM;
         }
     }
-    // the nodes' offsets, and for a handle built for differentiation (whose P2M
-    // reads them) their powers, 512 bytes per node, below kTpMaxBytes
     if (rc == GNK_OK && pool_alloc(reinterpret_cast<void**>(&t->tn), (size_t)b.N * sizeof(float4), st) != cudaSuccess) {
         cudaGetLastError();
         set_error("FMM: allocation of the node offsets failed");
@@ -2246,14 +2240,11 @@ int ensure_fmm(const Boundary& bc, int R, cudaStream_t st) {
         set_error("FMM: allocation of the leaves' paths failed");
         rc = GNK_ENOMEM;
     }
-    if (rc == GNK_OK && b.diff && (double)b.N * kFmmP * sizeof(float4) <= kTpMaxBytes &&
-        pool_alloc(reinterpret_cast<void**>(&t->tp), (size_t)b.N * kFmmP * sizeof(float4), st) != cudaSuccess)
-        t->tp = nullptr;
     if (rc == GNK_OK) {
         FmmArgs a;
         b.fmm = t;
         fmm_args(b, a);
-        fmm_tn_build_kernel<<<(b.N + 255) / 256, 256, 0, st>>>(a, t->tn, t->tp);
+        fmm_tn_build_kernel<<<(b.N + 255) / 256, 256, 0, st>>>(a, t->tn);
         fmm_path_kernel<<<(t->nleaf + 127) / 128, 128, 0, st>>>(a, t->path);
         count_launches(2);
         if (cudaGetLastError() != cudaSuccess) {
@@ -2281,9 +2272,9 @@ int ensure_fmm(const Boundary& bc, int R, cudaStream_t st) {
 // lane for an L2L transform (32 terms of the Pascal sum at 24 each, two exact
 // scalings at 30 and two double-float additions), 742 for an M2M (31 passes
 // of a double-float complex addition, 22 each, and the two scalings); P2M: 35
-// complex products a node (38 each) and 16 per order for the sums (from the
-// table of a handle built for differentiation 48 per order); L2P: 58 R per node
-// and order (a complex product and sum), twice that with the derivative.
+// complex products a node (38 each) and 16 per order for the sums (a handle built
+// for differentiation 38 per order for the powers and 48 for the sums); L2P: 58 R per
+// node and order (a complex product and sum), twice that with the derivative.
 // which = 0: M2L; 1: the upward pass (P2M and the M2M climb); 2: L2L; 3: L2P;
 // 4: L2P with the derivative.  (The near field: fmm_near_instr.)
 double fmm_instr(const Boundary& b, int R, int which) {
@@ -2292,7 +2283,7 @@ double fmm_instr(const Boundary& b, int R, int which) {
     const double P = kFmmP, m2m = 742.0 * P, l2l = 840.0 * P, m2l = (24.0 * P + 98.0) * P;
     switch (which) {
         case 0: return R * m2l * (double)t->m2l_pairs;
-        case 1: return R * m2m * (double)t->m2m_pairs + (double)b.N * (t->tp ? 48.0 * R * P : R * (38.0 * 35.0 + 16.0 * P));
+        case 1: return R * m2m * (double)t->m2m_pairs + (double)b.N * (b.diff ? (38.0 + 48.0 * R) * P : R * (38.0 * 35.0 + 16.0 * P));
         case 2: return R * l2l * (double)t->nleaf * (t->L - t->l0);
         default: return R * (double)b.N * P * 58.0 * (which == 4 ? 2.0 : 1.0);
     }
@@ -2482,7 +2473,7 @@ static int l2p_epi(const FmmArgs& a, const ReduceArgs& e, int nb, cudaStream_t s
 }
 
 // Bytes of cache per product up to which it is left to L2's own policy (a third
-// of the 129 MB, beside the power table and the expansions); a larger one is
+// of the 129 MB, beside the nodes and the expansions); a larger one is
 // streamed past it.
 constexpr double kNbKeepBytes = 48e6;
 
@@ -2512,8 +2503,7 @@ static int launch_near_bulk(const Boundary& b, const FmmArgs& a, bool adj, cudaS
 
 // Starts forming the near-field cache right after the tree, on a stream of its
 // own, so that it overlaps whatever the caller enqueues before the first cached
-// product (the power table, the right-hand side's circulant, the first
-// product's gather and far field); that product waits for it.  For callers
+// product (the right-hand side's circulant, the first product's far field); that product waits for it.  For callers
 // whose products are z = E(q x) (the FBIE and the equation's solves).
 int fmm_start_near_cache(const Boundary& bc, cudaStream_t st) {
     Boundary& b = const_cast<Boundary&>(bc);
@@ -2561,9 +2551,9 @@ static int fmm_product(const Boundary& b, FmmArgs& a, int R, bool EF, const Redu
     // level's M2L on a third stream beside the climb measured slower: the two
     // compete for the same SMs.)
     const ProfToken toku = prof_begin(fs, PK_FMMUP);
-    if (a.tp && R == 2)  // a handle built for differentiation
+    if (b.diff && R == 2)
         fmm_up_kernel<2><<<t->nleaf, kFmmUT, 0, fs>>>(a);
-    else if (a.tp)
+    else if (b.diff)
         fmm_up_kernel<1><<<t->nleaf, kFmmUT, 0, fs>>>(a);
     else if (R == 2)
         fmm_up_tc_kernel<2><<<t->nleaf, kFmmUT, 0, fs>>>(a);
@@ -2714,7 +2704,7 @@ static void fmm_args(const Boundary& b, FmmArgs& a) {
     a.nsplit = 1;
     a.near_scaled = 0;
     a.tn = t->tn;
-    a.tp = t->tp;
+    a.diff = b.diff;
     a.mult = t->mult;
     a.loc = t->loc;
     a.ws = t->ws;
@@ -2762,7 +2752,7 @@ int run_fmm(const Boundary& b, const PairJob& job, cudaStream_t st) {
         if (!adj || job.done != nullptr) GNK_TRY(ensure_near_cache(b, adj, st));
         if ((adj ? b.fmm->nt_state : b.fmm->nq_state) >= 1) {
             cached = (adj || im_only) ? 1 : 0;
-            a.gathered = (a.tp != nullptr);  // the table form of P2M reads the sorted weights
+            a.gathered = b.diff;  // its P2M reads the sorted weights
             a.near_scaled = 1;
             a.nsplit = fmm_near_splits(b, b.fmm->nitems);
         }

@@ -80,7 +80,6 @@ struct FmmTree {
     int* fault = nullptr;       // set by a bounded wait of an FMM kernel that gave up
     unsigned* path = nullptr;   // [nleaf][L - l0 + 1]: box | quadrant << 30 of each leaf and its ancestors
     float4* tn = nullptr;       // [N] offset of each node from its leaf centre in leaf widths
-    float4* tp = nullptr;       // [N][P] its powers (handles built for differentiation), or null
     cudaStream_t aux = nullptr; // high-priority stream of the far field (the near field runs beside it)
     cudaStream_t nst = nullptr; // the near field's stream inside a solve (which runs on aux)
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_solve = nullptr;

@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(KT) k_norm(const double* __restrict__ x, int N
             s->last_k = s->k;
             s->k = 0;
             if (!isfinite(nrm)) s->nonfinite = 1;
-            s->done = (!(nrm > s->tol * s->bnorm)) ? 1 : 0;  // also stops on NaN
+            s->done = (!(nrm / s->bnorm > s->tol)) ? 1 : 0;  // the host goes by it; also stops on NaN
             if (s->done) report_progress(s, 0, true);
             p.g[0] = nrm;
             for (int k = 1; k <= s->restart; ++k) p.g[k] = 0.0;
@@ -1344,7 +1344,9 @@ int gmres_on(Boundary& b, int adjoint /* OpId */, int prec, const double* rhs, d
             status = GNK_ENONFINITE;
             break;
         }
-        if (*relres <= tol) {
+        // The device's decision (relres <= tol, as rounded there), not one of the host's
+        // own: were the two to differ in the last bit, every further cycle would do nothing.
+        if (hs.done) {
             status = GNK_OK;
             break;
         }

@@ -197,8 +197,8 @@ struct Boundary {
     size_t partial_bytes = 0;
     // source-chunk override of the direct pair kernels for the current call
     // (gnk_options.tile_chunks; 0: the plans below) and the larger partial-sum
-    // workspace that it or the FP64 kernel may need (from the memory pool, kept
-    // until the handle is freed)
+    // workspace that it may need (from the memory pool, kept until the handle is
+    // freed)
     mutable int tile_chunks = 0;
     mutable void* partial_x = nullptr;
     mutable size_t partial_x_bytes = 0;

@@ -1507,7 +1507,7 @@ PairPlan make_plan(int N, int sms, int blocks_per_sm, int targets_per_block, int
 // domains take 32-node blocks of one warp (N = 768: 300 blocks instead of the
 // 18 of the ordered kernel).
 constexpr int kSymMaxBlocks = kSymCounts;
-constexpr size_t kSymArenaBytes = (size_t)64 << 20;
+constexpr size_t kSymArenaBytes = (size_t)4 << 20;  // N <= 2,048
 
 SymPlan make_sym_plan(int N, int sms) {
     static const int kShape[][2] = {{1, 1}, {2, 1}, {4, 1}, {8, 1}, {8, 2}, {8, 4}, {8, 8}, {8, 16}};
@@ -1535,8 +1535,8 @@ int pair_workspace_bytes(const Boundary& b, size_t* bytes) {
     const size_t b32 = (size_t)b.plan32.chunks * kMaxRHS * b.N * sizeof(float2);
     const size_t bdf = (size_t)b.plandf.chunks * kMaxRHS * b.N * sizeof(float4);
     *bytes = std::max(std::max(b64, b32), bdf);
-    // the sums of the kernel that takes each pair once, where they are small
-    // (larger ones come from the pool with the first FP64 product)
+    // the sums of the FP64 kernel that takes each pair once, where they are small
+    // (sym_workspace has larger ones from the pool for the one product)
     const size_t bs = (size_t)b.sym64.nt * kMaxRHS * b.N * sizeof(double2);
     if (b.sym64.W > 0 && bs <= kSymArenaBytes) *bytes = std::max(*bytes, bs);
     return GNK_OK;
@@ -1576,21 +1576,38 @@ static int launch_plan(const Boundary& b, const PairPlan& base, size_t elem_byte
     return partial_workspace(b, (size_t)p->chunks * kMaxRHS * b.N * elem_bytes, partial, st);
 }
 
-// The workspace of the kernels that take each pair once; null where the ordered
-// kernel, which needs far less, is to serve the call: no memory for it, or a
-// capturing stream and more than the handle's own workspace holds (the one from
-// the pool moves when a later product needs more, and a graph keeps its address).
-static int sym_workspace(const Boundary& b, size_t need, void** partial, cudaStream_t st) {
-    *partial = nullptr;
-    if (need > b.partial_bytes) {
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        GNK_TRY_CUDA(cudaStreamIsCapturing(st, &cs));
-        if (cs != cudaStreamCaptureStatusNone) return GNK_OK;
+// The workspace of the kernels that take each pair once: the handle's own where it
+// is large enough, else a block of the pool for the length of the product, given back
+// in the order of the stream (the sums are nt x N, up to 1 GB a right-hand side: a
+// program that keeps many handles must not keep one for each).  None where the
+// ordered kernel, which needs far less, is to serve the call: no memory for it, or a
+// capturing stream and more than the handle's own holds.
+struct SymSpace {
+    void* p = nullptr;
+    cudaStream_t st = nullptr;
+    bool lent = false;
+    SymSpace() = default;
+    SymSpace(const SymSpace&) = delete;
+    ~SymSpace() {
+        if (lent) pool_free(p, st);
     }
-    const int rc = partial_workspace(b, need, partial, st);
-    if (rc == GNK_OK) return GNK_OK;
-    *partial = nullptr;
-    return rc == GNK_ENOMEM ? GNK_OK : rc;
+};
+
+static int sym_workspace(const Boundary& b, size_t need, SymSpace* s, cudaStream_t st) {
+    if (need <= b.partial_bytes) {
+        s->p = b.partial;
+        return GNK_OK;
+    }
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    GNK_TRY_CUDA(cudaStreamIsCapturing(st, &cs));
+    if (cs != cudaStreamCaptureStatusNone) return GNK_OK;
+    s->st = st;
+    s->lent = pool_alloc(&s->p, need, st) == cudaSuccess;
+    if (!s->lent) {
+        cudaGetLastError();
+        s->p = nullptr;
+    }
+    return GNK_OK;
 }
 
 template <int R, int MODE, int COMP, int W>
@@ -1629,9 +1646,9 @@ static int run_pairsum64_sym(const Boundary& b, const PairJob& job, cudaStream_t
     *ran = false;
     const SymPlan& p = b.sym64;
     if (p.W == 0 || b.tile_chunks > 0) return GNK_OK;
-    void* partial = nullptr;
-    GNK_TRY(sym_workspace(b, (size_t)p.nt * job.R * b.N * sizeof(double2), &partial, st));
-    if (!partial) return GNK_OK;
+    SymSpace space;
+    GNK_TRY(sym_workspace(b, (size_t)p.nt * job.R * b.N * sizeof(double2), &space, st));
+    if (!space.p) return GNK_OK;
     Pair64SymArgs a;
     a.et = b.et;
     a.N = b.N;
@@ -1640,7 +1657,7 @@ static int run_pairsum64_sym(const Boundary& b, const PairJob& job, cudaStream_t
     a.x0 = job.x[0];
     a.x1 = job.x[1];
     a.s = job.s;
-    a.partial = static_cast<double2*>(partial);
+    a.partial = static_cast<double2*>(space.p);
     a.nt = p.nt;
     a.G = p.G;
     a.count = b.sym_count;
@@ -1666,7 +1683,7 @@ static int run_pairsum64_sym(const Boundary& b, const PairJob& job, cudaStream_t
     const bool fast = p.W > 1 || p.nt * (p.nt + 1) / 2 >= kSymFastBlocks * b.sms;
     const double per_pair = (fast ? 2.0 : 9.0) + ((job.comp && job.R == 1) ? 4.0 : 8.0 * job.R);
     prof_end(tok, PK_PAIR64, (double)job.R * b.N * (b.N - 1.0), st, 0.5 * per_pair * b.N * (b.N - 1.0));
-    if (p.W > 1) GNK_TRY_CUDA(launch_reduce(b, job, p.nt, 0, st, partial));  // else done by the kernel
+    if (p.W > 1) GNK_TRY_CUDA(launch_reduce(b, job, p.nt, 0, st, space.p));  // else done by the kernel
     count_launches(p.W > 1 ? 2 : 1);
     *ran = true;
     return GNK_OK;
@@ -1710,7 +1727,7 @@ int run_pairsum64(const Boundary& b, const PairJob& job, cudaStream_t st) {
     return GNK_OK;
 }
 
-constexpr int kSymMaxTiles = 256;  // N <= 65,536: 268 MB of double-float sums
+constexpr int kSymMaxTiles = 256;  // N <= 65,536: 268 MB of double-float sums a right-hand side
 
 // The FP32 sum with each pair taken once; *ran as for the double-float sum.
 static int run_pairsum32_sym(const Boundary& b, const PairJob& job, cudaStream_t st, bool* ran) {
@@ -1718,9 +1735,9 @@ static int run_pairsum32_sym(const Boundary& b, const PairJob& job, cudaStream_t
     const int nt = (b.N + kSrcTile32 - 1) / kSrcTile32, pairs = nt * (nt + 1) / 2;
     if (b.tile_chunks > 0 || b.f32_scalar || nt > kSymMaxTiles) return GNK_OK;
     if (job.mode == W_SCALED && job.s != b.q && job.s != b.A) return GNK_OK;  // refused by the caller
-    void* partial = nullptr;
-    GNK_TRY(sym_workspace(b, (size_t)nt * job.R * b.N * sizeof(float2), &partial, st));
-    if (!partial) return GNK_OK;
+    SymSpace space;
+    GNK_TRY(sym_workspace(b, (size_t)nt * job.R * b.N * sizeof(float2), &space, st));
+    if (!space.p) return GNK_OK;
     Pair32Args a;
     a.et32 = b.et32;
     a.ref32 = b.ref32;
@@ -1731,7 +1748,7 @@ static int run_pairsum32_sym(const Boundary& b, const PairJob& job, cudaStream_t
     a.x0 = job.x[0];
     a.x1 = job.x[1];
     a.s32 = (job.s == b.q) ? b.q32 : b.A32;
-    a.partial = static_cast<float2*>(partial);
+    a.partial = static_cast<float2*>(space.p);
     a.tiles_src = nt;
     a.tiles_per_chunk = 1;
     a.done = job.done;
@@ -1754,7 +1771,7 @@ static int run_pairsum32_sym(const Boundary& b, const PairJob& job, cudaStream_t
     // right-hand side (one part of z: 3)
     const double per_pair = 4.0 + ((job.comp && job.R == 1) ? 6.0 : 4.0 + 8.0 * job.R);
     prof_end(tok, PK_PAIR32, (double)job.R * b.N * (b.N - 1.0), st, 0.5 * per_pair * b.N * (b.N - 1.0));
-    GNK_TRY_CUDA(launch_reduce(b, job, nt, 1, st, partial));
+    GNK_TRY_CUDA(launch_reduce(b, job, nt, 1, st, space.p));
     count_launches(2);
     *ran = true;
     return GNK_OK;
@@ -1830,9 +1847,9 @@ static int run_pairsumdf_sym(const Boundary& b, const PairJob& job, cudaStream_t
     *ran = false;
     const int nt = (b.N + kSrcTile32 - 1) / kSrcTile32, pairs = nt * (nt + 1) / 2;
     if (b.tile_chunks > 0 || b.df_scalar || nt > kSymMaxTiles) return GNK_OK;
-    void* partial = nullptr;
-    GNK_TRY(sym_workspace(b, (size_t)nt * job.R * b.N * sizeof(float4), &partial, st));
-    if (!partial) return GNK_OK;
+    SymSpace space;
+    GNK_TRY(sym_workspace(b, (size_t)nt * job.R * b.N * sizeof(float4), &space, st));
+    if (!space.p) return GNK_OK;
     PairDFArgs a;
     a.et = b.et;
     a.ref64 = b.ref64;
@@ -1843,7 +1860,7 @@ static int run_pairsumdf_sym(const Boundary& b, const PairJob& job, cudaStream_t
     a.x0 = job.x[0];
     a.x1 = job.x[1];
     a.s = job.s;
-    a.partial = static_cast<float4*>(partial);
+    a.partial = static_cast<float4*>(space.p);
     a.tiles_src = nt;
     a.tiles_per_chunk = 1;
     a.done = job.done;
@@ -1866,7 +1883,7 @@ static int run_pairsumdf_sym(const Boundary& b, const PairJob& job, cudaStream_t
     // 48 (one part of z: 24)
     const double per_pair = 49.0 + ((job.comp && job.R == 1) ? 48.0 : 96.0 * job.R);
     prof_end(tok, PK_PAIRDF, (double)job.R * b.N * (b.N - 1.0), st, 0.5 * per_pair * b.N * (b.N - 1.0));
-    GNK_TRY_CUDA(launch_reduce(b, job, nt, 2, st, partial));
+    GNK_TRY_CUDA(launch_reduce(b, job, nt, 2, st, space.p));
     count_launches(2);
     *ran = true;
     return GNK_OK;

@@ -41,7 +41,9 @@ def build(force: bool = False, verbose: bool = False, extra_flags=None) -> str:
         return LIB
     os.makedirs(OUT_DIR, exist_ok=True)
     nvcc = nvcc_path()
-    flags = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
+    # device code above 10 MB an object would be compressed: fmm.cu's first kernel in a
+    # process then waited 8 ms for its module to be unpacked
+    flags = ARCH + ["-O3", "-lineinfo", "--compress-mode=none", "-std=c++17", "-Xcompiler", "-fPIC",
                     "-I", os.path.join(ROOT, "include")] + list(extra_flags or [])
 
     def compile_one(src):

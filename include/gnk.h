@@ -219,12 +219,13 @@ int gnk_build_boundary(gnk_boundary** out, int m1, int n,
  * (GNK_EINVAL): its geometry derivative is that of the subtracted form. */
 #define GNK_BUILD_PLAIN 0x200
 /* With GNK_BUILD_DIFF or-ed into `precision`, the FMM of a handle whose solution
- * will be differentiated keeps to one fixed sequence of operations.  Beside a
- * graded corner the nodes are as close as n^-3 and dL/d eta sums 1/d^2: the last
- * bit of mu or lambda moves it by 1e-7 of its norm at n = 2048.  Other handles
- * take faster sequences of the same accuracy (multipole-to-local translations on
- * the tensor cores; the solves of the adjoint and the transposed equation read
- * their near field from an operator cache). */
+ * will be differentiated keeps its translations and its directly summed near field
+ * to one fixed sequence of double-float operations.  Beside a graded corner the nodes
+ * are as close as n^-3 and dL/d eta sums 1/d^2: a change of the last bits of mu or
+ * lambda moves it by up to 1e-7 of its norm at n = 2048 (measured 3e-8).  Other handles
+ * take faster sequences of the same accuracy (translations on the tensor cores; the
+ * solves of the adjoint and the transposed equation read their near field from an
+ * operator cache). */
 #define GNK_BUILD_DIFF 0x400
 int gnk_build_boundary_ex(gnk_boundary** out, int m1, int n,
                           const double* et, const double* etp, const double* etpp,
@@ -332,7 +333,11 @@ int gnk_solve_ie_transpose(const gnk_boundary* b, const double* rhs, double* x,
  * K = 2I + diag(B1) - B and M = D - diag(D1) + Lhat, then one FP64 pass of six
  * Cauchy sums and six sums of the derivative kernel 1/(eta_i - eta_j)^2.
  * `opt` controls the transposed solve (its precision also sets the arithmetic
- * of M^T).  Host arrays are staged through temporary device buffers.  Returns
+ * of M^T).  With an FMM precision the handle may be built with GNK_BUILD_DIFF or
+ * without: dL/d eta of the two differs by less than 1e-7 of its norm at graded corners
+ * with n = 2048, below the error that the solves leave there (8e-6 at tol = 1e-12,
+ * 5e-7 at 1e-13, with the flag, without it and with direct FP64 sums alike).  Host
+ * arrays are staged through temporary device buffers.  Returns
  * GNK_OK or GNK_ENOTCONV (gradient from the best iterate). */
 int gnk_fbie_backward(const gnk_boundary* b, const double* mu, const double* gam,
                       const double* grad_mu, const double* grad_h, const double* grad_hk,

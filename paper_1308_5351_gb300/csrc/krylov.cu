@@ -1159,8 +1159,12 @@ struct Progress {
     }
 };
 
-// Steps enqueued ahead of the device: the host needs 10 to 20 us to enqueue one
-// and the device at least 25 us to run it.
+// Steps enqueued ahead of the device, which takes 35 us (N = 768, FP64) to 720 us
+// (N = 524,288) for one; the host enqueues one in 10 to 20 us.  Every step enqueued past
+// convergence costs its empty launches: with 2, 4, 8 steps and the whole cycle ahead the
+// FBIE at N = 768 takes 695, 707, 735, 762 us, the adjoint solve at N = 16,830 2.05, 2.06,
+// 2.16, 2.37 ms, the FBIE at N = 65,536 3.27, 3.29, 3.34, 3.51 ms.  With the host's 16
+// cores overloaded twice a step of the latter takes 7 to 8 ms with either lead.
 constexpr int kAhead = 2;
 
 // Test hook of gnk_debug_barrier_fault, read by every later solve.

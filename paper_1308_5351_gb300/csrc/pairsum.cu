@@ -1639,6 +1639,22 @@ static cudaError_t launch_sym64_w(int W, int sms, const Pair64SymArgs& a, const 
     }
 }
 
+// Whether the result of a job lies over one of its inputs.  The 32-node kernel writes
+// results while other blocks still read the inputs, so such a product goes through the
+// handle's scratch (the other kernels write their results in a launch of its own).
+static bool in_place(const PairJob& job, int N) {
+    const bool z = job.epi == EPI_Z;
+    const char* out = z ? reinterpret_cast<const char*>(job.out_c) : reinterpret_cast<const char*>(job.out);
+    const size_t nout = (size_t)N * (z ? job.R * sizeof(double2) : sizeof(double));
+    for (int r = 0; r < job.R; ++r) {
+        const char* in = job.mode == W_COMPLEX ? reinterpret_cast<const char*>(job.w[r])
+                                               : reinterpret_cast<const char*>(job.x[r]);
+        const size_t nin = (size_t)N * (job.mode == W_COMPLEX ? sizeof(double2) : sizeof(double));
+        if (in < out + nout && out < in + nin) return true;
+    }
+    return false;
+}
+
 // The FP64 sum with each pair taken once.  *ran = false where the ordered kernel
 // serves the call: a source-chunk override, more than 524,288 nodes, no memory for
 // the partial sums, or a capturing stream (sym_workspace).
@@ -1646,6 +1662,20 @@ static int run_pairsum64_sym(const Boundary& b, const PairJob& job, cudaStream_t
     *ran = false;
     const SymPlan& p = b.sym64;
     if (p.W == 0 || b.tile_chunks > 0) return GNK_OK;
+    if (p.W == 1 && in_place(job, b.N)) {
+        PairJob via = job;
+        const bool z = job.epi == EPI_Z;
+        if (z)
+            via.out_c = b.zbuf;
+        else
+            via.out = reinterpret_cast<double*>(b.zbuf);
+        GNK_TRY(run_pairsum64_sym(b, via, st, ran));
+        if (*ran)
+            GNK_TRY_CUDA(cudaMemcpyAsync(z ? (void*)job.out_c : (void*)job.out, b.zbuf,
+                                         (size_t)b.N * (z ? job.R * sizeof(double2) : sizeof(double)),
+                                         cudaMemcpyDeviceToDevice, st));
+        return GNK_OK;
+    }
     SymSpace space;
     GNK_TRY(sym_workspace(b, (size_t)p.nt * job.R * b.N * sizeof(double2), &space, st));
     if (!space.p) return GNK_OK;

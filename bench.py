@@ -62,13 +62,12 @@ PEAK_BASIS = {
     "pair64": "FP64 pipe: 152 SMs x 2 DFMA lanes x 2070 MHz; 2 + 8R FP64 instr per unordered pair (9 + 8R in small domains)",
     "pair32": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 8 + 8R FP32 instr per unordered pair (+1 MUFU)",
     "pairdf": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 49 + 96R FP32 instr per unordered double-float pair",
-    "fmm": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; per M2L pair and lane 24 FP32 instr for each "
-           "of the 32 double-float products of the real Pascal matrix + 98 for the two complex scalings "
-           "(equivalents: the matrix product itself runs on the tensor cores)",
-    "fmm_up": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 742 FP32 instr per lane per binomial M2M "
-              "transform (equivalents: on the tensor cores), 35 x 38 R + 16R per order and node in P2M",
-    "fmm_l2l": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 840 FP32 instr per lane per Pascal-matrix L2L transform "
-               "(equivalents: on the tensor cores)",
+    "fmm": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; per lane and tile of four M2L pairs 744 FP32 instr "
+           "(digits, scalings and sums around the matrix product on the tensor cores)",
+    "fmm_up": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 816 FP32 instr per lane and M2M tile (around the "
+              "matrix product on the tensor cores), 35 x 38 R per node and 16R per order and node in P2M",
+    "fmm_l2l": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 728 FP32 instr per lane and L2L tile (around the "
+               "matrix product on the tensor cores)",
     "fmm_l2p": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 58R FP32 instr per node and order (Horner)",
     "fmm_near": "FP32 pipe: 152 SMs x 128 lanes x 2070 MHz; 49 + 48R FP32 instr per double-float "
                 "near-field pair",

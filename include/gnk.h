@@ -38,6 +38,16 @@
  *   - GMRES orthogonalises in double-float (about 48 significant bits) for
  *     every precision but GNK_PREC_FP64, which keeps it in FP64.
  *   - The caller owns all arrays it passes; the handle owns its own copies.
+ *   - Direct sums take partial sums of (node blocks) x N from the library's memory
+ *     pool for the length of a product: per right-hand side up to 1.1 GB in FP64
+ *     (N = 524,288), 268 MB in double-float and 134 MB in FP32 (N = 65,536).  Where
+ *     there is no room for them, and in a product captured into a CUDA graph whose
+ *     partial sums exceed the handle's own few MB, a form that needs none serves
+ *     the call, at about half the speed and with other last bits.
+ *   - With the FMM a handle keeps operator caches of its near field: 16 bytes per
+ *     near pair after the first product with weights q x, 8 more after an adjoint or
+ *     a transposed solve (16 with GNK_BUILD_DIFF).  A cache above 16 GiB, or that
+ *     finds no memory, is left out and its sums are formed for every product.
  */
 #ifndef GNK_H
 #define GNK_H
@@ -163,11 +173,13 @@ int gnk_profile_mask(unsigned mask);
 int gnk_profile_query(int kind, long long* launches, double* total_ms,
                       double* work);
 /* As gnk_profile_query, plus the launches' algorithmic instruction count on
- * their limiting pipe (pair kernels: per ordered pair, FP64 (2 + 8R)/2 where
- * each pair is taken once (one part of z: 6/2; domains of up to about a thousand
- * nodes: 9 in place of 2), else 9 + 4R, FP32 6 + 4R,
- * double-float 49 + 48R, R the right-hand sides of the launch; the FMM
- * kernels: FP32-pipe instructions of their double-float arithmetic). */
+ * their limiting pipe (pair kernels, per ordered pair with R right-hand sides:
+ * where each pair is taken once FP64 (2 + 8R)/2, one part of z 6/2, with 9 in
+ * place of 2 up to 1,344 nodes; FP32 (8 + 8R)/2, one part 10/2; double-float
+ * (49 + 96R)/2, one part 97/2; else FP64 9 + 4R, FP32 6 + 4R, double-float
+ * 49 + 48R.  The FMM kernels: FP32-pipe instructions of their double-float
+ * arithmetic, for the translations on the tensor cores of the digits, the
+ * scalings and the sums around the matrix products). */
 int gnk_profile_query_ex(int kind, long long* launches, double* total_ms,
                          double* work, double* instr);
 /* As gnk_profile_query_ex, plus the algorithmic bytes the launches read and

@@ -2299,13 +2299,15 @@ int ensure_fmm(const Boundary& bc, int R, cudaStream_t st) {
     return rc;
 }
 
-// FP32-pipe instructions of one FMM product, for the roofline, in the
-// double-float form of the translations whichever form runs.  M2L, per pair
-// and lane: 32 (2 Dekker products and 2 compensated sums, 24) for the real
-// Pascal matrix, the two complex scalings (38 each) and the sum (22); 840 per
-// lane for an L2L transform (32 terms of the Pascal sum at 24 each, two exact
-// scalings at 30 and two double-float additions), 742 for an M2M (31 passes
-// of a double-float complex addition, 22 each, and the two scalings); P2M: 35
+// FP32-pipe instructions of one FMM product, for the roofline.  Translations on the
+// tensor cores, per lane and tile of four pairs: 400 for tc_transform (184 for the
+// digits, 216 for the sums), and around it 344 for M2L, 416 for M2M (one tile per box
+// with children), 328 for L2L (one per four leaves and level).  In double-float
+// (handles built for differentiation), per lane and pair: M2L 32 (2 Dekker products
+// and 2 compensated sums, 24) for the real Pascal matrix, the two complex scalings (38
+// each) and the sum (22); 840 for an L2L transform (32 terms of the Pascal sum at 24
+// each, two exact scalings at 30 and two double-float additions), 742 for an M2M (31
+// passes of a double-float complex addition, 22 each, and the two scalings).  P2M: 35
 // complex products a node (38 each) and 16 per order for the sums (a handle built
 // for differentiation 38 per order for the powers and 48 for the sums); L2P: 58 R per
 // node and order (a complex product and sum), twice that with the derivative.
@@ -2314,11 +2316,14 @@ int ensure_fmm(const Boundary& bc, int R, cudaStream_t st) {
 double fmm_instr(const Boundary& b, int R, int which) {
     const FmmTree* t = b.fmm;
     if (!t) return 0.0;
-    const double P = kFmmP, m2m = 742.0 * P, l2l = 840.0 * P, m2l = (24.0 * P + 98.0) * P;
+    const double P = kFmmP, levels = t->L - t->l0;
     switch (which) {
-        case 0: return R * m2l * (double)t->m2l_pairs;
-        case 1: return R * m2m * (double)t->m2m_pairs + (double)b.N * (b.diff ? (38.0 + 48.0 * R) * P : R * (38.0 * 35.0 + 16.0 * P));
-        case 2: return R * l2l * (double)t->nleaf * (t->L - t->l0);
+        case 0: return R * (double)t->m2l_pairs * (b.diff ? (24.0 * P + 98.0) * P : 744.0 * 32.0 / 4.0);
+        case 1:
+            if (b.diff) return R * 742.0 * P * (double)t->m2m_pairs + (double)b.N * (38.0 + 48.0 * R) * P;
+            return R * (816.0 * 32.0 * (double)(t->nbox - t->nleaf) + (double)b.N * (38.0 * 35.0 + 16.0 * P));
+        case 2:
+            return R * levels * (b.diff ? 840.0 * P * (double)t->nleaf : 728.0 * 32.0 * (double)((t->nleaf + 3) / 4));
         default: return R * (double)b.N * P * 58.0 * (which == 4 ? 2.0 : 1.0);
     }
 }

@@ -93,6 +93,7 @@ struct FmmTree {
 // GNK_OK, an error code, or kFmmUseHost when the tree is too deep for the
 // device lookup grids (then the host builder runs).
 constexpr int kFmmUseHost = 1;
+constexpr int kMaxGridLevel = 11;  // the deepest level of those grids
 
 // The topmost level with expansions.  From level 3 on in trees of level 4 and more (all of whose boxes then
 // interact where they are not adjacent, at most 60 each) the climb and the descent
@@ -111,8 +112,11 @@ int fmm_tree_device(const Boundary& b, FmmTree* t, cudaStream_t st);
 // Where the boxes fill the plane a level has up to four times the nodes of the next:
 // there the line is the geometric mean of the two (62): 400 close circles at N = 40,000,
 // 156 nodes per leaf 8.58 ms, 39 nodes 5.66; 576 at 36,864, 144 nodes 11.19, 36 nodes 8.14.
+// Levels beyond the device builder's grids want 64 too: the host builds such a tree
+// (196 small circles far apart, N = 156,800: the FBIE with its tree 6.96 ms with the 47
+// nodes of level 12, 2.66 with the 95 of level 11).
 inline bool fmm_level_wanted(const Boundary& b, int l, double mean_nodes, double parent_nodes) {
-    if (l < 4 || b.diff) return mean_nodes >= 64.0;
+    if (l < 4 || l > kMaxGridLevel || b.diff) return mean_nodes >= 64.0;
     return mean_nodes >= 44.0 || (mean_nodes >= 28.0 && mean_nodes * parent_nodes >= 62.0 * 62.0);
 }
 

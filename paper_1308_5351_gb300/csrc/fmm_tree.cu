@@ -30,7 +30,6 @@ namespace {
 constexpr int TB = 256;           // threads of the per-node kernels
 constexpr int RS_TILE = 2048;     // radix sort: nodes per block (8 warps x 256)
 constexpr int LV_BLOCK = 1024;    // level box ids: nodes per block
-constexpr int kMaxGridLevel = 11;
 
 __device__ __forceinline__ uint32_t spread16d(uint32_t v) {
     v &= 0xffffu;

@@ -683,11 +683,11 @@ __device__ __forceinline__ void tc_transform(const uint4* __restrict__ T, const 
     }
     // pair t: y = 2^(ex - 126) sum_s c_s 2^(-18 - 10 s)
     const int ext = __shfl_sync(full, ex, 8 * t);
-    const float2 dn = f2(__uint_as_float((unsigned)(min(ext, 253) + 1) << 23));
+    const float2 dn = f2(__uint_as_float((unsigned)ext << 23));  // 2^(ex - 127), and 2 in w
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         float2 v[kTcD + 1];
-        float w = 1.f / 262144.f;
+        float w = 2.f / 262144.f;
 #pragma unroll
         for (int s = 0; s <= kTcD; ++s) {
             v[s] = mul2(make_float2(c[s][i >> 1][2 * (i & 1)], c[s][i >> 1][2 * (i & 1) + 1]), f2(w));

@@ -31,7 +31,9 @@ struct CEArgs {
 
 // FP64 pipe bound: per pair 2 (z - eta) and 8 (two complex sums), 1/(z - eta) being
 // formed on the FP32 pipe (20,000 points, 5,120 nodes: 3.45 ms with all 17
-// instructions of a pair in FP64, 2.06 ms now).
+// instructions of a pair in FP64, 2.06 ms now).  The last tile ends with the nodes:
+// a source far away in its place would take inv_conj_f64's slow way (1,000 points, 258
+// nodes: 206 us with it, 169 without).
 __global__ void __launch_bounds__(CE_NT64) ceval64_kernel(CEArgs a) {
     __shared__ double2 s_pos[CE_S64];
     __shared__ double2 s_w[2][CE_S64];
@@ -48,22 +50,17 @@ __global__ void __launch_bounds__(CE_NT64) ceval64_kernel(CEArgs a) {
     }
     const int tb = blockIdx.y * a.tpc, te = min(tb + a.tpc, a.tiles_src);
     for (int tile = tb; tile < te; ++tile) {
-        const int j0 = tile * CE_S64;
+        const int j0 = tile * CE_S64, cnt = min(CE_S64, a.N - j0);
         __syncthreads();
-        for (int k = threadIdx.x; k < CE_S64; k += CE_NT64) {
+        for (int k = threadIdx.x; k < cnt; k += CE_NT64) {
             const int j = j0 + k;
-            if (j < a.N) {
-                const double2 e = a.etp[j], fv = a.f[j];
-                s_pos[k] = a.et[j];
-                s_w[0][k] = make_double2(fv.x * e.x - fv.y * e.y, fv.x * e.y + fv.y * e.x);
-                s_w[1][k] = e;
-            } else {
-                s_pos[k] = make_double2(1e150, 1e150);
-                s_w[0][k] = s_w[1][k] = make_double2(0.0, 0.0);
-            }
+            const double2 e = a.etp[j], fv = a.f[j];
+            s_pos[k] = a.et[j];
+            s_w[0][k] = make_double2(fv.x * e.x - fv.y * e.y, fv.x * e.y + fv.y * e.x);
+            s_w[1][k] = e;
         }
         __syncthreads();
-        for (int k = 0; k < CE_S64; ++k) {
+        for (int k = 0; k < cnt; ++k) {
             const double2 sp = s_pos[k];
 #pragma unroll
             for (int t = 0; t < CE_T64; ++t) {

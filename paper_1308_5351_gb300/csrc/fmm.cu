@@ -1461,7 +1461,9 @@ __global__ void __launch_bounds__(kNbThreads) fmm_near_bulk_kernel(FmmArgs a, co
         asm volatile("bar.sync 1, %0;" ::"r"(kFmmNT) : "memory");
         for (int c = seg; ok && c < se; ++c) {
             const int u = c - cb, st = u % kNbStages;
-            if (!mbar_wait(&full[st], (unsigned)((u / kNbStages) & 1), kNbSpin)) {
+            // one decision per warp: lanes that gave up alone would wait at the next barrier
+            // for the others, and these for them
+            if (!__all_sync(0xffffffffu, mbar_wait(&full[st], (unsigned)((u / kNbStages) & 1), kNbSpin))) {
                 atomicExch(a.fault, 1);
                 ok = false;
                 break;

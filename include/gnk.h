@@ -43,7 +43,7 @@
  *     (N = 524,288), 268 MB in double-float and 134 MB in FP32 (N = 65,536).  Where
  *     there is no room for them, and in a product captured into a CUDA graph whose
  *     partial sums exceed the handle's own few MB, a form that needs none serves
- *     the call, at about half the speed and with other last bits.
+ *     the call, at a quarter to two thirds of the speed and with other last bits.
  *   - With the FMM a handle keeps operator caches of its near field: 16 bytes per
  *     near pair after the first product with weights q x, 8 more after an adjoint or
  *     a transposed solve (16 with GNK_BUILD_DIFF).  A cache above 16 GiB, or that

@@ -313,9 +313,6 @@ double fmm_instr(const Boundary& b, int R, int which);
 double fmm_near_instr(const Boundary& b, int R);
 // Device word set by an FMM kernel whose bounded wait gave up (null before the tree).
 const int* fmm_fault_word(const Boundary& b);
-// the chunk reduction and epilogue of the pair sums, for products formed elsewhere
-cudaError_t launch_reduce_public(const Boundary& b, const PairJob& job, int chunks, int ptype,
-                                 cudaStream_t st);
 
 // ---------------------------------------------------------------- slit maps (slitmap.cu)
 int slit_data(int m1, int n, const double2* et, double2 alpha, const double* theta, int bounded, double2* A,

@@ -1999,11 +1999,6 @@ int pair_component_needed(const Boundary& b, const PairJob& job) {
     return 0;
 }
 
-cudaError_t launch_reduce_public(const Boundary& b, const PairJob& job, int chunks, int ptype,
-                                 cudaStream_t st) {
-    return launch_reduce(b, job, chunks, ptype, st);
-}
-
 int run_pairsum(const Boundary& b, const PairJob& job, int precision, cudaStream_t st) {
     if (precision == GNK_PREC_FMM) return run_fmm(b, job, st);
     GNK_TRY(run_job_sides(b, job, st));
